@@ -8,7 +8,8 @@ import subprocess
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB_PATH = os.path.join(HERE, "libbpd.so")
-SOURCES = ["bpd.cu", "noalloc.cu"]
+OBJ_DIR = os.path.join(HERE, "build")
+SOURCES = ["layer_stack.cu", "fused_layer.cu", "gemm_tc.cu", "bpd.cu", "noalloc.cu"]
 
 
 def _nvcc() -> str:
@@ -31,16 +32,25 @@ def build_library(force: bool = False, verbose: bool = False) -> str:
     """Build ``libbpd.so`` next to this file if it is missing or older than its sources."""
     if not force and not _stale():
         return LIB_PATH
-    cmd = [_nvcc(), "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
-           "-Xcompiler", "-fPIC", "-shared", "-o", LIB_PATH]
+    flags = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17", "-Xcompiler", "-fPIC"]
     if verbose:
-        cmd += ["-Xptxas", "-v"]
-    cmd += [os.path.join(CSRC, s) for s in SOURCES]
-    proc = subprocess.run(cmd, capture_output=True, text=True)
-    if proc.returncode != 0:
-        raise RuntimeError("nvcc failed:\n" + proc.stdout + proc.stderr)
-    if verbose:
-        print(proc.stderr)
+        flags += ["-Xptxas", "-v"]
+    os.makedirs(OBJ_DIR, exist_ok=True)
+    objs = [os.path.join(OBJ_DIR, s[:-3] + ".o") for s in SOURCES]
+    # one nvcc per translation unit, side by side
+    procs = [(s, subprocess.Popen([_nvcc(), *flags, "-c", "-o", o, os.path.join(CSRC, s)], stdout=subprocess.PIPE,
+                                  stderr=subprocess.STDOUT, text=True)) for s, o in zip(SOURCES, objs)]
+    for name, proc in procs:
+        out, _ = proc.communicate()
+        if proc.returncode != 0:
+            for _, other in procs:
+                other.kill()
+            raise RuntimeError(f"nvcc failed on {name}:\n{out}")
+        if verbose:
+            print(out)
+    link = subprocess.run([_nvcc(), *flags, "-shared", "-o", LIB_PATH, *objs], capture_output=True, text=True)
+    if link.returncode != 0:
+        raise RuntimeError("linking failed:\n" + link.stdout + link.stderr)
     return LIB_PATH
 
 

@@ -139,10 +139,11 @@ struct Arena {
 
 static int pages_per_row(const Config& c, int max_tgt) { return ceil_div(max_tgt + 1 + c.k_model, kPage); }
 
-// Sessions whose widest pass has more than 64 rows plan their projections for full token tiles.
-static int session_wide_ttiles(const Config& c, int B) {
+// Sessions whose widest pass has more than 16 rows run their projections in the wide kernel; the K splits are planned
+// for that many rows.  0: the few-row kernel.
+static int session_wide_rows(const Config& c, int B) {
   const int rmax = B * c.k_model;
-  return rmax > 64 ? tc::token_tiles(rmax) : 0;
+  return rmax > tc::kNarrowBN ? rmax : 0;
 }
 
 // Lays the session out; with base == nullptr only measures.
@@ -195,25 +196,16 @@ static size_t plan_session(const Config& c, int B, int max_src, int max_tgt, cha
   float* part_val = a.take<float>(tiles * R2);
   int* part_idx = a.take<int>(tiles * R2);
   unsigned* counters = a.take<unsigned>(ceil_div((int)R2, kRC) + 1);
-  // split-K workspace of the tensor-core projections: the largest any launch of this session can need
+  // split-K workspace of the few-row projection kernel: the largest any launch of this session can need
   size_t ws = 0, ncnt = 1;
-  if (c.dtype == 1) {
-    const int wide = session_wide_ttiles(c, B);
-    auto need = [&](int N, int K, size_t T, int z) {
-      ws = std::max(ws, tc::ws_floats(N, K, (int)T, z, wide));
-      ncnt = std::max(ncnt, tc::counters_needed(N, (int)T, z));
+  if (c.dtype == 1 && !session_wide_rows(c, B)) {
+    auto need = [&](int N, int K, int z) {
+      ws = std::max(ws, tc::ws_floats(N, K, z));
+      ncnt = std::max(ncnt, tc::counters_needed(N, z));
     };
     const int dd = c.d, ff = c.d_ff, fh = c.d_hidden, km = c.k_model;
-    for (size_t T : {Rmax, E}) {
-      need(3 * dd, dd, T, 1); need(dd, dd, T, 1); need(ff, dd, T, 1); need(dd, ff, T, 1); need(2 * dd, dd, T, 1);
-    }
-    for (int kh = 1; kh <= km; ++kh) {
-      need(kh * fh, dd, Rmax, 1); need(km * fh, dd, Rmax, 1);
-      need(kh * dd, km * fh, Rmax, 1);
-      if (wide) ws = std::max(ws, tc::ws_floats(kh * dd, km * fh, B, 1, 1, tc::kSlots));   // stage 2 of the lazy heads
-      need(dd, fh, Rmax, kh);
-    }
-    need(c.V, dd, R2, 1);
+    need(3 * dd, dd, 1); need(dd, dd, 1); need(ff, dd, 1); need(dd, ff, 1);
+    need(km * fh, dd, 1); need(km * dd, km * fh, 1); need(dd, fh, km);
   }
   float* tc_ws = a.take<float>(ws);
   unsigned* tc_counters = a.take<unsigned>(ncnt);
@@ -476,7 +468,7 @@ static tc::Scratch tc_scratch(bpd_session* s) {
   sc.ws = s->tc_ws; sc.ws_floats = s->tc_ws_floats; sc.tile_counters = s->tc_counters; sc.n_counters = s->tc_n_counters;
   sc.done_counter = s->tc_done; sc.best = s->tc_best; sc.best_elems = s->tc_best_elems;
   sc.error = s->st.error;
-  sc.wide_ttiles = session_wide_ttiles(s->m->cfg, s->B);
+  sc.wide_rows = session_wide_rows(s->m->cfg, s->B);
   sc.l2_hints = s->opt.l2_stream_hints;
   return sc;
 }
@@ -500,7 +492,8 @@ static int run_encoder_tc(bpd_session* s) {
   const Config& c = m->cfg;
   cudaStream_t st = s->stream;
   const int E = s->B * s->max_src, d = c.d, f = c.d_ff;
-  const tc::Scratch sc = tc_scratch(s);
+  tc::Scratch sc = tc_scratch(s);
+  sc.wide_rows = E;
   const bool pdl = s->use_pdl != 0;   // every kernel after the first may start while its predecessor ends
   EmbedParams ep;
   memset(&ep, 0, sizeof(ep));
@@ -556,11 +549,6 @@ static int run_encoder_tc(bpd_session* s) {
 }
 
 // ------------------------------------------------------------------ fused decoder layers (few rows per pass)
-template <typename P>
-static int fused_attr(void (*kernel)(P), size_t smem) {
-  return ensure_smem_limit(reinterpret_cast<const void*>(kernel), smem);
-}
-
 // Embedding, then three launches per decoder layer (self-attention block, cross-attention block, feed-forward
 // block); leaves the residual stream in s->x like the kernel-per-projection path.
 static int run_layers_fused(bpd_session* s, const PassArgs& a) {
@@ -581,26 +569,17 @@ static int run_layers_fused(bpd_session* s, const PassArgs& a) {
   const size_t smem_self = fused::attn_layout<true>(d, nt, s->B * s->ppr).total;
   const size_t smem_cross = fused::attn_layout<false>(d, nt, 0, s->B * cross_smax).total;
   const size_t smem_ffn = fused::ffn_layout(d, nt).total;
+  // every position the cache can hold (max_tgt + k + 1 of them) within kC chunks of 32: the short schedule only
+  const bool short_only = s->max_tgt + c.k_model + 1 <= fused::kC * 32;
+  const bool roomy = c.H * fused::kC <= 74;      // an attention launch leaves half the SMs free
+  const bool ffn_small = fused::kC * (c.d_ff / (fused::kC * fused::kHS)) <= 148;   // one CTA per SM is enough for the feed-forward launch
+  const void* k_self = fused::attn_kernel(true, nt, short_only ? 1 : 2, roomy ? 1 : 2);
+  const void* k_cross = fused::attn_kernel(false, nt, cross_smax > 0 ? 1 : 0, 2);
+  const void* k_ffn = fused::ffn_kernel(nt, ffn_small ? 2 : 3);
   // the opt-in shared-memory limit of each kernel grows with the widest model seen so far
-  {
-    BPD_TRY(fused_attr(fused::attn_block_kernel<true, 1, 1>, smem_self));
-    BPD_TRY(fused_attr(fused::attn_block_kernel<true, 2, 1>, smem_self));
-    BPD_TRY(fused_attr(fused::attn_block_kernel<true, 1, 2>, smem_self));
-    BPD_TRY(fused_attr(fused::attn_block_kernel<true, 2, 2>, smem_self));
-    BPD_TRY(fused_attr(fused::attn_block_kernel<true, 1, 2, 1>, smem_self));
-    BPD_TRY(fused_attr(fused::attn_block_kernel<true, 2, 2, 1>, smem_self));
-    BPD_TRY(fused_attr(fused::attn_block_kernel<false, 1, 1>, smem_cross));
-    BPD_TRY(fused_attr(fused::attn_block_kernel<false, 2, 1>, smem_cross));
-    if (nt == 1) {
-      BPD_TRY(fused_attr(fused::attn_block_kernel<false, 1>, smem_cross));
-      BPD_TRY(fused_attr(fused::ffn_block_kernel<1>, smem_ffn));
-      BPD_TRY(fused_attr(fused::ffn_block_kernel<1, 2>, smem_ffn));
-    } else {
-      BPD_TRY(fused_attr(fused::attn_block_kernel<false, 2>, smem_cross));
-      BPD_TRY(fused_attr(fused::ffn_block_kernel<2>, smem_ffn));
-      BPD_TRY(fused_attr(fused::ffn_block_kernel<2, 2>, smem_ffn));
-    }
-  }
+  BPD_TRY(ensure_smem_limit(k_self, smem_self));
+  BPD_TRY(ensure_smem_limit(k_cross, smem_cross));
+  BPD_TRY(ensure_smem_limit(k_ffn, smem_ffn));
   EmbedParams ep;
   memset(&ep, 0, sizeof(ep));
   ep.table = m->tgt_embed; ep.pe = s->pe; ep.npos = s->npos; ep.x = s->x; ep.rows = R; ep.rows_per_b = a.kcur;
@@ -635,29 +614,9 @@ static int run_layers_fused(bpd_session* s, const PassArgs& a) {
     pf.w1 = static_cast<const bf16*>(L.w1); pf.w2 = static_cast<const bf16*>(L.w2); pf.b2 = static_cast<const bf16*>(L.b2);
     pf.d = d; pf.ff = c.d_ff; pf.R = R; pf.NJ = (int)grid_ffn.y; pf.eps = c.eps;
     pf.ws = s->fused_ws; pf.counters = s->fused_counters; pf.all_done = done;
-    // every position the cache can hold (max_tgt + k + 1 of them) within kC chunks of 32: the short schedule only
-    const bool short_only = s->max_tgt + c.k_model + 1 <= fused::kC * 32;
-    const bool roomy = c.H * fused::kC <= 74;      // an attention launch leaves half the SMs free
-    const bool ffn_small = grid_ffn.x * grid_ffn.y <= 148;   // one CTA per SM is enough for the feed-forward launch
-    if (nt == 1) {
-      if (short_only) BPD_CUDA(launch_k(fused::attn_block_kernel<true, 1, 1>, grid_attn, block, smem_self, st, pdl, ps));
-      else if (roomy) BPD_CUDA(launch_k(fused::attn_block_kernel<true, 1, 2, 1>, grid_attn, block, smem_self, st, pdl, ps));
-      else BPD_CUDA(launch_k(fused::attn_block_kernel<true, 1, 2>, grid_attn, block, smem_self, st, pdl, ps));
-      if (cross_smax > 0) BPD_CUDA(launch_k(fused::attn_block_kernel<false, 1, 1>, grid_attn, block, smem_cross, st, pdl, pc));
-      else
-      BPD_CUDA(launch_k(fused::attn_block_kernel<false, 1>, grid_attn, block, smem_cross, st, pdl, pc));
-      if (ffn_small) BPD_CUDA(launch_k(fused::ffn_block_kernel<1, 2>, grid_ffn, block, smem_ffn, st, pdl, pf));
-      else BPD_CUDA(launch_k(fused::ffn_block_kernel<1>, grid_ffn, block, smem_ffn, st, pdl, pf));
-    } else {
-      if (short_only) BPD_CUDA(launch_k(fused::attn_block_kernel<true, 2, 1>, grid_attn, block, smem_self, st, pdl, ps));
-      else if (roomy) BPD_CUDA(launch_k(fused::attn_block_kernel<true, 2, 2, 1>, grid_attn, block, smem_self, st, pdl, ps));
-      else BPD_CUDA(launch_k(fused::attn_block_kernel<true, 2, 2>, grid_attn, block, smem_self, st, pdl, ps));
-      if (cross_smax > 0) BPD_CUDA(launch_k(fused::attn_block_kernel<false, 2, 1>, grid_attn, block, smem_cross, st, pdl, pc));
-      else
-      BPD_CUDA(launch_k(fused::attn_block_kernel<false, 2>, grid_attn, block, smem_cross, st, pdl, pc));
-      if (ffn_small) BPD_CUDA(launch_k(fused::ffn_block_kernel<2, 2>, grid_ffn, block, smem_ffn, st, pdl, pf));
-      else BPD_CUDA(launch_k(fused::ffn_block_kernel<2>, grid_ffn, block, smem_ffn, st, pdl, pf));
-    }
+    BPD_CUDA(launch_kc(k_self, grid_attn, block, smem_self, st, pdl, ps));
+    BPD_CUDA(launch_kc(k_cross, grid_attn, block, smem_cross, st, pdl, pc));
+    BPD_CUDA(launch_kc(k_ffn, grid_ffn, block, smem_ffn, st, pdl, pf));
     g_launches += 3;
     if (a.layer_dump)
       BPD_CUDA(cudaMemcpyAsync(a.layer_dump + (size_t)l * R * d, s->x, sizeof(float) * R * d, cudaMemcpyDeviceToDevice, st));
@@ -716,22 +675,10 @@ static bool stack_plan(const Config& c, int rows, int nb, int ppr, int cross_row
   return true;
 }
 
-// The persistent kernel's instantiations: token tiles (1 or 2 of 8 rows), reduction steps per panel (2: d_model 256,
-// else 4), CTAs per SM (1 or 2), lean (short sequences and staged encoder rows only).  `f` gets the kernel.
-template <typename F>
-static int stack_variant(int nt, int ksteps, int minb, bool lean, F&& f) {
-#define BPD_V(NT, KS, MB, LN) if (nt == NT && ksteps == KS && minb == MB && lean == LN) return f(stack::layer_stack_kernel<NT, KS, MB, LN>)
-  BPD_V(1, 2, 1, false); BPD_V(2, 2, 1, false); BPD_V(1, 4, 1, false); BPD_V(2, 4, 1, false);
-  BPD_V(1, 2, 2, false); BPD_V(2, 2, 2, false); BPD_V(1, 4, 2, false); BPD_V(2, 4, 2, false);
-  BPD_V(1, 2, 1, true); BPD_V(2, 2, 1, true); BPD_V(1, 4, 1, true); BPD_V(2, 4, 1, true);
-  BPD_V(1, 2, 2, true); BPD_V(2, 2, 2, true); BPD_V(1, 4, 2, true); BPD_V(2, 4, 2, true);
-#undef BPD_V
-  return fail(BPD_E_UNSUPPORTED, "no persistent layer kernel for %d token tiles, %d steps, %d CTAs per SM", nt, ksteps, minb);
-}
-
-template <typename K>
-static int stack_clusters(K kernel, size_t smem, int H, int* out) {
-  BPD_TRY(ensure_smem_limit(reinterpret_cast<const void*>(kernel), smem));
+// How many clusters of the given instantiation can be resident at once.
+static int stack_clusters(const void* kernel, size_t smem, int H, int* out) {
+  if (!kernel) return fail(BPD_E_UNSUPPORTED, "no such instantiation of the persistent layer kernel");
+  BPD_TRY(ensure_smem_limit(kernel, smem));
   cudaLaunchConfig_t cfg;
   memset(&cfg, 0, sizeof(cfg));
   cfg.gridDim = dim3(fused::kC, H); cfg.blockDim = dim3(stack::kThreads); cfg.dynamicSmemBytes = smem;
@@ -799,8 +746,8 @@ static int stack_setup(bpd_session* s) {
       const size_t sm = (size_t)lay.total;
       const bool lean = !long_seq && cross_rows > 0;
       const int ksteps = c.d == 256 ? 2 : 4, H = c.H;
-      BPD_TRY(stack_variant(1, ksteps, minb, lean, [&](auto kernel) { return stack_clusters(kernel, sm, H, &n1); }));
-      BPD_TRY(stack_variant(2, ksteps, minb, lean, [&](auto kernel) { return stack_clusters(kernel, sm, H, &n2); }));
+      BPD_TRY(stack_clusters(stack::kernel_for(1, ksteps, minb, lean), sm, H, &n1));
+      BPD_TRY(stack_clusters(stack::kernel_for(2, ksteps, minb, lean), sm, H, &n2));
       ok = n1 >= c.H && n2 >= c.H;
     }
     if (ok) break;
@@ -887,11 +834,9 @@ static int run_layers_stack(bpd_session* s, const PassArgs& a) {
   // reduction panels of 32 columns (two steps of 16) for d_model 256, else 64 (four steps); one or two CTAs per SM
   const int nt = p.R > 8 ? 2 : 1, ksteps = c.d == 256 ? 2 : 4;
   const bool lean = !s->stack_long && s->stack_cross_rows > 0;
-  cudaStream_t stream = s->stream;
-  BPD_TRY(stack_variant(nt, ksteps, s->stack_minb, lean, [&](auto kernel) {
-    BPD_CUDA(launch_k(kernel, grid, block, smem, stream, pdl, maps, p));
-    return (int)BPD_OK;
-  }));
+  const void* kernel = stack::kernel_for(nt, ksteps, s->stack_minb, lean);
+  if (!kernel) return fail(BPD_E_UNSUPPORTED, "no such instantiation of the persistent layer kernel");
+  BPD_CUDA(launch_kc(kernel, grid, block, smem, s->stream, pdl, maps, p));
   ++g_launches;
   return BPD_OK;
 }
@@ -918,8 +863,9 @@ static int run_pass_tc(bpd_session* s, const PassArgs& a) {
   ep.d = d; ep.vocab = c.V; ep.st = s->st; ep.forced = a.forced; ep.forced_rows = a.forced_rows;
   ep.kforced = a.kforced; ep.src = nullptr; ep.all_done = done;
   if (fold) { ep.gain = static_cast<const bf16*>(m->dec[0].ln1g); ep.xg_hi = static_cast<bf16*>(s->xn); ep.xg_plane = s->pl_xn; }
-  // passes of more than 16 rows: layer-norm statistics travel as per-tile partial results (see TcParams::stat_out)
-  const bool wide = fold && R > 16;
+  // sessions with passes of more than 16 rows: layer-norm statistics travel as per-tile partial results (see
+  // TcParams::stat_out)
+  const bool wide = fold && sc.wide_rows > 0;
   const int parts = d / 128;
   if (wide) { ep.stat_out = s->ln_stats; ep.stat_T = R; }
   auto stats_from = [&](tc::TcParams& q) { if (wide) { q.ln_x = nullptr; q.stat_in = s->ln_stats; q.stat_parts = parts; q.stat_T = R; } };
@@ -995,12 +941,15 @@ static int run_pass_tc(bpd_session* s, const PassArgs& a) {
   prof_mark(s, kProfHeadW1, 1);
   // output layers + shared vocabulary projection with a fused top-1 for T rows and kh heads
   // Sessions that evaluate the heads lazily never use head 1 of a launch over all heads, so there the output
-  // layers of head 1 alone (greedy passes, stage 1) are planned for their own size, and stage 2 (plan_tt = 1:
-  // one token tile) for its own; everywhere else every launch is planned for the full matrix, so that head 1
+  // layers of head 1 alone (greedy passes, stage 1) are planned for their own size, and stage 2 (one row per
+  // sequence) for its own; everywhere else every launch is planned for the full matrix, so that head 1
   // is the same sum whether it is evaluated alone or with the others.
-  const bool own_plan = s->lazy_heads != 0 && tc_scratch(s).wide_ttiles > 0;
+  const bool own_plan = s->lazy_heads != 0 && sc.wide_rows > 0;
+  // the vocabulary projection takes the wide kernel in every session: k x k rows in all, or (lazy heads) k
+  tc::Scratch sv = sc;
+  sv.wide_rows = s->B * c.k_model * (s->lazy_heads ? 1 : c.k_model);
   auto heads = [&](const void* u_planes, long long u_plane, int u_rows, const float* hres, int T, int kh, int* table_out,
-                   bool rank, float* logits, int plan_tt) -> int {
+                   bool rank, float* logits, int plan_rows) -> int {
     prof_mark(s, kProfHeadW2, 0);
     tc::Operands uo{m->head_w2, km * d, u_planes, u_plane, ldu, u_rows, ldu};
     tc::TcParams ph = tc_params(m->head_b2, 0, done);
@@ -1008,7 +957,7 @@ static int run_pass_tc(bpd_session* s, const PassArgs& a) {
     ph.h = hres; ph.d = d; ph.head_identity = c.p1_identity;
     if (c.head_layout == 0) {
       BPD_TRY(tc::launch<tc::kTcHeadOut>(uo, kh * d, km * fhd, T, ph, sc, st, 1, 0, 0, pdl, own_plan ? kh * d : km * d,
-                                         own_plan ? plan_tt : 0));
+                                         own_plan ? plan_rows : 0));
     } else {
       ph.zofs_n = d;
       BPD_TRY(tc::launch<tc::kTcHeadOut>(uo, d, fhd, T, ph, sc, st, kh, d, fhd, pdl));
@@ -1025,7 +974,7 @@ static int run_pass_tc(bpd_session* s, const PassArgs& a) {
       ++g_launches;
       pv.rank = s->rank; pv.rank_kh = kh;
     }
-    BPD_TRY(tc::launch<tc::kTcArgmax>(oo, c.V, d, T * kh, pv, sc, st, 1, 0, 0, pdl)); ++g_launches;
+    BPD_TRY(tc::launch<tc::kTcArgmax>(oo, c.V, d, T * kh, pv, sv, st, 1, 0, 0, pdl)); ++g_launches;
     prof_mark(s, kProfVocab, 1);
     return BPD_OK;
   };
@@ -1043,7 +992,7 @@ static int run_pass_tc(bpd_session* s, const PassArgs& a) {
                     s->st, s->B, a.kcur, done};
     launch_k(gather_selected_kernel, dim3(s->B, 16), dim3(256), 0, st, pdl, gp);
     ++g_launches;
-    BPD_TRY(heads(s->u2, s->pl_u2, s->B, s->h2, s->B, a.kh, s->table2, false, nullptr, 1));
+    BPD_TRY(heads(s->u2, s->pl_u2, s->B, s->h2, s->B, a.kh, s->table2, false, nullptr, s->B));
     SelectParams sp{s->st, s->st.table, s->table2, s->table_full, s->B, a.kcur, a.kh, a.knext, done};
     launch_k(select_next_kernel, dim3(1), dim3(32 * ceil_div(s->B, 32)), 0, st, pdl, sp);
     ++g_launches;
@@ -1654,27 +1603,6 @@ int bpd_fetch_output(bpd_session* s, int max_new, int32_t* out_ids, int32_t* out
   return fetch(s, max_new, out_ids, out_len, stats, ms);
 }
 
-#ifdef BPD_STACK_TRACE
-// Development builds only: where the persistent layer kernel writes its per-CTA step timestamps (device memory,
-// clusters * 8 * 256 unsigned 64-bit words), or null to stop.
-int bpd_debug_set_stack_trace(void* dev_buffer) {
-  unsigned long long* ptr = static_cast<unsigned long long*>(dev_buffer);
-  BPD_CUDA(cudaMemcpyToSymbol(stack::g_stack_trace, &ptr, sizeof(ptr)));
-
-  return BPD_OK;
-}
-#endif
-
-#ifdef BPD_TC_TRACE
-// Development builds only: where the projection kernel writes its per-CTA step timestamps (4096 * 16 unsigned 64-bit
-// words of device memory), or null to stop.
-int bpd_debug_set_tc_trace(void* dev_buffer) {
-  unsigned long long* ptr = static_cast<unsigned long long*>(dev_buffer);
-  BPD_CUDA(cudaMemcpyToSymbol(tc::g_tc_trace, &ptr, sizeof(ptr)));
-  return BPD_OK;
-}
-#endif
-
 // ------------------------------------------------------------------ self test of the bounded waits
 int bpd_debug_wait_timeout(int32_t* dev_word, int limit_us, void* cuda_stream) {
   if (!dev_word) return fail(BPD_E_INVALID, "device word is null");
@@ -1703,25 +1631,16 @@ int bpd_debug_wait_timeout(int32_t* dev_word, int limit_us, void* cuda_stream) {
 }
 
 // ------------------------------------------------------------------ single operators
-// Scratch layout of the bf16 (tensor-core) operators: a zero "lo" plane for the caller's single-plane bf16
-// activations, the split-K workspace, tile counters, the top-1 merge counter and partials, an error word.
+// Scratch layout of the bf16 (tensor-core) operators: the top-1 keys, the merge counter and an error word.
 struct OpScratch {
-  size_t zero_off, ws_off, cnt_off, done_off, pv_off, pi_off, err_off, total;
-  size_t ws_floats, n_counters, part_elems;
+  size_t best_off, done_off, err_off, total;
 };
-static OpScratch op_scratch_layout(int rows, int in_f, int out_f) {
+static OpScratch op_scratch_layout(int rows, bool top1) {
   OpScratch o;
   size_t off = 0;
   auto take = [&](size_t bytes) { size_t at = off; off = align_up(off + bytes); return at; };
-  o.ws_floats = tc::ws_floats(out_f, in_f, rows, 1);
-  o.n_counters = tc::counters_needed(out_f, rows, 1);
-  o.part_elems = (size_t)rows;
-  o.zero_off = take((size_t)rows * in_f * sizeof(bf16));
-  o.ws_off = take(o.ws_floats * sizeof(float));
-  o.cnt_off = take(o.n_counters * sizeof(unsigned));
+  o.best_off = take(top1 ? (size_t)rows * tc::kBestStride * sizeof(unsigned long long) : 0);
   o.done_off = take(sizeof(unsigned));
-  o.pv_off = take(o.part_elems * tc::kBestStride * sizeof(unsigned long long));
-  o.pi_off = o.pv_off;
   o.err_off = take(sizeof(int));
   o.total = off;
   return o;
@@ -1738,7 +1657,7 @@ static int op_tc_finish(char* scratch, const OpScratch& L, cudaStream_t st) {
 
 size_t bpd_op_vocab_argmax_scratch_bytes(int rows, int d, int vocab, int dtype) {
   if (rows < 1 || vocab < 1 || d < 1) return 0;
-  if (op_use_tc(dtype)) return op_scratch_layout(rows, d, vocab).total;
+  if (op_use_tc(dtype)) return op_scratch_layout(rows, true).total;
   const size_t tiles = ceil_div(vocab, kVocTile);
   return align_up(tiles * rows * sizeof(float)) + align_up(tiles * rows * sizeof(int)) +
          align_up((ceil_div(rows, kRC) + 1) * sizeof(unsigned));
@@ -1754,12 +1673,11 @@ int bpd_op_vocab_argmax(const void* x, const void* w, int rows, int d, int vocab
   cudaStream_t st = (cudaStream_t)cuda_stream;
   char* p = static_cast<char*>(scratch);
   if (op_use_tc(dtype)) {
-    const OpScratch L = op_scratch_layout(rows, d, vocab);
+    const OpScratch L = op_scratch_layout(rows, true);
     BPD_CUDA(cudaMemsetAsync(p, 0, L.total, st));
-    tc::Scratch sc{reinterpret_cast<float*>(p + L.ws_off), L.ws_floats, reinterpret_cast<unsigned*>(p + L.cnt_off),
-                   L.n_counters, reinterpret_cast<unsigned*>(p + L.done_off),
-                   reinterpret_cast<unsigned long long*>(p + L.pv_off), L.part_elems, reinterpret_cast<int*>(p + L.err_off), 0, 1};
-    tc::Operands op{w, vocab, x, 0, d, rows, d, p + L.zero_off};   // the lo plane is the scratch's zero block
+    tc::Scratch sc{nullptr, 0, nullptr, 0, reinterpret_cast<unsigned*>(p + L.done_off), reinterpret_cast<unsigned long long*>(p + L.best_off),
+                   (size_t)rows, reinterpret_cast<int*>(p + L.err_off), rows, 1};
+    tc::Operands op{w, vocab, x, 0, d, rows, d};   // one plane
     tc::TcParams tp;
     memset(&tp, 0, sizeof(tp));
     tp.out_idx = out_idx; tp.out_val = out_val;
@@ -1783,7 +1701,7 @@ int bpd_op_vocab_argmax(const void* x, const void* w, int rows, int d, int vocab
 
 size_t bpd_op_linear_scratch_bytes(int rows, int in_f, int out_f, int dtype) {
   if (rows < 1 || in_f < 1 || out_f < 1) return 0;
-  if (op_use_tc(dtype)) return op_scratch_layout(rows, in_f, out_f).total;
+  if (op_use_tc(dtype)) return op_scratch_layout(rows, false).total;
   return 256;
 }
 
@@ -1796,14 +1714,13 @@ int bpd_op_linear(const void* x, const void* w, const void* bias, int rows, int 
   cudaStream_t st = (cudaStream_t)cuda_stream;
   if (op_use_tc(dtype)) {
     if (!scratch || (uintptr_t)scratch % 256) return fail(BPD_E_INVALID, "scratch is null or misaligned");
-    const OpScratch L = op_scratch_layout(rows, in_f, out_f);
+    const OpScratch L = op_scratch_layout(rows, false);
     if (scratch_bytes < L.total) return fail(BPD_E_NOMEM, "scratch too small");
     char* p = static_cast<char*>(scratch);
     BPD_CUDA(cudaMemsetAsync(p, 0, L.total, st));
-    tc::Scratch sc{reinterpret_cast<float*>(p + L.ws_off), L.ws_floats, reinterpret_cast<unsigned*>(p + L.cnt_off),
-                   L.n_counters, reinterpret_cast<unsigned*>(p + L.done_off),
-                   reinterpret_cast<unsigned long long*>(p + L.pv_off), L.part_elems, reinterpret_cast<int*>(p + L.err_off), 0, 1};
-    tc::Operands op{w, out_f, x, 0, in_f, rows, in_f, p + L.zero_off};   // the lo plane is the scratch's zero block
+    tc::Scratch sc{nullptr, 0, nullptr, 0, reinterpret_cast<unsigned*>(p + L.done_off), reinterpret_cast<unsigned long long*>(p + L.best_off),
+                   (size_t)rows, reinterpret_cast<int*>(p + L.err_off), rows, 1};
+    tc::Operands op{w, out_f, x, 0, in_f, rows, in_f};   // one plane
     tc::TcParams tp;
     memset(&tp, 0, sizeof(tp));
     tp.bias = static_cast<const bf16*>(bias); tp.relu = relu; tp.out_f32 = y; tp.ldo = out_f;

@@ -936,5 +936,9 @@ __host__ inline bool supported(int d, int H, int ff, int rows) {
          rows * (d / kC) <= 8 * kThreads;   // planes: at most two groups of four columns per thread
 }
 
+// The instantiations above by their properties (fused_layer.cu); null if there is none.
+const void* attn_kernel(bool self, int nt, int lean, int minb);
+const void* ffn_kernel(int nt, int minb);
+
 }  // namespace fused
 }  // namespace bpd

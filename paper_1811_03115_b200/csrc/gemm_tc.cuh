@@ -42,7 +42,7 @@ constexpr int kBM = 128;          // features per tile (MMA M)
 constexpr int kBK = 64;           // K elements per pipeline stage (128 bytes of bf16: one swizzle row)
 constexpr int kMaxStages = 4;     // pipeline depth is chosen per launch (2..4) so that two CTAs fit on an SM when possible
 constexpr int kThreads = 192;     // warp 0: TMA, warp 1: MMA + tensor-memory allocation, warps 2-5: epilogue
-constexpr int kMaxBN = 128;       // tokens per CTA (MMA N), a multiple of 16
+constexpr int kMaxBN = 16;        // tokens per CTA (MMA N); wider launches take gemm_wide.cuh
 // Words between the top-1 keys of successive tokens: every key has a 128-byte line of its own.  Hundreds of
 // tiles send one atomic max per token; keys that share a line queue behind one another in L2.
 constexpr int kBestStride = 16;
@@ -208,33 +208,12 @@ __device__ __forceinline__ float unpack_value(unsigned long long key) {
   return __uint_as_float((ord & 0x80000000u) ? (ord & 0x7fffffffu) : ~ord);
 }
 
-// Warp-wide (value, index) maximum with ties to the lower index, for lanes whose indices grow with the lane
-// number: one integer max-reduction on the orderable pattern of the value, one ballot for the first lane that
-// holds it -- instead of a five-level shuffle butterfly on two registers.
-__device__ __forceinline__ void warp_argmax_lanes(float& v, int& idx) {
-  const unsigned b = __float_as_uint(v);
-  const unsigned ord = (b & 0x80000000u) ? ~b : (b | 0x80000000u);
-  const unsigned m = __reduce_max_sync(0xffffffffu, ord);
-  const int src = __ffs(__ballot_sync(0xffffffffu, ord == m)) - 1;
-  idx = __shfl_sync(0xffffffffu, idx, src);
-  v = __uint_as_float((m & 0x80000000u) ? (m & 0x7fffffffu) : ~m);
-}
-
 // Arrival on a device-wide counter with release (our earlier writes, and those of the CTA's other threads
 // ordered before us by the barrier, become visible) and acquire (we see what earlier arrivals released).
 __device__ __forceinline__ unsigned atom_add_acq_rel(unsigned* addr, unsigned v) {
   unsigned old;
   asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], %2;" : "=r"(old) : "l"(addr), "r"(v) : "memory");
   return old;
-}
-
-// Top-n acceptance: among this warp's 32 features, how many beat the proposal that follows token t's position.
-__device__ __forceinline__ void count_beats(const TcParams& p, int t, int n, float x, int lane) {
-  if (!p.rank.cnt || t >= p.T || (t % p.rank_kh) != 0) return;   // uniform over the warp
-  const int pr = t / p.rank_kh, tok = p.rank.tok[pr];
-  const bool beat = tok >= 0 && n < p.N && n != tok && better(x, n, p.rank.thr[pr], tok);
-  const unsigned m = __ballot_sync(0xffffffffu, beat);
-  if (lane == 0 && m) atomicAdd(&p.rank.cnt[pr], __popc(m));
 }
 
 __device__ __forceinline__ void split_bf16(float v, bf16& hi, bf16& lo) {
@@ -244,7 +223,7 @@ __device__ __forceinline__ void split_bf16(float v, bf16& hi, bf16& lo) {
 
 // Shared-memory footprint of one CTA.
 __host__ __device__ inline size_t stage_bytes(int bn) { return (size_t)kBM * 128 + 2 * (size_t)bn * 128; }
-__host__ __device__ inline int stages_for(int bn) { return bn <= 16 ? 5 : (bn <= 32 ? 4 : (bn <= 64 ? 3 : 4)); }
+__host__ __device__ inline int stages_for(int) { return 5; }
 __host__ __device__ inline size_t smem_bytes(int bn) { return stages_for(bn) * stage_bytes(bn) + 1024 /*alignment*/ + 256; }
 
 // ---------------------------------------------------------------- final epilogue for one (feature, token)
@@ -317,226 +296,6 @@ __device__ __forceinline__ void tc_store8(const TcParams& p, int z, int t_first,
   }
 }
 
-// ---------------------------------------------------------------- final epilogue of a wide tile
-// The tile lies in shared memory with one row per token (row stride tstride floats, a multiple of 4).  An item is
-// (token, four consecutive features); the 128 epilogue threads take the items in order, so a warp finishes 128
-// consecutive features of a token with one 16-byte (fp32) or 8-byte (bf16) access per lane instead of 32-lane
-// scalar stores per token.  Same arithmetic per element as tc_store8 (no folded layer norm here).
-__device__ __forceinline__ uint2 pack4_bf16(const bf16 (&b)[4]) {
-  return make_uint2((uint32_t)__bfloat16_as_ushort(b[0]) | ((uint32_t)__bfloat16_as_ushort(b[1]) << 16),
-                    (uint32_t)__bfloat16_as_ushort(b[2]) | ((uint32_t)__bfloat16_as_ushort(b[3]) << 16));
-}
-// A 16-byte load from L2 that stays where it is written: the compiler otherwise sinks such loads to their first use,
-// which turns a batch of independent loads into a chain of round trips.
-__device__ __forceinline__ float4 ld_cg_v4_here(const float* ptr) {
-  float4 v;
-  asm volatile("ld.global.cg.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(ptr) : "memory");
-  return v;
-}
-
-// Per-thread constants of an item's four features.
-struct FinishCtx {
-  float bias[4], gn[4], lns[4];
-  bool folded;     // y = rstd * (acc - mean * ln_s) + ln_c; ln_c holds the bias
-  int n, g;
-};
-template <int EPI>
-__device__ __forceinline__ bool tc_finish_setup(const TcParams& p, int z, int tile, int et, FinishCtx& c) {
-  c.g = et & 31;
-  c.n = tile * kBM + c.g * 4;                       // first of this item's four features (within the slice)
-  if (c.n >= p.N) return false;
-#pragma unroll
-  for (int e = 0; e < 4; ++e) { c.bias[e] = 0.f; c.gn[e] = 0.f; c.lns[e] = 0.f; }
-  c.folded = (p.stat_in != nullptr);
-  if (c.folded) {
-    const float4 s4 = *reinterpret_cast<const float4*>(p.ln_s + c.n), c4 = *reinterpret_cast<const float4*>(p.ln_c + c.n);
-    c.lns[0] = s4.x; c.lns[1] = s4.y; c.lns[2] = s4.z; c.lns[3] = s4.w;
-    c.bias[0] = c4.x; c.bias[1] = c4.y; c.bias[2] = c4.z; c.bias[3] = c4.w;
-  } else if (p.bias) {
-    const uint2 bw = *reinterpret_cast<const uint2*>(p.bias + c.n + p.zofs_n * z);
-    c.bias[0] = __uint_as_float(bw.x << 16); c.bias[1] = __uint_as_float(bw.x & 0xffff0000u);
-    c.bias[2] = __uint_as_float(bw.y << 16); c.bias[3] = __uint_as_float(bw.y & 0xffff0000u);
-  }
-  if (EPI == kTcResidual && p.g_next) {
-    const uint2 gw = *reinterpret_cast<const uint2*>(p.g_next + c.n);
-    c.gn[0] = __uint_as_float(gw.x << 16); c.gn[1] = __uint_as_float(gw.x & 0xffff0000u);
-    c.gn[2] = __uint_as_float(gw.y << 16); c.gn[3] = __uint_as_float(gw.y & 0xffff0000u);
-  }
-  return true;
-}
-// Finishes one item: token t (row tr of the tile), features c.n .. c.n + 3, accumulated values a; `old` is the
-// residual stream's current content (only read by the caller when the new value is needed: residual with g_next).
-template <int EPI>
-__device__ __forceinline__ void tc_finish_item(const TcParams& p, const FinishCtx& c, int z, int t, int tr, const float4& a,
-                                               float4& old, const unsigned long long* s_slot, const float* s_mean,
-                                               const float* s_rstd) {
-  const int n = c.n;
-  float v[4] = {a.x + c.bias[0], a.y + c.bias[1], a.z + c.bias[2], a.w + c.bias[3]};
-  if (c.folded) {
-    const float mu = s_mean[tr], rs = s_rstd[tr];
-    v[0] = rs * (a.x - mu * c.lns[0]) + c.bias[0]; v[1] = rs * (a.y - mu * c.lns[1]) + c.bias[1];
-    v[2] = rs * (a.z - mu * c.lns[2]) + c.bias[2]; v[3] = rs * (a.w - mu * c.lns[3]) + c.bias[3];
-  }
-  if (p.relu) {
-#pragma unroll
-    for (int e = 0; e < 4; ++e) v[e] = fmaxf(v[e], 0.f);
-  }
-  if (EPI == kTcPlanes || EPI == kTcHeadOut) {
-    const int nz = n + p.zofs_n * z;
-    if (EPI == kTcHeadOut) {
-      const float4 h = __ldg(reinterpret_cast<const float4*>(p.h + (size_t)t * p.d + (n % p.d)));
-      const float pre[4] = {h.x, h.y, h.z, h.w};
-#pragma unroll
-      for (int e = 0; e < 4; ++e) v[e] = (p.head_identity && nz < p.d) ? pre[e] : v[e] + pre[e];
-    }
-    bf16 hi[4], lo[4];
-#pragma unroll
-    for (int e = 0; e < 4; ++e) split_bf16(v[e], hi[e], lo[e]);
-    const long long o = (long long)t * p.ldo + nz;
-    *reinterpret_cast<uint2*>(p.out_hi + o) = pack4_bf16(hi);
-    *reinterpret_cast<uint2*>(p.out_hi + o + p.plane) = pack4_bf16(lo);
-  } else if (EPI == kTcF32) {
-    *reinterpret_cast<float4*>(p.out_f32 + (long long)t * p.ldo + n) = make_float4(v[0], v[1], v[2], v[3]);
-  } else if (EPI == kTcResidual) {
-    float4* xp = reinterpret_cast<float4*>(p.out_f32 + (long long)t * p.ldo + n);
-    if (!p.g_next) {
-      // one writer per element: x += v as a 16-byte reduction, nothing to read back
-      asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(xp), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]) : "memory");
-      return;
-    }
-    const float xn[4] = {old.x + v[0], old.y + v[1], old.z + v[2], old.w + v[3]};
-    *xp = make_float4(xn[0], xn[1], xn[2], xn[3]);
-    {
-      bf16 hi[4], lo[4];
-#pragma unroll
-      for (int e = 0; e < 4; ++e) split_bf16(xn[e] * c.gn[e], hi[e], lo[e]);
-      *reinterpret_cast<uint2*>(p.xg_hi + (long long)t * p.ldo + n) = pack4_bf16(hi);
-      *reinterpret_cast<uint2*>(p.xg_hi + (long long)t * p.ldo + n + p.xg_plane) = pack4_bf16(lo);
-    }
-    old = make_float4(xn[0], xn[1], xn[2], xn[3]);   // handed back for the per-tile statistics
-  } else if (EPI == kTcQkv) {
-    const int d = p.d;
-    if (n < d) {
-      *reinterpret_cast<float4*>(p.out_f32 + (long long)t * p.ldo + n) = make_float4(v[0], v[1], v[2], v[3]);
-    } else {
-      const bf16 b4[4] = {__float2bfloat16_rn(v[0]), __float2bfloat16_rn(v[1]), __float2bfloat16_rn(v[2]), __float2bfloat16_rn(v[3])};
-      bf16* dst = (n < 2 * d) ? p.kcache + s_slot[tr] + (n - d) : p.vcache + s_slot[tr] + (n - 2 * d);
-      *reinterpret_cast<uint2*>(dst) = pack4_bf16(b4);
-    }
-  }
-}
-// Per-tile statistics of TB tokens at once (kTcResidual with stat_out): the warp holds the tile's 128 new values of
-// each token, four per lane (N is a multiple of 128 here: every lane is live).  Sums of deviations from the token's
-// first value in the tile, and of their squares, are reduced for all TB tokens together so that the shuffles of one
-// token hide behind those of the others; mean and squared deviations about the mean follow exactly from the two.
-template <int TB>
-__device__ __forceinline__ void tc_tile_stats(const TcParams& p, const FinishCtx& c, int t0, int tb, int nt, const float4 (&xn)[TB]) {
-  float s1[TB], s2[TB], pivot[TB];
-#pragma unroll
-  for (int i = 0; i < TB; ++i) {
-    pivot[i] = __shfl_sync(0xffffffffu, xn[i].x, 0);
-    const float d0 = xn[i].x - pivot[i], d1 = xn[i].y - pivot[i], d2 = xn[i].z - pivot[i], d3 = xn[i].w - pivot[i];
-    s1[i] = (d0 + d1) + (d2 + d3);
-    s2[i] = (d0 * d0 + d1 * d1) + (d2 * d2 + d3 * d3);
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-#pragma unroll
-    for (int i = 0; i < TB; ++i) {
-      s1[i] += __shfl_xor_sync(0xffffffffu, s1[i], o);
-      s2[i] += __shfl_xor_sync(0xffffffffu, s2[i], o);
-    }
-  }
-  if (c.g == 0) {
-#pragma unroll
-    for (int i = 0; i < TB; ++i) {
-      const int tr = tb + 4 * i;
-      if (tr < nt) {
-        const float dm = s1[i] * (1.0f / kBM);              // mean - pivot
-        reinterpret_cast<float2*>(p.stat_out)[(size_t)(c.n / kBM) * p.stat_T + t0 + tr] =
-            make_float2(pivot[i] + dm, fmaxf(s2[i] - s1[i] * dm, 0.f));
-      }
-    }
-  }
-}
-
-// The complete tile lies in shared memory (one row per token).  Warp w of the four takes tokens w, w + 4, ...; four
-// tokens are in flight per lane so that the loads of the old residual values overlap.
-template <int EPI>
-__device__ __forceinline__ void tc_finish_tile(const TcParams& p, int z, int t0, int nt, int tile, const float* s_t, int tstride,
-                                               const unsigned long long* s_slot, int et, const float* s_mean,
-                                               const float* s_rstd) {
-  FinishCtx c;
-  if (!tc_finish_setup<EPI>(p, z, tile, et, c)) return;
-  const bool need_old = (EPI == kTcResidual) && p.g_next != nullptr;
-  constexpr int TB = 4;
-  for (int tb = et >> 5; tb < nt; tb += 4 * TB) {
-    float4 old[TB];
-#pragma unroll
-    for (int i = 0; i < TB; ++i) {
-      const int tr = tb + 4 * i;
-      old[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (need_old && tr < nt) old[i] = ld_cg_v4_here(p.out_f32 + (long long)(t0 + tr) * p.ldo + c.n);
-    }
-#pragma unroll
-    for (int i = 0; i < TB; ++i) {
-      const int tr = tb + 4 * i;
-      if (tr < nt) {
-        const float4 a = *reinterpret_cast<const float4*>(s_t + tr * tstride + c.g * 4);
-        tc_finish_item<EPI>(p, c, z, t0 + tr, tr, a, old[i], s_slot, s_mean, s_rstd);
-      }
-    }
-    if (EPI == kTcResidual && p.stat_out) tc_tile_stats<TB>(p, c, t0, tb, nt, old);
-  }
-}
-// The tile is the sum of `splits` partial tiles in the workspace ([split][token][128 features]): the CTA that
-// arrived last adds them in split order and finishes the items straight from registers -- TB tokens x up to four
-// splits of 16-byte loads (and the old residual values) are in flight per lane.
-template <int EPI, int TB>
-__device__ __forceinline__ void tc_merge_finish_tile(const TcParams& p, int z, int t0, int nt, int tile, const float* wsz, int bn,
-                                                     const unsigned long long* s_slot, int et, const float* s_mean,
-                                                     const float* s_rstd) {
-  FinishCtx c;
-  if (!tc_finish_setup<EPI>(p, z, tile, et, c)) return;
-  const bool need_old = (EPI == kTcResidual) && p.g_next != nullptr;
-  constexpr int SB = 16 / TB;                       // 16 partial loads in flight
-  if (et == 0) BPD_TC_STAMP(8);
-  for (int tb = et >> 5; tb < nt; tb += 4 * TB) {
-    float4 old[TB], acc[TB];
-#pragma unroll
-    for (int i = 0; i < TB; ++i) {
-      const int tr = tb + 4 * i;
-      old[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-      acc[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (need_old && tr < nt) old[i] = ld_cg_v4_here(p.out_f32 + (long long)(t0 + tr) * p.ldo + c.n);
-    }
-    for (int s0 = 0; s0 < p.splits; s0 += SB) {
-      float4 v[SB][TB];
-#pragma unroll
-      for (int ss = 0; ss < SB; ++ss)
-#pragma unroll
-        for (int i = 0; i < TB; ++i) {
-          const int tr = tb + 4 * i;
-          v[ss][i] = (s0 + ss < p.splits && tr < nt) ? ld_cg_v4_here(wsz + ((size_t)(s0 + ss) * bn + tr) * kBM + c.g * 4)
-                                                      : make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-#pragma unroll
-      for (int ss = 0; ss < SB; ++ss)
-#pragma unroll
-        for (int i = 0; i < TB; ++i) {
-          acc[i].x += v[ss][i].x; acc[i].y += v[ss][i].y; acc[i].z += v[ss][i].z; acc[i].w += v[ss][i].w;
-        }
-    }
-#pragma unroll
-    for (int i = 0; i < TB; ++i) {
-      const int tr = tb + 4 * i;
-      if (tr < nt) tc_finish_item<EPI>(p, c, z, t0 + tr, tr, acc[i], old[i], s_slot, s_mean, s_rstd);
-    }
-    if (EPI == kTcResidual && p.stat_out) tc_tile_stats<TB>(p, c, t0, tb, nt, old);
-  }
-  if (et == 0) BPD_TC_STAMP(12);
-}
-
 // ---------------------------------------------------------------- bounded-wait self test
 // One CTA waits on an mbarrier that nothing ever arrives on, gives up after `limit_cycles`, records the same
 // error code the projection kernel would and returns normally: the context stays usable.
@@ -550,29 +309,20 @@ static __global__ void wait_probe_kernel(int* error, unsigned long long limit_cy
   }
 }
 
-// Top-1 epilogue: threads that share a token (a power of two, at most 8, with tpt * bn <= 128).
-__host__ __device__ inline int topk_threads_per_token(int bn) { return bn <= 16 ? 8 : (bn <= 32 ? 4 : (bn <= 64 ? 2 : 1)); }
-
 // ---------------------------------------------------------------- epilogue of one (tile, split) unit
-// Shared by the one-shot projection kernel and the persistent layer kernel.  Called by the four epilogue warps
-// (128 threads, named barrier 1).
+// Called by the four epilogue warps (128 threads, named barrier 1).
 struct EpiShared {
-  float* s_t;                   // top-1: the tile transposed, [token][128 features], rows of topk_stride() floats
   float* s_mean; float* s_rstd;
   unsigned long long* s_slot;
-  volatile uint32_t* ctl;       // [1] reduces the tile, [2] merges the top-1, [3] accumulator arrived
+  volatile uint32_t* ctl;       // [1] reduces the tile, [3] accumulator arrived
 };
 struct EpiUnit {
   uint32_t tmem, acc_bar, acc_parity;
-  int tile, split, slice, zidx, ntiles, zcount, t0, nt, bn, nchunks;
+  int tile, split, slice, zidx, ntiles, t0, nt, bn, nchunks;
   bool skip;
 };
-// WIDE: the launch has token tiles of 32 or more tokens.  Everything that only such tiles use (the way out through
-// shared memory, per-tile statistics, the merge that finishes items from registers) is compiled into that variant
-// alone, so that the few-row launches of the weight-streaming kernels carry none of it.
-template <int EPI, bool WIDE>
+template <int EPI>
 __device__ __forceinline__ void tc_epilogue(const TcParams& p, const EpiShared& sh, const EpiUnit& u, int warp, int lane) {
-  float* s_t = sh.s_t;
   float* s_mean = sh.s_mean;
   float* s_rstd = sh.s_rstd;
   unsigned long long* s_slot = sh.s_slot;
@@ -584,42 +334,12 @@ __device__ __forceinline__ void tc_epilogue(const TcParams& p, const EpiShared& 
   const int row = q * 32 + lane;
   const int n = tile * kBM + row;                  // feature index within the slice
   const int et = threadIdx.x - 64;                 // 0..127
-  const int tpt = topk_threads_per_token(bn), tstride = kBM + tpt;   // row stride = tpt mod 32: conflict-free scans
-  // the debug dump of the logits and the rank counting of top-n acceptance are rare: kept out of the common loops
-  const bool extras = (EPI == kTcArgmax) && (p.logits != nullptr || p.rank.cnt != nullptr);
-  // wide tiles of the other epilogues leave through shared memory too (see tc_finish_tile)
-  const bool vec = WIDE && (EPI != kTcArgmax) && p.vec && bn >= 32 && !p.ln_x;   // a folded layer norm on wide tiles comes with stat_in
-  constexpr int vstride = kBM + 4;
   if (EPI == kTcQkv && !skip && et < nt) {
     const int t = t0 + et;
     const int b = t / p.rows_per_b, i = t % p.rows_per_b;
     const int pos = p.st.len[b] + i;
     const int page = p.st.page_table[b * p.st.pages_per_row + pos / kPage];
     s_slot[et] = ((unsigned long long)page * kPage + (pos % kPage)) * p.d;
-  }
-  if (WIDE && p.stat_in && !skip && et < nt) {
-    // per-token statistics from the per-tile partial results of the kernel that wrote the stream: merged in
-    // tile order (pairwise update of mean and sum of squared deviations), the same for every consumer
-    const float2* sp = reinterpret_cast<const float2*>(p.stat_in) + (t0 + et);
-    float2 part[8];
-    float mean = 0.f, m2 = 0.f, cnt = 0.f;
-    for (int i0 = 0; i0 < p.stat_parts; i0 += 8) {
-#pragma unroll
-      for (int i = 0; i < 8; ++i)
-        if (i0 + i < p.stat_parts) part[i] = __ldcg(sp + (size_t)(i0 + i) * p.stat_T);
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        if (i0 + i < p.stat_parts) {
-          const float nb = (float)kBM, tot = cnt + nb;
-          const float delta = part[i].x - mean;
-          mean += delta * (nb / tot);
-          m2 += part[i].y + delta * delta * (cnt * nb / tot);
-          cnt = tot;
-        }
-      }
-    }
-    s_mean[et] = mean;
-    s_rstd[et] = rsqrtf(m2 / cnt + p.ln_eps);
   }
   if (p.ln_x && !skip) {
     // per-token mean and 1/std of the residual stream, computed while the main loop runs: 8 threads per
@@ -667,26 +387,11 @@ __device__ __forceinline__ void tc_epilogue(const TcParams& p, const EpiShared& 
       for (int cb = 0; cb < bn; cb += 16) {
         float v[16];
         tmem_ld16(tmem + ((uint32_t)(q * 32) << 16) + cb, v);
-        if (EPI != kTcArgmax && vec) {
-#pragma unroll
-          for (int c = 0; c < 16; ++c) s_t[(cb + c) * vstride + row] = v[c];
-        } else if (EPI != kTcArgmax) {
-          if (n < p.N) {
-            const float lo8[8] = {v[0], v[1], v[2], v[3], v[4], v[5], v[6], v[7]};
-            const float hi8[8] = {v[8], v[9], v[10], v[11], v[12], v[13], v[14], v[15]};
-            tc_store8<EPI>(p, slice, t0 + cb, min(8, nt - cb), n, lo8, s_mean, s_rstd, cb, s_slot);
-            tc_store8<EPI>(p, slice, t0 + cb + 8, min(8, nt - cb - 8), n, hi8, s_mean, s_rstd, cb + 8, s_slot);
-          }
-        } else {
-#pragma unroll
-          for (int c = 0; c < 16; ++c) s_t[(cb + c) * tstride + row] = (n < p.N) ? v[c] : -INFINITY;
-          if (extras) {
-#pragma unroll
-            for (int c = 0; c < 16; ++c) {
-              if (p.logits && cb + c < nt && n < p.N) p.logits[(size_t)(t0 + cb + c) * p.N + n] = v[c];
-              if (cb + c < nt) count_beats(p, t0 + cb + c, n, (n < p.N) ? v[c] : -INFINITY, lane);
-            }
-          }
+        if (n < p.N) {
+          const float lo8[8] = {v[0], v[1], v[2], v[3], v[4], v[5], v[6], v[7]};
+          const float hi8[8] = {v[8], v[9], v[10], v[11], v[12], v[13], v[14], v[15]};
+          tc_store8<EPI>(p, slice, t0 + cb, min(8, nt - cb), n, lo8, s_mean, s_rstd, cb, s_slot);
+          tc_store8<EPI>(p, slice, t0 + cb + 8, min(8, nt - cb - 8), n, hi8, s_mean, s_rstd, cb + 8, s_slot);
         }
       }
     } else {
@@ -713,123 +418,27 @@ __device__ __forceinline__ void tc_epilogue(const TcParams& p, const EpiShared& 
       if (ctl[1]) {
         // Splits are added in split order.  The partial tiles sit in L2 and every load is a round trip of about a
         // microsecond, so as many as the registers hold are issued together: G tokens x SB splits = 64 per thread.
-        auto emit8 = [&](const float (&acc)[8], int cg) {
-          if (EPI != kTcArgmax && vec) {
+        constexpr int G = 8, SB = 8;
+        for (int cg = 0; cg < nt; cg += G) {
+          float acc[G];
 #pragma unroll
-            for (int c = 0; c < 8; ++c)
-              if (cg + c < nt) s_t[(cg + c) * vstride + row] = acc[c];
-          } else if (EPI != kTcArgmax) {
-            if (n < p.N) tc_store8<EPI>(p, slice, t0 + cg, min(8, nt - cg), n, acc, s_mean, s_rstd, cg, s_slot);
-          } else {
+          for (int c = 0; c < G; ++c) acc[c] = 0.f;
+          for (int s0 = 0; s0 < p.splits; s0 += SB) {
+            float v[SB][G];
 #pragma unroll
-            for (int c = 0; c < 8; ++c)
-              if (cg + c < nt) s_t[(cg + c) * tstride + row] = (n < p.N) ? acc[c] : -INFINITY;
-            if (extras) {
+            for (int ss = 0; ss < SB; ++ss)
 #pragma unroll
-              for (int c = 0; c < 8; ++c) {
-                if (cg + c >= nt) break;
-                if (p.logits && n < p.N) p.logits[(size_t)(t0 + cg + c) * p.N + n] = acc[c];
-                count_beats(p, t0 + cg + c, n, (n < p.N) ? acc[c] : -INFINITY, lane);
-              }
-            }
+              for (int c = 0; c < G; ++c)
+                v[ss][c] = (s0 + ss < p.splits && cg + c < nt)
+                               ? __ldcg(&wsz[((size_t)(s0 + ss) * bn + cg + c) * kBM + row]) : 0.f;
+#pragma unroll
+            for (int ss = 0; ss < SB; ++ss)
+#pragma unroll
+              for (int c = 0; c < G; ++c) acc[c] += v[ss][c];
           }
-        };
-        auto merge = [&](auto g_tag, auto sb_tag) {
-          constexpr int G = decltype(g_tag)::value, SB = decltype(sb_tag)::value;
-          for (int cg = 0; cg < nt; cg += G) {
-            float acc[G];
-#pragma unroll
-            for (int c = 0; c < G; ++c) acc[c] = 0.f;
-            for (int s0 = 0; s0 < p.splits; s0 += SB) {
-              float v[SB][G];
-#pragma unroll
-              for (int ss = 0; ss < SB; ++ss)
-#pragma unroll
-                for (int c = 0; c < G; ++c)
-                  v[ss][c] = (s0 + ss < p.splits && cg + c < nt)
-                                 ? __ldcg(&wsz[((size_t)(s0 + ss) * bn + cg + c) * kBM + row]) : 0.f;
-#pragma unroll
-              for (int ss = 0; ss < SB; ++ss)
-#pragma unroll
-                for (int c = 0; c < G; ++c) acc[c] += v[ss][c];
-            }
-#pragma unroll
-            for (int g8 = 0; g8 < G; g8 += 8) {
-              if (cg + g8 < nt) {
-                const float a8[8] = {acc[g8], acc[g8 + 1], acc[g8 + 2], acc[g8 + 3], acc[g8 + 4], acc[g8 + 5], acc[g8 + 6], acc[g8 + 7]};
-                emit8(a8, cg + g8);
-              }
-            }
-          }
-        };
-        if (WIDE && EPI != kTcArgmax && vec) {
-          tc_merge_finish_tile<EPI, 4>(p, slice, t0, nt, tile, wsz, bn, s_slot, et, s_mean, s_rstd);
-        } else if (!WIDE || nt <= 8) merge(std::integral_constant<int, 8>{}, std::integral_constant<int, 8>{});
-        else if (p.splits <= 2) merge(std::integral_constant<int, 32>{}, std::integral_constant<int, 2>{});
-        else if (p.splits <= 4) merge(std::integral_constant<int, 16>{}, std::integral_constant<int, 4>{});
-        else merge(std::integral_constant<int, 8>{}, std::integral_constant<int, 8>{});
+          if (n < p.N) tc_store8<EPI>(p, slice, t0 + cg, min(8, nt - cg), n, acc, s_mean, s_rstd, cg, s_slot);
+        }
         if (et == 0) p.tile_counters[(size_t)u.zidx * ntiles + tile] = 0;   // ready for the next launch
-      }
-    }
-    if (WIDE && EPI != kTcArgmax && vec && direct) {
-      asm volatile("bar.sync 1, 128;" ::: "memory");
-      if (et == 0) BPD_TC_STAMP(8);
-      tc_finish_tile<EPI>(p, slice, t0, nt, tile, s_t, vstride, s_slot, et, s_mean, s_rstd);
-    }
-    if (EPI == kTcArgmax && (direct || ctl[1])) {
-      // The tile sits in shared memory with one row per token.  tpt threads share a token: each scans every
-      // tpt-th feature in ascending order (a strict comparison keeps the lowest index among equals), then the
-      // tpt partial results are merged with the same ordering.  No shuffle per token, no work for absent tokens.
-      // Then the CTA that completes the last tile merges all tiles.
-      asm volatile("bar.sync 1, 128;" ::: "memory");
-      {
-        const int token = et / tpt, part = et % tpt;            // tokens >= bn do not occur: tpt * bn <= 128
-        const float* rowp = s_t + token * tstride;
-        float x = -INFINITY;
-        int ix = 0x7fffffff;
-        if (token < nt) {
-          // four independent running maxima (features part + tpt * (4j + a)), merged by (value, lower index)
-          float xa[4];
-          int ia[4];
-#pragma unroll
-          for (int a = 0; a < 4; ++a) { ia[a] = part + tpt * a; xa[a] = rowp[ia[a]]; }
-          for (int f = part + 4 * tpt; f < kBM; f += 4 * tpt) {
-#pragma unroll
-            for (int a = 0; a < 4; ++a) {
-              const float y = rowp[f + tpt * a];
-              if (y > xa[a]) { xa[a] = y; ia[a] = f + tpt * a; }
-            }
-          }
-          x = xa[0];
-          ix = ia[0];
-#pragma unroll
-          for (int a = 1; a < 4; ++a)
-            if (better(xa[a], ia[a], x, ix)) { x = xa[a]; ix = ia[a]; }
-          ix = (tile * kBM + ix < p.N) ? tile * kBM + ix : 0x7fffffff;
-        }
-        for (int o = 1; o < tpt; o <<= 1) {                     // partners are neighbouring lanes of one warp
-          const float ov = __shfl_xor_sync(0xffffffffu, x, o);
-          const int oi = __shfl_xor_sync(0xffffffffu, ix, o);
-          if (better(ov, oi, x, ix)) { x = ov; ix = oi; }
-        }
-        // one 64-bit atomic max per (tile, token): larger value wins, equal values go to the lower index;
-        // max is order independent, so the result does not depend on which tile arrives first
-        if (token < nt && part == 0) atomicMax(&p.best[(size_t)(t0 + token) * kBestStride], pack_best(x, ix));
-      }
-      asm volatile("bar.sync 1, 128;" ::: "memory");
-      if (et == 0) {
-        const unsigned prev = atom_add_acq_rel(p.done_counter, 1u);
-        ctl[2] = (prev == (unsigned)(ntiles * u.zcount) - 1) ? 1u : 0u;
-      }
-      asm volatile("bar.sync 1, 128;" ::: "memory");
-      if (ctl[2]) {
-        for (int t = et; t < p.T; t += 128) {
-          const unsigned long long key = __ldcg(&p.best[(size_t)t * kBestStride]);
-          p.out_idx[t] = (int)(0xffffffffu - (unsigned)(key & 0xffffffffull));
-          if (p.out_val) p.out_val[t] = unpack_value(key);
-          p.best[(size_t)t * kBestStride] = 0ull;                       // ready for the next launch
-        }
-        if (et == 0) *p.done_counter = 0;
       }
     }
   }
@@ -838,7 +447,7 @@ __device__ __forceinline__ void tc_epilogue(const TcParams& p, const EpiShared& 
 // ---------------------------------------------------------------- the kernel
 // grid = (feature tiles, K splits, z), z = token tile * zslices + slice (slices: block-diagonal heads).
 // tmA: weights [N, K]; tmBh / tmBl: activation planes [rows, K]; box = (64, 128) and (64, bn).
-template <int EPI, bool WIDE>
+template <int EPI>
 __global__ void __launch_bounds__(kThreads)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmBh,
                const __grid_constant__ CUtensorMap tmBl, TcParams p, int zslices, int a_rows_per_slice,
@@ -862,9 +471,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   const uint32_t stage_sz = (uint32_t)stage_bytes(bn);
   const uint32_t bars = base + kStages * stage_sz;                   // full[kStages], empty[kStages], accum
   volatile uint32_t* ctl = reinterpret_cast<volatile uint32_t*>(gen_base + kStages * stage_sz + 128);
-  // ctl[0] = tensor-memory base, ctl[1] = "this CTA reduces the tile", ctl[2] = "this CTA merges the top-1",
-  // ctl[3] = "the accumulator arrived"
-  __shared__ float s_mean[WIDE ? kMaxBN : 16], s_rstd[WIDE ? kMaxBN : 16];
+  // ctl[0] = tensor-memory base, ctl[1] = "this CTA reduces the tile", ctl[3] = "the accumulator arrived"
+  __shared__ float s_mean[kMaxBN], s_rstd[kMaxBN];
   __shared__ unsigned long long s_slot[kMaxBN];   // kTcQkv: cache slot (element offset) of every token of the tile
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -876,7 +484,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   const int c0 = split * p.chunks_per_split;
   const int c1 = min(total_chunks, c0 + p.chunks_per_split);
   const int nchunks = max(0, c1 - c0);
-  const uint32_t ncols = bn <= 32 ? 32u : (bn <= 64 ? 64u : 128u);
+  const uint32_t ncols = 32;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages; ++s) {
@@ -886,7 +494,6 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     mbar_init(bars + 8 * 2 * kStages, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     ctl[1] = 0;
-    ctl[2] = 0;
   }
   if (warp == 1) tmem_alloc(base + kStages * stage_sz + 128, ncols);
   tc_fence_before();
@@ -963,11 +570,10 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   } else if (warp >= 2) {
     // ---------------- epilogue: thread = one feature row, registers = tokens
     pdl_wait();
-    // the stages are free once the accumulator is complete: the top-1 epilogue transposes the tile into them
-    const EpiShared sh{reinterpret_cast<float*>(gen_base), s_mean, s_rstd, s_slot, ctl};
+    const EpiShared sh{s_mean, s_rstd, s_slot, ctl};
     const EpiUnit u{tmem, bars + 8 * 2 * kStages, 0u, tile, split, slice, (int)blockIdx.z, (int)gridDim.x,
-                    (int)gridDim.z / zslices, t0, nt, bn, nchunks, p.all_done && *p.all_done};
-    tc_epilogue<EPI, WIDE>(p, sh, u, warp, lane);
+                    t0, nt, bn, nchunks, p.all_done && *p.all_done};
+    tc_epilogue<EPI>(p, sh, u, warp, lane);
   }
   tc_fence_before();
   __syncthreads();

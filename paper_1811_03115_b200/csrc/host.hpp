@@ -46,6 +46,45 @@ inline cudaError_t launch_k(void (*kernel)(KArgs...), dim3 grid, dim3 block, siz
   return cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
 }
 
+// The same for a kernel known by its address alone (instantiated in another translation unit): the arguments must have
+// exactly the types of the kernel's parameters.
+template <typename... Args>
+inline cudaError_t launch_kc(const void* kernel, dim3 grid, dim3 block, size_t smem, cudaStream_t st, bool pdl, Args... args) {
+  cudaLaunchConfig_t cfg;
+  memset(&cfg, 0, sizeof(cfg));
+  cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = pdl ? 1 : 0;
+  void* ptrs[] = {static_cast<void*>(&args)...};
+  return cudaLaunchKernelExC(&cfg, kernel, ptrs);
+}
+
+// ... and with clusters of (1, cluster, 1) CTAs.
+template <typename... Args>
+inline cudaError_t launch_cluster(const void* kernel, dim3 grid, dim3 block, size_t smem, cudaStream_t st, bool pdl, int cluster,
+                                  Args... args) {
+  cudaLaunchConfig_t cfg;
+  memset(&cfg, 0, sizeof(cfg));
+  cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  int n = 0;
+  if (pdl) {
+    attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[n++].val.programmaticStreamSerializationAllowed = 1;
+  }
+  if (cluster > 1) {
+    attr[n].id = cudaLaunchAttributeClusterDimension;
+    attr[n].val.clusterDim.x = 1; attr[n].val.clusterDim.y = (unsigned)cluster; attr[n++].val.clusterDim.z = 1;
+  }
+  cfg.attrs = attr;
+  cfg.numAttrs = (unsigned)n;
+  void* ptrs[] = {static_cast<void*>(&args)...};
+  return cudaLaunchKernelExC(&cfg, kernel, ptrs);
+}
+
 // Opt-in dynamic shared-memory limit of a kernel: only ever raised, tracked per (device, kernel), so that
 // sessions of different models and several devices in one process cannot lower or miss each other's limit.
 int ensure_smem_limit(const void* kernel, size_t bytes);

@@ -1326,5 +1326,9 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
   cluster.sync();
 }
 
+// The kernel's instantiations (layer_stack.cu): token tiles (1 or 2 of 8 rows), reduction steps per panel (2: d_model
+// 256, else 4), CTAs per SM (1 or 2), lean (short sequences and staged encoder rows only); null if there is none.
+const void* kernel_for(int nt, int ksteps, int minb, bool lean);
+
 }  // namespace stack
 }  // namespace bpd

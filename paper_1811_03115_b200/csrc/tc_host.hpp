@@ -2,84 +2,110 @@
 #pragma once
 #include <cuda.h>
 #include <cuda_runtime.h>
+#include <math.h>
 
+#include <algorithm>
 #include <map>
 #include <mutex>
 #include <tuple>
 
-#include "gemm_tc.cuh"
+#include "gemm_wide.cuh"
 #include "host.hpp"
 
 namespace bpd {
 namespace tc {
 
 // Resident CTA slots the planner aims to fill: 2 CTAs on each of the 148 SMs of a B200.
-constexpr int kSlots = 296;
+constexpr int kSms = 148;
+constexpr int kSlots = 2 * kSms;
 constexpr int kMinChunksPerSplit = 2;
 
 struct Plan {
   int tiles, chunks, splits, chunks_per_split;
 };
-// Depends on (N, K) only -- never on the number of tokens -- so that a position
-// scored alone and the same position scored inside a block add up in the same order.
-// wide_ttiles: 0 for sessions whose passes carry few rows (one token tile, two CTAs per SM, split K finely);
-// otherwise the number of token tiles the split is planned for (the session's widest pass, unless the launch
-// says otherwise): those launches already have tiles x token tiles CTAs, so K is split only as far as that
-// leaves of the `slots` CTA slots idle.  Both are properties of the session and of the matrix, so greedy and
-// blockwise passes of one session still agree.
-inline Plan plan_splits(int N, int K, int wide_ttiles = 0, int slots = kSlots / 2) {
+// Launches of at most 16 token rows (gemm_tc.cuh): one token tile, two CTAs per SM, K split finely.  Depends on (N, K)
+// only -- never on the number of tokens -- so that a position scored alone and the same position scored inside a
+// block add up in the same order.
+inline Plan plan_splits(int N, int K) {
   Plan pl;
   pl.tiles = (N + kBM - 1) / kBM;
   pl.chunks = (K + kBK - 1) / kBK;
-  int splits;
-  if (wide_ttiles > 0) splits = std::max(1, std::min(pl.chunks / 8, slots / (pl.tiles * wide_ttiles)));
-  else splits = std::max(1, std::min(pl.chunks / kMinChunksPerSplit, kSlots / pl.tiles));
+  const int splits = std::max(1, std::min(pl.chunks / kMinChunksPerSplit, kSlots / pl.tiles));
   pl.chunks_per_split = (pl.chunks + splits - 1) / splits;
   pl.splits = (pl.chunks + pl.chunks_per_split - 1) / pl.chunks_per_split;
   return pl;
 }
-inline int token_bn(int T, int ttiles);
-// Token tiling of a launch: as few tiles of at most 128 tokens as possible, but -- in sessions with many rows --
-// the tiling (tiles of 32 to 64 tokens) that leaves the busiest SM the fewest bytes to stage: with
-// `ctas_per_ttile` CTAs per token tile, a CTA stages 16 KB of weights and bn / 4 KB of activation planes per
-// K chunk, and the busiest SM runs ceil(CTAs / 148) of them.  Ties go to the finer tiling (more loads in
-// flight).  The tile width only changes the MMA's N; every output element is still the same sum in the same order.
-inline int token_tiles(int T, int ctas_per_ttile = 0) {
-  int tt = std::max(1, (T + kMaxBN - 1) / kMaxBN);
-  if (ctas_per_ttile > 0) {
-    // at most 64 tokens per tile: two CTAs fit on an SM, and one's epilogue overlaps the other's main loop
-    // (measured on the batch-32 workload: 1428 -> 1338 us per iteration against tiles of 80-112 tokens)
-    tt = std::max(tt, (T + 63) / 64);
-    const int hi = std::max(tt, (T + 31) / 32);
-    long best_cost = -1;
-    int best_tt = tt;
-    for (int cand = tt; cand <= hi; ++cand) {
-      const int bn = token_bn(T, cand);
-      if ((long)(cand - 1) * bn >= T) continue;                   // its last tile would be empty
-      const long per_sm = ((long)ctas_per_ttile * cand + 147) / 148;
-      const long cost = per_sm * (64 + bn);                       // quarter KB per K chunk
-      if (best_cost < 0 || cost <= best_cost) { best_cost = cost; best_tt = cand; }
+
+// Launches of the wide kernel (gemm_wide.cuh).  A tiling is (tokens per tile, CTAs per cluster = K splits); its cost in
+// microseconds is estimated from what bounds these launches: shared-memory fill (every CTA stages 16 KB of weights and
+// bn x planes x 128 bytes of activations per K chunk) and the exchange of the partial tiles inside the cluster.
+struct WidePlan {
+  int tiles, chunks, splits, chunks_per_split, bn, ttiles, stages;
+  float cost;
+};
+constexpr size_t kWideSmemHalf = 108 * 1024;    // dynamic shared memory with two CTAs per SM (static: 4.3 KB, reserved: 1 KB)
+constexpr size_t kWideSmemFull = 221 * 1024;
+inline WidePlan wide_tiling(int N, int K, int T, int z, int planes, int splits, int ttiles) {
+  WidePlan w;
+  w.tiles = (N + kBM - 1) / kBM;
+  w.chunks = (K + kBK - 1) / kBK;
+  w.splits = splits;
+  w.chunks_per_split = (w.chunks + splits - 1) / splits;
+  w.ttiles = ttiles;
+  w.bn = std::max(16, ((T + ttiles - 1) / ttiles + 15) / 16 * 16);
+  // two CTAs per SM where at least two stages of each fit, else one with as many stages as there is room for
+  int per_sm = 2;
+  size_t room = kWideSmemHalf;
+  if (wide_smem_bytes(w.bn, planes, std::min(2, w.chunks_per_split)) > kWideSmemHalf) { per_sm = 1; room = kWideSmemFull; }
+  w.stages = 1;
+  while (w.stages < kWideStages && w.stages < w.chunks_per_split && wide_smem_bytes(w.bn, planes, w.stages + 1) <= room) ++w.stages;
+  // Fitted to 2300 timings of dependent launches (N 256..40960, K 512..40960, T 10..2560; the tiling it picks is on
+  // average 2.6 % slower than the best one measured): a first round trip, the bytes of a chunk at what one SM takes in,
+  // a refill of the ring per chunk beyond its depth, the exchange inside the cluster; all CTA slots of the GPU (clusters
+  // of 4 and 8 do not fill every SM) in waves, and no faster than L2 and HBM deliver.
+  const double ctas = (double)w.tiles * w.splits * w.ttiles * z;
+  const double kb = wide_stage_bytes(w.bn, planes) / 1024.0;
+  const int full = kSms * per_sm, slots = splits >= 8 ? full * 8 / 9 : (splits == 4 ? full * 11 / 12 : full);
+  const double waves = ceil(ctas / slots), resident = std::min<double>(per_sm, ceil(ctas / kSms));
+  const double in = 2.26 + w.chunks_per_split * kb * resident / 165.0 + std::max(0, w.chunks_per_split - w.stages) * 1.2 / w.stages;
+  const double out = 0.0017 * w.bn / splits + (splits > 1 ? 0.022 * w.bn * (splits - 1) / splits : 0.0);
+  const double deliver = std::max(ctas * w.chunks_per_split * kb / 13200.0, (double)z * w.tiles * w.chunks * 16.0 / 7600.0);
+  w.cost = (float)std::max(waves * (in + out) * (per_sm == 1 ? 1.2 : 1.0), deliver + 2.26 + out);
+  return w;
+}
+// The split of a matrix: chosen for `rows` token rows (the session's widest pass) and kept for every launch on it.
+inline int wide_splits(int N, int K, int rows, int z, int planes) {
+  int best = 1;
+  float cost = 0;
+  for (int s = 1; s <= 8; s *= 2) {
+    if (s > 1 && s > (K + kBK - 1) / kBK) break;
+    for (int tt = (rows + kWideBN - 1) / kWideBN; tt <= (rows + 31) / 32 || tt == 1; ++tt) {
+      const WidePlan w = wide_tiling(N, K, rows, z, planes, s, tt);
+      if ((long)(tt - 1) * w.bn >= rows) continue;                   // its last tile would be empty
+      if (cost == 0 || w.cost < cost) { cost = w.cost; best = s; }
     }
-    tt = best_tt;
   }
-  return tt;
+  return best;
 }
-inline int token_bn(int T, int ttiles) {
-  const int per = (T + ttiles - 1) / ttiles;
-  return std::max(16, (per + 15) / 16 * 16);
+// The token tiling of a launch of T rows, its split given.
+inline WidePlan wide_plan(int N, int K, int T, int z, int planes, int splits) {
+  WidePlan best;
+  best.cost = -1;
+  for (int tt = (T + kWideBN - 1) / kWideBN; tt <= (T + 31) / 32 || tt == 1; ++tt) {
+    const WidePlan w = wide_tiling(N, K, T, z, planes, splits, tt);
+    if ((long)(tt - 1) * w.bn >= T) continue;
+    if (best.cost < 0 || w.cost < best.cost) best = w;
+  }
+  return best;
 }
-inline int token_bn(int T) { return token_bn(T, token_tiles(T)); }
-inline int max_token_tiles(int T) { return std::max(token_tiles(T), (T + 31) / 32); }
-// fp32 elements of split-K workspace a launch with these sizes needs.
-inline size_t ws_floats(int N, int K, int T, int zslices, int wide_ttiles = 0, int slots = kSlots / 2) {
-  const Plan pl = plan_splits(N, K, wide_ttiles, slots);
-  if (pl.splits == 1) return 0;
-  // upper bound over every token tiling the launch may pick: tiles * bn <= T + 16 per tile
-  return (size_t)zslices * pl.tiles * pl.splits * ((size_t)T + 16 * max_token_tiles(T)) * kBM;
+
+// fp32 elements of split-K workspace and arrival counters a launch of the few-row kernel needs.
+constexpr int kNarrowBN = 16;
+inline size_t ws_floats(int N, int K, int zslices) {
+  const Plan pl = plan_splits(N, K);
+  return pl.splits == 1 ? 0 : (size_t)zslices * pl.tiles * pl.splits * kNarrowBN * kBM;
 }
-inline size_t counters_needed(int N, int T, int zslices) {
-  return (size_t)max_token_tiles(T) * zslices * ((N + kBM - 1) / kBM);
-}
+inline size_t counters_needed(int N, int zslices) { return (size_t)zslices * ((N + kBM - 1) / kBM); }
 
 struct Scratch {
   float* ws; size_t ws_floats;
@@ -87,7 +113,7 @@ struct Scratch {
   unsigned* done_counter;
   unsigned long long* best; size_t best_elems;
   int* error;
-  int wide_ttiles;   // see plan_splits
+  int wide_rows;     // > 0: the wide kernel, its splits chosen for this many token rows; 0: the few-row kernel
   int l2_hints;      // 1: weights that a launch reads once are loaded "evict first"
 };
 
@@ -200,65 +226,94 @@ inline int make_map_3d(const void* ptr, int elem_bytes, uint64_t layers, uint64_
 
 struct Operands {
   const void* w; int w_rows;            // weights [w_rows, K] (all slices stacked)
-  const void* x; long long x_plane;     // activation planes: hi at x, lo at x + x_plane (elements)
+  const void* x; long long x_plane;     // activation planes: hi at x, lo at x + x_plane (elements); 0: one plane (wide kernel only)
   long long ldx; int x_rows; int x_cols;  // allocated rows, total columns per row
-  const void* x_lo = nullptr;           // the lo plane when it lives in another allocation (x_plane unused then)
 };
 
+// plan_n: the feature count the K split is planned for.  A launch that computes only the first features of a matrix
+// (fewer heads) passes the full count so that every feature is summed in the same order either way.
+// plan_rows: in a session with many rows, the row count the split is planned for when its results need not agree bit
+// for bit with any other launch (the second stage of the lazy heads).
 template <int EPI>
 int launch(const Operands& op, int N, int K, int T, TcParams p, const Scratch& sc, cudaStream_t st, int zslices = 1,
-           int a_rows_per_slice = 0, int b_cols_per_slice = 0, bool pdl = false, int plan_n = 0, int plan_tt = 0) {
-  {
-    int rc0 = ensure_smem_limit(reinterpret_cast<const void*>(gemm_tc_kernel<EPI, false>), smem_bytes(16));
-    if (!rc0) rc0 = ensure_smem_limit(reinterpret_cast<const void*>(gemm_tc_kernel<EPI, true>), std::max(smem_bytes(kMaxBN), smem_bytes(64)));
-    if (rc0) return rc0;
-  }
-  // plan_n: the feature count the K split is planned for.  A launch that computes only the first features of a
-  // matrix (fewer heads) passes the full count so that every feature is summed in the same order either way.
-  // plan_tt: in a session with many rows, a launch whose results need not agree bit for bit with any other
-  // launch (the second stage of the lazy heads) plans its K split for its own token tiles and for two CTAs per SM.
-  Plan pl = (sc.wide_ttiles && plan_tt > 0) ? plan_splits(plan_n > 0 ? plan_n : N, K, plan_tt, kSlots)
-                                            : plan_splits(plan_n > 0 ? plan_n : N, K, sc.wide_ttiles);
-  pl.tiles = (N + kBM - 1) / kBM;
-  const int ttiles = token_tiles(T, sc.wide_ttiles ? pl.tiles * pl.splits * zslices : 0), bn = token_bn(T, ttiles);
-  const size_t need_ws = pl.splits == 1 ? 0 : (size_t)ttiles * zslices * pl.tiles * pl.splits * bn * kBM;
-  const size_t need_cnt = (size_t)ttiles * zslices * pl.tiles;
-  if (need_ws > sc.ws_floats || need_cnt > sc.n_counters)
-    return fail(BPD_E_NOMEM, "split-K workspace too small (%zu floats, %zu counters needed)", need_ws, need_cnt);
+           int a_rows_per_slice = 0, int b_cols_per_slice = 0, bool pdl = false, int plan_n = 0, int plan_rows = 0) {
+  const int pn = plan_n > 0 ? plan_n : N;
+  const int planes = op.x_plane > 0 ? 2 : 1;
+  const bool wide = sc.wide_rows > 0;
+  if (!wide && (T > kNarrowBN || planes != 2)) return fail(BPD_E_UNSUPPORTED, "%d token rows in a launch of the few-row projection kernel", T);
   if (EPI == kTcArgmax && (size_t)T > sc.best_elems) return fail(BPD_E_NOMEM, "top-1 workspace too small");
+  WidePlan wp;
+  Plan pl;
+  int bn = kNarrowBN;
+  if (wide) {
+    wp = wide_plan(N, K, T, zslices, planes, wide_splits(pn, K, plan_rows > 0 ? plan_rows : sc.wide_rows, zslices, planes));
+    bn = wp.bn;
+  } else {
+    pl = plan_splits(pn, K);
+    pl.tiles = (N + kBM - 1) / kBM;
+    const size_t need_ws = pl.splits == 1 ? 0 : (size_t)zslices * pl.tiles * pl.splits * bn * kBM;
+    const size_t need_cnt = (size_t)zslices * pl.tiles;
+    if (need_ws > sc.ws_floats || need_cnt > sc.n_counters)
+      return fail(BPD_E_NOMEM, "split-K workspace too small (%zu floats, %zu counters needed)", need_ws, need_cnt);
+  }
   CUtensorMap ma, mh, ml;
   int rc = make_map(op.w, (uint64_t)op.w_rows, (uint64_t)K, (uint64_t)K, kBM, &ma);
   if (rc) return rc;
   rc = make_map(op.x, (uint64_t)op.x_rows, (uint64_t)op.x_cols, (uint64_t)op.ldx, (uint32_t)bn, &mh);
   if (rc) return rc;
-  rc = make_map(op.x_lo ? static_cast<const bf16*>(op.x_lo) : static_cast<const bf16*>(op.x) + op.x_plane, (uint64_t)op.x_rows, (uint64_t)op.x_cols, (uint64_t)op.ldx,
-                (uint32_t)bn, &ml);
+  ml = mh;
+  if (planes == 2) rc = make_map(static_cast<const bf16*>(op.x) + op.x_plane, (uint64_t)op.x_rows, (uint64_t)op.x_cols, (uint64_t)op.ldx, (uint32_t)bn, &ml);
   if (rc) return rc;
-  p.T = T; p.N = N; p.K = K; p.bn = bn; p.splits = pl.splits; p.chunks_per_split = pl.chunks_per_split;
+  p.T = T; p.N = N; p.K = K; p.bn = bn;
+  p.splits = wide ? wp.splits : pl.splits; p.chunks_per_split = wide ? wp.chunks_per_split : pl.chunks_per_split;
 #ifdef BPD_TC_TRACE
   { static int next_trace_id = 0; p.trace_id = next_trace_id++ & 127; }
 #endif
   p.ws = sc.ws; p.tile_counters = sc.tile_counters; p.done_counter = sc.done_counter;
   p.best = sc.best; p.error = sc.error;
-  p.stream_weights = (ttiles == 1 && sc.l2_hints) ? 1 : 0;
+  p.stream_weights = ((!wide || wp.ttiles == 1) && sc.l2_hints) ? 1 : 0;
+  if (!wide) {
+    if (p.stat_in || p.stat_out) return fail(BPD_E_UNSUPPORTED, "per-tile layer-norm statistics in a launch of the few-row projection kernel");
+    if constexpr (EPI == kTcArgmax) {
+      return fail(BPD_E_UNSUPPORTED, "the few-row projection kernel has no top-1 epilogue");
+    } else {
+      if ((rc = ensure_smem_limit(reinterpret_cast<const void*>(gemm_tc_kernel<EPI>), smem_bytes(bn)))) return rc;
+      BPD_CUDA(launch_k(gemm_tc_kernel<EPI>, dim3(pl.tiles, pl.splits, zslices), dim3(kThreads), smem_bytes(bn), st, pdl, ma, mh, ml, p,
+                        zslices, a_rows_per_slice, b_cols_per_slice));
+      return BPD_OK;
+    }
+  }
   {
-    // vector stores in the epilogue of wide tiles: every row offset and pointer involved must allow them
+    // vector stores in the epilogue: every row offset and pointer involved must allow them
     auto al = [](const void* q, size_t a) { return q == nullptr || (uintptr_t)q % a == 0; };
     p.vec = (N % 4 == 0 && p.ldo % 4 == 0 && p.plane % 4 == 0 && p.xg_plane % 4 == 0 && p.zofs_n % 4 == 0 &&
              (p.d % 4 == 0) && al(p.out_f32, 16) && al(p.out_hi, 8) && al(p.xg_hi, 8) && al(p.h, 16) && al(p.bias, 8) &&
              al(p.g_next, 8) && al(p.kcache, 8) && al(p.vcache, 8)) ? 1 : 0;
   }
-  if ((p.stat_in || p.stat_out) && !(p.vec && bn >= 32 && N % kBM == 0 && EPI != kTcArgmax && !p.ln_x))
-    return fail(BPD_E_UNSUPPORTED, "per-tile layer-norm statistics need wide, vectorisable tiles (N = %d, %d tokens per tile)", N, bn);
-  dim3 grid(pl.tiles, pl.splits, ttiles * zslices);
-  if (bn >= 32)
-    BPD_CUDA(launch_k(gemm_tc_kernel<EPI, true>, grid, dim3(kThreads), smem_bytes(bn), st, pdl, ma, mh, ml, p, zslices,
-                      a_rows_per_slice, b_cols_per_slice));
-  else
-    BPD_CUDA(launch_k(gemm_tc_kernel<EPI, false>, grid, dim3(kThreads), smem_bytes(bn), st, pdl, ma, mh, ml, p, zslices,
-                      a_rows_per_slice, b_cols_per_slice));
+  if (p.ln_x || (!p.vec && EPI != kTcF32 && EPI != kTcArgmax)) return fail(BPD_E_UNSUPPORTED, "operands of the wide projection kernel are misaligned");
+  if ((p.stat_in || p.stat_out) && !(p.vec && N % kBM == 0 && EPI != kTcArgmax))
+    return fail(BPD_E_UNSUPPORTED, "per-tile layer-norm statistics need whole, aligned feature tiles (N = %d)", N);
+  const void* kernel = planes == 2 ? reinterpret_cast<const void*>(gemm_wide_kernel<EPI, 2>) : nullptr;
+  if constexpr (EPI == kTcF32 || EPI == kTcArgmax) {
+    if (planes == 1) kernel = reinterpret_cast<const void*>(gemm_wide_kernel<EPI, 1>);
+  }
+  if (!kernel) return fail(BPD_E_UNSUPPORTED, "single-plane activations with this epilogue");
+  const size_t smem = wide_smem_bytes(bn, planes, wp.stages);
+  if ((rc = ensure_smem_limit(kernel, smem))) return rc;
+  BPD_CUDA(launch_cluster(kernel, dim3(wp.ttiles * zslices, wp.splits, wp.tiles), dim3(kWideThreads), smem, st, pdl, wp.splits,
+                          ma, mh, ml, p, wp.ttiles, wp.stages, a_rows_per_slice, b_cols_per_slice));
   return BPD_OK;
 }
+
+#define BPD_TC_LAUNCH(EPI) \
+  template int launch<EPI>(const Operands&, int, int, int, TcParams, const Scratch&, cudaStream_t, int, int, int, bool, int, int)
+// instantiated in gemm_tc.cu
+extern BPD_TC_LAUNCH(kTcPlanes);
+extern BPD_TC_LAUNCH(kTcF32);
+extern BPD_TC_LAUNCH(kTcResidual);
+extern BPD_TC_LAUNCH(kTcQkv);
+extern BPD_TC_LAUNCH(kTcHeadOut);
+extern BPD_TC_LAUNCH(kTcArgmax);
 
 }  // namespace tc
 }  // namespace bpd
