@@ -470,6 +470,7 @@ static tc::Scratch tc_scratch(bpd_session* s) {
   sc.error = s->st.error;
   sc.wide_rows = session_wide_rows(s->m->cfg, s->B);
   sc.l2_hints = s->opt.l2_stream_hints;
+  sc.error_on_host = 0;
   return sc;
 }
 
@@ -1098,6 +1099,70 @@ static int fetch(bpd_session* s, int max_new, int32_t* out_ids, int32_t* out_len
   return BPD_OK;
 }
 
+// ------------------------------------------------------------------ single operators
+// Scratch layout of the bf16 (tensor-core) top-1: the keys and the merge counter.
+struct OpScratch {
+  size_t best_off, done_off, total;
+};
+static OpScratch op_scratch_layout(int rows) {
+  OpScratch o;
+  o.best_off = 0;
+  o.done_off = (size_t)rows * tc::kBestStride * sizeof(unsigned long long);
+  o.total = align_up(o.done_off + sizeof(unsigned));
+  return o;
+}
+static bool op_use_tc(int dtype) { return dtype == 1; }
+
+// Error words of the operator calls in flight: words of pinned host memory, so that a call reads its word after
+// waiting for the stream instead of copying it back first (the copy of a device word took 12 of the call's 32 us).
+// Pages of 1024 words are added when more calls than that are in flight and kept for later calls.
+class ErrorWords {
+ public:
+  int take(volatile int** host, int** dev) {
+    std::lock_guard<std::mutex> lock(mu_);
+    if (free_.empty()) {
+      int* page = nullptr;
+      BPD_CUDA(cudaHostAlloc(reinterpret_cast<void**>(&page), 4096, cudaHostAllocMapped | cudaHostAllocPortable));
+      for (int i = 0; i < 1024; ++i) free_.push_back(page + i);
+    }
+    int* w = free_.back();
+    void* d = nullptr;
+    BPD_CUDA(cudaHostGetDevicePointer(&d, w, 0));
+    free_.pop_back();
+    *w = 0;
+    *host = w;
+    *dev = static_cast<int*>(d);
+    return BPD_OK;
+  }
+  void give_back(volatile int* w) {
+    std::lock_guard<std::mutex> lock(mu_);
+    free_.push_back(const_cast<int*>(w));
+  }
+ private:
+  std::mutex mu_;
+  std::vector<int*> free_;
+};
+static ErrorWords g_error_words;
+
+// Launches a projection with an error word of its own, waits for the stream and reports what the word says.
+template <int EPI>
+static int op_tc(const tc::Operands& op, int N, int K, int rows, const tc::TcParams& tp, tc::Scratch sc, cudaStream_t st) {
+  volatile int* word = nullptr;
+  BPD_TRY(g_error_words.take(&word, &sc.error));
+  sc.error_on_host = 1;
+  sc.wide_rows = rows;
+  sc.l2_hints = 1;
+  int rc = tc::launch<EPI>(op, N, K, rows, tp, sc, st);
+  if (!rc) {
+    ++g_launches;
+    const cudaError_t e = cudaStreamSynchronize(st);
+    if (e != cudaSuccess) rc = fail(BPD_E_CUDA, "operator failed: %s", cudaGetErrorString(e));
+    else if (*word) rc = fail(BPD_E_TIMEOUT, "a bounded wait inside the projection kernel expired (code %d)", (int)*word);
+  }
+  g_error_words.give_back(word);
+  return rc;
+}
+
 }  // namespace bpd
 
 using namespace bpd;
@@ -1631,33 +1696,9 @@ int bpd_debug_wait_timeout(int32_t* dev_word, int limit_us, void* cuda_stream) {
 }
 
 // ------------------------------------------------------------------ single operators
-// Scratch layout of the bf16 (tensor-core) operators: the top-1 keys, the merge counter and an error word.
-struct OpScratch {
-  size_t best_off, done_off, err_off, total;
-};
-static OpScratch op_scratch_layout(int rows, bool top1) {
-  OpScratch o;
-  size_t off = 0;
-  auto take = [&](size_t bytes) { size_t at = off; off = align_up(off + bytes); return at; };
-  o.best_off = take(top1 ? (size_t)rows * tc::kBestStride * sizeof(unsigned long long) : 0);
-  o.done_off = take(sizeof(unsigned));
-  o.err_off = take(sizeof(int));
-  o.total = off;
-  return o;
-}
-static bool op_use_tc(int dtype) { return dtype == 1; }
-
-static int op_tc_finish(char* scratch, const OpScratch& L, cudaStream_t st) {
-  int err = 0;
-  BPD_CUDA(cudaMemcpyAsync(&err, scratch + L.err_off, sizeof(int), cudaMemcpyDeviceToHost, st));
-  BPD_CUDA(cudaStreamSynchronize(st));
-  if (err) return fail(BPD_E_TIMEOUT, "a bounded wait inside the projection kernel expired (code %d)", err);
-  return BPD_OK;
-}
-
 size_t bpd_op_vocab_argmax_scratch_bytes(int rows, int d, int vocab, int dtype) {
   if (rows < 1 || vocab < 1 || d < 1) return 0;
-  if (op_use_tc(dtype)) return op_scratch_layout(rows, true).total;
+  if (op_use_tc(dtype)) return op_scratch_layout(rows).total;
   const size_t tiles = ceil_div(vocab, kVocTile);
   return align_up(tiles * rows * sizeof(float)) + align_up(tiles * rows * sizeof(int)) +
          align_up((ceil_div(rows, kRC) + 1) * sizeof(unsigned));
@@ -1673,18 +1714,16 @@ int bpd_op_vocab_argmax(const void* x, const void* w, int rows, int d, int vocab
   cudaStream_t st = (cudaStream_t)cuda_stream;
   char* p = static_cast<char*>(scratch);
   if (op_use_tc(dtype)) {
-    const OpScratch L = op_scratch_layout(rows, true);
+    const OpScratch L = op_scratch_layout(rows);
     BPD_CUDA(cudaMemsetAsync(p, 0, L.total, st));
-    tc::Scratch sc{nullptr, 0, nullptr, 0, reinterpret_cast<unsigned*>(p + L.done_off), reinterpret_cast<unsigned long long*>(p + L.best_off),
-                   (size_t)rows, reinterpret_cast<int*>(p + L.err_off), rows, 1};
-    tc::Operands op{w, vocab, x, 0, d, rows, d};   // one plane
+    tc::Scratch sc{};
+    sc.done_counter = reinterpret_cast<unsigned*>(p + L.done_off);
+    sc.best = reinterpret_cast<unsigned long long*>(p + L.best_off);
+    sc.best_elems = (size_t)rows;
     tc::TcParams tp;
     memset(&tp, 0, sizeof(tp));
     tp.out_idx = out_idx; tp.out_val = out_val;
-    int rc = tc::launch<tc::kTcArgmax>(op, vocab, d, rows, tp, sc, st);
-    if (rc) return rc;
-    ++g_launches;
-    return op_tc_finish(p, L, st);
+    return op_tc<tc::kTcArgmax>(tc::Operands{w, vocab, x, 0, d, rows, d}, vocab, d, rows, tp, sc, st);
   }
   const size_t tiles = ceil_div(vocab, kVocTile);
   float* pv = reinterpret_cast<float*>(p);
@@ -1699,10 +1738,10 @@ int bpd_op_vocab_argmax(const void* x, const void* w, int rows, int d, int vocab
   return BPD_OK;
 }
 
-size_t bpd_op_linear_scratch_bytes(int rows, int in_f, int out_f, int dtype) {
-  if (rows < 1 || in_f < 1 || out_f < 1) return 0;
-  if (op_use_tc(dtype)) return op_scratch_layout(rows, false).total;
-  return 256;
+// The projection keeps its partial sums on the chip: the scratch is not touched, but still has to be there.
+constexpr size_t kOpLinearScratch = 256;
+size_t bpd_op_linear_scratch_bytes(int rows, int in_f, int out_f, int) {
+  return (rows < 1 || in_f < 1 || out_f < 1) ? 0 : kOpLinearScratch;
 }
 
 int bpd_op_linear(const void* x, const void* w, const void* bias, int rows, int in_f, int out_f, int dtype, int relu,
@@ -1714,20 +1753,11 @@ int bpd_op_linear(const void* x, const void* w, const void* bias, int rows, int 
   cudaStream_t st = (cudaStream_t)cuda_stream;
   if (op_use_tc(dtype)) {
     if (!scratch || (uintptr_t)scratch % 256) return fail(BPD_E_INVALID, "scratch is null or misaligned");
-    const OpScratch L = op_scratch_layout(rows, false);
-    if (scratch_bytes < L.total) return fail(BPD_E_NOMEM, "scratch too small");
-    char* p = static_cast<char*>(scratch);
-    BPD_CUDA(cudaMemsetAsync(p, 0, L.total, st));
-    tc::Scratch sc{nullptr, 0, nullptr, 0, reinterpret_cast<unsigned*>(p + L.done_off), reinterpret_cast<unsigned long long*>(p + L.best_off),
-                   (size_t)rows, reinterpret_cast<int*>(p + L.err_off), rows, 1};
-    tc::Operands op{w, out_f, x, 0, in_f, rows, in_f};   // one plane
+    if (scratch_bytes < kOpLinearScratch) return fail(BPD_E_NOMEM, "scratch too small");
     tc::TcParams tp;
     memset(&tp, 0, sizeof(tp));
     tp.bias = static_cast<const bf16*>(bias); tp.relu = relu; tp.out_f32 = y; tp.ldo = out_f;
-    int rc = tc::launch<tc::kTcF32>(op, out_f, in_f, rows, tp, sc, st);
-    if (rc) return rc;
-    ++g_launches;
-    return op_tc_finish(p, L, st);
+    return op_tc<tc::kTcF32>(tc::Operands{w, out_f, x, 0, in_f, rows, in_f}, out_f, in_f, rows, tp, tc::Scratch{}, st);
   }
   LinearParams p = lin(x, in_f, w, in_f, out_f, bias, rows, y, out_f, relu, nullptr);
   if (dtype == 0) launch_linear<float, float, kEpiStoreF32>(p, 1, st);

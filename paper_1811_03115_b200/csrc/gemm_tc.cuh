@@ -95,7 +95,8 @@ struct TcParams {
 #ifdef BPD_TC_TRACE
   int trace_id;
 #endif
-  int* error;                  // device error word
+  int* error;                  // error word
+  int error_on_host;           // 1 (wide kernel only): the word lies in pinned host memory
   const int* all_done;
   int stream_weights;          // 1: the weights are read once per launch (one token tile): load them "evict first"
   int vec;                     // 1: wide token tiles finish through shared memory with 8- and 16-byte stores (the

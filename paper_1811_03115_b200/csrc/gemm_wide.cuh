@@ -57,6 +57,12 @@ __device__ __forceinline__ float4 ld_cg_v4_here(const float* ptr) {
   return v;
 }
 
+// Error code of a launch: a device word that keeps the first code, or (single operators) a word of pinned host memory.
+__device__ __forceinline__ void report(const TcParams& p, int code) {
+  if (p.error_on_host) *reinterpret_cast<volatile int*>(p.error) = code;
+  else atomicCAS(p.error, 0, code);
+}
+
 // ---------------------------------------------------------------- finishing (token, four features) items
 // A warp finishes the 128 features of a token, four consecutive ones per lane.  Per-thread constants of the four:
 struct FinishCtx {
@@ -352,7 +358,7 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         load_w(it, s);
         load_x(it, s);
       }
-      if (!ok) atomicCAS(p.error, 0, 101);
+      if (!ok) report(p, 101);
       if (!ok || skip) {
         // nobody will consume what is in flight: give it a bounded chance to land before shared memory goes away
         for (int it = max(0, issued - stages); it < issued; ++it) mbar_wait(bars + 8 * (it % stages), (it / stages) & 1);
@@ -378,7 +384,7 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         umma_commit(bars + 8 * (kWideStages + s));    // frees the stage once these MMAs have read it
       }
       umma_commit(acc_bar);                           // accumulator complete
-      if (!ok) atomicCAS(p.error, 0, 102);
+      if (!ok) report(p, 102);
     }
     __syncwarp();
   } else {
@@ -423,7 +429,7 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     }
     bool done = !skip;
     if (done && nchunks > 0) done = mbar_wait(acc_bar, 0);
-    if (!done && !skip && lane == 0) atomicCAS(p.error, 0, 103);
+    if (!done && !skip && lane == 0) report(p, 103);
     tc_fence_after();
     // the stages are free once the accumulator is complete: the tile goes there, one row per token.  A warp reads the
     // 32 tensor-memory lanes (features) its number allows; two warps share them and take every other 16 tokens.

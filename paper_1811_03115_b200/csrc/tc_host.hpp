@@ -99,6 +99,19 @@ inline WidePlan wide_plan(int N, int K, int T, int z, int planes, int splits) {
   return best;
 }
 
+// The same with the split chosen for (plan_n, rows); a thread that repeats a launch keeps its plan (an operator call is
+// a few microseconds, the search over tilings one or two).
+inline WidePlan wide_plan_for(int N, int K, int T, int z, int planes, int plan_n, int rows) {
+  struct Last { int key[7]; WidePlan plan; };
+  static thread_local Last last = {{0, 0, 0, 0, 0, 0, 0}, {}};
+  const int key[7] = {N, K, T, z, planes, plan_n, rows};
+  if (memcmp(key, last.key, sizeof(key)) != 0) {
+    last.plan = wide_plan(N, K, T, z, planes, wide_splits(plan_n, K, rows, z, planes));
+    memcpy(last.key, key, sizeof(key));
+  }
+  return last.plan;
+}
+
 // fp32 elements of split-K workspace and arrival counters a launch of the few-row kernel needs.
 constexpr int kNarrowBN = 16;
 inline size_t ws_floats(int N, int K, int zslices) {
@@ -115,6 +128,7 @@ struct Scratch {
   int* error;
   int wide_rows;     // > 0: the wide kernel, its splits chosen for this many token rows; 0: the few-row kernel
   int l2_hints;      // 1: weights that a launch reads once are loaded "evict first"
+  int error_on_host; // 1: `error` lies in pinned host memory (wide kernel only)
 };
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
@@ -246,7 +260,7 @@ int launch(const Operands& op, int N, int K, int T, TcParams p, const Scratch& s
   Plan pl;
   int bn = kNarrowBN;
   if (wide) {
-    wp = wide_plan(N, K, T, zslices, planes, wide_splits(pn, K, plan_rows > 0 ? plan_rows : sc.wide_rows, zslices, planes));
+    wp = wide_plan_for(N, K, T, zslices, planes, pn, plan_rows > 0 ? plan_rows : sc.wide_rows);
     bn = wp.bn;
   } else {
     pl = plan_splits(pn, K);
@@ -270,7 +284,7 @@ int launch(const Operands& op, int N, int K, int T, TcParams p, const Scratch& s
   { static int next_trace_id = 0; p.trace_id = next_trace_id++ & 127; }
 #endif
   p.ws = sc.ws; p.tile_counters = sc.tile_counters; p.done_counter = sc.done_counter;
-  p.best = sc.best; p.error = sc.error;
+  p.best = sc.best; p.error = sc.error; p.error_on_host = sc.error_on_host;
   p.stream_weights = ((!wide || wp.ttiles == 1) && sc.l2_hints) ? 1 : 0;
   if (!wide) {
     if (p.stat_in || p.stat_out) return fail(BPD_E_UNSUPPORTED, "per-tile layer-norm statistics in a launch of the few-row projection kernel");
