@@ -272,7 +272,7 @@ int bpd_op_vocab_argmax(const void* x, const void* w, int rows, int d, int vocab
  * device-wide synchronisation an allocation may cause, or a plug-in callback
  * that is only allowed to enqueue work.  (The paper has no counterpart; this is
  * a deployment convenience.)  The cross-CTA reduction workspace is a fixed
- * 512 KiB array inside the library image, resident on every GPU that loads the
+ * 33 KiB array inside the library image, resident on every GPU that loads the
  * library until the process exits.  Limits: rows <= 256, vocab <= 65536
  * (beyond them the call returns BPD_E_NOMEM) and d <= 1024, a multiple of 8
  * (BPD_E_SHAPE, as for bpd_op_vocab_argmax); a refused call leaves the outputs

@@ -192,10 +192,6 @@ static size_t plan_session(const Config& c, int B, int max_src, int max_tgt, cha
   int* src_dev = a.take<int>(E);
   int* tail_dev = a.take<int>((size_t)B * kMaxK);
   int* plan_dev = a.take<int>((size_t)B * max_tgt * (kMaxK - 1));
-  const size_t tiles = std::max(ceil_div(c.V, kVocTile), ceil_div(c.V, tc::kBM));
-  float* part_val = a.take<float>(tiles * R2);
-  int* part_idx = a.take<int>(tiles * R2);
-  unsigned* counters = a.take<unsigned>(ceil_div((int)R2, kRC) + 1);
   // split-K workspace of the few-row projection kernel: the largest any launch of this session can need
   size_t ws = 0, ncnt = 1;
   if (c.dtype == 1 && !session_wide_rows(c, B)) {
@@ -210,7 +206,7 @@ static size_t plan_session(const Config& c, int B, int max_src, int max_tgt, cha
   float* tc_ws = a.take<float>(ws);
   unsigned* tc_counters = a.take<unsigned>(ncnt);
   unsigned* tc_done = a.take<unsigned>(1);
-  unsigned long long* tc_best = a.take<unsigned long long>(R2 * tc::kBestStride);
+  unsigned long long* tc_best = a.take<unsigned long long>(R2 * kBestStride);
   // fused decoder layers (few rows per pass): per-head / per-cluster shares of the output projections, slice counters
   const bool fused_ok = c.dtype == 1 && fused::supported(c.d, c.H, c.d_ff, (int)Rmax);
   const size_t fused_parts = std::max<size_t>(c.H, c.d_ff / (fused::kC * fused::kHS));
@@ -227,10 +223,10 @@ static size_t plan_session(const Config& c, int B, int max_src, int max_tgt, cha
     s->fused_ws = fused_ws; s->fused_counters = fused_counters;
     s->x = x; s->h_f32 = h_f32; s->xn = xn; s->qbuf = qbuf; s->attn = attn; s->ffh = ffh; s->u = u; s->o = o;
     s->crosskv = crosskv; s->kcache = kc; s->vcache = vc; s->st = st; s->src_dev = src_dev;
-    s->tail_dev = tail_dev; s->plan_dev = plan_dev; s->part_val = part_val; s->part_idx = part_idx;
+    s->tail_dev = tail_dev; s->plan_dev = plan_dev;
     s->rank = rank;
     s->u2 = u2; s->pl_u2 = (long long)B * c.k_model * c.d_hidden; s->h2 = h2; s->table2 = table2; s->table_full = table_full;
-    s->counters = counters; s->ppr = ppr; s->part_elems = tiles * R2; s->pe = pe; s->npos = (int)npos;
+    s->ppr = ppr; s->pe = pe; s->npos = (int)npos;
     s->tc_ws = tc_ws; s->tc_ws_floats = ws; s->tc_counters = tc_counters; s->tc_n_counters = ncnt; s->tc_done = tc_done; s->tc_best = tc_best; s->tc_best_elems = R2;
     s->pl_xn = (long long)(Rall * d); s->pl_attn = (long long)(Rall * d); s->pl_ffh = (long long)(Rall * c.d_ff);
     s->pl_u = (long long)(Rmax * c.k_model * c.d_hidden); s->pl_o = (long long)(R2 * d);
@@ -245,9 +241,8 @@ static size_t weight_bytes_for(const ParsedBlob& pb) { return align_up(pb.total)
 // ------------------------------------------------------------------ launches
 std::atomic<long long> g_launches{0};
 template <typename WT, typename AT, int EPI>
-static void launch_linear(const LinearParams& p, int zcount, cudaStream_t st) {
-  dim3 grid(ceil_div(p.N, kLinWarps * kFPW), ceil_div(p.rows, kRC), zcount);
-  linear_kernel<WT, AT, EPI><<<grid, kLinWarps * 32, 0, st>>>(p);
+static void launch_linear(const LinearParams& p, int zcount, cudaStream_t st, bool pdl = false) {
+  launch_linear_tiles<WT, AT, EPI>(p, zcount, st, pdl);
   ++g_launches;
 }
 
@@ -268,15 +263,17 @@ static void launch_ln(const float* x, const void* g, const void* b, void* y, flo
   ++g_launches;
 }
 
-template <typename WT, typename AT>
-static void launch_vocab_argmax(const void* x, const void* w, int rows, int d, int V, float* part_val, int* part_idx,
-                                unsigned* counters, int* out_idx, float* out_val, float* logits, const int* all_done,
-                                cudaStream_t st, const RankState* rank = nullptr, int rank_kh = 1) {
-  ArgmaxParams p{x, (long long)d, w, rows, d, V, part_val, part_idx, counters, out_idx, out_val, logits, all_done};
-  if (rank) { p.rank = *rank; p.rank_kh = rank_kh; }
-  dim3 grid(ceil_div(V, kVocTile), ceil_div(rows, kRC));
-  vocab_argmax_kernel<WT, AT><<<grid, kLinWarps * 32, (size_t)kRC * d * sizeof(float), st>>>(p);
-  ++g_launches;
+// The layer norm in front of a projection, applied to its input on the way in.
+static LinearParams with_ln(LinearParams p, const void* g, const void* b, float eps) {
+  p.ln_g = g; p.ln_b = b; p.ln_eps = eps;
+  return p;
+}
+// Vocabulary projection with a top-1 per row.
+static LinearParams lin_top1(const void* x, const void* w, int rows, int d, int V, unsigned long long* best, unsigned* done_counter,
+                             int* out_idx, float* out_val, const int* all_done) {
+  LinearParams p = lin(x, d, w, d, V, nullptr, rows, nullptr, 0, 0, all_done);
+  p.best = best; p.done_counter = done_counter; p.out_idx = out_idx; p.out_val = out_val; p.rank_kh = 1;
+  return p;
 }
 
 // Optional per-phase timing: pairs of events around a phase of the pass, on the session's stream.
@@ -304,6 +301,7 @@ static int run_encoder(bpd_session* s) {
   const Config& c = m->cfg;
   cudaStream_t st = s->stream;
   const int E = s->B * s->max_src, d = c.d;
+  const bool pdl = s->use_pdl != 0;   // every kernel after the first may start while its predecessor ends
   EmbedParams ep;
   memset(&ep, 0, sizeof(ep));
   ep.table = m->src_embed; ep.pe = s->pe; ep.npos = s->npos; ep.x = s->x; ep.rows = E; ep.rows_per_b = s->max_src;
@@ -312,8 +310,7 @@ static int run_encoder(bpd_session* s) {
   ++g_launches;
   for (int l = 0; l < c.n_enc; ++l) {
     const EncLayer& L = m->enc[l];
-    launch_ln<WT, float>(s->x, L.ln1g, L.ln1b, s->xn, nullptr, E, d, c.eps, nullptr, st);
-    launch_linear<WT, float, kEpiStoreAct>(lin(s->xn, d, L.wqkv, d, 3 * d, nullptr, E, s->qbuf, 3 * d, 0, nullptr), 1, st);
+    launch_linear<WT, float, kEpiStoreAct>(with_ln(lin(s->x, d, L.wqkv, d, 3 * d, nullptr, E, s->qbuf, 3 * d, 0, nullptr), L.ln1g, L.ln1b, c.eps), 1, st, pdl);
     AttnParams ap;
     memset(&ap, 0, sizeof(ap));
     ap.q = s->qbuf; ap.ldq = 3 * d; ap.out = s->attn; ap.ldo = d; ap.rows = E; ap.rows_per_b = s->max_src;
@@ -321,17 +318,16 @@ static int run_encoder(bpd_session* s) {
     ap.k = static_cast<float*>(s->qbuf) + d; ap.v = static_cast<float*>(s->qbuf) + 2 * d;
     ap.ldkv = 3 * d; ap.bstride = (long long)s->max_src * 3 * d; ap.paged = 0; ap.st = s->st;
     ap.scale = 1.0f / sqrtf((float)ap.dh); ap.by_rows = (s->B >= 8) ? 1 : 0;
-    launch_attention<float, float>(ap, st);
+    launch_attention<float, float>(ap, st, pdl);
     ++g_launches;
     LinearParams po = lin(s->attn, d, L.wo, d, d, nullptr, E, s->x, d, 0, nullptr);
-    launch_linear<WT, float, kEpiResidual>(po, 1, st);
-    launch_ln<WT, float>(s->x, L.ln2g, L.ln2b, s->xn, nullptr, E, d, c.eps, nullptr, st);
-    launch_linear<WT, float, kEpiStoreAct>(lin(s->xn, d, L.w1, d, c.d_ff, L.b1, E, s->ffh, c.d_ff, 1, nullptr), 1, st);
-    launch_linear<WT, float, kEpiResidual>(lin(s->ffh, c.d_ff, L.w2, c.d_ff, d, L.b2, E, s->x, d, 0, nullptr), 1, st);
+    launch_linear<WT, float, kEpiResidual>(po, 1, st, pdl);
+    launch_linear<WT, float, kEpiStoreAct>(with_ln(lin(s->x, d, L.w1, d, c.d_ff, L.b1, E, s->ffh, c.d_ff, 1, nullptr), L.ln2g, L.ln2b, c.eps), 1, st, pdl);
+    launch_linear<WT, float, kEpiResidual>(lin(s->ffh, c.d_ff, L.w2, c.d_ff, d, L.b2, E, s->x, d, 0, nullptr), 1, st, pdl);
   }
-  launch_ln<WT, float>(s->x, m->enc_lnf_g, m->enc_lnf_b, s->xn, nullptr, E, d, c.eps, nullptr, st);
   for (int l = 0; l < c.n_dec; ++l)
-    launch_linear<WT, float, kEpiStoreAct>(lin(s->xn, d, m->dec[l].cwkv, d, 2 * d, nullptr, E, s->crosskv[l], 2 * d, 0, nullptr), 1, st);
+    launch_linear<WT, float, kEpiStoreAct>(with_ln(lin(s->x, d, m->dec[l].cwkv, d, 2 * d, nullptr, E, s->crosskv[l], 2 * d, 0, nullptr),
+                                                   m->enc_lnf_g, m->enc_lnf_b, c.eps), 1, st, pdl);
   BPD_CUDA(cudaGetLastError());
   return BPD_OK;
 }
@@ -384,6 +380,7 @@ static int run_pass(bpd_session* s, const PassArgs& a) {
   cudaStream_t st = s->stream;
   const int d = c.d, R = s->B * a.kcur, R2 = R * a.kh;
   const int* done = s->st.all_done;
+  const bool pdl = s->use_pdl != 0;   // every kernel after the first may start while its predecessor ends
   EmbedParams ep;
   memset(&ep, 0, sizeof(ep));
   ep.table = m->tgt_embed; ep.pe = s->pe; ep.npos = s->npos; ep.x = s->x; ep.rows = R; ep.rows_per_b = a.kcur;
@@ -395,67 +392,66 @@ static int run_pass(bpd_session* s, const PassArgs& a) {
   for (int l = 0; l < c.n_dec; ++l) {
     const DecLayer& L = m->dec[l];
     // self-attention over the cache plus the causal part of the block
-    launch_ln<WT, float>(s->x, L.ln1g, L.ln1b, s->xn, nullptr, R, d, c.eps, done, st);
-    LinearParams pq = lin(s->xn, d, L.wqkv, d, 3 * d, nullptr, R, s->qbuf, d, 0, done);
+    LinearParams pq = with_ln(lin(s->x, d, L.wqkv, d, 3 * d, nullptr, R, s->qbuf, d, 0, done), L.ln1g, L.ln1b, c.eps);
     pq.d = d; pq.kcache = s->kcache[l]; pq.vcache = s->vcache[l]; pq.st = s->st; pq.rows_per_b = a.kcur;
-    launch_linear<WT, float, kEpiQkv>(pq, 1, st);
+    launch_linear<WT, float, kEpiQkv>(pq, 1, st, pdl);
     AttnParams ap;
     memset(&ap, 0, sizeof(ap));
     ap.q = s->qbuf; ap.ldq = d; ap.out = s->attn; ap.ldo = d; ap.rows = R; ap.rows_per_b = a.kcur;
     ap.H = c.H; ap.dh = d / c.H; ap.causal = 1; ap.local_q = c.local_q; ap.local_m = c.local_m;
     ap.k = s->kcache[l]; ap.v = s->vcache[l]; ap.ldkv = d;
     ap.paged = 1; ap.st = s->st; ap.scale = 1.0f / sqrtf((float)ap.dh); ap.by_rows = (s->B >= 8) ? 1 : 0; ap.all_done = done;
-    launch_attention<float, WT>(ap, st);
+    launch_attention<float, WT>(ap, st, pdl);
     ++g_launches;
-    launch_linear<WT, float, kEpiResidual>(lin(s->attn, d, L.wo, d, d, nullptr, R, s->x, d, 0, done), 1, st);
+    launch_linear<WT, float, kEpiResidual>(lin(s->attn, d, L.wo, d, d, nullptr, R, s->x, d, 0, done), 1, st, pdl);
     // cross-attention over the encoder memory
-    launch_ln<WT, float>(s->x, L.ln2g, L.ln2b, s->xn, nullptr, R, d, c.eps, done, st);
-    launch_linear<WT, float, kEpiStoreAct>(lin(s->xn, d, L.cwq, d, d, nullptr, R, s->qbuf, d, 0, done), 1, st);
+    launch_linear<WT, float, kEpiStoreAct>(with_ln(lin(s->x, d, L.cwq, d, d, nullptr, R, s->qbuf, d, 0, done), L.ln2g, L.ln2b, c.eps), 1, st, pdl);
     ap.causal = 0; ap.limit_b = s->st.src_len; ap.k = s->crosskv[l]; ap.v = static_cast<float*>(s->crosskv[l]) + d;
     ap.ldkv = 2 * d; ap.bstride = (long long)s->max_src * 2 * d; ap.paged = 0;
-    launch_attention<float, float>(ap, st);
+    launch_attention<float, float>(ap, st, pdl);
     ++g_launches;
-    launch_linear<WT, float, kEpiResidual>(lin(s->attn, d, L.cwo, d, d, nullptr, R, s->x, d, 0, done), 1, st);
+    launch_linear<WT, float, kEpiResidual>(lin(s->attn, d, L.cwo, d, d, nullptr, R, s->x, d, 0, done), 1, st, pdl);
     // feed-forward
-    launch_ln<WT, float>(s->x, L.ln3g, L.ln3b, s->xn, nullptr, R, d, c.eps, done, st);
-    launch_linear<WT, float, kEpiStoreAct>(lin(s->xn, d, L.w1, d, c.d_ff, L.b1, R, s->ffh, c.d_ff, 1, done), 1, st);
-    launch_linear<WT, float, kEpiResidual>(lin(s->ffh, c.d_ff, L.w2, c.d_ff, d, L.b2, R, s->x, d, 0, done), 1, st);
+    launch_linear<WT, float, kEpiStoreAct>(with_ln(lin(s->x, d, L.w1, d, c.d_ff, L.b1, R, s->ffh, c.d_ff, 1, done), L.ln3g, L.ln3b, c.eps), 1, st, pdl);
+    launch_linear<WT, float, kEpiResidual>(lin(s->ffh, c.d_ff, L.w2, c.d_ff, d, L.b2, R, s->x, d, 0, done), 1, st, pdl);
     if (a.layer_dump)
       BPD_CUDA(cudaMemcpyAsync(a.layer_dump + (size_t)l * R * d, s->x, sizeof(float) * R * d, cudaMemcpyDeviceToDevice, st));
   }
-  launch_ln<WT, float>(s->x, m->dec_lnf_g, m->dec_lnf_b, s->xn, s->h_f32, R, d, c.eps, done, st);
+  launch_ln<WT, float>(s->x, m->dec_lnf_g, m->dec_lnf_b, s->xn, s->h_f32, R, d, c.eps, done, st, 0, pdl);
   prof_mark(s, kProfLayers, 1);
   // proposal heads: hidden layer, k output layers with a residual from the decoder output
   const int fh = c.d_hidden;
   const long long ldu = (long long)c.k_model * fh;
   const int hid = (c.head_layout == 0) ? c.k_model * fh : a.kh * fh;
   prof_mark(s, kProfHeadW1, 0);
-  launch_linear<WT, float, kEpiStoreAct>(lin(s->xn, d, m->head_w1, d, hid, m->head_b1, R, s->u, ldu, 1, done), 1, st);
+  launch_linear<WT, float, kEpiStoreAct>(lin(s->xn, d, m->head_w1, d, hid, m->head_b1, R, s->u, ldu, 1, done), 1, st, pdl);
   prof_mark(s, kProfHeadW1, 1);
   prof_mark(s, kProfHeadW2, 0);
   if (c.head_layout == 0) {
     LinearParams ph = lin(s->u, ldu, m->head_w2, c.k_model * fh, a.kh * d, m->head_b2, R, s->o, (long long)a.kh * d, 0, done);
     ph.h = s->h_f32; ph.d = d; ph.head_identity = c.p1_identity;
-    launch_linear<WT, float, kEpiHeadOut>(ph, 1, st);
+    launch_linear<WT, float, kEpiHeadOut>(ph, 1, st, pdl);
   } else {
     LinearParams ph = lin(s->u, ldu, m->head_w2, fh, d, m->head_b2, R, s->o, (long long)a.kh * d, 0, done);
     ph.xz = fh; ph.wz = (long long)d * fh; ph.bz = d; ph.yz = d;
     ph.h = s->h_f32; ph.d = d; ph.head_identity = c.p1_identity;
-    launch_linear<WT, float, kEpiHeadOut>(ph, a.kh, st);
+    launch_linear<WT, float, kEpiHeadOut>(ph, a.kh, st, pdl);
   }
   prof_mark(s, kProfHeadW2, 1);
   // shared vocabulary projection with a fused top-1: table[b][r][i]
   prof_mark(s, kProfVocab, 0);
   if (wants_rank(a)) {
     ProposalLogitParams pl{s->o, 0, m->out_proj, s->st, s->rank, s->B, a.kcur, a.kh, d, done};
-    proposal_logit_kernel<WT><<<ceil_div(R, 4), 128, 0, st>>>(pl);
+    launch_k(proposal_logit_kernel<WT>, dim3(ceil_div(R, 4)), dim3(128), 0, st, pdl, pl);
     ++g_launches;
   }
-  launch_vocab_argmax<WT, float>(s->o, m->out_proj, R2, d, c.V, s->part_val, s->part_idx, s->counters, s->st.table,
-                              nullptr, a.logits_dump, done, st, wants_rank(a) ? &s->rank : nullptr, a.kh);
+  LinearParams pt = lin_top1(s->o, m->out_proj, R2, d, c.V, s->tc_best, s->tc_done, s->st.table, nullptr, done);
+  pt.logits = a.logits_dump;
+  if (wants_rank(a)) { pt.rank = s->rank; pt.rank_kh = a.kh; }
+  launch_linear<WT, float, kEpiArgmax>(pt, 1, st, pdl);
   prof_mark(s, kProfVocab, 1);
   VerifyParams vp = verify_params(s, a);
-  verify_commit_kernel<<<1, 32 * ceil_div(s->B, 32), 0, st>>>(vp);
+  launch_k(verify_commit_kernel, dim3(1), dim3(32 * ceil_div(s->B, 32)), 0, st, pdl, vp);
   ++g_launches;
   BPD_CUDA(cudaGetLastError());
   s->invocations += 1;
@@ -1100,14 +1096,14 @@ static int fetch(bpd_session* s, int max_new, int32_t* out_ids, int32_t* out_len
 }
 
 // ------------------------------------------------------------------ single operators
-// Scratch layout of the bf16 (tensor-core) top-1: the keys and the merge counter.
+// Scratch layout of the top-1: the keys and the merge counter.
 struct OpScratch {
   size_t best_off, done_off, total;
 };
 static OpScratch op_scratch_layout(int rows) {
   OpScratch o;
   o.best_off = 0;
-  o.done_off = (size_t)rows * tc::kBestStride * sizeof(unsigned long long);
+  o.done_off = (size_t)rows * kBestStride * sizeof(unsigned long long);
   o.total = align_up(o.done_off + sizeof(unsigned));
   return o;
 }
@@ -1696,12 +1692,9 @@ int bpd_debug_wait_timeout(int32_t* dev_word, int limit_us, void* cuda_stream) {
 }
 
 // ------------------------------------------------------------------ single operators
-size_t bpd_op_vocab_argmax_scratch_bytes(int rows, int d, int vocab, int dtype) {
+size_t bpd_op_vocab_argmax_scratch_bytes(int rows, int d, int vocab, int) {
   if (rows < 1 || vocab < 1 || d < 1) return 0;
-  if (op_use_tc(dtype)) return op_scratch_layout(rows).total;
-  const size_t tiles = ceil_div(vocab, kVocTile);
-  return align_up(tiles * rows * sizeof(float)) + align_up(tiles * rows * sizeof(int)) +
-         align_up((ceil_div(rows, kRC) + 1) * sizeof(unsigned));
+  return op_scratch_layout(rows).total;
 }
 
 int bpd_op_vocab_argmax(const void* x, const void* w, int rows, int d, int vocab, int dtype, void* scratch,
@@ -1713,27 +1706,19 @@ int bpd_op_vocab_argmax(const void* x, const void* w, int rows, int d, int vocab
   if (scratch_bytes < bpd_op_vocab_argmax_scratch_bytes(rows, d, vocab, dtype)) return fail(BPD_E_NOMEM, "scratch too small");
   cudaStream_t st = (cudaStream_t)cuda_stream;
   char* p = static_cast<char*>(scratch);
+  const OpScratch L = op_scratch_layout(rows);
+  BPD_CUDA(cudaMemsetAsync(p, 0, L.total, st));
+  unsigned* done = reinterpret_cast<unsigned*>(p + L.done_off);
+  unsigned long long* best = reinterpret_cast<unsigned long long*>(p + L.best_off);
   if (op_use_tc(dtype)) {
-    const OpScratch L = op_scratch_layout(rows);
-    BPD_CUDA(cudaMemsetAsync(p, 0, L.total, st));
     tc::Scratch sc{};
-    sc.done_counter = reinterpret_cast<unsigned*>(p + L.done_off);
-    sc.best = reinterpret_cast<unsigned long long*>(p + L.best_off);
-    sc.best_elems = (size_t)rows;
+    sc.done_counter = done; sc.best = best; sc.best_elems = (size_t)rows;
     tc::TcParams tp;
     memset(&tp, 0, sizeof(tp));
     tp.out_idx = out_idx; tp.out_val = out_val;
     return op_tc<tc::kTcArgmax>(tc::Operands{w, vocab, x, 0, d, rows, d}, vocab, d, rows, tp, sc, st);
   }
-  const size_t tiles = ceil_div(vocab, kVocTile);
-  float* pv = reinterpret_cast<float*>(p);
-  p += align_up(tiles * rows * sizeof(float));
-  int* pi = reinterpret_cast<int*>(p);
-  p += align_up(tiles * rows * sizeof(int));
-  unsigned* cnt = reinterpret_cast<unsigned*>(p);
-  BPD_CUDA(cudaMemsetAsync(cnt, 0, (ceil_div(rows, kRC) + 1) * sizeof(unsigned), st));
-  if (dtype == 0) launch_vocab_argmax<float, float>(x, w, rows, d, vocab, pv, pi, cnt, out_idx, out_val, nullptr, nullptr, st);
-  else launch_vocab_argmax<bf16, bf16>(x, w, rows, d, vocab, pv, pi, cnt, out_idx, out_val, nullptr, nullptr, st);
+  launch_linear<float, float, kEpiArgmax>(lin_top1(x, w, rows, d, vocab, best, done, out_idx, out_val, nullptr), 1, st);
   BPD_CUDA(cudaGetLastError());
   return BPD_OK;
 }
@@ -1760,8 +1745,7 @@ int bpd_op_linear(const void* x, const void* w, const void* bias, int rows, int 
     return op_tc<tc::kTcF32>(tc::Operands{w, out_f, x, 0, in_f, rows, in_f}, out_f, in_f, rows, tp, tc::Scratch{}, st);
   }
   LinearParams p = lin(x, in_f, w, in_f, out_f, bias, rows, y, out_f, relu, nullptr);
-  if (dtype == 0) launch_linear<float, float, kEpiStoreF32>(p, 1, st);
-  else launch_linear<bf16, bf16, kEpiStoreF32>(p, 1, st);
+  launch_linear<float, float, kEpiStoreF32>(p, 1, st);
   BPD_CUDA(cudaGetLastError());
   return BPD_OK;
 }

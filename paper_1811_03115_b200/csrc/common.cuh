@@ -89,6 +89,26 @@ __device__ __forceinline__ void warp_argmax(float& v, int& i) {
   }
 }
 
+// (value, index) packed so that an unsigned 64-bit max picks the larger value and, among equal values, the lower index.
+// Zero is below every real entry.  Every row's key has a 128-byte line of its own: hundreds of tiles send one atomic
+// max per row, and keys that share a line queue behind one another in L2.
+constexpr int kBestStride = 16;
+__device__ __forceinline__ unsigned order_bits(float v) {
+  const unsigned b = __float_as_uint(v);
+  return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
+}
+__device__ __forceinline__ float unpack_value(unsigned long long key) {
+  const unsigned ord = (unsigned)(key >> 32);
+  return __uint_as_float((ord & 0x80000000u) ? (ord & 0x7fffffffu) : ~ord);
+}
+// Arrival on a device-wide counter with release (our earlier writes, and those of the CTA's other threads ordered
+// before us by the barrier, become visible) and acquire (we see what earlier arrivals released).
+__device__ __forceinline__ unsigned atom_add_acq_rel(unsigned* addr, unsigned v) {
+  unsigned old;
+  asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], %2;" : "=r"(old) : "l"(addr), "r"(v) : "memory");
+  return old;
+}
+
 // Programmatic dependent launch: a kernel launched with the stream-serialization attribute may start while
 // its predecessor still runs.  launch_dependents lets the successor start early; wait blocks until the
 // predecessor grids have completed and their writes are visible.  Both are no-ops without the attribute.

@@ -759,7 +759,7 @@ __global__ void __cluster_dims__(kC, 1, 1) __launch_bounds__(kThreads, MINB) att
       }
   }
   __syncthreads();
-  if (tid == 0) *flag = (tc::atom_add_acq_rel(&p.counters[c], 1u) == (unsigned)p.H - 1) ? 1 : 0;
+  if (tid == 0) *flag = (atom_add_acq_rel(&p.counters[c], 1u) == (unsigned)p.H - 1) ? 1 : 0;
   __syncthreads();
   if (*flag) {                           // last head to arrive at this slice: heads are added in head order
     merge_slice<16>(p.x, p.ws, nullptr, p.H, p.R, d, c * slice, slice);
@@ -922,7 +922,7 @@ __global__ void __cluster_dims__(kC, 1, 1) __launch_bounds__(kThreads, MINB) ffn
       }
   }
   __syncthreads();
-  if (tid == 0) *flag = (tc::atom_add_acq_rel(&p.counters[c], 1u) == (unsigned)p.NJ - 1) ? 1 : 0;
+  if (tid == 0) *flag = (atom_add_acq_rel(&p.counters[c], 1u) == (unsigned)p.NJ - 1) ? 1 : 0;
   __syncthreads();
   if (*flag) {               // last cluster to arrive at this slice: clusters are added in cluster order
     merge_slice<12>(p.x, p.ws, p.b2, p.NJ, p.R, d, c * slice, slice);

@@ -43,9 +43,6 @@ constexpr int kBK = 64;           // K elements per pipeline stage (128 bytes of
 constexpr int kMaxStages = 4;     // pipeline depth is chosen per launch (2..4) so that two CTAs fit on an SM when possible
 constexpr int kThreads = 192;     // warp 0: TMA, warp 1: MMA + tensor-memory allocation, warps 2-5: epilogue
 constexpr int kMaxBN = 16;        // tokens per CTA (MMA N); wider launches take gemm_wide.cuh
-// Words between the top-1 keys of successive tokens: every key has a 128-byte line of its own.  Hundreds of
-// tiles send one atomic max per token; keys that share a line queue behind one another in L2.
-constexpr int kBestStride = 16;
 constexpr unsigned long long kSpinCycles = 2000000000ull;   // about a second
 
 enum TcEpilogue {
@@ -195,26 +192,6 @@ __device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t saddr) {
 // Instruction descriptor: bf16 x bf16 -> fp32, both operands K-major, M = 128.
 __device__ __forceinline__ uint32_t instr_desc_bf16(int n) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(kBM >> 4) << 24);
-}
-
-// (value, index) packed so that an unsigned 64-bit max picks the larger value and, among equal values, the
-// lower index.  Zero is below every real entry.
-__device__ __forceinline__ unsigned long long pack_best(float v, int idx) {
-  const unsigned b = __float_as_uint(v);
-  const unsigned ord = (b & 0x80000000u) ? ~b : (b | 0x80000000u);
-  return ((unsigned long long)ord << 32) | (unsigned long long)(0xffffffffu - (unsigned)idx);
-}
-__device__ __forceinline__ float unpack_value(unsigned long long key) {
-  const unsigned ord = (unsigned)(key >> 32);
-  return __uint_as_float((ord & 0x80000000u) ? (ord & 0x7fffffffu) : ~ord);
-}
-
-// Arrival on a device-wide counter with release (our earlier writes, and those of the CTA's other threads
-// ordered before us by the barrier, become visible) and acquire (we see what earlier arrivals released).
-__device__ __forceinline__ unsigned atom_add_acq_rel(unsigned* addr, unsigned v) {
-  unsigned old;
-  asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], %2;" : "=r"(old) : "l"(addr), "r"(v) : "memory");
-  return old;
 }
 
 __device__ __forceinline__ void split_bf16(float v, bf16& hi, bf16& lo) {

@@ -229,7 +229,8 @@ enum Epilogue {
   kEpiStoreF32 = 1,  // y_f32[r][n] = act(v + bias)
   kEpiResidual = 2,  // x_f32[r][n] += v + bias
   kEpiQkv = 3,       // n < d: q[r][n]; else key / value into the paged cache at position len[b] + i
-  kEpiHeadOut = 4    // o[r][n] = v + bias + h[r][n mod d]   (residual to each of the k outputs)
+  kEpiHeadOut = 4,   // o[r][n] = v + bias + h[r][n mod d]   (residual to each of the k outputs)
+  kEpiArgmax = 5     // per-row top-1 over all features, optional logits dump and rank counting
 };
 
 struct LinearParams {
@@ -245,12 +246,21 @@ struct LinearParams {
   void* kcache; void* vcache;     // kEpiQkv
   RowState st; int rows_per_b;
   const int* all_done;
+  // layer norm of x's rows on the way in (K is the model width then), or null
+  const void* ln_g; const void* ln_b; float ln_eps;
+  // kEpiArgmax: packed (orderable value, ~index) per row, kBestStride words apart, zero between launches; CTAs that are
+  // done, zero between launches
+  unsigned long long* best; unsigned* done_counter;
+  int* out_idx; float* out_val; float* logits;
+  RankState rank; int rank_kh;    // top-n acceptance: count entries beating each proposal (rank.cnt null = off)
 };
 
-constexpr int kRC = 8;      // rows per CTA pass
-constexpr int kFPW = 4;     // output features per warp
-constexpr int kKT = 512;    // K tile staged in shared memory
-constexpr int kLinWarps = 8;
+constexpr int kTileN = 32;      // features per CTA
+constexpr int kTileK = 64;      // K columns staged at a time
+constexpr int kTilePitch = kTileK + 4;   // floats between staged rows: 16-byte reads of 8 consecutive rows hit all banks once
+constexpr int kTileGroups = 4;  // thread groups that share a K tile
+constexpr int kTileThreads = 256;
+constexpr int kArgmaxMaxD = 1024;
 
 template <typename WT, typename AT, int EPI>
 __device__ __forceinline__ void linear_epilogue(const LinearParams& p, int z, int r, int n, float v) {
@@ -284,72 +294,208 @@ __device__ __forceinline__ void linear_epilogue(const LinearParams& p, int z, in
   }
 }
 
-// One warp owns kFPW output features and kRC rows; its lanes split K, each
-// accumulating in increasing-k order, then a butterfly sum.  The order depends
-// only on K, never on the number of rows.
-template <typename WT, typename AT, int EPI>
-__global__ void __launch_bounds__(kLinWarps * 32) linear_kernel(LinearParams p) {
+// A CTA computes 32 features x 8 RPT rows.  K tiles of 64 columns of both operands are staged in shared memory, the
+// loads of the next ones in flight; four groups of 64 threads take 16 columns of every tile each, a thread 4 features x
+// RPT rows of it.  The groups' sums are added in group order: the order of a sum depends on K alone, never on the number
+// of rows.  The model's own layer norm is applied to x on the way in where a projection follows one, which saves its
+// launch.  Shared-memory reads bound the loop (4 + RPT 16-byte reads for 16 RPT FMAs), so launches of few rows take a tile
+// of few rows; the rest of a small launch is latency (about 2.5 us in a dependent chain), which is why the first weight
+// tiles are requested before the dependency wait.
+template <typename WT, typename AT, int EPI, int RPT>
+__global__ void __launch_bounds__(kTileThreads, 2) linear_kernel(const __grid_constant__ LinearParams p) {
   pdl_launch_dependents();
-  pdl_wait();
-  if (p.all_done && *p.all_done) return;
-  __shared__ __align__(16) float xs[kRC][kKT];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  constexpr int TR = 8 * RPT, AHEAD = RPT == 1 ? 4 : (RPT == 2 ? 3 : (RPT == 4 ? 2 : 1));
+  constexpr int kStage = (kTileN + TR) * kTilePitch, kSums = kTileGroups * TR * kTileN;
+  __shared__ __align__(16) float s_stage[kStage > kSums ? kStage : kSums];           // weight tile, activation tile; then the groups' sums
+  __shared__ float s_mean[TR], s_rstd[TR];
+  __shared__ unsigned s_last;
+  float* ws = s_stage;
+  float* xs = s_stage + kTileN * kTilePitch;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int z = blockIdx.z;
   const AT* X = reinterpret_cast<const AT*>(p.x) + z * p.xz;
   const WT* W = reinterpret_cast<const WT*>(p.w) + z * p.wz;
-  const int r0 = blockIdx.y * kRC;
-  const int nr = min(kRC, p.rows - r0);
-  const int n0 = blockIdx.x * (kLinWarps * kFPW) + warp * kFPW;
-  float acc[kFPW][kRC];
+  const int n0 = blockIdx.x * kTileN, r0 = blockIdx.y * TR;
+  const int nr = min(TR, p.rows - r0);
+  // staging: thread -> row tid / 8, eight columns (tid % 8) * 8 of it
+  const int srow = tid >> 3, scol = (tid & 7) * 8;
+  constexpr int XS = TR <= 32 ? 1 : TR / 32;          // rows of x a thread stages
+  const bool w_live = n0 + srow < p.N;
+  const WT* wsrc = W + (long long)(n0 + srow) * p.ldw + scol;
+  const AT* xsrc = X + (long long)(r0 + srow) * p.ldx + scol;
+  float wv[AHEAD][8], xv[AHEAD][XS][8];
+  auto fetch_w = [&](int kt, float (&v)[8]) {
+    if (w_live && kt + scol < p.K) load8_stream(wsrc + kt, v);
+    else {
 #pragma unroll
-  for (int f = 0; f < kFPW; ++f)
-#pragma unroll
-    for (int r = 0; r < kRC; ++r) acc[f][r] = 0.f;
-
-  for (int kt = 0; kt < p.K; kt += kKT) {
-    __syncthreads();
-    for (int v = threadIdx.x; v < kRC * kKT / 8; v += kLinWarps * 32) {
-      const int r = v / (kKT / 8), kk = (v % (kKT / 8)) * 8;
-      float t[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-      if (r < nr && kt + kk < p.K) load8(X + (long long)(r0 + r) * p.ldx + kt + kk, t);
-      *reinterpret_cast<float4*>(&xs[r][kk]) = make_float4(t[0], t[1], t[2], t[3]);
-      *reinterpret_cast<float4*>(&xs[r][kk + 4]) = make_float4(t[4], t[5], t[6], t[7]);
+      for (int e = 0; e < 8; ++e) v[e] = 0.f;
     }
-    __syncthreads();
+  };
+  auto fetch_x = [&](int kt, float (&v)[XS][8]) {
 #pragma unroll
-    for (int c = 0; c < kKT / 256; ++c) {
-      const int kk = c * 256 + lane * 8;
-      if (kt + kk < p.K) {
-        float wv[kFPW][8];
+    for (int q = 0; q < XS; ++q) {
+      if (srow + 32 * q < nr && kt + scol < p.K) load8(xsrc + (long long)(32 * q) * p.ldx + kt, v[q]);
+      else {
 #pragma unroll
-        for (int f = 0; f < kFPW; ++f) {
-          if (n0 + f < p.N) {
-            load8_stream(W + (long long)(n0 + f) * p.ldw + kt + kk, wv[f]);
-          } else {
-#pragma unroll
-            for (int e = 0; e < 8; ++e) wv[f][e] = 0.f;
-          }
-        }
-#pragma unroll
-        for (int r = 0; r < kRC; ++r) {
-          const float4 a = *reinterpret_cast<const float4*>(&xs[r][kk]);
-          const float4 b = *reinterpret_cast<const float4*>(&xs[r][kk + 4]);
-          const float xv[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
-#pragma unroll
-          for (int f = 0; f < kFPW; ++f)
-#pragma unroll
-            for (int e = 0; e < 8; ++e) acc[f][r] = fmaf(wv[f][e], xv[e], acc[f][r]);
-        }
+        for (int e = 0; e < 8; ++e) v[q][e] = 0.f;
       }
     }
-  }
+  };
 #pragma unroll
-  for (int f = 0; f < kFPW; ++f)
+  for (int s = 0; s < AHEAD; ++s) fetch_w(s * kTileK, wv[s]);    // weights do not depend on the preceding launch
+  pdl_wait();
+  if (p.all_done && *p.all_done) return;
 #pragma unroll
-    for (int r = 0; r < kRC; ++r) {
-      const float v = warp_sum(acc[f][r]);
-      if (lane == f * kRC + r && r < nr && n0 + f < p.N) linear_epilogue<WT, AT, EPI>(p, z, r0 + r, n0 + f, v);
+  for (int s = 0; s < AHEAD; ++s) fetch_x(s * kTileK, xv[s]);
+  if (p.ln_g) {
+    // statistics of the rows: a warp takes RPT of them, one after the other, two passes over a row held in registers
+#pragma unroll 1
+    for (int q = 0; q < RPT; ++q) {
+      const float* row = reinterpret_cast<const float*>(p.x) + (long long)min(r0 + warp * RPT + q, p.rows - 1) * p.ldx;
+      float4 v[kArgmaxMaxD / 128];
+      float sum = 0.f, sq = 0.f;
+#pragma unroll
+      for (int i = 0; i < kArgmaxMaxD / 128; ++i) {
+        const int c = i * 128 + lane * 4;
+        v[i] = c < p.K ? *reinterpret_cast<const float4*>(row + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+        sum += (v[i].x + v[i].y) + (v[i].z + v[i].w);
+      }
+      const float mean = warp_sum(sum) / (float)p.K;
+#pragma unroll
+      for (int i = 0; i < kArgmaxMaxD / 128; ++i) {
+        if (i * 128 + lane * 4 < p.K) {
+          const float a = v[i].x - mean, b = v[i].y - mean, c = v[i].z - mean, d = v[i].w - mean;
+          sq += (a * a + b * b) + (c * c + d * d);
+        }
+      }
+      sq = warp_sum(sq);
+      if (lane == 0) { s_mean[warp * RPT + q] = mean; s_rstd[warp * RPT + q] = rsqrtf(sq / (float)p.K + p.ln_eps); }
     }
+    __syncthreads();
+  }
+  const int grp = tid >> 6, fx = tid & 7, ry = (tid >> 3) & 7;   // K group, features fx + 8 i, rows ry + 8 j
+  float acc[4][RPT];
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < RPT; ++j) acc[i][j] = 0.f;
+  for (int kt0 = 0; kt0 < p.K; kt0 += AHEAD * kTileK) {
+#pragma unroll
+  for (int s = 0; s < AHEAD; ++s) {
+    const int kt = kt0 + s * kTileK;
+    if (kt >= p.K) break;
+    if (kt > 0) __syncthreads();               // the previous tile has been used
+    float* wd = ws + srow * kTilePitch + scol;
+    *reinterpret_cast<float4*>(wd) = make_float4(wv[s][0], wv[s][1], wv[s][2], wv[s][3]);
+    *reinterpret_cast<float4*>(wd + 4) = make_float4(wv[s][4], wv[s][5], wv[s][6], wv[s][7]);
+#pragma unroll
+    for (int q = 0; q < XS; ++q) {
+      const int row = srow + 32 * q;
+      if (TR < 32 && row >= TR) break;
+      float (&v)[8] = xv[s][q];
+      if (p.ln_g && row < nr && kt + scol < p.K) {
+        float g[8], b[8];
+        load8(reinterpret_cast<const WT*>(p.ln_g) + kt + scol, g);
+        load8(reinterpret_cast<const WT*>(p.ln_b) + kt + scol, b);
+        const float mean = s_mean[row], rstd = s_rstd[row];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) v[e] = (v[e] - mean) * rstd * g[e] + b[e];
+      }
+      float* xd = xs + row * kTilePitch + scol;
+      *reinterpret_cast<float4*>(xd) = make_float4(v[0], v[1], v[2], v[3]);
+      *reinterpret_cast<float4*>(xd + 4) = make_float4(v[4], v[5], v[6], v[7]);
+    }
+    __syncthreads();
+    if (kt + AHEAD * kTileK < p.K) { fetch_w(kt + AHEAD * kTileK, wv[s]); fetch_x(kt + AHEAD * kTileK, xv[s]); }
+#pragma unroll
+    for (int kk = 0; kk < kTileK / kTileGroups; kk += 4) {
+      const int col = grp * (kTileK / kTileGroups) + kk;
+      float4 a[4], b[RPT];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) a[i] = *reinterpret_cast<const float4*>(ws + (fx + 8 * i) * kTilePitch + col);
+#pragma unroll
+      for (int j = 0; j < RPT; ++j) b[j] = *reinterpret_cast<const float4*>(xs + (ry + 8 * j) * kTilePitch + col);
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < RPT; ++j) {
+          acc[i][j] = fmaf(a[i].x, b[j].x, acc[i][j]);
+          acc[i][j] = fmaf(a[i].y, b[j].y, acc[i][j]);
+          acc[i][j] = fmaf(a[i].z, b[j].z, acc[i][j]);
+          acc[i][j] = fmaf(a[i].w, b[j].w, acc[i][j]);
+        }
+    }
+  }
+  }
+  // the groups' sums: [group][row][feature], added in group order; a warp finishes 32 consecutive features of a row
+  __syncthreads();
+  float* red = s_stage;
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < RPT; ++j) red[(grp * TR + ry + 8 * j) * kTileN + fx + 8 * i] = acc[i][j];
+  __syncthreads();
+  const int n = n0 + lane;
+  float out[RPT];
+#pragma unroll
+  for (int q = 0; q < RPT; ++q) {
+    const int row = warp + 8 * q;
+    out[q] = red[row * kTileN + lane];
+#pragma unroll
+    for (int g = 1; g < kTileGroups; ++g) out[q] += red[(g * TR + row) * kTileN + lane];
+  }
+  if constexpr (EPI != kEpiArgmax) {
+#pragma unroll
+    for (int q = 0; q < RPT; ++q) {
+      const int row = warp + 8 * q;
+      if (row < nr && n < p.N) linear_epilogue<WT, AT, EPI>(p, z, r0 + row, n, out[q]);
+    }
+  } else {
+#pragma unroll
+    for (int q = 0; q < RPT; ++q) {
+      const int row = warp + 8 * q, r = r0 + row;
+      if (row >= nr) break;                                     // uniform over the warp
+      const unsigned ord = n < p.N ? order_bits(out[q]) : 0u;
+      const unsigned m = __reduce_max_sync(0xffffffffu, ord);
+      const int first = __ffs(__ballot_sync(0xffffffffu, ord == m)) - 1;   // lanes grow with the feature index
+      if (lane == 0)
+        atomicMax(&p.best[(size_t)r * kBestStride], ((unsigned long long)m << 32) | (unsigned long long)(0xffffffffu - (unsigned)(n0 + first)));
+      if (p.logits && n < p.N) p.logits[(size_t)r * p.N + n] = out[q];
+      if (p.rank.cnt && r % p.rank_kh == 0) {
+        const int pr = r / p.rank_kh, tok = p.rank.tok[pr];
+        const unsigned beats = __ballot_sync(0xffffffffu, tok >= 0 && n < p.N && n != tok && better(out[q], n, p.rank.thr[pr], tok));
+        if (lane == 0 && beats) atomicAdd(&p.rank.cnt[pr], __popc(beats));
+      }
+    }
+    // the CTA that completes the last tile hands the winners out
+    __syncthreads();
+    if (tid == 0) s_last = (atom_add_acq_rel(p.done_counter, 1u) == gridDim.x * gridDim.y - 1) ? 1u : 0u;
+    __syncthreads();
+    if (s_last) {
+      for (int r = tid; r < p.rows; r += kTileThreads) {
+        const unsigned long long key = __ldcg(&p.best[(size_t)r * kBestStride]);
+        p.out_idx[r] = (int)(0xffffffffu - (unsigned)(key & 0xffffffffull));
+        if (p.out_val) p.out_val[r] = unpack_value(key);
+        p.best[(size_t)r * kBestStride] = 0ull;                 // ready for the next launch
+      }
+      if (tid == 0) *p.done_counter = 0;
+    }
+  }
+}
+
+// Rows per thread for a launch of `rows` rows: the smallest tile that holds them; beyond 64 rows the reads per FMA of the
+// widest tile count for more than the CTAs it saves on.
+inline int linear_rows_per_thread(int rows) { return rows <= 8 ? 1 : (rows <= 16 ? 2 : (rows <= 64 ? 4 : 8)); }
+template <typename WT, typename AT, int EPI>
+inline void launch_linear_tiles(const LinearParams& p, int zcount, cudaStream_t st, bool pdl) {
+  const int rpt = linear_rows_per_thread(p.rows);
+  const dim3 grid((p.N + kTileN - 1) / kTileN, (p.rows + 8 * rpt - 1) / (8 * rpt), zcount), block(kTileThreads);
+  switch (rpt) {
+    case 1: launch_k(linear_kernel<WT, AT, EPI, 1>, grid, block, 0, st, pdl, p); break;
+    case 2: launch_k(linear_kernel<WT, AT, EPI, 2>, grid, block, 0, st, pdl, p); break;
+    case 4: launch_k(linear_kernel<WT, AT, EPI, 4>, grid, block, 0, st, pdl, p); break;
+    default: launch_k(linear_kernel<WT, AT, EPI, 8>, grid, block, 0, st, pdl, p); break;
+  }
 }
 
 // ------------------------------------------------------------------ attention (one warp per (row, head))
@@ -1015,132 +1161,6 @@ __global__ void __launch_bounds__(128) proposal_logit_kernel(ProposalLogitParams
     thr = warp_sum(acc);
   }
   if (lane == 0) { p.rank.tok[pr] = tok; p.rank.thr[pr] = thr; p.rank.cnt[pr] = 0; }
-}
-
-// ------------------------------------------------------------------ vocabulary projection + top-1
-struct ArgmaxParams {
-  const void* x; long long ldx;   // [rows, d] activations
-  const void* w;                  // [V, d]
-  int rows, d, V;
-  float* part_val; int* part_idx; // [tiles][rows] workspace
-  unsigned* counters;             // [row chunks], zero between launches
-  int* out_idx; float* out_val;   // [rows]
-  float* logits;                  // optional dump [rows, V]
-  const int* all_done;
-  RankState rank; int rank_kh;    // top-n acceptance: count entries beating each proposal (rank.cnt null = off)
-};
-constexpr int kVocTile = 256;     // vocabulary rows per CTA
-constexpr int kArgmaxMaxD = 1024;
-
-template <typename WT, typename AT>
-__global__ void __launch_bounds__(kLinWarps * 32) vocab_argmax_kernel(ArgmaxParams p) {
-  pdl_launch_dependents();
-  pdl_wait();
-  if (p.all_done && *p.all_done) return;
-  extern __shared__ __align__(16) float xs_dyn[];   // [kRC][d]
-  __shared__ float sv[kLinWarps][kRC];
-  __shared__ int si[kLinWarps][kRC];
-  __shared__ unsigned ticket;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int r0 = blockIdx.y * kRC;
-  const int nr = min(kRC, p.rows - r0);
-  const int d = p.d;
-  const AT* X = reinterpret_cast<const AT*>(p.x);
-  const WT* W = reinterpret_cast<const WT*>(p.w);
-  for (int v = threadIdx.x; v < kRC * d / 8; v += kLinWarps * 32) {
-    const int r = v / (d / 8), kk = (v % (d / 8)) * 8;
-    float t[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    if (r < nr) load8(X + (long long)(r0 + r) * p.ldx + kk, t);
-    *reinterpret_cast<float4*>(&xs_dyn[r * d + kk]) = make_float4(t[0], t[1], t[2], t[3]);
-    *reinterpret_cast<float4*>(&xs_dyn[r * d + kk + 4]) = make_float4(t[4], t[5], t[6], t[7]);
-  }
-  __syncthreads();
-  float bv[kRC];
-  int bi[kRC];
-#pragma unroll
-  for (int r = 0; r < kRC; ++r) { bv[r] = -INFINITY; bi[r] = 0x7fffffff; }
-  const int tile0 = blockIdx.x * kVocTile;
-  for (int g = 0; g < kVocTile / (kLinWarps * kFPW); ++g) {
-    const int n0 = tile0 + g * (kLinWarps * kFPW) + warp * kFPW;   // ascending over g for a given warp
-    if (n0 >= p.V) break;
-    float acc[kFPW][kRC];
-#pragma unroll
-    for (int f = 0; f < kFPW; ++f)
-#pragma unroll
-      for (int r = 0; r < kRC; ++r) acc[f][r] = 0.f;
-    for (int kk = lane * 8; kk < d; kk += 256) {
-      float wv[kFPW][8];
-#pragma unroll
-      for (int f = 0; f < kFPW; ++f) {
-        if (n0 + f < p.V) {
-          load8_stream(W + (size_t)(n0 + f) * d + kk, wv[f]);
-        } else {
-#pragma unroll
-          for (int e = 0; e < 8; ++e) wv[f][e] = 0.f;
-        }
-      }
-#pragma unroll
-      for (int r = 0; r < kRC; ++r) {
-        const float4 a = *reinterpret_cast<const float4*>(&xs_dyn[r * d + kk]);
-        const float4 b = *reinterpret_cast<const float4*>(&xs_dyn[r * d + kk + 4]);
-        const float xv[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
-#pragma unroll
-        for (int f = 0; f < kFPW; ++f)
-#pragma unroll
-          for (int e = 0; e < 8; ++e) acc[f][r] = fmaf(wv[f][e], xv[e], acc[f][r]);
-      }
-    }
-#pragma unroll
-    for (int f = 0; f < kFPW; ++f)
-#pragma unroll
-      for (int r = 0; r < kRC; ++r) {
-        const float v = warp_sum(acc[f][r]);
-        if (n0 + f < p.V) {
-          if (p.rank.cnt && lane == 0 && r < nr && (r0 + r) % p.rank_kh == 0) {
-            const int pr = (r0 + r) / p.rank_kh, tok = p.rank.tok[pr];
-            if (tok >= 0 && tok != n0 + f && better(v, n0 + f, p.rank.thr[pr], tok)) atomicAdd(&p.rank.cnt[pr], 1);
-          }
-          if (better(v, n0 + f, bv[r], bi[r])) { bv[r] = v; bi[r] = n0 + f; }
-          if (p.logits && lane == f * kRC + r && r < nr) p.logits[(size_t)(r0 + r) * p.V + n0 + f] = v;
-        }
-      }
-  }
-  if (lane == 0) {
-#pragma unroll
-    for (int r = 0; r < kRC; ++r) { sv[warp][r] = bv[r]; si[warp][r] = bi[r]; }
-  }
-  __syncthreads();
-  if (threadIdx.x < nr) {
-    const int r = threadIdx.x;
-    float v = sv[0][r];
-    int ix = si[0][r];
-    for (int w2 = 1; w2 < kLinWarps; ++w2)
-      if (better(sv[w2][r], si[w2][r], v, ix)) { v = sv[w2][r]; ix = si[w2][r]; }
-    p.part_val[(size_t)blockIdx.x * p.rows + r0 + r] = v;
-    p.part_idx[(size_t)blockIdx.x * p.rows + r0 + r] = ix;
-  }
-  // The CTA that finishes last for this row chunk merges all tiles (no waiting on anyone).
-  __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0) ticket = atomicAdd(&p.counters[blockIdx.y], 1u);
-  __syncthreads();
-  if (ticket != gridDim.x - 1) return;
-  __threadfence();
-  for (int r = warp; r < nr; r += kLinWarps) {
-    float v = -INFINITY;
-    int ix = 0x7fffffff;
-    for (int t = lane; t < (int)gridDim.x; t += 32) {
-      const float tv = __ldcg(&p.part_val[(size_t)t * p.rows + r0 + r]);
-      const int ti = __ldcg(&p.part_idx[(size_t)t * p.rows + r0 + r]);
-      if (better(tv, ti, v, ix)) { v = tv; ix = ti; }
-    }
-    warp_argmax(v, ix);
-    if (lane == 0) {
-      p.out_idx[r0 + r] = ix;
-      if (p.out_val) p.out_val[r0 + r] = v;
-    }
-  }
-  if (threadIdx.x == 0) p.counters[blockIdx.y] = 0;
 }
 
 // ------------------------------------------------------------------ verify / accept / commit / select next

@@ -10,13 +10,10 @@ namespace bpd {
 
 constexpr int kNoAllocMaxRows = 256;
 constexpr int kNoAllocMaxVocab = 65536;
-constexpr int kNoAllocMaxTiles = kNoAllocMaxVocab / kVocTile;
-constexpr size_t kNoAllocValBytes = (size_t)kNoAllocMaxTiles * kNoAllocMaxRows * sizeof(float);
-constexpr size_t kNoAllocIdxBytes = (size_t)kNoAllocMaxTiles * kNoAllocMaxRows * sizeof(int);
-constexpr size_t kNoAllocCntBytes = 256;   // one counter per group of kRC rows: 32 of them, padded
-constexpr size_t kNoAllocBytes = kNoAllocValBytes + kNoAllocIdxBytes + kNoAllocCntBytes;
+constexpr size_t kNoAllocKeys = (size_t)kNoAllocMaxRows * kBestStride * sizeof(unsigned long long);
+constexpr size_t kNoAllocBytes = kNoAllocKeys + 256;   // the counter first, the keys behind it
 
-// 512 KiB + 256 B of global memory on every GPU that loads this library, held until the process exits.
+// 32 KiB of global memory on every GPU that loads this library, held until the process exits.
 // In host code this name is only a handle for the runtime, not a device address.
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocBytes];
 
@@ -59,16 +56,15 @@ extern "C" int bpd_op_vocab_argmax_noalloc(const void* x, const void* w, int row
   int rc = noalloc_scratch(&base);
   if (rc) return rc;
   cudaStream_t st = (cudaStream_t)cuda_stream;
-  float* part_val = reinterpret_cast<float*>(base);
-  int* part_idx = reinterpret_cast<int*>(base + kNoAllocValBytes);
-  unsigned* counters = reinterpret_cast<unsigned*>(base + kNoAllocValBytes + kNoAllocIdxBytes);
-  // the array keeps whatever the previous call left: the arrival counters must start at zero
-  BPD_CUDA(cudaMemsetAsync(counters, 0, kNoAllocCntBytes, st));
-  ArgmaxParams p{x, (long long)d, w, rows, d, vocab, part_val, part_idx, counters, out_idx, out_val, nullptr, nullptr};
-  dim3 grid((vocab + kVocTile - 1) / kVocTile, (rows + kRC - 1) / kRC);
-  const size_t smem = (size_t)kRC * d * sizeof(float);
-  if (dtype == 0) vocab_argmax_kernel<float, float><<<grid, kLinWarps * 32, smem, st>>>(p);
-  else vocab_argmax_kernel<bf16, bf16><<<grid, kLinWarps * 32, smem, st>>>(p);
+  // the array keeps whatever the previous call left: counter and keys must start at zero
+  BPD_CUDA(cudaMemsetAsync(base, 0, 256 + (size_t)rows * kBestStride * sizeof(unsigned long long), st));
+  LinearParams p;
+  memset(&p, 0, sizeof(p));
+  p.x = x; p.ldx = d; p.w = w; p.ldw = d; p.rows = rows; p.K = d; p.N = vocab;
+  p.done_counter = reinterpret_cast<unsigned*>(base); p.best = reinterpret_cast<unsigned long long*>(base + 256);
+  p.out_idx = out_idx; p.out_val = out_val; p.rank_kh = 1;
+  if (dtype == 0) launch_linear_tiles<float, float, kEpiArgmax>(p, 1, st, false);
+  else launch_linear_tiles<bf16, bf16, kEpiArgmax>(p, 1, st, false);
   ++g_launches;
   BPD_CUDA(cudaGetLastError());
   return BPD_OK;

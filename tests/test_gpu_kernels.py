@@ -29,3 +29,23 @@ def test_wide_projection_at_tile_edges(bpd, rows, in_f, out_f):
     picked = logits[np.arange(rows), idx.cpu().numpy()]
     np.testing.assert_allclose(picked, logits.max(-1), atol=1e-4)
     np.testing.assert_allclose(val.cpu().numpy(), logits.max(-1), atol=1e-4)
+
+
+# row tiles of 8, 16, 32 and 64 rows, K tiles of 64 columns, feature tiles of 32
+@pytest.mark.parametrize("rows,in_f,out_f", [(1, 8, 1), (8, 64, 32), (9, 72, 33), (16, 1024, 31), (17, 136, 65), (64, 200, 96), (65, 64, 40),
+                                             (129, 520, 7)])
+def test_fp32_projection_at_tile_edges(bpd, rows, in_f, out_f):
+    import torch
+    g = torch.Generator().manual_seed(rows + in_f)
+    x = torch.randn(rows, in_f, generator=g)
+    w = torch.randn(out_f, in_f, generator=g) * 0.05
+    b = torch.randn(out_f, generator=g) * 0.1
+    want = x.double().numpy() @ w.double().numpy().T
+    got = bpd.bpd_op_linear(x.cuda(), w.cuda(), b.cuda(), relu=True).cpu().numpy()
+    np.testing.assert_allclose(got, np.maximum(want + b.double().numpy(), 0), atol=2e-6 * np.sqrt(in_f))
+    idx, val = bpd.bpd_op_vocab_argmax(x.cuda(), w.cuda(), want_val=True)
+    idx2, val2 = torch.zeros(rows, dtype=torch.int32, device="cuda"), torch.zeros(rows, device="cuda")
+    bpd.bpd_op_vocab_argmax_noalloc(x.cuda(), w.cuda(), idx2, val2)
+    for i, v in ((idx, val), (idx2, val2)):
+        np.testing.assert_allclose(want[np.arange(rows), i.cpu().numpy()], want.max(-1), atol=1e-5)
+        np.testing.assert_allclose(v.cpu().numpy(), want.max(-1), atol=1e-5)
