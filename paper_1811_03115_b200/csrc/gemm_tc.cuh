@@ -59,6 +59,10 @@ struct TcParams {
   int bn;                      // MMA N: T rounded up to 16 (per token tile)
   int splits;                  // grid.y
   int chunks_per_split;        // K chunks (of kBK) each split owns
+  // few-row kernel: a split's chunks are summed in `groups` (1 or 8) groups of group_chunks, the groups' sums as a binary
+  // tree; `fine` CTAs share a split, each a subtree, so a launch of few feature tiles can use more CTAs and still
+  // add up in the order of the launch it was planned for
+  int groups, group_chunks, fine;
   const bf16* bias;            // [N] or null
   int relu;
   // outputs
@@ -297,8 +301,35 @@ struct EpiShared {
 struct EpiUnit {
   uint32_t tmem, acc_bar, acc_parity;
   int tile, split, slice, zidx, ntiles, t0, nt, bn, nchunks;
+  int acc_groups, acc_live;     // sub-accumulators of this CTA (16 columns each), those with chunks
   bool skip;
 };
+// Sum of the CTA's sub-accumulators (16 tensor-memory columns each) for this thread's lane: a binary tree over `groups`
+// (1, 2, 4 or 8), of which the first `live` hold anything.
+__device__ __forceinline__ void sum_groups(uint32_t taddr, int groups, int live, float (&v)[16]) {
+  auto leaf = [&](int g, float (&x)[16]) {
+    if (g < live) tmem_ld16(taddr + g * 16, x);
+    else {
+#pragma unroll
+      for (int c = 0; c < 16; ++c) x[c] = 0.f;
+    }
+  };
+  auto add = [](float (&x)[16], const float (&y)[16]) {
+#pragma unroll
+    for (int c = 0; c < 16; ++c) x[c] += y[c];
+  };
+  leaf(0, v);
+  if (groups > 1) { float a[16]; leaf(1, a); add(v, a); }
+  if (groups > 2) { float a[16], b[16]; leaf(2, a); leaf(3, b); add(a, b); add(v, a); }
+  if (groups > 4) {
+    float a[16], b[16], c[16];
+    leaf(4, a); leaf(5, b); add(a, b);
+    leaf(6, b); leaf(7, c); add(b, c);
+    add(a, b);
+    add(v, a);
+  }
+}
+
 template <int EPI>
 __device__ __forceinline__ void tc_epilogue(const TcParams& p, const EpiShared& sh, const EpiUnit& u, int warp, int lane) {
   float* s_mean = sh.s_mean;
@@ -361,30 +392,20 @@ __device__ __forceinline__ void tc_epilogue(const TcParams& p, const EpiShared& 
   const bool direct = (p.splits == 1);
   float* wsz = p.ws + ((size_t)u.zidx * ntiles + tile) * p.splits * (size_t)bn * kBM;
   if (ok) {
+    float v[16];
+    sum_groups(tmem + ((uint32_t)(q * 32) << 16), u.acc_groups, u.acc_live, v);
     if (direct) {
-      for (int cb = 0; cb < bn; cb += 16) {
-        float v[16];
-        tmem_ld16(tmem + ((uint32_t)(q * 32) << 16) + cb, v);
-        if (n < p.N) {
-          const float lo8[8] = {v[0], v[1], v[2], v[3], v[4], v[5], v[6], v[7]};
-          const float hi8[8] = {v[8], v[9], v[10], v[11], v[12], v[13], v[14], v[15]};
-          tc_store8<EPI>(p, slice, t0 + cb, min(8, nt - cb), n, lo8, s_mean, s_rstd, cb, s_slot);
-          tc_store8<EPI>(p, slice, t0 + cb + 8, min(8, nt - cb - 8), n, hi8, s_mean, s_rstd, cb + 8, s_slot);
-        }
+      if (n < p.N) {
+        const float lo8[8] = {v[0], v[1], v[2], v[3], v[4], v[5], v[6], v[7]};
+        const float hi8[8] = {v[8], v[9], v[10], v[11], v[12], v[13], v[14], v[15]};
+        tc_store8<EPI>(p, slice, t0, min(8, nt), n, lo8, s_mean, s_rstd, 0, s_slot);
+        tc_store8<EPI>(p, slice, t0 + 8, min(8, nt - 8), n, hi8, s_mean, s_rstd, 8, s_slot);
       }
     } else {
       // partial tile -> workspace [split][token][128], coalesced over features
-      for (int cb = 0; cb < bn; cb += 16) {
-        float v[16];
-        if (nchunks > 0) tmem_ld16(tmem + ((uint32_t)(q * 32) << 16) + cb, v);
-        else {
 #pragma unroll
-          for (int c = 0; c < 16; ++c) v[c] = 0.f;
-        }
-#pragma unroll
-        for (int c = 0; c < 16; ++c)
-          if (cb + c < nt) wsz[((size_t)split * bn + cb + c) * kBM + row] = v[c];
-      }
+      for (int c = 0; c < 16; ++c)
+        if (c < nt) wsz[((size_t)split * bn + c) * kBM + row] = v[c];
       asm volatile("bar.sync 1, 128;" ::: "memory");
       if (et == 0) {
         BPD_TC_STAMP(6);
@@ -409,10 +430,30 @@ __device__ __forceinline__ void tc_epilogue(const TcParams& p, const EpiShared& 
               for (int c = 0; c < G; ++c)
                 v[ss][c] = (s0 + ss < p.splits && cg + c < nt)
                                ? __ldcg(&wsz[((size_t)(s0 + ss) * bn + cg + c) * kBM + row]) : 0.f;
+            // the `fine` parts of a split first (a binary tree), then the splits in order
+            if (p.fine > 1) {
 #pragma unroll
-            for (int ss = 0; ss < SB; ++ss)
+              for (int ss = 0; ss < SB; ss += 2)
 #pragma unroll
-              for (int c = 0; c < G; ++c) acc[c] += v[ss][c];
+                for (int c = 0; c < G; ++c) v[ss][c] += v[ss + 1][c];
+            }
+            if (p.fine > 2) {
+#pragma unroll
+              for (int ss = 0; ss < SB; ss += 4)
+#pragma unroll
+                for (int c = 0; c < G; ++c) v[ss][c] += v[ss + 2][c];
+            }
+            if (p.fine > 4) {
+#pragma unroll
+              for (int c = 0; c < G; ++c) v[0][c] += v[4][c];
+            }
+#pragma unroll
+            for (int ss = 0; ss < SB; ++ss) {
+              if (ss % p.fine == 0) {
+#pragma unroll
+                for (int c = 0; c < G; ++c) acc[c] += v[ss][c];
+              }
+            }
           }
           if (n < p.N) tc_store8<EPI>(p, slice, t0 + cg, min(8, nt - cg), n, acc, s_mean, s_rstd, cg, s_slot);
         }
@@ -459,10 +500,12 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   const int t0 = ttile * bn;
   const int nt = min(bn, p.T - t0);                                  // live tokens in this tile
   const int total_chunks = (p.K + kBK - 1) / kBK;
-  const int c0 = split * p.chunks_per_split;
-  const int c1 = min(total_chunks, c0 + p.chunks_per_split);
+  // this CTA's part of its split: acc_groups of the groups
+  const int acc_groups = p.groups / p.fine, part0 = (split / p.fine) * p.chunks_per_split;
+  const int c0 = part0 + (split % p.fine) * acc_groups * p.group_chunks;
+  const int c1 = min(min(total_chunks, part0 + p.chunks_per_split), c0 + acc_groups * p.group_chunks);
   const int nchunks = max(0, c1 - c0);
-  const uint32_t ncols = 32;
+  const uint32_t ncols = acc_groups > 4 ? 128 : (acc_groups > 2 ? 64 : 32);
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages; ++s) {
@@ -525,9 +568,11 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     const uint32_t idesc = instr_desc_bf16(bn);
     pdl_wait();
     const bool skip = p.all_done && *p.all_done;
-    for (int it = 0; it < nchunks && !skip; ++it) {
+    uint32_t acc = tmem;
+    for (int it = 0, in_group = 0; it < nchunks && !skip; ++it, ++in_group) {
       const int s = it % kStages;
       const uint32_t ph = (it / kStages) & 1;
+      if (in_group == p.group_chunks) { in_group = 0; acc += 16; }
       if (!mbar_wait(bars + 8 * s, ph)) { ok = false; break; }
       tc_fence_after();
       if (it == 0) BPD_TC_STAMP(3);
@@ -537,8 +582,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         const uint64_t ad = smem_desc_sw128(sa + kk * 32);
         const uint64_t bh = smem_desc_sw128(sa + kBM * 128 + kk * 32);
         const uint64_t bl = smem_desc_sw128(sa + kBM * 128 + bn * 128 + kk * 32);
-        umma_f16(tmem, ad, bh, idesc, (it > 0 || kk > 0) ? 1u : 0u);
-        umma_f16(tmem, ad, bl, idesc, 1u);
+        umma_f16(acc, ad, bh, idesc, (in_group > 0 || kk > 0) ? 1u : 0u);
+        umma_f16(acc, ad, bl, idesc, 1u);
       }
       umma_commit(bars + 8 * (kStages + s));       // frees the stage once these MMAs have read it
     }
@@ -550,7 +595,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     pdl_wait();
     const EpiShared sh{s_mean, s_rstd, s_slot, ctl};
     const EpiUnit u{tmem, bars + 8 * 2 * kStages, 0u, tile, split, slice, (int)blockIdx.z, (int)gridDim.x,
-                    t0, nt, bn, nchunks, p.all_done && *p.all_done};
+                    t0, nt, bn, nchunks, acc_groups, (nchunks + p.group_chunks - 1) / p.group_chunks, p.all_done && *p.all_done};
     tc_epilogue<EPI>(p, sh, u, warp, lane);
   }
   tc_fence_before();

@@ -22,6 +22,7 @@ constexpr int kMinChunksPerSplit = 2;
 
 struct Plan {
   int tiles, chunks, splits, chunks_per_split;
+  int groups, group_chunks;   // of a split's chunks, see TcParams
 };
 // Launches of at most 16 token rows (gemm_tc.cuh): one token tile, two CTAs per SM, K split finely.  Depends on (N, K)
 // only -- never on the number of tokens -- so that a position scored alone and the same position scored inside a
@@ -33,7 +34,15 @@ inline Plan plan_splits(int N, int K) {
   const int splits = std::max(1, std::min(pl.chunks / kMinChunksPerSplit, kSlots / pl.tiles));
   pl.chunks_per_split = (pl.chunks + splits - 1) / splits;
   pl.splits = (pl.chunks + pl.chunks_per_split - 1) / pl.chunks_per_split;
+  pl.groups = pl.chunks_per_split >= 32 ? 8 : 1;
+  pl.group_chunks = (pl.chunks_per_split + pl.groups - 1) / pl.groups;
   return pl;
+}
+// CTAs that share a split in a launch of `tiles` feature tiles: as many as the slots hold.
+inline int plan_fine(const Plan& pl, int tiles) {
+  int fine = 1;
+  while (fine < pl.groups && tiles * pl.splits * fine * 2 <= kSlots) fine *= 2;
+  return fine;
 }
 
 // Launches of the wide kernel (gemm_wide.cuh).  A tiling is (tokens per tile, CTAs per cluster = K splits); its cost in
@@ -116,7 +125,8 @@ inline WidePlan wide_plan_for(int N, int K, int T, int z, int planes, int plan_n
 constexpr int kNarrowBN = 16;
 inline size_t ws_floats(int N, int K, int zslices) {
   const Plan pl = plan_splits(N, K);
-  return pl.splits == 1 ? 0 : (size_t)zslices * pl.tiles * pl.splits * kNarrowBN * kBM;
+  // launches of fewer tiles may split finer, up to kSlots CTAs
+  return pl.splits == 1 && pl.groups == 1 ? 0 : std::max((size_t)zslices * pl.tiles * pl.splits, (size_t)kSlots) * kNarrowBN * kBM;
 }
 inline size_t counters_needed(int N, int zslices) { return (size_t)zslices * ((N + kBM - 1) / kBM); }
 
@@ -265,6 +275,9 @@ int launch(const Operands& op, int N, int K, int T, TcParams p, const Scratch& s
   } else {
     pl = plan_splits(pn, K);
     pl.tiles = (N + kBM - 1) / kBM;
+    p.fine = plan_fine(pl, pl.tiles * zslices);
+    p.groups = pl.groups; p.group_chunks = pl.group_chunks;
+    pl.splits *= p.fine;
     const size_t need_ws = pl.splits == 1 ? 0 : (size_t)zslices * pl.tiles * pl.splits * bn * kBM;
     const size_t need_cnt = (size_t)zslices * pl.tiles;
     if (need_ws > sc.ws_floats || need_cnt > sc.n_counters)
