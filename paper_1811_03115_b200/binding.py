@@ -113,7 +113,8 @@ def _host_i32(a, shape=None) -> np.ndarray:
 
 
 def _ptr(a: Optional[np.ndarray]):
-    return None if a is None else a.ctypes.data_as(C.c_void_p)
+    """Address of an array as the integer a void pointer argument takes (data_as builds a ctypes object: 1.5 us each)."""
+    return None if a is None else a.__array_interface__["data"][0]
 
 
 def _stream() -> int:
@@ -265,15 +266,14 @@ class Session:
         out.khat, out.accepted, out.table, out.next_block, out.block = (_ptr(khat), _ptr(acc), _ptr(table),
                                                                         _ptr(nxt), _ptr(blk))
         logits = hidden = layers = None
-        V, d = self.vocab, self.d_model
         if want_layers:
-            layers = torch.empty((self.n_dec, B, k, d), dtype=torch.float32, device=self.model.device)
+            layers = torch.empty((self.n_dec, B, k, self.d_model), dtype=torch.float32, device=self.model.device)
             out.layers_dev = layers.data_ptr()
         if want_logits:
-            logits = torch.empty((B, k, k, V), dtype=torch.float32, device=self.model.device)
+            logits = torch.empty((B, k, k, self.vocab), dtype=torch.float32, device=self.model.device)
             out.logits_dev = logits.data_ptr()
         if want_hidden:
-            hidden = torch.empty((B, k, d), dtype=torch.float32, device=self.model.device)
+            hidden = torch.empty((B, k, self.d_model), dtype=torch.float32, device=self.model.device)
             out.hidden_dev = hidden.data_ptr()
         tail = None if forced_tail is None else _host_i32(forced_tail, (B, k - 1))
         _check(lib.bpd_iteration(self.handle, k, accept_mode, max_new, eos_id, _ptr(tail), C.byref(out)))

@@ -137,6 +137,24 @@ struct Arena {
   void* take_bytes(size_t n) { return take<char>(n); }
 };
 
+// Where the words lie that decode calls (everything up to the error word) and bpd_iteration (everything from it on) hand
+// to the caller; the session's pinned memory mirrors it.
+struct Report {
+  size_t out_ids, j, error, khat, block, cur, table, table_full, total;
+  Report(int B, int max_tgt) {
+    const size_t b = B;
+    out_ids = 2 * (4 + kMaxK + 1);               // behind the statistics (64-bit words)
+    j = out_ids + b * max_tgt;
+    error = j + b;
+    khat = error + 1;
+    block = khat + b;
+    cur = block + b * kMaxK;
+    table = cur + b * kMaxK;
+    table_full = table + b * kMaxK * kMaxK;
+    total = table_full + b * kMaxK * kMaxK;
+  }
+};
+
 static int pages_per_row(const Config& c, int max_tgt) { return ceil_div(max_tgt + 1 + c.k_model, kPage); }
 
 // Sessions whose widest pass has more than 16 rows run their projections in the wide kernel; the K splits are planned
@@ -174,22 +192,22 @@ static size_t plan_session(const Config& c, int B, int max_src, int max_tgt, cha
   float* pe = a.take<float>(npos * d);
   int* page_table = a.take<int>((size_t)B * ppr);
   RowState st;
-  st.len = a.take<int>(B); st.j = a.take<int>(B); st.finished = a.take<int>(B); st.src_len = a.take<int>(B);
-  st.block = a.take<int>((size_t)B * kMaxK); st.cur_block = a.take<int>((size_t)B * kMaxK);
-  st.khat = a.take<int>(B);
-  st.table = a.take<int>((size_t)B * kMaxK * kMaxK);
-  st.out_ids = a.take<int>((size_t)B * max_tgt);
-  st.all_done = a.take<int>(1); st.error = a.take<int>(1);
+  st.len = a.take<int>(B); st.finished = a.take<int>(B); st.src_len = a.take<int>(B); st.all_done = a.take<int>(1);
+  // what calls read back lies in one piece (see Report), so that a call makes one copy
+  const Report rep(B, max_tgt);
+  int* report = a.take<int>(rep.total);
+  st.stats = reinterpret_cast<long long*>(report);
+  st.out_ids = report + rep.out_ids; st.j = report + rep.j; st.error = report + rep.error; st.khat = report + rep.khat;
+  st.block = report + rep.block; st.cur_block = report + rep.cur; st.table = report + rep.table;
+  int* table_full = report + rep.table_full;
   st.signal = a.take<int>(2); st.host_flags = nullptr;
-  st.stats = a.take<long long>(4 + kMaxK + 1);
   st.page_table = page_table; st.pages_per_row = ppr; st.max_tgt = max_tgt;
   void* u2 = a.take_bytes((size_t)B * c.k_model * c.d_hidden * ea);
   float* h2 = a.take<float>((size_t)B * d);
   int* table2 = a.take<int>((size_t)B * kMaxK);
-  int* table_full = a.take<int>((size_t)B * kMaxK * kMaxK);
   RankState rank;
   rank.thr = a.take<float>(Rmax); rank.tok = a.take<int>(Rmax); rank.cnt = a.take<int>(Rmax);
-  int* src_dev = a.take<int>(E);
+  int* src_dev = a.take<int>(E + B);     // source ids, then source lengths: one copy
   int* tail_dev = a.take<int>((size_t)B * kMaxK);
   int* plan_dev = a.take<int>((size_t)B * max_tgt * (kMaxK - 1));
   // split-K workspace of the few-row projection kernel: the largest any launch of this session can need
@@ -1052,40 +1070,48 @@ static int dispatch_pass(bpd_session* s, const PassArgs& a) {
   return BPD_OK;
 }
 
-static int check_device_error(bpd_session* s) {
-  int err = 0;
-  BPD_CUDA(cudaMemcpyAsync(&s->pinned[64], s->st.error, sizeof(int), cudaMemcpyDeviceToHost, s->stream));
-  BPD_CUDA(cudaStreamSynchronize(s->stream));
-  err = s->pinned[64];
+static int device_error(int err) {
+  if (err == 0) return BPD_OK;
   if (err == 1) return fail(BPD_E_INVALID, "a token id outside the vocabulary reached the decoder");
   if (err >= 101 && err <= 103) return fail(BPD_E_TIMEOUT, "a bounded wait inside the projection kernel expired (code %d)", err);
   if (err >= 104 && err <= 106) {
     const char* what[] = {"device-wide join", "weight tile", "exchange inside the cluster"};
     return fail(BPD_E_TIMEOUT, "a bounded wait inside the persistent layer kernel expired (code %d: %s)", err, what[err - 104]);
   }
-  if (err != 0) return fail(BPD_E_CUDA, "device-side error word %d", err);
-  return BPD_OK;
+  return fail(BPD_E_CUDA, "device-side error word %d", err);
 }
 
-static int fetch(bpd_session* s, int max_new, int32_t* out_ids, int32_t* out_len, bpd_stats* stats, float ms) {
+// Words [from, to) of the report into the session's pinned mirror.
+static cudaError_t copy_report(bpd_session* s, size_t from, size_t to) {
+  return cudaMemcpyAsync(s->mirror + from, reinterpret_cast<int*>(s->st.stats) + from, (to - from) * sizeof(int), cudaMemcpyDeviceToHost, s->stream);
+}
+
+// The results of a decode: one copy behind whatever is enqueued, one wait.  `timed`: the decode's events bracket it.
+static int fetch(bpd_session* s, int max_new, int32_t* out_ids, int32_t* out_len, bpd_stats* stats, bool timed) {
   const int B = s->B;
-  std::vector<int> ids, jj(B);
-  std::vector<long long> sv(4 + kMaxK + 1);
+  const Report rep(B, s->max_tgt);
   if (out_ids) {
-    ids.resize((size_t)B * s->max_tgt);
-    BPD_CUDA(cudaMemcpyAsync(ids.data(), s->st.out_ids, ids.size() * sizeof(int), cudaMemcpyDeviceToHost, s->stream));
+    BPD_CUDA(copy_report(s, 0, rep.khat));
+  } else {
+    BPD_CUDA(copy_report(s, 0, rep.out_ids));
+    BPD_CUDA(copy_report(s, rep.j, rep.khat));
   }
-  BPD_CUDA(cudaMemcpyAsync(jj.data(), s->st.j, B * sizeof(int), cudaMemcpyDeviceToHost, s->stream));
-  BPD_CUDA(cudaMemcpyAsync(sv.data(), s->st.stats, sv.size() * sizeof(long long), cudaMemcpyDeviceToHost, s->stream));
   BPD_CUDA(cudaStreamSynchronize(s->stream));
+  BPD_TRY(device_error(s->mirror[rep.error]));
+  const int* jj = s->mirror + rep.j;
   for (int b = 0; b < B; ++b) {
     const int n = std::min(jj[b], max_new);
     if (out_len) out_len[b] = n;
     if (out_ids) {
-      for (int t = 0; t < max_new; ++t) out_ids[(size_t)b * max_new + t] = (t < n) ? ids[(size_t)b * s->max_tgt + t] : -1;
+      const int* ids = s->mirror + rep.out_ids + (size_t)b * s->max_tgt;
+      memcpy(out_ids + (size_t)b * max_new, ids, sizeof(int) * n);
+      for (int t = n; t < max_new; ++t) out_ids[(size_t)b * max_new + t] = -1;
     }
   }
   if (stats) {
+    float ms = 0.f;
+    if (timed) BPD_CUDA(cudaEventElapsedTime(&ms, s->ev0, s->ev1));
+    const long long* sv = reinterpret_cast<const long long*>(s->mirror);
     memset(stats, 0, sizeof(*stats));
     stats->row_iterations = sv[0]; stats->tokens = sv[1]; stats->iterations = sv[2];
     for (int i = 0; i <= kMaxK; ++i) stats->khat_hist[i] = sv[4 + i];
@@ -1330,15 +1356,18 @@ int bpd_session_create_opt(const bpd_model* model, int batch, int max_src, int m
       pe[(size_t)pos * model->cfg.d + 2 * i] = (float)sin(ang);
       pe[(size_t)pos * model->cfg.d + 2 * i + 1] = (float)cos(ang);
     }
-  cudaError_t e = cudaMallocHost(reinterpret_cast<void**>(&s->pinned), (256 + (size_t)batch * kMaxK) * sizeof(int));
+  // pinned: the passes' flags, forced tails, sources with their lengths, the report's mirror
+  const size_t tails = 64, sources = tails + (size_t)batch * kMaxK, mirror = align_up(sources + (size_t)batch * max_src + batch, 64);
+  const size_t pinned_ints = mirror + Report(batch, max_tgt).total;
+  cudaError_t e = cudaMallocHost(reinterpret_cast<void**>(&s->pinned), pinned_ints * sizeof(int));
   if (e == cudaSuccess) {
-    memset(s->pinned, 0, (256 + (size_t)batch * kMaxK) * sizeof(int));
+    memset(s->pinned, 0, pinned_ints * sizeof(int));
+    s->tail_stage = s->pinned + tails; s->src_stage = s->pinned + sources; s->mirror = s->pinned + mirror;
     void* dev_view = nullptr;
     e = cudaHostGetDevicePointer(&dev_view, s->pinned, 0);
     s->st.host_flags = static_cast<int*>(dev_view);
     s->epoch = 0;
   }
-  for (int i = 0; i < 8 && e == cudaSuccess; ++i) e = cudaEventCreateWithFlags(&s->ev_flag[i], cudaEventDisableTiming);
   if (e == cudaSuccess) e = cudaEventCreate(&s->ev0);
   if (e == cudaSuccess) e = cudaEventCreate(&s->ev1);
   if (e == cudaSuccess) e = cudaMemsetAsync(s->base, 0, need, s->stream);
@@ -1364,35 +1393,39 @@ int bpd_session_destroy(bpd_session* s) {
     if (kv.second.exec) cudaGraphExecDestroy(kv.second.exec);
   if (s->enc_graph.exec) cudaGraphExecDestroy(s->enc_graph.exec);
   if (s->pinned) cudaFreeHost(s->pinned);
-  for (int i = 0; i < 8; ++i) cudaEventDestroy(s->ev_flag[i]);
   cudaEventDestroy(s->ev0);
   cudaEventDestroy(s->ev1);
   delete s;
   return BPD_OK;
 }
 
+// Numbers the decode that follows a reset of the rows.  The kernel that resets them puts the number where the verify
+// kernels read it, so a decode starts without a copy of its own.
+static int new_epoch(bpd_session* s) { return s->epoch = (s->epoch % 0x0fffffff) + 1; }
+
 int bpd_encode(bpd_session* s, const int32_t* src_ids, const int32_t* src_len) {
   if (!s || !src_ids || !src_len) return fail(BPD_E_INVALID, "null argument");
   const Config& c = s->m->cfg;
   const int B = s->B, S = s->max_src;
-  std::vector<int> ids((size_t)B * S, 0), lens(B);
   for (int b = 0; b < B; ++b) {
     if (src_len[b] < 1 || src_len[b] > S) return fail(BPD_E_SHAPE, "src_len[%d] = %d outside 1..%d", b, src_len[b], S);
-    lens[b] = src_len[b];
     for (int t = 0; t < src_len[b]; ++t) {
       const int id = src_ids[(size_t)b * S + t];
       if (id < 0 || id >= c.V) return fail(BPD_E_INVALID, "source id %d at row %d position %d outside the vocabulary", id, b, t);
-      ids[(size_t)b * S + t] = id;
     }
   }
-  // staging through pinned memory keeps the copies asynchronous and ordered on the stream
+  // ids and lengths go through pinned memory in one asynchronous copy; the wait keeps an earlier call's copy intact
   BPD_CUDA(cudaStreamSynchronize(s->stream));
-  BPD_CUDA(cudaMemcpyAsync(s->src_dev, ids.data(), ids.size() * sizeof(int), cudaMemcpyHostToDevice, s->stream));
-  BPD_CUDA(cudaMemcpyAsync(s->tail_dev, lens.data(), B * sizeof(int), cudaMemcpyHostToDevice, s->stream));
-  ResetParams rp{s->st, B, s->ppr, s->tail_dev, s->stack_bar};
+  for (int b = 0; b < B; ++b) {
+    int* row = s->src_stage + (size_t)b * S;
+    memcpy(row, src_ids + (size_t)b * S, sizeof(int) * src_len[b]);
+    memset(row + src_len[b], 0, sizeof(int) * (S - src_len[b]));
+    s->src_stage[(size_t)B * S + b] = src_len[b];
+  }
+  BPD_CUDA(cudaMemcpyAsync(s->src_dev, s->src_stage, ((size_t)B * S + B) * sizeof(int), cudaMemcpyHostToDevice, s->stream));
+  ResetParams rp{s->st, B, s->ppr, s->src_dev + (size_t)B * S, s->stack_bar, new_epoch(s)};
   reset_rows_kernel<<<1, 32 * ceil_div(B, 32), 0, s->stream>>>(rp);
   ++g_launches;
-  BPD_CUDA(cudaStreamSynchronize(s->stream));   // host vectors go out of scope
   int rc = BPD_OK;
   auto eager = [&]() { return s->tc ? run_encoder_tc(s) : ((c.dtype == 0) ? run_encoder<float>(s) : run_encoder<bf16>(s)); };
   GraphEntry& ge = s->enc_graph;
@@ -1427,7 +1460,7 @@ int bpd_encode(bpd_session* s, const int32_t* src_ids, const int32_t* src_len) {
 int bpd_rewind(bpd_session* s) {
   if (!s) return fail(BPD_E_INVALID, "session is null");
   if (s->phase < kPhaseEncoded) return fail(BPD_E_STATE, "nothing encoded yet");
-  ResetParams rp{s->st, s->B, s->ppr, s->st.src_len, s->stack_bar};
+  ResetParams rp{s->st, s->B, s->ppr, s->st.src_len, s->stack_bar, new_epoch(s)};
   reset_rows_kernel<<<1, 32 * ceil_div(s->B, 32), 0, s->stream>>>(rp);
   ++g_launches;
   BPD_CUDA(cudaGetLastError());
@@ -1505,20 +1538,17 @@ static int wait_pass_flag(bpd_session* s, int slot, int* finished) {
     }
   }
 }
-static int decode_loop(bpd_session* s, const PassArgs* cycle, int n_cycle, int max_passes) {
-  // a new epoch and pass counter for this decode, ordered on the stream behind whatever the previous one left
-  s->epoch = (s->epoch % 0x0fffffff) + 1;
-  int* stage = &s->pinned[200 + 2 * (s->epoch & 1)];
-  stage[0] = s->epoch; stage[1] = 0;
-  BPD_CUDA(cudaMemcpyAsync(s->st.signal, stage, 2 * sizeof(int), cudaMemcpyHostToDevice, s->stream));
-  for (int it = 0; it < max_passes; ++it) {
+// The passes of a decode: `first` (the priming pass) if there is one, then the cycle.
+static int decode_loop(bpd_session* s, const PassArgs* first, const PassArgs* cycle, int n_cycle, int max_passes) {
+  const int lead = first ? 1 : 0;
+  for (int it = 0; it < max_passes + lead; ++it) {
     if (it >= 2) {
       int finished = 0;
       int rc = wait_pass_flag(s, (it - 2) % 8, &finished);
       if (rc) return rc;
       if (finished) break;
     }
-    int rc = dispatch_pass(s, cycle[it % n_cycle]);
+    int rc = dispatch_pass(s, it < lead ? *first : cycle[(it - lead) % n_cycle]);
     if (rc) return rc;
   }
   return BPD_OK;
@@ -1528,12 +1558,7 @@ static int finish_decode(bpd_session* s, int max_new, int32_t* out_ids, int32_t*
   BPD_CUDA(cudaEventRecord(s->ev1, s->stream));
   s->timed = 1;
   if (!out_ids && !out_len && !stats) return BPD_OK;
-  BPD_CUDA(cudaEventSynchronize(s->ev1));
-  float ms = 0.f;
-  BPD_CUDA(cudaEventElapsedTime(&ms, s->ev0, s->ev1));
-  int rc = check_device_error(s);
-  if (rc) return rc;
-  return fetch(s, max_new, out_ids, out_len, stats, ms);
+  return fetch(s, max_new, out_ids, out_len, stats, true);
 }
 
 int bpd_decode_greedy(bpd_session* s, int max_new, int32_t eos_id, int32_t* out_ids, int32_t* out_len, bpd_stats* stats) {
@@ -1543,7 +1568,7 @@ int bpd_decode_greedy(bpd_session* s, int max_new, int32_t eos_id, int32_t* out_
   s->phase = kPhaseGreedy;
   BPD_CUDA(cudaEventRecord(s->ev0, s->stream));
   PassArgs a{kModeGreedy, 1, 1, 1, nullptr, 0, 0, max_new, eos_id, nullptr};
-  rc = decode_loop(s, &a, 1, max_new);
+  rc = decode_loop(s, nullptr, &a, 1, max_new);
   if (rc) return rc;
   return finish_decode(s, max_new, out_ids, out_len, stats);
 }
@@ -1559,12 +1584,10 @@ int bpd_decode_blockwise(bpd_session* s, int k, int accept_mode, int max_new, in
   if (s->plan_len && s->plan_k != k) return fail(BPD_E_SHAPE, "forced plan was installed for k = %d", s->plan_k);
   s->phase = kPhaseBlockwise;
   BPD_CUDA(cudaEventRecord(s->ev0, s->stream));
-  PassArgs prime{kModePrime, 1, k, k, nullptr, 0, 0, max_new, eos_id, nullptr};
-  rc = dispatch_pass(s, prime);
-  if (rc) return rc;
+  const PassArgs prime{kModePrime, 1, k, k, nullptr, 0, 0, max_new, eos_id, nullptr};
   PassArgs a{kModeBlock, k, k, k, s->plan_len ? s->plan_dev : nullptr, s->plan_len, k, max_new, eos_id, nullptr,
              acc.accept_kind, acc.accept_param, acc.min_block};
-  rc = decode_loop(s, &a, 1, max_new);
+  rc = decode_loop(s, &prime, &a, 1, max_new);
   if (rc) return rc;
   return finish_decode(s, max_new, out_ids, out_len, stats);
 }
@@ -1581,15 +1604,13 @@ int bpd_decode_blockwise_twocall(bpd_session* s, int k, int accept_mode, int max
   s->phase = kPhaseBlockwise;
   BPD_CUDA(cudaEventRecord(s->ev0, s->stream));
   // the first Predict scores the start token: the priming pass
-  PassArgs prime{kModePrime, 1, k, k, nullptr, 0, 0, max_new, eos_id, nullptr};
-  rc = dispatch_pass(s, prime);
-  if (rc) return rc;
+  const PassArgs prime{kModePrime, 1, k, k, nullptr, 0, 0, max_new, eos_id, nullptr};
   // Verify: p_1 alone at the k block positions, then accept; Predict: all k heads at the last accepted token
   PassArgs cycle[2] = {
       PassArgs{kModeBlock, k, 1, 1, s->plan_len ? s->plan_dev : nullptr, s->plan_len, k, max_new, eos_id, nullptr,
                acc.accept_kind, acc.accept_param, acc.min_block},
       PassArgs{kModePredict, 1, k, k, nullptr, 0, 0, max_new, eos_id, nullptr}};
-  rc = decode_loop(s, cycle, 2, 2 * max_new);
+  rc = decode_loop(s, &prime, cycle, 2, 2 * max_new);
   if (rc) return rc;
   return finish_decode(s, max_new, out_ids, out_len, stats);
 }
@@ -1617,8 +1638,8 @@ int bpd_iteration(bpd_session* s, int k, int accept_mode, int max_new, int32_t e
              acc.accept_kind, acc.accept_param, acc.min_block, out ? out->layers_dev : nullptr};
   if (forced_tail && k > 1) {
     BPD_CUDA(cudaStreamSynchronize(s->stream));   // the staging slots may still be in flight
-    memcpy(&s->pinned[128], forced_tail, sizeof(int) * B * (k - 1));
-    BPD_CUDA(cudaMemcpyAsync(s->tail_dev, &s->pinned[128], sizeof(int) * B * (k - 1), cudaMemcpyHostToDevice, s->stream));
+    memcpy(s->tail_stage, forced_tail, sizeof(int) * B * (k - 1));
+    BPD_CUDA(cudaMemcpyAsync(s->tail_dev, s->tail_stage, sizeof(int) * B * (k - 1), cudaMemcpyHostToDevice, s->stream));
     a.forced = s->tail_dev; a.forced_rows = 1; a.kforced = k;
   } else if (s->plan_len) {
     if (s->plan_k != k) return fail(BPD_E_SHAPE, "forced plan was installed for k = %d", s->plan_k);
@@ -1629,15 +1650,18 @@ int bpd_iteration(bpd_session* s, int k, int accept_mode, int max_new, int32_t e
   if (!out) return BPD_OK;
   if (out->hidden_dev)
     BPD_CUDA(cudaMemcpyAsync(out->hidden_dev, s->h_f32, sizeof(float) * B * k * s->m->cfg.d, cudaMemcpyDeviceToDevice, s->stream));
-  std::vector<int> khat(B), table((size_t)B * k * k), blk((size_t)B * kMaxK), cur((size_t)B * kMaxK);
-  BPD_CUDA(cudaMemcpyAsync(khat.data(), s->st.khat, B * sizeof(int), cudaMemcpyDeviceToHost, s->stream));
-  BPD_CUDA(cudaMemcpyAsync(table.data(), s->last_pass_lazy ? s->table_full : s->st.table, table.size() * sizeof(int),
-                           cudaMemcpyDeviceToHost, s->stream));
-  BPD_CUDA(cudaMemcpyAsync(blk.data(), s->st.block, blk.size() * sizeof(int), cudaMemcpyDeviceToHost, s->stream));
-  BPD_CUDA(cudaMemcpyAsync(cur.data(), s->st.cur_block, cur.size() * sizeof(int), cudaMemcpyDeviceToHost, s->stream));
+  // the accepted counts, blocks and table in one copy (two where the heads were evaluated lazily), one wait
+  const Report rep(B, s->max_tgt);
+  const size_t at = s->last_pass_lazy ? rep.table_full : rep.table, n_table = (size_t)B * k * k;
+  if (s->last_pass_lazy) {
+    BPD_CUDA(copy_report(s, rep.error, rep.table));
+    BPD_CUDA(copy_report(s, at, at + n_table));
+  } else {
+    BPD_CUDA(copy_report(s, rep.error, at + n_table));
+  }
   BPD_CUDA(cudaStreamSynchronize(s->stream));
-  rc = check_device_error(s);
-  if (rc) return rc;
+  if ((rc = device_error(s->mirror[rep.error]))) return rc;
+  const int *khat = s->mirror + rep.khat, *blk = s->mirror + rep.block, *cur = s->mirror + rep.cur;
   for (int b = 0; b < B; ++b) {
     if (out->khat) out->khat[b] = khat[b];
     for (int i = 0; i < k; ++i) {
@@ -1646,7 +1670,7 @@ int bpd_iteration(bpd_session* s, int k, int accept_mode, int max_new, int32_t e
       if (out->block) out->block[b * k + i] = cur[b * kMaxK + i];
     }
   }
-  if (out->table) memcpy(out->table, table.data(), table.size() * sizeof(int));
+  if (out->table) memcpy(out->table, s->mirror + at, n_table * sizeof(int));
   return BPD_OK;
 }
 
@@ -1654,14 +1678,8 @@ int bpd_fetch_output(bpd_session* s, int max_new, int32_t* out_ids, int32_t* out
   if (!s) return fail(BPD_E_INVALID, "session is null");
   if (max_new < 1 || max_new > s->max_tgt) return fail(BPD_E_SHAPE, "max_new = %d outside 1..%d", max_new, s->max_tgt);
   if (s->phase < kPhaseEncoded) return fail(BPD_E_STATE, "nothing encoded yet");
-  float ms = 0.f;
-  if (s->phase != kPhaseEncoded && s->timed) {   // a decode call bracketed its loop with events; bpd_iteration does not
-    BPD_CUDA(cudaEventSynchronize(s->ev1));
-    BPD_CUDA(cudaEventElapsedTime(&ms, s->ev0, s->ev1));
-  }
-  int rc = check_device_error(s);
-  if (rc) return rc;
-  return fetch(s, max_new, out_ids, out_len, stats, ms);
+  // a decode call bracketed its loop with events; bpd_iteration does not
+  return fetch(s, max_new, out_ids, out_len, stats, s->phase != kPhaseEncoded && s->timed);
 }
 
 // ------------------------------------------------------------------ self test of the bounded waits

@@ -172,9 +172,10 @@ struct bpd_session {
   unsigned* tc_done;
   unsigned long long* tc_best; size_t tc_best_elems;
   // host side
-  int* pinned;             // pinned ring of all_done flags + staging
-  cudaEvent_t ev_flag[8];
-  int epoch;               // decodes started on this session (the verify kernel tags its reports with it)
+  int* pinned;             // pinned: the passes' flags (8 words), then
+  int *tail_stage, *src_stage;   // staging of forced tails and sources
+  int* mirror;             // and what calls read back (see Report)
+  int epoch;               // resets of this session's rows so far (the verify kernel tags its reports with it)
   cudaEvent_t ev0, ev1;
   int timed;               // ev0 / ev1 bracket a finished decode loop
   int64_t invocations;

@@ -1339,6 +1339,7 @@ struct ResetParams {
   int B, ppr;
   const int* src_len;
   unsigned* join_words;   // control words of the persistent layer kernel (64), or null
+  int epoch;              // number of the decode that follows
 };
 static __global__ void reset_rows_kernel(ResetParams p) {
   const int b = threadIdx.x;
@@ -1353,6 +1354,8 @@ static __global__ void reset_rows_kernel(ResetParams p) {
   if (threadIdx.x == 0) {
     *p.st.all_done = 0;
     *p.st.error = 0;
+    p.st.signal[0] = p.epoch;
+    p.st.signal[1] = 0;
     for (int i = 0; i < 4 + kMaxK + 1; ++i) p.st.stats[i] = 0;
   }
   // the abort word is cleared; word 32 numbers the kernel's reductions over the whole life of the session (its
