@@ -13,6 +13,7 @@
 #include <utility>
 
 #include "host.hpp"
+#include "attention.cuh"
 #include "kernels_simt.cuh"
 #include "tc_host.hpp"
 #include "fused_layer.cuh"
@@ -312,6 +313,19 @@ static void prof_clear(bpd_session* s) {
   }
 }
 
+#define BPD_TRY(expr) do { int rc__ = (expr); if (rc__) return rc__; } while (0)
+
+// Attention of a pass or of the encoder.  max_keys, block: the most keys a row of the session can see, and the most rows
+// of a sequence in one launch; kv_static: keys and
+// values (of cached positions, in self-attention) do not come from the preceding launch.
+template <typename CT>
+static int attend(const AttnParams& a, int max_keys, int block, bool kv_static, cudaStream_t st, bool pdl) {
+  ++g_launches;
+  if (attn::applies(a, max_keys, block)) return attn::launch<CT>(a, max_keys, kv_static, st, pdl);
+  launch_attention<float, CT>(a, st, pdl);
+  return BPD_OK;
+}
+
 // ------------------------------------------------------------------ encoder
 template <typename WT>
 static int run_encoder(bpd_session* s) {
@@ -336,8 +350,7 @@ static int run_encoder(bpd_session* s) {
     ap.k = static_cast<float*>(s->qbuf) + d; ap.v = static_cast<float*>(s->qbuf) + 2 * d;
     ap.ldkv = 3 * d; ap.bstride = (long long)s->max_src * 3 * d; ap.paged = 0; ap.st = s->st;
     ap.scale = 1.0f / sqrtf((float)ap.dh); ap.by_rows = (s->B >= 8) ? 1 : 0;
-    launch_attention<float, float>(ap, st, pdl);
-    ++g_launches;
+    BPD_TRY(attend<float>(ap, s->max_src, s->max_src, false, st, pdl));
     LinearParams po = lin(s->attn, d, L.wo, d, d, nullptr, E, s->x, d, 0, nullptr);
     launch_linear<WT, float, kEpiResidual>(po, 1, st, pdl);
     launch_linear<WT, float, kEpiStoreAct>(with_ln(lin(s->x, d, L.w1, d, c.d_ff, L.b1, E, s->ffh, c.d_ff, 1, nullptr), L.ln2g, L.ln2b, c.eps), 1, st, pdl);
@@ -419,15 +432,13 @@ static int run_pass(bpd_session* s, const PassArgs& a) {
     ap.H = c.H; ap.dh = d / c.H; ap.causal = 1; ap.local_q = c.local_q; ap.local_m = c.local_m;
     ap.k = s->kcache[l]; ap.v = s->vcache[l]; ap.ldkv = d;
     ap.paged = 1; ap.st = s->st; ap.scale = 1.0f / sqrtf((float)ap.dh); ap.by_rows = (s->B >= 8) ? 1 : 0; ap.all_done = done;
-    launch_attention<float, WT>(ap, st, pdl);
-    ++g_launches;
+    BPD_TRY(attend<WT>(ap, s->max_tgt + 1 + c.k_model, c.k_model, true, st, pdl));
     launch_linear<WT, float, kEpiResidual>(lin(s->attn, d, L.wo, d, d, nullptr, R, s->x, d, 0, done), 1, st, pdl);
     // cross-attention over the encoder memory
     launch_linear<WT, float, kEpiStoreAct>(with_ln(lin(s->x, d, L.cwq, d, d, nullptr, R, s->qbuf, d, 0, done), L.ln2g, L.ln2b, c.eps), 1, st, pdl);
     ap.causal = 0; ap.limit_b = s->st.src_len; ap.k = s->crosskv[l]; ap.v = static_cast<float*>(s->crosskv[l]) + d;
     ap.ldkv = 2 * d; ap.bstride = (long long)s->max_src * 2 * d; ap.paged = 0;
-    launch_attention<float, float>(ap, st, pdl);
-    ++g_launches;
+    BPD_TRY(attend<float>(ap, s->max_src, c.k_model, true, st, pdl));
     launch_linear<WT, float, kEpiResidual>(lin(s->attn, d, L.cwo, d, d, nullptr, R, s->x, d, 0, done), 1, st, pdl);
     // feed-forward
     launch_linear<WT, float, kEpiStoreAct>(with_ln(lin(s->x, d, L.w1, d, c.d_ff, L.b1, R, s->ffh, c.d_ff, 1, done), L.ln3g, L.ln3b, c.eps), 1, st, pdl);
@@ -495,13 +506,6 @@ static tc::TcParams tc_params(const void* bias, int relu, const int* all_done) {
   return p;
 }
 
-#define BPD_TRY(expr) do { int rc__ = (expr); if (rc__) return rc__; } while (0)
-
-// The opt-in shared-memory limit of the staged attention kernel grows with the longest source seen so far.
-static int cross_staged_attr(size_t smem) {
-  return ensure_smem_limit(reinterpret_cast<const void*>(cross_attention_staged_kernel<float>), smem);
-}
-
 static int run_encoder_tc(bpd_session* s) {
   const bpd_model* m = s->m;
   const Config& c = m->cfg;
@@ -533,15 +537,7 @@ static int run_encoder_tc(bpd_session* s) {
     ap.k = static_cast<float*>(s->qbuf) + d; ap.v = static_cast<float*>(s->qbuf) + 2 * d;
     ap.ldkv = 3 * d; ap.bstride = (long long)s->max_src * 3 * d; ap.paged = 0; ap.st = s->st;
     ap.scale = 1.0f / sqrtf((float)ap.dh); ap.by_rows = (s->B >= 8) ? 1 : 0;
-    // many sequences, head width 64: a CTA per (sequence, head) with the sequence's keys and values in shared memory
-    if (ap.by_rows && ap.dh == 64 && cross_staged_smem(s->max_src) <= 160 * 1024 && s->opt.stage_encoder_rows) {
-      const size_t smem = cross_staged_smem(s->max_src);
-      BPD_TRY(cross_staged_attr(smem));
-      BPD_CUDA(launch_k(cross_attention_staged_kernel<float>, dim3(s->B * c.H), dim3(kAttnWarps * 32), smem, st, pdl, ap, s->max_src, 0));
-    } else {
-      launch_attention<float, float>(ap, st, pdl);
-    }
-    ++g_launches;
+    BPD_TRY(attend<float>(ap, s->max_src, s->max_src, false, st, pdl));
     tc::TcParams po = tc_params(nullptr, 0, nullptr);
     po.out_f32 = s->x; po.ldo = d;
     BPD_TRY(tc::launch<tc::kTcResidual>(with_w(at, L.wo, d), d, d, E, po, sc, st, 1, 0, 0, pdl)); ++g_launches;
@@ -904,8 +900,7 @@ static int run_pass_tc(bpd_session* s, const PassArgs& a) {
     ap.rows_per_b = a.kcur; ap.H = c.H; ap.dh = d / c.H; ap.causal = 1; ap.local_q = c.local_q; ap.local_m = c.local_m;
     ap.k = s->kcache[l]; ap.v = s->vcache[l];
     ap.ldkv = d; ap.paged = 1; ap.st = s->st; ap.scale = 1.0f / sqrtf((float)ap.dh); ap.by_rows = (s->B >= 8) ? 1 : 0; ap.all_done = done;
-    PROF(kProfSelfAttn, launch_attention<float, bf16>(ap, st, pdl););
-    ++g_launches;
+    PROF(kProfSelfAttn, BPD_TRY(attend<bf16>(ap, s->max_tgt + 1 + c.k_model, c.k_model, true, st, pdl)););
     tc::TcParams po = tc_params(nullptr, 0, done);
     po.out_f32 = s->x; po.ldo = d;
     if (fold) { po.g_next = static_cast<const bf16*>(L.ln2g); po.xg_hi = static_cast<bf16*>(s->xn); po.xg_plane = s->pl_xn; stats_to(po); }
@@ -917,17 +912,7 @@ static int run_pass_tc(bpd_session* s, const PassArgs& a) {
     PROF(kProfCrossQ, BPD_TRY(tc::launch<tc::kTcF32>(with_w(xn, L.cwq, d), d, d, R, pc, sc, st, 1, 0, 0, pdl)); ++g_launches);
     ap.causal = 0; ap.limit_b = s->st.src_len; ap.k = s->crosskv[l]; ap.v = static_cast<float*>(s->crosskv[l]) + d;
     ap.ldkv = 2 * d; ap.bstride = (long long)s->max_src * 2 * d; ap.paged = 0;
-    // many sequences, head width 64: the encoder's keys and values are staged before the dependency wait
-    const bool staged_cross = ap.by_rows && ap.dh == 64 && a.kcur <= 16 && cross_staged_smem(s->max_src) <= 160 * 1024 &&
-                              s->opt.stage_encoder_rows;
-    if (staged_cross) {
-      const size_t smem = cross_staged_smem(s->max_src);
-      BPD_TRY(cross_staged_attr(smem));
-      PROF(kProfCrossAttn, BPD_CUDA(launch_k(cross_attention_staged_kernel<float>, dim3(s->B * c.H), dim3(kAttnWarps * 32), smem, st, pdl, ap, s->max_src, 1)););
-    } else {
-      PROF(kProfCrossAttn, launch_attention<float, float>(ap, st, pdl););
-    }
-    ++g_launches;
+    PROF(kProfCrossAttn, BPD_TRY(attend<float>(ap, s->max_src, c.k_model, s->opt.stage_encoder_rows != 0, st, pdl)););
     if (fold) { po.g_next = static_cast<const bf16*>(L.ln3g); stats_to(po); }
     PROF(kProfCrossO, BPD_TRY(tc::launch<tc::kTcResidual>(with_w(at, L.cwo, d), d, d, R, po, sc, st, 1, 0, 0, pdl)); ++g_launches);
     if (!fold) PROF(kProfLn, launch_ln<bf16, float>(s->x, L.ln3g, L.ln3b, s->xn, nullptr, R, d, c.eps, done, st, s->pl_xn, pdl););

@@ -49,3 +49,39 @@ def test_fp32_projection_at_tile_edges(bpd, rows, in_f, out_f):
     for i, v in ((idx, val), (idx2, val2)):
         np.testing.assert_allclose(want[np.arange(rows), i.cpu().numpy()], want.max(-1), atol=1e-5)
         np.testing.assert_allclose(v.cpu().numpy(), want.max(-1), atol=1e-5)
+
+
+# attention of many-row sessions against the oracle's decoder: one chunk and several (96 encoder rows per chunk), query tiles
+# of up to 16 rows, sources from one id on, sequences long enough for a second chunk of 256 cached keys, local attention
+@pytest.mark.parametrize("batch,k,max_src,tgt,local", [(3, 8, 33, 20, 0), (9, 2, 100, 12, 0), (10, 16, 17, 40, 0), (19, 3, 5, 300, 0), (19, 3, 97, 290, 64)])
+def test_many_row_attention_decodes_like_the_oracle(bpd, batch, k, max_src, tgt, local):
+    from bpd_inputs import ModelConfig, Workload, make_weights
+    from oracle.decode import TransformerScorer
+    from oracle.model import parse_blob
+    cfg = ModelConfig(1, 2, 256, 4, 256, 300, k, 64, local_q=local, local_m=local // 2)
+    w = Workload("attn", cfg, 0.06, 5, 6, 7, batch=batch, src_lo=1, src_hi=max_src, n_decode=tgt)
+    blob = make_weights(cfg, 5, 0.06)
+    rng = np.random.default_rng(batch)
+    lens = rng.integers(1, max_src + 1, batch).astype(np.int32)
+    lens[:2] = 1, max_src
+    src = rng.integers(2, 300, (batch, max_src)).astype(np.int32)
+    model = bpd.Model(blob)
+    s = bpd.Session(model, batch, max_src, tgt)
+    s.bpd_encode(src, lens)
+    model_o, rows = parse_blob(blob), (0, 1, batch - 1)
+    scorers = {b: TransformerScorer(model_o, src[b], int(lens[b]), cached=True, capacity=tgt + k + 2) for b in rows}
+    inputs = {b: [0] for b in rows}
+    for b in rows:
+        scorers[b](inputs[b], 1)
+    while True:
+        r = s.bpd_iteration(k, tgt, want_hidden=True, accept_mode=k << 16)      # minimum block k: every proposal is kept
+        for b in rows:
+            block = [int(t) for t in r["block"][b]]
+            scorers[b](inputs[b] + block, k)
+            n = int(r["khat"][b])
+            np.testing.assert_allclose(r["hidden"][b].cpu().numpy(), scorers[b].last_hidden, atol=8e-3)     # the cache is bf16
+            inputs[b] += block[:n]
+        if len(inputs[0]) > tgt:
+            break
+    s.close()
+    model.close()
