@@ -638,10 +638,11 @@ static int run_layers_fused(bpd_session* s, const PassArgs& a) {
 // ------------------------------------------------------------------ persistent layer stack (few rows per pass)
 // Shared-memory plan of the persistent kernel for a session whose widest pass has `rows` rows; `budget` bytes per
 // CTA.  Returns false when the working buffers and a ring that holds at least the two largest tiles do not fit.
-static bool stack_plan(const Config& c, int rows, int nb, int ppr, int cross_rows, bool long_seq, size_t budget,
+// lean: the kernel's variant (1: short sequences, 2: one long sequence, 3: one short sequence, 0: general).
+static bool stack_plan(const Config& c, int rows, int nb, int ppr, int cross_rows, bool long_seq, int lean, size_t budget,
                        stack::Layout* out) {
   const int NT = rows > 8 ? 2 : 1, RP = NT * 8;
-  const stack::Geo g = stack::make_geo(c.d, c.H, c.d_ff, c.n_dec, cross_rows);
+  const stack::Geo g = stack::make_geo(c.d, c.H, c.d_ff, c.n_dec, cross_rows, lean >= 2);
   auto up = [](size_t v, size_t a) { return (v + a - 1) / a * a; };
   size_t off = 0;
   stack::Layout L;
@@ -654,15 +655,27 @@ static bool stack_plan(const Config& c, int rows, int nb, int ppr, int cross_row
   L.ol = take((size_t)RP * 128);
   L.hid = take((size_t)fused::kC * 2 * RP * g.UPR * 2);
   const size_t chunk = std::max((size_t)NT * 3 * fused::kDH * 4, (size_t)g.UPR * RP * 4);
-  L.outbox = take(fused::kC * chunk);
-  L.inbox = take(fused::kC * chunk);
+  const size_t states = (size_t)fused::kC * rows * stack::kState * 4;
+  const size_t window = lean == 2 ? stack::kLongKeys : stack::kShortKeys;
+  if (lean >= 2) {
+    // scores share the outbox, the ranks' states the inbox: their uses never overlap (see share_states)
+    L.outbox = L.sc = take(std::max(fused::kC * chunk, (size_t)16 * (window + 4) * 4));
+    L.inbox = L.lvl2 = take(std::max(fused::kC * chunk, states));
+    L.qp = take((size_t)3 * 16 * (attn::kPitch + stack::kLongCross + 8) * 2);
+    L.kv = take(window * 256);
+    L.attn = take(48 * 4);
+    L.wst = L.lvl1 = L.attn;
+  } else {
+    L.outbox = take(fused::kC * chunk);
+    L.inbox = take(fused::kC * chunk);
+    L.attn = take(sizeof(AttnSmem<fused::kDH, stack::kWarps>));
+    L.wst = take((size_t)stack::kWarps * NT * stack::kState * 4);
+    const size_t lvl = long_seq ? states : 0;
+    L.lvl1 = take(lvl);
+    L.lvl2 = take(lvl);
+  }
   L.kvq = take((size_t)RP * 512);
   L.stats = take((size_t)fused::kC * fused::kMaxRows * 2 * 4 + 4 * fused::kMaxRows * 4);
-  L.attn = take(sizeof(AttnSmem<fused::kDH, stack::kWarps>));
-  L.wst = take((size_t)stack::kWarps * NT * stack::kState * 4);
-  const size_t lvl = long_seq ? (size_t)fused::kC * rows * stack::kState * 4 : 0;
-  L.lvl1 = take(lvl);
-  L.lvl2 = take(lvl);
   L.pt = take((size_t)nb * ppr * 4);
   L.layers = take((size_t)c.n_dec * sizeof(stack::LayerPtrs));
   L.misc = take(sizeof(stack::Ctl));
@@ -679,7 +692,7 @@ static bool stack_plan(const Config& c, int rows, int nb, int ppr, int cross_row
   if (ring < (size_t)largest + second) return false;
   L.ring_bytes = (int)ring;
   int* fields[] = {&L.x, &L.xh, &L.xl, &L.oh, &L.ol, &L.hid, &L.outbox, &L.inbox, &L.kvq, &L.stats, &L.attn, &L.wst, &L.lvl1,
-                   &L.lvl2, &L.pt, &L.layers, &L.misc};
+                   &L.lvl2, &L.pt, &L.layers, &L.misc, &L.kv, &L.qp, &L.sc};
   for (int* f : fields) *f += (int)ring;
   L.total = (int)(ring + work);
   *out = L;
@@ -732,8 +745,14 @@ static int stack_setup(bpd_session* s) {
   const int rows = s->B * c.k_model;
   if (!s->tc || !s->opt.persistent_layers || !stack_shapes_ok(c, rows)) return BPD_OK;
   const bool long_seq = s->max_tgt + 1 + c.k_model > 32 * fused::kC;
-  const bool only_lean = s->opt.persistent_layers < 0;   // the library's own choice: sessions the lean kernel takes
-  if (only_lean && (long_seq || !s->opt.stage_encoder_rows || s->B * s->max_src > 256)) return BPD_OK;
+  const bool only_lean = s->opt.persistent_layers < 0;   // the library's own choice: sessions a lean kernel takes
+  const bool stageable = s->opt.stage_encoder_rows && s->B * s->max_src <= 256;
+  // one sequence: the variants that split the keys over the ranks (they need an SM per CTA; measured against the short
+  // one on one box: 138 -> 134 us for the base model's layers, and 272 -> 201 against the cluster launches for a long
+  // sequence); otherwise the short one
+  const int split = (s->B == 1 && s->max_src <= fused::kC * stack::kLongCross) ? (long_seq ? 2 : 3) : 0;
+  const int want = split ? split : (stageable && !long_seq ? 1 : 0);
+  if (only_lean && want == 0) return BPD_OK;
   cudaDeviceProp prop;
   int dev = 0;
   BPD_CUDA(cudaGetDevice(&dev));
@@ -744,18 +763,20 @@ static int stack_setup(bpd_session* s) {
   const size_t budgets[2] = {optin, std::min(optin, per_sm / 2 - 1024)};
   stack::Layout lay;
   bool ok = false;
-  int cross_rows = 0;
-  int minb = 0;
+  int cross_rows = 0, staged = 0, minb = 0, lean = 0;
   for (size_t budget : budgets) {
     ++minb;                                    // first one CTA per SM, then two
-    for (int staged = s->opt.stage_encoder_rows ? 1 : 0; staged >= (only_lean ? 1 : 0) && !ok; --staged) {
-      cross_rows = (staged && s->B * s->max_src <= 256) ? s->B * s->max_src : 0;
-      if (staged && !cross_rows) continue;
-      if (budget <= 1024 || !stack_plan(c, rows, s->B, s->ppr, cross_rows, long_seq, budget - 1024, &lay)) continue;
+    for (int attempt = 0; attempt < 3 && !ok; ++attempt) {
+      // the lean variant, else the general one with and without staged encoder rows
+      lean = attempt == 0 ? want : 0;
+      if (lean >= 2 && minb == 2) lean = (stageable && !long_seq) ? 1 : 0;
+      if ((attempt == 0 && !lean) || (attempt > 0 && only_lean) || (attempt == 1 && !stageable)) continue;
+      staged = lean >= 2 ? s->opt.stage_encoder_rows : (attempt < 2 ? 1 : 0);
+      cross_rows = lean >= 2 ? (ceil_div(s->max_src, fused::kC) + 7) / 8 * 8 : (staged ? s->B * s->max_src : 0);
+      if (budget <= 1024 || !stack_plan(c, rows, s->B, s->ppr, staged ? cross_rows : 0, long_seq, lean, budget - 1024, &lay)) continue;
       lay.total += 1024;                       // slack for aligning the ring to 1024 bytes
       int n1 = 0, n2 = 0;
       const size_t sm = (size_t)lay.total;
-      const bool lean = !long_seq && cross_rows > 0;
       const int ksteps = c.d == 256 ? 2 : 4, H = c.H;
       BPD_TRY(stack_clusters(stack::kernel_for(1, ksteps, minb, lean), sm, H, &n1));
       BPD_TRY(stack_clusters(stack::kernel_for(2, ksteps, minb, lean), sm, H, &n2));
@@ -767,7 +788,7 @@ static int stack_setup(bpd_session* s) {
   // tensor maps over all layers at once: weight slices as boxes of 64 (32 for d_model 256) reduction columns,
   // encoder keys / values.  The layers' tensors must lie at a constant stride (they do in a blob written tensor
   // by tensor, layer after layer; the session's encoder keys / values are laid out the same way).
-  const stack::Geo g = stack::make_geo(c.d, c.H, c.d_ff, c.n_dec, cross_rows);
+  const stack::Geo g = stack::make_geo(c.d, c.H, c.d_ff, c.n_dec, staged ? cross_rows : 0, lean >= 2);
   std::vector<stack::LayerPtrs> lp(c.n_dec);
   const int d = c.d, f = c.d_ff, nl = c.n_dec;
   auto stride_of = [&](auto get, long long* out) {
@@ -811,7 +832,7 @@ static int stack_setup(bpd_session* s) {
   BPD_CUDA(cudaStreamSynchronize(s->stream));
   static_assert(sizeof(stack::Layout) <= sizeof(s->stack_layout), "layout does not fit its opaque copy");
   memcpy(s->stack_layout, &lay, sizeof(lay));
-  s->stack_cross_rows = cross_rows; s->stack_long = long_seq ? 1 : 0; s->stack_minb = minb;
+  s->stack_cross_rows = cross_rows; s->stack_staged = staged; s->stack_long = long_seq ? 1 : 0; s->stack_minb = minb; s->stack_lean = lean;
   s->stack = 1;
   s->stack_dev = dev;
   stack_live(dev, +1);
@@ -830,7 +851,7 @@ static int run_layers_stack(bpd_session* s, const PassArgs& a) {
   p.tgt_embed = static_cast<const bf16*>(m->tgt_embed); p.pe = s->pe; p.npos = s->npos; p.vocab = c.V;
   p.st = s->st; p.forced = a.forced; p.forced_rows = a.forced_rows; p.kforced = a.kforced;
   p.local_q = c.local_q; p.local_m = c.local_m; p.max_src = s->max_src; p.scale = 1.0f / sqrtf((float)fused::kDH);
-  p.cross_rows = s->stack_cross_rows; p.long_seq = s->stack_long;
+  p.cross_rows = s->stack_cross_rows; p.cross_staged = s->stack_staged; p.cross_split = s->stack_lean >= 2; p.long_seq = s->stack_long;
   p.lnf_g = static_cast<const bf16*>(m->dec_lnf_g); p.lnf_b = static_cast<const bf16*>(m->dec_lnf_b);
   p.xn_hi = static_cast<bf16*>(s->xn); p.xn_plane = s->pl_xn; p.h_f32 = s->h_f32;
   p.layer_dump = a.layer_dump;
@@ -844,8 +865,7 @@ static int run_layers_stack(bpd_session* s, const PassArgs& a) {
   const size_t smem = (size_t)p.lay.total;
   // reduction panels of 32 columns (two steps of 16) for d_model 256, else 64 (four steps); one or two CTAs per SM
   const int nt = p.R > 8 ? 2 : 1, ksteps = c.d == 256 ? 2 : 4;
-  const bool lean = !s->stack_long && s->stack_cross_rows > 0;
-  const void* kernel = stack::kernel_for(nt, ksteps, s->stack_minb, lean);
+  const void* kernel = stack::kernel_for(nt, ksteps, s->stack_minb, s->stack_lean);
   if (!kernel) return fail(BPD_E_UNSUPPORTED, "no such instantiation of the persistent layer kernel");
   BPD_CUDA(launch_kc(kernel, grid, block, smem, s->stream, pdl, maps, p));
   ++g_launches;

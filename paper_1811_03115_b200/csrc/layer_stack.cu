@@ -5,13 +5,15 @@
 namespace bpd {
 namespace stack {
 
-const void* kernel_for(int nt, int ksteps, int minb, bool lean) {
+const void* kernel_for(int nt, int ksteps, int minb, int lean) {
 #define BPD_V(NT, KS, MB, LN) \
   if (nt == NT && ksteps == KS && minb == MB && lean == LN) return reinterpret_cast<const void*>(layer_stack_kernel<NT, KS, MB, LN>)
-  BPD_V(1, 2, 1, false); BPD_V(2, 2, 1, false); BPD_V(1, 4, 1, false); BPD_V(2, 4, 1, false);
-  BPD_V(1, 2, 2, false); BPD_V(2, 2, 2, false); BPD_V(1, 4, 2, false); BPD_V(2, 4, 2, false);
-  BPD_V(1, 2, 1, true); BPD_V(2, 2, 1, true); BPD_V(1, 4, 1, true); BPD_V(2, 4, 1, true);
-  BPD_V(1, 2, 2, true); BPD_V(2, 2, 2, true); BPD_V(1, 4, 2, true); BPD_V(2, 4, 2, true);
+  BPD_V(1, 2, 1, 0); BPD_V(2, 2, 1, 0); BPD_V(1, 4, 1, 0); BPD_V(2, 4, 1, 0);
+  BPD_V(1, 2, 2, 0); BPD_V(2, 2, 2, 0); BPD_V(1, 4, 2, 0); BPD_V(2, 4, 2, 0);
+  BPD_V(1, 2, 1, 1); BPD_V(2, 2, 1, 1); BPD_V(1, 4, 1, 1); BPD_V(2, 4, 1, 1);
+  BPD_V(1, 2, 2, 1); BPD_V(2, 2, 2, 1); BPD_V(1, 4, 2, 1); BPD_V(2, 4, 2, 1);
+  BPD_V(1, 2, 1, 2); BPD_V(2, 2, 1, 2); BPD_V(1, 4, 1, 2); BPD_V(2, 4, 1, 2);
+  BPD_V(1, 2, 1, 3); BPD_V(2, 2, 1, 3); BPD_V(1, 4, 1, 3); BPD_V(2, 4, 1, 3);
 #undef BPD_V
   return nullptr;
 }

@@ -42,6 +42,7 @@
 #include <cooperative_groups.h>
 #include <cuda.h>
 
+#include "attention.cuh"
 #include "fused_layer.cuh"
 
 namespace bpd {
@@ -83,7 +84,9 @@ struct LayerPtrs {
 // Byte offsets inside dynamic shared memory (the ring first, 1024-byte aligned).
 struct Layout {
   int ring_bytes;
-  int x, xh, xl, oh, ol, hid, outbox, inbox, kvq, stats, attn, wst, lvl1, lvl2, pt, layers, misc, total;
+  int x, xh, xl, oh, ol, hid, outbox, inbox, kvq, stats, attn, wst, lvl1, lvl2, pt, layers, misc;
+  int kv, qp, sc;                          // lean long-sequence variant: keys and values, query planes, scores
+  int total;
 };
 
 struct StackParams {
@@ -97,7 +100,8 @@ struct StackParams {
   // attention
   int local_q, local_m, max_src;
   float scale;
-  int cross_rows;                          // encoder rows staged per CTA (nb * max_src), 0: read from L2
+  int cross_rows, cross_split;             // encoder rows per CTA: all nb * max_src, or (split) rows rank * cross_rows ..
+  int cross_staged;                        // 1: in a tile of the ring, 0: read from L2
   int long_seq;                            // 1: sequences may exceed 256 keys (buffers of the shared-key schedule exist)
   // final layer norm -> planes for the head's first projection and the fp32 residual of the heads
   const bf16 *lnf_g, *lnf_b;
@@ -183,12 +187,12 @@ struct Ctl {
 };
 
 struct Geo {                               // derived sizes, the same in every CTA
-  int ks, PW, P, HCt, PH, UPR, ntl, staged, total_tiles;
+  int ks, PW, P, HCt, PH, UPR, ntl, staged, split, total_tiles;
   int lg_n4, lg_pw, lg_upr;                // log2 of ks / 4, PW, UPR (all powers of two)
   uint32_t xmask, hmask;                   // swizzle masks of the x planes (and weight panels over x), of the hidden planes
 };
 __host__ __device__ inline int ilog2(int v) { int l = 0; while ((1 << l) < v) ++l; return l; }
-__host__ __device__ inline Geo make_geo(int d, int H, int ff, int L, int cross_rows) {
+__host__ __device__ inline Geo make_geo(int d, int H, int ff, int L, int cross_rows, int split) {
   Geo g;
   g.ks = d / kC;
   g.PW = g.ks < 64 ? g.ks : 64;
@@ -197,6 +201,7 @@ __host__ __device__ inline Geo make_geo(int d, int H, int ff, int L, int cross_r
   g.PH = g.HCt / 64;
   g.UPR = g.HCt / kC;
   g.staged = cross_rows > 0 ? 1 : 0;
+  g.split = split;
   g.ntl = 2 * g.P + g.PH + 3 + g.staged;
   g.total_tiles = g.ntl * L;
   g.xmask = g.PW == 64 ? 7u : 3u;
@@ -226,7 +231,7 @@ __host__ __device__ inline TileDesc make_tile(const Geo& g, int i, int cross_row
   if (g.staged) {
     if (i == 0) {                                              // encoder keys (two halves of 32 floats), then values
       const int kb = round1k(cross_rows * 128);
-      t.map = kMapCk; t.nbox = 2; t.box_bytes = cross_rows * 128; t.x = j * kDH; t.y = 0; t.dx = 32; t.dstep = kb;
+      t.map = kMapCk; t.nbox = 2; t.box_bytes = cross_rows * 128; t.x = j * kDH; t.y = g.split ? c * cross_rows : 0; t.dx = 32; t.dstep = kb;
       t.map2 = kMapCv; t.x2 = d + j * kDH; t.off2 = 2 * kb; t.bytes2 = cross_rows * 256;
       t.bytes = 2 * kb + round1k(cross_rows * 256);
       return t;
@@ -283,7 +288,7 @@ __device__ __forceinline__ void pump(const Cta& k, int stop_before = 0x7fffffff)
     const int dy = (t.map == kMapQkv) ? dmodel : 0;
     for (int b = 0; b < t.nbox; ++b)
       tma_load_3d(dst + b * t.dstep, &k.maps->m[t.map], bar, t.x + b * t.dx, t.y + b * dy, layer, k.policy);
-    if (t.map2 >= 0) tma_load_3d(dst + t.off2, &k.maps->m[t.map2], bar, t.x2, 0, layer, k.policy);
+    if (t.map2 >= 0) tma_load_3d(dst + t.off2, &k.maps->m[t.map2], bar, t.x2, t.y, layer, k.policy);
     if (++idx == ntl) { idx = 0; ++layer; }
     ++issued;
   }
@@ -705,6 +710,273 @@ __device__ __forceinline__ void send_rows(const Cta& k, int n, uint8_t* buf0, ui
   xchg_wait(k, n);
 }
 
+// ------------------------------------------------------------------ attention over a rank's share of the keys (LEAN = 2, 3)
+// One sequence of at most 16 block rows.  Self-attention: chunk ch of 32 absolute positions belongs to rank ch mod 8;
+// cross-attention: encoder row r to rank r / cross_rows.  A rank computes the scores of all rows against its keys as one
+// product on mma.sync, the softmax weights against its own maximum, and the weighted values as a second product; the
+// ranks' states (maximum, weight sum, weighted values) are shared and merged in rank order.  A fold of one row and one
+// chunk on CUDA cores took 700 cycles, ten rows one after the other; a step here takes all rows and up to kLongKeys
+// keys.  Operands as in attention.cuh: three bf16 planes for whatever is not a bf16 cache entry, so nothing is rounded
+// that a CUDA-core kernel would not round.  Committed keys and values are fetched one block ahead.
+constexpr int kLongKeys = 224;             // keys of one step (KW) for long sequences: 56 KB of keys and values
+constexpr int kShortKeys = 32;             // ... for sessions of at most 256 positions: a rank has one chunk at most
+constexpr int kLongCross = 32;             // encoder rows of a rank at most
+
+struct LongCtx {
+  uint8_t *kb, *vb;                        // keys, values [KW][128 B], 16-byte pieces swizzled by the row
+  bf16 *qs, *ps;                           // query planes [3][16][72]; weight planes, in the keys' place
+  float *sc, *red;                         // scores [16][KW + 4]; maximum, sum, correction of 16 rows
+  const int* pt;
+  int len, first_ch, n_my;                 // committed positions; this rank's first chunk that any row sees, number of chunks
+  int local_q, local_m;
+};
+__device__ __forceinline__ int long_first_key(const LongCtx& lc, int pos) {
+  return lc.local_q <= 0 ? 0 : max(0, (pos / lc.local_q) * lc.local_q - lc.local_m);
+}
+template <int KW>
+__device__ __forceinline__ LongCtx long_ctx(const Cta& k, const AttnParams& ap, uint8_t* ssm, const int* s_pt, int len) {
+  LongCtx lc;
+  const Layout& L = k.p->lay;
+  lc.kb = ssm + L.kv; lc.vb = lc.kb + KW * 128;
+  lc.ps = reinterpret_cast<bf16*>(lc.kb);
+  lc.qs = reinterpret_cast<bf16*>(ssm + L.qp);
+  lc.sc = reinterpret_cast<float*>(ssm + L.sc);
+  lc.red = reinterpret_cast<float*>(ssm + L.attn);
+  lc.pt = s_pt; lc.len = len; lc.local_q = ap.local_q; lc.local_m = ap.local_m;
+  const int nch = (len + k.p->rows_per_b + 31) >> 5, ch0 = long_first_key(lc, len) >> 5;
+  lc.first_ch = ch0 + ((k.c - ch0) & (kC - 1));
+  lc.n_my = lc.first_ch < nch ? (nch - lc.first_ch + kC - 1) / kC : 0;
+  return lc;
+}
+// Absolute position of this rank's key `i`.
+__device__ __forceinline__ int long_pos(const LongCtx& lc, int i) { return ((lc.first_ch + kC * (i >> 5)) << 5) + (i & 31); }
+
+// Committed keys and values of this rank's keys i0 .. i0 + KW - 1 on their way into shared memory.
+template <int KW>
+__device__ __forceinline__ void long_prefetch(const Cta& k, const LongCtx& lc, const LayerPtrs& LP, int i0) {
+  const int n = min(KW, lc.n_my * 32 - i0), d = k.p->d;
+  const uint32_t ks = tc::smem_u32(lc.kb), vs = tc::smem_u32(lc.vb);
+  for (int w = k.tid; w < n * 8; w += kThreads) {
+    const int i = w >> 3, piece = w & 7, pos = long_pos(lc, i0 + i);
+    if (pos >= lc.len) continue;
+    const size_t at = ((size_t)lc.pt[pos / kPage] * kPage + (pos % kPage)) * d + k.j * kDH + piece * 8;
+    attn::cp_async16(ks + attn::swz(i, piece), LP.kcache + at);
+    attn::cp_async16(vs + attn::swz(i, piece), LP.vcache + at);
+  }
+}
+
+// Planes of the scaled queries (fp32, in the rows of kvq): 16 threads per row.
+__device__ __forceinline__ void long_queries(const Cta& k, const LongCtx& lc, const uint8_t* kvq) {
+  const int row = k.tid >> 4, col = (k.tid & 15) * 4;
+  float4 q = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (row < k.p->R) q = *reinterpret_cast<const float4*>(kvq + row * 512 + 256 + col * 4);
+  uint32_t a[3], b[3];
+  attn::split3_pair(q.x, q.y, a);
+  attn::split3_pair(q.z, q.w, b);
+#pragma unroll
+  for (int s = 0; s < 3; ++s) *reinterpret_cast<uint2*>(lc.qs + (s * 16 + row) * attn::kPitch + col) = make_uint2(a[s], b[s]);
+  if (k.tid < 16) { lc.red[k.tid] = -INFINITY; lc.red[16 + k.tid] = 0.f; }
+}
+
+// Softmax weights of the scores against the running maximum, as planes; key i of this step counts for row r if
+// visible(r, i).  PP: elements between the rows of a weight plane.
+template <int KW, int PP, typename F>
+__device__ __forceinline__ void long_weights(const Cta& k, const LongCtx& lc, int nk16, F&& visible) {
+  constexpr int sp = KW + 4, pp = PP;
+  const int row = k.tid >> 4, t = k.tid & 15;
+  const float m_old = lc.red[row];
+  float m_new = m_old, sum = 0.f;
+  for (int i = t * 2; i < nk16; i += 32) {
+    const float2 v = *reinterpret_cast<const float2*>(lc.sc + row * sp + i);
+    if (visible(row, i)) m_new = fmaxf(m_new, v.x);
+    if (visible(row, i + 1)) m_new = fmaxf(m_new, v.y);
+  }
+#pragma unroll
+  for (int o = 8; o > 0; o >>= 1) m_new = fmaxf(m_new, __shfl_xor_sync(0xffffffffu, m_new, o));
+  for (int i = t * 2; i < nk16; i += 32) {
+    const float2 v = *reinterpret_cast<const float2*>(lc.sc + row * sp + i);
+    const float e0 = visible(row, i) ? expf(v.x - m_new) : 0.f, e1 = visible(row, i + 1) ? expf(v.y - m_new) : 0.f;
+    sum += e0 + e1;
+    uint32_t w[3];
+    attn::split3_pair(e0, e1, w);
+#pragma unroll
+    for (int s = 0; s < 3; ++s) *reinterpret_cast<uint32_t*>(lc.ps + (s * 16 + row) * pp + i) = w[s];
+  }
+#pragma unroll
+  for (int o = 8; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+  if (t == 0) {
+    const float corr = m_new == -INFINITY ? 1.f : expf(m_old - m_new);          // nothing visible yet: nothing to rescale
+    lc.red[row] = m_new;
+    lc.red[16 + row] = lc.red[16 + row] * corr + sum;
+    lc.red[32 + row] = corr;
+  }
+}
+__device__ __forceinline__ void long_rescale(const Cta& k, const LongCtx& lc, float (&acc)[4][4]) {
+  const float f0 = lc.red[32 + (k.lane >> 2)], f1 = lc.red[32 + (k.lane >> 2) + 8];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) { acc[i][0] *= f0; acc[i][1] *= f0; acc[i][2] *= f1; acc[i][3] *= f1; }
+}
+// This rank's state into its block of the table: warp w holds dims 8w .. 8w + 7 of all rows.
+__device__ __forceinline__ void long_state(const Cta& k, const LongCtx& lc, const float (&acc)[4][4], float* lvl2) {
+  const int g = k.lane >> 2, R = k.p->R;
+#pragma unroll
+  for (int half = 0; half < 2; ++half) {
+    const int row = g + 8 * half;
+    if (row < R) *reinterpret_cast<float2*>(lvl2 + (size_t)(k.c * R + row) * kState + k.warp * 8 + (k.lane & 3) * 2) =
+        make_float2(attn::sum4(acc, 2 * half), attn::sum4(acc, 2 * half + 1));
+  }
+  if (k.tid < R) {
+    lvl2[(size_t)(k.c * R + k.tid) * kState + kDH] = lc.red[k.tid];
+    lvl2[(size_t)(k.c * R + k.tid) * kState + kDH + 1] = lc.red[16 + k.tid];
+  }
+}
+
+template <int KW>
+__device__ __forceinline__ void long_self_attention(const Cta& k, const LongCtx& lc, const LayerPtrs& LP, const uint8_t* kvq, float* lvl2) {
+  constexpr int sp = KW + 4, pp = KW + 8;
+  const int lane = k.lane, warp = k.warp, g = lane >> 2, t4 = lane & 3, rpb = k.p->rows_per_b;
+  const uint32_t ks = tc::smem_u32(lc.kb), vs = tc::smem_u32(lc.vb);
+  float acc[4][4] = {};
+  long_queries(k, lc, kvq);
+  const int total = lc.n_my * 32;
+  for (int i0 = 0; i0 < total || i0 == 0; i0 += KW) {
+    const int nk = min(KW, total - i0);             // a multiple of 32
+    if (i0 > 0) {
+      __syncthreads();                                     // the step before has used keys, values and weights
+      long_prefetch<KW>(k, lc, LP, i0);
+    }
+    // the block's own rows come from the exchange; what no row can see becomes zero
+    for (int w = k.tid; w < nk * 8; w += kThreads) {
+      const int i = w >> 3, piece = w & 7, pos = long_pos(lc, i0 + i);
+      if (pos < lc.len) continue;
+      const bool live = pos < lc.len + rpb;
+      const uint8_t* row = kvq + (live ? pos - lc.len : 0) * 512 + piece * 16;
+      *reinterpret_cast<uint4*>(lc.kb + attn::swz(i, piece)) = live ? *reinterpret_cast<const uint4*>(row) : make_uint4(0u, 0u, 0u, 0u);
+      *reinterpret_cast<uint4*>(lc.vb + attn::swz(i, piece)) = live ? *reinterpret_cast<const uint4*>(row + 128) : make_uint4(0u, 0u, 0u, 0u);
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();
+    for (int n0 = warp * 8; n0 < nk; n0 += 64) {
+      float c[4][4] = {};
+#pragma unroll
+      for (int k2 = 0; k2 < 2; ++k2) {
+        uint32_t b[4];
+        attn::ldsm4(ks + attn::swz(n0 + (lane & 7), k2 * 4 + (lane >> 3)), b);
+#pragma unroll
+        for (int kk = 0; kk < 2; ++kk)
+#pragma unroll
+          for (int s = 0; s < 3; ++s) {
+            uint32_t a[4];
+            attn::ldsm4(tc::smem_u32(lc.qs + (s * 16 + (lane & 15)) * attn::kPitch + (k2 * 2 + kk) * 16 + (lane >> 4) * 8), a);
+            attn::mma_bf16(c[s], a, b[kk * 2], b[kk * 2 + 1]);
+          }
+      }
+      *reinterpret_cast<float2*>(lc.sc + g * sp + n0 + t4 * 2) = make_float2(attn::sum4(c, 0), attn::sum4(c, 1));
+      *reinterpret_cast<float2*>(lc.sc + (g + 8) * sp + n0 + t4 * 2) = make_float2(attn::sum4(c, 2), attn::sum4(c, 3));
+    }
+    __syncthreads();
+    long_weights<KW, pp>(k, lc, nk, [&](int row, int i) {
+      const int pos = long_pos(lc, i0 + i), own = lc.len + row;
+      return row < rpb && pos <= own && pos >= long_first_key(lc, own);
+    });
+    __syncthreads();
+    long_rescale(k, lc, acc);
+    for (int k0 = 0; k0 < nk; k0 += 16) {
+      uint32_t b0, b1;
+      attn::ldsm2_trans(vs + attn::swz(k0 + (lane & 15), warp), b0, b1);
+#pragma unroll
+      for (int s = 0; s < 3; ++s) {
+        uint32_t a[4];
+        attn::ldsm4(tc::smem_u32(lc.ps + (s * 16 + (lane & 15)) * pp + k0 + (lane >> 4) * 8), a);
+        attn::mma_bf16(acc[s], a, b0, b1);
+      }
+    }
+  }
+  long_state(k, lc, acc, lvl2);
+  __syncthreads();                                         // keys, values and weights are free for the next block's
+}
+
+// Encoder rows of this rank: keys as two tiles of 32 columns in TMA's 128-byte swizzle, values [rows][64] (both fp32).
+template <int KW>
+__device__ __forceinline__ void long_cross_attention(const Cta& k, const LongCtx& lc, const LayerPtrs& LP, const uint8_t* kvq, const uint8_t* k0t,
+                                                     const uint8_t* k1t, const uint8_t* vt, int limit, float* lvl2) {
+  constexpr int sp = KW + 4, pp = kLongCross + 8;
+  const int lane = k.lane, warp = k.warp, g = lane >> 2, t4 = lane & 3, R = k.p->R;
+  const int rows = k.p->cross_rows, first = k.c * rows, nk16 = (rows + 15) & ~15;   // at most kLongCross
+  float acc[4][4] = {};
+  long_queries(k, lc, kvq);
+  // the weights take a place of their own here: the keys' buffer is being filled for the next layer's self-attention
+  LongCtx cc = lc;
+  cc.ps = lc.qs + 3 * 16 * attn::kPitch;
+  __syncthreads();
+  for (int n0 = warp * 8; n0 < nk16; n0 += 64) {
+    float c[4][4] = {};
+    const int row = min(n0 + g, rows - 1);                 // rows beyond the last repeat it with weight 0
+    const float* unstaged = LP.crosskv + (size_t)min(first + row, k.p->max_src - 1) * (2 * k.p->d) + k.j * kDH;
+#pragma unroll
+    for (int kk = 0; kk < 4; ++kk) {
+      const uint8_t* base = kk < 2 ? k0t : k1t;
+      const int col = (kk & 1) * 64 + t4 * 8;              // bytes
+      const bool st = k.g.staged != 0;
+      const float2 x = st ? *reinterpret_cast<const float2*>(base + swz(row * 128 + col, 7u)) : *reinterpret_cast<const float2*>(unstaged + kk * 16 + t4 * 2);
+      const float2 y = st ? *reinterpret_cast<const float2*>(base + swz(row * 128 + col + 32, 7u)) : *reinterpret_cast<const float2*>(unstaged + kk * 16 + t4 * 2 + 8);
+      uint32_t b0[3], b1[3];
+      attn::split3_pair(x.x, x.y, b0);
+      attn::split3_pair(y.x, y.y, b1);
+#pragma unroll
+      for (int s = 0; s < 3; ++s) {
+        uint32_t a[4];
+        attn::ldsm4(tc::smem_u32(lc.qs + (s * 16 + (lane & 15)) * attn::kPitch + kk * 16 + (lane >> 4) * 8), a);
+#pragma unroll
+        for (int q = 0; q < 3 - s; ++q) attn::mma_bf16(c[attn::product_slot(s, q, true)], a, b0[q], b1[q]);
+      }
+    }
+    *reinterpret_cast<float2*>(lc.sc + g * sp + n0 + t4 * 2) = make_float2(attn::sum4(c, 0), attn::sum4(c, 1));
+    *reinterpret_cast<float2*>(lc.sc + (g + 8) * sp + n0 + t4 * 2) = make_float2(attn::sum4(c, 2), attn::sum4(c, 3));
+  }
+  __syncthreads();
+  long_weights<KW, pp>(k, cc, nk16, [&](int row, int i) { return row < R && i < rows && first + i < limit; });
+  __syncthreads();
+  for (int k0 = 0; k0 < nk16; k0 += 16) {
+    uint32_t b0[3], b1[3];
+    auto at = [&](int r) {
+      const int row = min(k0 + r, rows - 1), dim = warp * 8 + g;
+      if (k.g.staged) return *reinterpret_cast<const float*>(vt + (size_t)row * 256 + dim * 4);
+      return LP.crosskv[(size_t)min(first + row, k.p->max_src - 1) * (2 * k.p->d) + k.p->d + k.j * kDH + dim];
+    };
+    attn::split3_pair(at(t4 * 2), at(t4 * 2 + 1), b0);
+    attn::split3_pair(at(t4 * 2 + 8), at(t4 * 2 + 9), b1);
+#pragma unroll
+    for (int s = 0; s < 3; ++s) {
+      uint32_t a[4];
+      attn::ldsm4(tc::smem_u32(cc.ps + (s * 16 + (lane & 15)) * pp + k0 + (lane >> 4) * 8), a);
+#pragma unroll
+      for (int q = 0; q < 3 - s; ++q) attn::mma_bf16(acc[attn::product_slot(s, q, true)], a, b0[q], b1[q]);
+    }
+  }
+  long_state(k, lc, acc, lvl2);
+}
+
+// The ranks' states to every rank (exchange n), merged in rank order into the planes of the attention output.
+__device__ __forceinline__ void share_states(const Cta& k, int n, float* lvl2, uint8_t* oh, uint8_t* ol, int nfree = 0) {
+  const int R = k.p->R;
+  float* mine = lvl2 + (size_t)k.c * R * kState;
+  const uint32_t bytes = (uint32_t)(R * kState * 4);
+  fence_async_smem();
+  __syncthreads();
+  if (k.tid == kPumpThread && nfree) release_tiles(k, nfree);
+  if (k.tid == 0) xchg_expect(k, n, (kC - 1) * bytes);
+  if (k.tid < kC && k.tid != k.c) xchg_send(k, n, k.tid, mine, mine, bytes);
+  xchg_wait(k, n);
+  for (int idx = k.tid; idx < R * kDH; idx += kThreads) {
+    const int row = idx / kDH, dim = idx % kDH;
+    float M, num, den;
+    fused::states_merge(lvl2 + row * kState, R * kState, dim, M, num, den);
+    store_attn_out(oh, ol, row, dim, num / den);
+  }
+  __syncthreads();
+}
+
 // ------------------------------------------------------------------ development trace
 #ifdef BPD_STACK_TRACE
 __device__ unsigned long long* g_stack_trace = nullptr;
@@ -719,10 +991,11 @@ constexpr int kTracePts = 256;
 // grid = (8, H), clusters of 8 along x.  All clusters must be resident at once (the host checks the occupancy).
 // MINB: CTAs per SM the kernel is compiled for.  Models with at most 15 heads have an SM to themselves per CTA (no
 // register limit to speak of); 16 clusters only fit with two CTAs on some SMs, which caps the registers at 128.
-// LEAN: sessions whose cache holds at most 256 positions and whose encoder rows are staged by TMA carry only that
-// path (the short self-attention schedule, the staged cross-attention); the general kernel needs far more than the
-// 128 registers a thread has when two CTAs share an SM.
-template <int NT, int KS, int MINB, bool LEAN>
+// LEAN = 1: sessions whose cache holds at most 256 positions and whose encoder rows are staged by TMA carry only that
+// path (the short self-attention schedule, the staged cross-attention); the general kernel (0) needs far more than the
+// 128 registers a thread has when two CTAs share an SM.  LEAN = 2, 3: sessions of one sequence of any length (2)
+// or of at most 256 positions (3); both attentions split the keys over the ranks and run on mma.sync.
+template <int NT, int KS, int MINB, int LEAN>
 __global__ void __cluster_dims__(kC, 1, 1) __launch_bounds__(kThreads, MINB)
 layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant__ StackParams p) {
   extern __shared__ __align__(1024) uint8_t ssm_raw[];
@@ -733,7 +1006,7 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
   Cta k;
   k.p = &p;
   k.maps = &maps;
-  k.g = make_geo(p.d, p.H, p.ff, p.L, p.cross_rows);
+  k.g = make_geo(p.d, p.H, p.ff, p.L, p.cross_staged ? p.cross_rows : 0, p.cross_split);
   k.sm = ssm;
   k.ctl = reinterpret_cast<Ctl*>(ssm + p.lay.misc);
   k.ring = tc::smem_u32(ssm);
@@ -844,10 +1117,15 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
   ap.rows = R; ap.rows_per_b = rpb; ap.H = p.H; ap.dh = kDH; ap.causal = 1; ap.local_q = p.local_q; ap.local_m = p.local_m;
   ap.ldkv = d; ap.paged = 1; ap.st = p.st; ap.st.page_table = s_pt; ap.scale = p.scale;
   bool one_chunk_per_rank = true;
-  if (!LEAN) {
+  if (LEAN == 0) {
     for (int b = 0; b < nb; ++b)
       one_chunk_per_rank = one_chunk_per_rank && ((s_len[b] + rpb + 31) >> 5) - (attn_first_key(ap, s_len[b]) >> 5) <= kC;
   }
+
+  constexpr bool SPLIT = LEAN >= 2;         // keys split over the ranks
+  constexpr int KW = LEAN == 2 ? kLongKeys : kShortKeys;
+  const LongCtx lc = SPLIT ? long_ctx<KW>(k, ap, ssm, s_pt, s_len[0]) : LongCtx{};
+  if (SPLIT) long_prefetch<KW>(k, lc, layers_s[0], 0);
 
   unsigned nbar = 0;                        // joins passed so far in this launch
   int seq = 0;                              // next tile to consume
@@ -956,7 +1234,12 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
       ap.k = LP.kcache; ap.v = LP.vcache;
       const bf16* Kc = LP.kcache;
       const bf16* Vc = LP.vcache;
-      if (LEAN || one_chunk_per_rank) {
+      if constexpr (SPLIT) {
+        long_self_attention<KW>(k, lc, LP, kvq, lvl2);
+        if (l + 1 < p.L) long_prefetch<KW>(k, lc, layers_s[l + 1], 0);
+        share_states(k, xn, lvl2, oh, ol);
+        ++xn;
+      } else if (LEAN == 1 || one_chunk_per_rank) {
         // this rank attends for its own rows; warp w folds the chunk that belongs to rank w
         for (int slot = 0; slot < NT; ++slot) {
           const int token = slot * kC + c;
@@ -1113,6 +1396,21 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
       const int kb = round1k(p.cross_rows * 128);
       ap.causal = 0; ap.limit_b = s_src; ap.k = LP.crosskv; ap.v = LP.crosskv + d; ap.ldkv = 2 * d;
       ap.bstride = (long long)p.max_src * 2 * d; ap.paged = 0;
+      if constexpr (SPLIT) {
+        // every rank needs all queries: finished rows travel like the keys and values of the self-attention block
+        for (int slot = 0; slot < NT; ++slot) {
+          const int token = slot * kC + c;
+          if (token < R && tid < kDH) {
+            float a = 0.f;
+#pragma unroll
+            for (int src = 0; src < kC; ++src) a += inbox[(src * NT + slot) * kDH + tid];
+            reinterpret_cast<float*>(kvq + token * 512 + 256)[tid] = (s_rstd[token] * (a - s_mean[token] * fs) + fc) * p.scale;
+          }
+        }
+        send_rows<NT>(k, xn, kvq, nullptr, 512, 0);
+        ++xn;
+        long_cross_attention<KW>(k, lc, LP, kvq, ckv_g, ckv_g + kb, ckv_g + 2 * kb, s_src[0], lvl2);
+      } else {
       for (int slot = 0; slot < NT; ++slot) {
         const int token = slot * kC + c;
         if (token < R) {                     // uniform over the CTA
@@ -1125,16 +1423,21 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
           __syncthreads();
           const int b = token / rpb;
           float ov;
-          if (LEAN || g.staged) ov = cross_attention_tile(ckv_g, ckv_g + kb, ckv_g + 2 * kb, b * p.max_src, s_src[b], sm);
+          if (LEAN == 1 || g.staged) ov = cross_attention_tile(ckv_g, ckv_g + kb, ckv_g + 2 * kb, b * p.max_src, s_src[b], sm);
           else ov = attention_head<float, kDH, kWarps, false>(ap, b, j, 0, s_src[b], sm);
           if (tid < kDH) store_attn_out(oh, ol, token, tid, ov);
           __syncthreads();
         }
       }
+      }
       ap.causal = 1; ap.ldkv = d; ap.paged = 1;
       seq += g.staged;
     }
-    send_rows<NT>(k, xn, oh, ol, 128, g.staged);
+    if constexpr (SPLIT) {
+      share_states(k, xn, lvl2, oh, ol, g.staged);
+    } else {
+      send_rows<NT>(k, xn, oh, ol, 128, g.staged);
+    }
     ++xn;
     BPD_TR();
     {
@@ -1328,7 +1631,7 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
 
 // The kernel's instantiations (layer_stack.cu): token tiles (1 or 2 of 8 rows), reduction steps per panel (2: d_model
 // 256, else 4), CTAs per SM (1 or 2), lean (short sequences and staged encoder rows only); null if there is none.
-const void* kernel_for(int nt, int ksteps, int minb, bool lean);
+const void* kernel_for(int nt, int ksteps, int minb, int lean);
 
 }  // namespace stack
 }  // namespace bpd

@@ -63,8 +63,10 @@ extern "C" int bpd_op_vocab_argmax_noalloc(const void* x, const void* w, int row
   p.x = x; p.ldx = d; p.w = w; p.ldw = d; p.rows = rows; p.K = d; p.N = vocab;
   p.done_counter = reinterpret_cast<unsigned*>(base); p.best = reinterpret_cast<unsigned long long*>(base + 256);
   p.out_idx = out_idx; p.out_val = out_val; p.rank_kh = 1;
-  if (dtype == 0) launch_linear_tiles<float, float, kEpiArgmax>(p, 1, st, false);
-  else launch_linear_tiles<bf16, bf16, kEpiArgmax>(p, 1, st, false);
+  // one instantiation per data type whatever the row count: what the set-up call loaded is all the later calls need
+  const dim3 grid((vocab + kTileN - 1) / kTileN, (rows + 31) / 32), block(kTileThreads);
+  if (dtype == 0) launch_k(linear_kernel<float, float, kEpiArgmax, 4>, grid, block, 0, st, false, p);
+  else launch_k(linear_kernel<bf16, bf16, kEpiArgmax, 4>, grid, block, 0, st, false, p);
   ++g_launches;
   BPD_CUDA(cudaGetLastError());
   return BPD_OK;

@@ -74,7 +74,8 @@ inline WidePlan wide_tiling(int N, int K, int T, int z, int planes, int splits, 
   // of 4 and 8 do not fill every SM) in waves, and no faster than L2 and HBM deliver.
   const double ctas = (double)w.tiles * w.splits * w.ttiles * z;
   const double kb = wide_stage_bytes(w.bn, planes) / 1024.0;
-  const int full = kSms * per_sm, slots = splits >= 8 ? full * 8 / 9 : (splits == 4 ? full * 11 / 12 : full);
+  // (15 clusters of 8 are resident at one CTA per SM, 33 at two)
+  const int full = kSms * per_sm, slots = splits >= 8 ? (per_sm == 1 ? 120 : 264) : (splits == 4 ? full * 11 / 12 : full);
   const double waves = ceil(ctas / slots), resident = std::min<double>(per_sm, ceil(ctas / kSms));
   const double in = 2.26 + w.chunks_per_split * kb * resident / 165.0 + std::max(0, w.chunks_per_split - w.stages) * 1.2 / w.stages;
   const double out = 0.0017 * w.bn / splits + (splits > 1 ? 0.022 * w.bn * (splits - 1) / splits : 0.0);
