@@ -315,18 +315,36 @@ def bpd_kernel_launches() -> int:
     return int(lib.bpd_kernel_launches())
 
 
+_top1_scratch = {}      # (device, stream) -> scratch tensor, address, bytes: kept from call to call (see _scratch_for)
+
+
+def _scratch_for(device, stream: int, nbytes: int):
+    """A scratch of at least ``nbytes`` for calls on this device and stream.  Calls on one stream run one after the
+    other and each leaves the scratch cleared, so they may share it -- also when several threads enqueue on the same
+    stream.  At most 64 are kept."""
+    key = (device, stream)
+    have = _top1_scratch.get(key)
+    if have is None or have[2] < nbytes:
+        import torch
+        if len(_top1_scratch) >= 64:
+            _top1_scratch.clear()
+        t = torch.empty(nbytes, dtype=torch.uint8, device=device)
+        have = _top1_scratch[key] = (t, t.data_ptr(), nbytes)
+    return have
+
+
 def bpd_op_vocab_argmax(x, w, want_val: bool = False):
     """x [rows, d], w [vocab, d]: CUDA tensors, both float32 or both bfloat16.  Returns idx (and val)."""
     import torch
     rows, d = x.shape
     vocab = w.shape[0]
     dtype = 0 if x.dtype == torch.float32 else 1
-    nbytes = lib.bpd_op_vocab_argmax_scratch_bytes(rows, d, vocab, dtype)
-    scratch = torch.empty(max(nbytes, 256), dtype=torch.uint8, device=x.device)
-    idx = torch.empty(rows, dtype=torch.int32, device=x.device)
-    val = torch.empty(rows, dtype=torch.float32, device=x.device) if want_val else None
-    _check(lib.bpd_op_vocab_argmax(x.data_ptr(), w.data_ptr(), rows, d, vocab, dtype, scratch.data_ptr(), nbytes,
-                                   idx.data_ptr(), None if val is None else val.data_ptr(), _stream()))
+    device, stream = x.device, _stream()
+    scratch = _scratch_for(device, stream, max(lib.bpd_op_vocab_argmax_scratch_bytes(rows, d, vocab, dtype), 256))
+    idx = torch.empty(rows, dtype=torch.int32, device=device)
+    val = torch.empty(rows, dtype=torch.float32, device=device) if want_val else None
+    _check(lib.bpd_op_vocab_argmax(x.data_ptr(), w.data_ptr(), rows, d, vocab, dtype, scratch[1], scratch[2],
+                                   idx.data_ptr(), None if val is None else val.data_ptr(), stream))
     return (idx, val) if want_val else idx
 
 
