@@ -480,7 +480,7 @@ static int run_pass(bpd_session* s, const PassArgs& a) {
   launch_linear<WT, float, kEpiArgmax>(pt, 1, st, pdl);
   prof_mark(s, kProfVocab, 1);
   VerifyParams vp = verify_params(s, a);
-  launch_k(verify_commit_kernel, dim3(1), dim3(32 * ceil_div(s->B, 32)), 0, st, pdl, vp);
+  launch_k(verify_commit_kernel, dim3(1), dim3(32 * std::min(s->B, 32)), 0, st, pdl, vp);
   ++g_launches;
   BPD_CUDA(cudaGetLastError());
   s->invocations += 1;
@@ -1005,7 +1005,7 @@ static int run_pass_tc(bpd_session* s, const PassArgs& a) {
     PassArgs a1 = a;
     a1.kh = 1; a1.knext = 1;
     VerifyParams v1 = verify_params(s, a1);
-    launch_k(verify_commit_kernel, dim3(1), dim3(32 * ceil_div(s->B, 32)), 0, st, pdl, v1);
+    launch_k(verify_commit_kernel, dim3(1), dim3(32 * std::min(s->B, 32)), 0, st, pdl, v1);
     ++g_launches;
     // stage 2: all heads at the last accepted position of every row
     GatherParams gp{static_cast<const bf16*>(s->u), s->pl_u, ldu, static_cast<bf16*>(s->u2), s->pl_u2, s->h_f32, s->h2, d,
@@ -1022,7 +1022,7 @@ static int run_pass_tc(bpd_session* s, const PassArgs& a) {
   }
   BPD_TRY(heads(s->u, s->pl_u, s->rows_dec, s->h_f32, R, a.kh, s->st.table, wants_rank(a), a.logits_dump, 0));
   VerifyParams vp = verify_params(s, a);
-  PROF(kProfVerify, launch_k(verify_commit_kernel, dim3(1), dim3(32 * ceil_div(s->B, 32)), 0, st, pdl, vp););
+  PROF(kProfVerify, launch_k(verify_commit_kernel, dim3(1), dim3(32 * std::min(s->B, 32)), 0, st, pdl, vp););
   ++g_launches;
   BPD_CUDA(cudaGetLastError());
   s->invocations += 1;

@@ -1079,96 +1079,100 @@ struct VerifyParams {
 };
 
 // Tells the host that one more pass has been verified, and whether every row is finished.
-__device__ __forceinline__ void signal_host(const RowState& st, int done) {
-  const int seq = st.signal[1];
+__device__ __forceinline__ void signal_host(const RowState& st, int epoch, int seq, int done) {
   st.signal[1] = seq + 1;
   // a plain store: the host only needs to see it some time before it enqueues the pass after the next, and no
   // other data rides on it (a system-wide fence here cost 3 us per pass)
-  *reinterpret_cast<volatile int*>(st.host_flags + (seq & 7)) = (st.signal[0] << 2) | (done ? 2 : 1);
+  *reinterpret_cast<volatile int*>(st.host_flags + (seq & 7)) = (epoch << 2) | (done ? 2 : 1);
 }
+__device__ __forceinline__ void signal_host(const RowState& st, int done) { signal_host(st, st.signal[0], st.signal[1], done); }
 
-static __global__ void verify_commit_kernel(VerifyParams p) {
+// One CTA of whole warps, a warp per row: lane i holds proposal i and the predictions of all positions for the token i
+// places ahead.  Everything a row needs is requested at once -- one thread walking the block took a round trip per
+// accepted proposal, 4 us of every pass.
+__device__ __forceinline__ void verify_commit(const VerifyParams& p) {
+  __shared__ int any_open;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
+  int epoch = 0, seq = 0;
+  if (threadIdx.x == 0) { any_open = 0; epoch = p.st.signal[0]; seq = p.st.signal[1]; }
+  __syncthreads();
+  const bool whole_block = p.mode != kModePrime && p.mode != kModePredict && p.mode != kModeGreedy;
+  for (int b = warp; b < p.B; b += nwarps) {
+    int* blk = p.st.block + b * kMaxK;
+    const int* A = p.st.table + (size_t)b * p.kcur * p.kh;
+    int tab[kMaxK];                                   // tab[r]: prediction of position r for the token `lane` places ahead
+#pragma unroll
+    for (int r = 0; r < kMaxK; ++r) tab[r] = (r < p.kcur && lane < p.kh) ? A[r * p.kh + lane] : 0;
+    const int own = lane < p.kcur ? p.st.cur_block[b * kMaxK + lane] : 0;
+    const int cnt = (whole_block && p.accept_kind == kAcceptTopN && lane >= 1 && lane < p.kcur) ? p.rank.cnt[b * p.kcur + lane - 1] : 0;
+    // p_1 for proposal `lane` sits at the position of the proposal before it
+    const int before = (lane >= 1 && lane < p.kcur) ? A[(lane - 1) * p.kh] : 0;
+    const int finished = p.st.finished[b], j = p.st.j[b], len = p.st.len[b];
+    if (finished) {
+      if (lane == 0) p.st.khat[b] = 0;
+    } else if (p.mode != kModePrime && p.mode != kModePredict && j >= p.max_new) {
+      // the caller lowered max_new below what the row already holds (bpd_iteration takes it per call): the row
+      // is complete, nothing is appended or committed
+      if (lane == 0) { p.st.khat[b] = 0; p.st.finished[b] = 1; }
+    } else if (!whole_block && p.mode != kModeGreedy) {
+      // priming: the start token becomes part of the prefix; its row of predictions is the first block.
+      // Predict call of the two-call form: the row of the last accepted token (the length was stepped back onto
+      // it) is part of the prefix again; its predictions are the next block.  The accepted count stays.
+      if (lane < p.knext) blk[lane] = tab[0];
+      if (lane == 0) {
+        p.st.len[b] = len + 1;
+        if (p.mode == kModePrime) p.st.khat[b] = 0;
+        any_open = 1;
+      }
+    } else {
+      int khat = 1, fin, mine = own;
+      if (p.mode == kModeGreedy) {
+        mine = tab[0];                                // the token itself, not a proposal
+        fin = (j + 1 >= p.max_new) || (p.eos >= 0 && __shfl_sync(0xffffffffu, mine, 0) == p.eos);
+      } else {
+        // longest prefix of the block that the base model would have produced itself
+        bool okay;
+        if (p.accept_kind == kAcceptTopN) okay = cnt < p.accept_param;
+        else if (p.accept_kind == kAcceptDistance) okay = abs(own - before) <= p.accept_param;
+        else okay = own == before;
+        const unsigned refused = __ballot_sync(0xffffffffu, lane >= 1 && lane < p.kcur && !okay && lane >= p.min_block);
+        khat = min(refused ? __ffs(refused) - 1 : p.kcur, p.max_new - j);
+        fin = (j + khat >= p.max_new);
+        const unsigned ends = __ballot_sync(0xffffffffu, p.eos >= 0 && lane < khat && own == p.eos);
+        if (ends) { khat = __ffs(ends); fin = 1; }
+      }
+      if (lane < khat) p.st.out_ids[(size_t)b * p.st.max_tgt + j + lane] = mine;
+      int next = tab[0];
+#pragma unroll
+      for (int r = 1; r < kMaxK; ++r) if (r == khat - 1) next = tab[r];
+      if (lane < p.knext) blk[lane] = next;
+      if (lane == 0) {
+        p.st.j[b] = j + khat;
+        p.st.len[b] = len + khat;     // keys/values of rejected positions stay behind the length and get overwritten
+        p.st.khat[b] = khat;
+        p.st.finished[b] = fin;
+        if (!fin) any_open = 1;
+        atomicAdd((unsigned long long*)&p.st.stats[0], 1ull);
+        atomicAdd((unsigned long long*)&p.st.stats[1], (unsigned long long)khat);
+        atomicAdd((unsigned long long*)&p.st.stats[4 + khat], 1ull);
+      }
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    atomicAdd((unsigned long long*)&p.st.stats[(p.mode == kModePrime || p.mode == kModePredict) ? 3 : 2], 1ull);
+    if (!any_open) *p.st.all_done = 1;
+    signal_host(p.st, epoch, seq, !any_open);
+  }
+}
+static __global__ void __launch_bounds__(1024) verify_commit_kernel(VerifyParams p) {
   pdl_launch_dependents();
   pdl_wait();
   if (*p.st.all_done) {
     if (threadIdx.x == 0) signal_host(p.st, 1);
     return;
   }
-  __shared__ int any_open;
-  if (threadIdx.x == 0) any_open = 0;
-  __syncthreads();
-  const int b = threadIdx.x;
-  if (b < p.B) {
-    int* blk = p.st.block + b * kMaxK;
-    const int* cur = p.st.cur_block + b * kMaxK;
-    const int* A = p.st.table + (size_t)b * p.kcur * p.kh;
-    if (p.st.finished[b]) {
-      p.st.khat[b] = 0;
-    } else if (p.mode != kModePrime && p.mode != kModePredict && p.st.j[b] >= p.max_new) {
-      // the caller lowered max_new below what the row already holds (bpd_iteration takes it per call): the row
-      // is complete, nothing is appended or committed
-      p.st.khat[b] = 0;
-      p.st.finished[b] = 1;
-    } else if (p.mode == kModePrime || p.mode == kModePredict) {
-      // priming: the start token becomes part of the prefix; its row of predictions is the first block.
-      // Predict call of the two-call form: the row of the last accepted token (the length was stepped back onto
-      // it) is part of the prefix again; its predictions are the next block.  The accepted count stays.
-      p.st.len[b] += 1;
-      if (p.mode == kModePrime) p.st.khat[b] = 0;
-      for (int i = 0; i < p.knext; ++i) blk[i] = A[i];
-      atomicOr(&any_open, 1);
-    } else if (p.mode == kModeGreedy) {
-      const int tok = A[0];
-      const int j = p.st.j[b];
-      p.st.out_ids[(size_t)b * p.st.max_tgt + j] = tok;
-      p.st.j[b] = j + 1;
-      p.st.len[b] += 1;
-      p.st.khat[b] = 1;
-      blk[0] = tok;
-      const int fin = (j + 1 >= p.max_new) || (p.eos >= 0 && tok == p.eos);
-      p.st.finished[b] = fin;
-      if (!fin) atomicOr(&any_open, 1);
-      atomicAdd((unsigned long long*)&p.st.stats[0], 1ull);
-      atomicAdd((unsigned long long*)&p.st.stats[1], 1ull);
-      atomicAdd((unsigned long long*)&p.st.stats[4 + 1], 1ull);
-    } else {
-      // longest prefix of the block that the base model would have produced itself:
-      // proposal i+1 is checked against head 1 at the position of proposal i
-      int khat = 1;
-      while (khat < p.kcur) {
-        const int top1 = A[(khat - 1) * p.kh];
-        bool okay;
-        if (p.accept_kind == kAcceptTopN) okay = p.rank.cnt[b * p.kcur + khat - 1] < p.accept_param;
-        else if (p.accept_kind == kAcceptDistance) okay = abs(cur[khat] - top1) <= p.accept_param;
-        else okay = (cur[khat] == top1);
-        if (!okay && khat >= p.min_block) break;
-        ++khat;
-      }
-      const int j = p.st.j[b];
-      khat = min(khat, p.max_new - j);
-      int fin = (j + khat >= p.max_new);
-      if (p.eos >= 0) {
-        for (int i = 0; i < khat; ++i)
-          if (cur[i] == p.eos) { khat = i + 1; fin = 1; break; }
-      }
-      for (int i = 0; i < khat; ++i) p.st.out_ids[(size_t)b * p.st.max_tgt + j + i] = cur[i];
-      p.st.j[b] = j + khat;
-      p.st.len[b] += khat;      // keys/values of rejected positions stay behind the length and get overwritten
-      p.st.khat[b] = khat;
-      for (int i = 0; i < p.knext; ++i) blk[i] = A[(khat - 1) * p.kh + i];
-      p.st.finished[b] = fin;
-      if (!fin) atomicOr(&any_open, 1);
-      atomicAdd((unsigned long long*)&p.st.stats[0], 1ull);
-      atomicAdd((unsigned long long*)&p.st.stats[1], (unsigned long long)khat);
-      atomicAdd((unsigned long long*)&p.st.stats[4 + khat], 1ull);
-    }
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    p.st.stats[(p.mode == kModePrime || p.mode == kModePredict) ? 3 : 2] += 1;
-    if (!any_open) *p.st.all_done = 1;
-    signal_host(p.st, !any_open);
-  }
+  verify_commit(p);
 }
 
 // Before a Predict call of the two-call form (Section 3): the single row it scores is the last accepted token, which
