@@ -18,7 +18,6 @@
 #include "tc_host.hpp"
 #include "fused_layer.cuh"
 #include "layer_stack.cuh"
-#include "tiny.cuh"
 
 namespace bpd {
 
@@ -1030,50 +1029,6 @@ static int run_pass_tc(bpd_session* s, const PassArgs& a) {
   return BPD_OK;
 }
 
-// ------------------------------------------------------------------ small fp32 models: a pass as one launch
-static size_t tiny_smem(const Config& c, int rows, int kh) {
-  return tiny::smem_floats(rows, kh, c.d, c.d_ff, c.k_model * c.d_hidden, c.n_dec) * sizeof(float);
-}
-// Bytes of weights a pass reads.
-static size_t tiny_weights(const Config& c) {
-  const size_t d = c.d, f = c.d_ff, k = c.k_model, fh = c.d_hidden;
-  return 4 * (c.n_dec * (6 * d * d + 2 * d * f) + k * fh * d + (c.head_layout == 0 ? k * d * k * fh : k * d * fh) + c.V * d);
-}
-// With more weights than this the eight SMs of the cluster take longer to read them (about 0.8 TB/s) than the launches
-// of a pass that uses all SMs cost.
-static bool tiny_applies(const Config& c, int B) {
-  const int rows = B * c.k_model, dh = c.d / c.H;
-  return c.dtype == 0 && rows <= tiny::kMaxRows && c.n_dec <= tiny::kMaxLayers && (dh == 16 || dh == 32) && tiny_weights(c) <= tiny::kMaxWeights &&
-         tiny_smem(c, rows, c.k_model) <= 200 * 1024;
-}
-static int run_pass_tiny(bpd_session* s, const PassArgs& a) {
-  const bpd_model* m = s->m;
-  const Config& c = m->cfg;
-  tiny::Params p;
-  memset(&p, 0, sizeof(p));
-  auto f = [](const void* q) { return static_cast<const float*>(q); };
-  for (int l = 0; l < c.n_dec; ++l) {
-    const DecLayer& L = m->dec[l];
-    p.layers[l] = tiny::Layer{f(L.ln1g), f(L.ln1b), f(L.wqkv), f(L.wo), f(L.ln2g), f(L.ln2b), f(L.cwq), f(L.cwo), f(L.ln3g), f(L.ln3b), f(L.w1), f(L.b1),
-                              f(L.w2), f(L.b2), static_cast<float*>(s->kcache[l]), static_cast<float*>(s->vcache[l]), f(s->crosskv[l])};
-  }
-  p.L = c.n_dec; p.d = c.d; p.H = c.H; p.ff = c.d_ff; p.V = c.V; p.km = c.k_model; p.fh = c.d_hidden; p.blockdiag = c.head_layout;
-  p.p1_identity = c.p1_identity; p.R = s->B * a.kcur; p.rpb = a.kcur; p.kh = a.kh; p.max_src = s->max_src;
-  p.local_q = c.local_q; p.local_m = c.local_m; p.eps = c.eps; p.scale = 1.0f / sqrtf((float)(c.d / c.H));
-  p.embed = f(m->tgt_embed); p.pe = s->pe; p.npos = s->npos;
-  p.lnfg = f(m->dec_lnf_g); p.lnfb = f(m->dec_lnf_b); p.hw1 = f(m->head_w1); p.hb1 = f(m->head_b1); p.hw2 = f(m->head_w2); p.hb2 = f(m->head_b2);
-  p.out_proj = f(m->out_proj);
-  p.forced = a.forced; p.forced_rows = a.forced_rows; p.kforced = a.kforced;
-  p.h_f32 = s->h_f32; p.verify = verify_params(s, a);
-  const void* kernel = c.d / c.H == 16 ? reinterpret_cast<const void*>(tiny::tiny_pass_kernel<16>) : reinterpret_cast<const void*>(tiny::tiny_pass_kernel<32>);
-  const size_t smem = tiny_smem(c, p.R, a.kh);
-  BPD_TRY(ensure_smem_limit(kernel, smem));
-  BPD_CUDA(launch_kc(kernel, dim3(tiny::kCtas), dim3(tiny::kThreads), smem, s->stream, false, p));
-  ++g_launches;
-  s->invocations += 1;
-  return BPD_OK;
-}
-
 #undef PROF
 static int dispatch_eager(bpd_session* s, const PassArgs& a) {
   if (a.mode == kModePredict) {
@@ -1083,7 +1038,6 @@ static int dispatch_eager(bpd_session* s, const PassArgs& a) {
     BPD_CUDA(cudaGetLastError());
   }
   if (s->tc) return run_pass_tc(s, a);
-  if (s->tiny && !s->profiling && !a.logits_dump && !a.layer_dump && !wants_rank(a)) return run_pass_tiny(s, a);
   return s->m->cfg.dtype == 0 ? run_pass<float>(s, a) : run_pass<bf16>(s, a);
 }
 
@@ -1392,7 +1346,6 @@ int bpd_session_create_opt(const bpd_model* model, int batch, int max_src, int m
   s->opt.stage_encoder_rows = o.stage_encoder_rows != 0 ? 1 : 0;
   s->opt.l2_stream_hints = o.l2_stream_hints != 0 ? 1 : 0;
   s->stack = 0; s->stack_dump = nullptr;
-  s->tiny = (o.persistent_layers != 0 && tiny_applies(model->cfg, batch)) ? 1 : 0;
   s->timed = 0;
   s->phase = kPhaseCreated; s->plan_len = 0; s->plan_k = 0; s->invocations = 0; s->pinned = nullptr;
   plan_session(model->cfg, batch, max_src, max_tgt, s->base, s);

@@ -194,7 +194,6 @@ struct bpd_session {
   // cluster occupancy do not allow it
   struct { int persistent_layers, stage_encoder_rows, l2_stream_hints; } opt;   // resolved session options
   int stack;
-  int tiny;                // small fp32 model: a pass as one launch (see tiny.cuh)
   unsigned char stack_maps[8 * 128] __attribute__((aligned(64)));   // stack::StackMaps (eight tensor maps over all layers)
   void* stack_layers;      // device: stack::LayerPtrs [n_dec]
   unsigned long long* stack_ws;   // device: [2][H][16][d] words (value, tag): the clusters' shares of the projection outputs

@@ -221,207 +221,3 @@ __device__ __forceinline__ float attend(const Params& p, const float* q, int fir
   for (int o = DH; o < 32; o <<= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
   return acc / l;
 }
-
-template <int DH>
-__global__ void __cluster_dims__(kCtas, 1, 1) __launch_bounds__(kThreads) tiny_pass_kernel(const __grid_constant__ Params p) {
-  pdl_launch_dependents();
-  const RowState& st = p.verify.st;
-  const int rank = blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  extern __shared__ __align__(16) float sm[];
-  __shared__ int s_len[kMaxRows], s_src[kMaxRows];
-  const int R = p.R, d = p.d, ff = p.ff, kh = p.kh, hid = (p.blockdiag ? kh : p.km) * p.fh, R2 = R * kh, K2 = p.blockdiag ? p.fh : hid;
-  const Split s_qkv = split_of(3 * d, d, rank), s_d = split_of(d, d, rank), s_f1 = split_of(ff, d, rank), s_f2 = split_of(d, ff, rank);
-  const Split s_h1 = split_of(hid, d, rank), s_h2 = split_of(kh * d, K2, rank), s_v = split_of(p.V, d, rank);
-  float* xbuf[2] = {sm, sm + R * d};
-  float* xn = sm + 2 * R * d;
-  float* qkv = xn + R * d;
-  float* att = qkv + 3 * R * d;
-  float* hidden = att + R * d;
-  float* u = hidden + R * ff;
-  float* o = u + R * hid;
-  unsigned long long* best = reinterpret_cast<unsigned long long*>(o + R2 * d);      // [8 CTAs][R2]
-  unsigned long long* wbest = best + kCtas * R2;                                     // [8 warps][16]
-  float* vec = reinterpret_cast<float*>(wbest + 8 * 16);                             // layer norms and biases
-  float* stage = vec + ((p.L * layer_vectors(d, ff) + 2 * d + hid + kh * d + 3) & ~3);   // a step's results
-  int cur = 0;
-  auto x_row = [&](const float* base, int ld) { return [=](int, int r) { return base + r * ld; }; };
-  auto w_row = [](const float* w, int ld) { return [=](int n) { return w + (size_t)n * ld; }; };
-
-  // weights do not depend on anything earlier in the stream
-  Ahead ah = fetch(s_qkv, d, w_row(p.layers[0].wqkv, d));
-  float* lnf = vec + p.L * layer_vectors(d, ff);
-  float* hb1 = lnf + 2 * d;
-  float* hb2 = hb1 + hid;
-  {
-    auto copy = [&](float* to, const float* from, int n) { for (int i = tid; i < n; i += kThreads) to[i] = from[i]; };
-    for (int l = 0; l < p.L; ++l) {
-      const Layer& L = p.layers[l];
-      float* v = vec + l * layer_vectors(d, ff);
-      copy(v, L.ln1g, d); copy(v + d, L.ln1b, d); copy(v + 2 * d, L.ln2g, d); copy(v + 3 * d, L.ln2b, d);
-      copy(v + 4 * d, L.ln3g, d); copy(v + 5 * d, L.ln3b, d); copy(v + 6 * d, L.b2, d); copy(v + 7 * d, L.b1, ff);
-    }
-    copy(lnf, p.lnfg, d); copy(lnf + d, p.lnfb, d); copy(hb1, p.hb1, hid); copy(hb2, p.hb2, kh * d);
-  }
-  pdl_wait();
-  if (*st.all_done) {
-    if (rank == 0 && tid == 0) signal_host(st, 1);
-    return;
-  }
-  if (tid < R / p.rpb) { s_len[tid] = st.len[tid]; s_src[tid] = st.src_len[tid]; }
-  __syncthreads();
-  // embedding: every CTA for itself
-  for (int r = warp; r < R; r += kThreads / 32) {
-    const int b = r / p.rpb, i = r % p.rpb;
-    int tok = st.block[b * kMaxK + i], pos = s_len[b] + i;
-    if (p.forced && i >= 1 && i < p.kforced) {
-      const int jb = st.j[b];
-      if (p.forced_rows == 1) tok = p.forced[(size_t)b * (p.kforced - 1) + (i - 1)];
-      else if (jb < p.forced_rows) tok = p.forced[((size_t)b * p.forced_rows + jb) * (p.kforced - 1) + (i - 1)];
-    }
-    if (rank == 0 && lane == 0) st.cur_block[b * kMaxK + i] = tok;
-    if (tok < 0 || tok >= p.V || pos >= p.npos) {           // never index outside the tables; report instead
-      if (rank == 0 && lane == 0) atomicCAS(st.error, 0, 1);
-      tok = 0;
-      pos = 0;
-    }
-    const float scale = sqrtf((float)d);
-    for (int c = lane; c < d; c += 32) xbuf[0][r * d + c] = p.embed[(size_t)tok * d + c] * scale + p.pe[(size_t)pos * d + c];
-  }
-  __syncthreads();
-  arrive();
-  wait();                                                   // every CTA runs: its shared memory may be written
-
-  // a step's end: its results go to every CTA; the next step's weights are requested while the barrier closes
-  auto turn = [&](const Split& mine, const float* in, int ld_in, float* out, int ld_out, const Split& next, int K, auto row) {
-    share(mine, R, in, ld_in, out, ld_out);
-    arrive();
-    ah = fetch(next, K, row);
-    wait();
-  };
-  const int ldd = ((s_d.n1 - s_d.n0) + 3) & ~3, ldq = ((s_qkv.n1 - s_qkv.n0) + 3) & ~3, ldf = ((s_f1.n1 - s_f1.n0) + 3) & ~3;
-  const int item0 = rank + kCtas * warp;                    // this warp's first (row, head)
-  auto share_head = [&](int r, int h, float y) {
-    if (lane < DH) {
-#pragma unroll
-      for (int c = 0; c < kCtas; ++c) asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(remote(att + r * d + h * DH + lane, c)), "f"(y) : "memory");
-    }
-  };
-  for (int l = 0; l < p.L; ++l) {
-    const Layer& L = p.layers[l];
-    const float* v = vec + l * layer_vectors(d, ff);
-    // committed keys and values, encoder rows: straight from L2, requested ahead
-    auto place = [&](int b, int pos) { return ((size_t)st.page_table[b * st.pages_per_row + pos / kPage] * kPage + pos % kPage) * d; };
-    auto self_first = [&](int own) { return p.local_q > 0 ? max(0, (own / p.local_q) * p.local_q - p.local_m) : 0; };
-    AttnAhead<DH> aa;
-    if (item0 < R * p.H) {
-      const int r = item0 / p.H, h = item0 % p.H, b = r / p.rpb;
-      aa = attn_fetch<DH>(self_first(s_len[b] + r % p.rpb), s_len[b], [&](int pos) { return L.kcache + place(b, pos) + h * DH; },
-                          [&](int pos) { return L.vcache + place(b, pos) + h * DH; });
-    }
-    normalise(p, xbuf[cur], xn, v, v + d);
-    project<4>(s_qkv, d, R, ah, w_row(L.wqkv, d), x_row(xn, d), [&](int n, int r, float y) {
-      stage[r * ldq + n - s_qkv.n0] = y;
-      if (n >= d) {
-        const int b = r / p.rpb;
-        const size_t at = place(b, s_len[b] + r % p.rpb);
-        (n < 2 * d ? L.kcache + at + (n - d) : L.vcache + at + (n - 2 * d))[0] = y;
-      }
-    });
-    turn(s_qkv, stage, ldq, qkv, 3 * d, s_d, d, w_row(L.wo, d));
-    for (int item = item0; item < R * p.H; item += kCtas * (kThreads / 32)) {
-      const int r = item / p.H, h = item % p.H, b = r / p.rpb, len = s_len[b], own = len + r % p.rpb;
-      auto at = [&](const float* cache, int which, int pos) {
-        if (pos >= len) return (const float*)(qkv + (b * p.rpb + pos - len) * 3 * d + which * d + h * DH);
-        return cache + place(b, pos) + h * DH;
-      };
-      share_head(r, h, attend<DH>(p, qkv + r * 3 * d + h * DH, self_first(own), own + 1, item == item0 ? len : 0, aa,
-                                  [&](int pos) { return at(L.kcache, 1, pos); }, [&](int pos) { return at(L.vcache, 2, pos); }));
-    }
-    arrive();
-    if (item0 < R * p.H) {
-      const int h = item0 % p.H, b = item0 / p.H / p.rpb;
-      const float* kv = L.crosskv + (size_t)b * p.max_src * 2 * d + h * DH;
-      aa = attn_fetch<DH>(0, s_src[b], [&](int pos) { return kv + (size_t)pos * 2 * d; }, [&](int pos) { return kv + (size_t)pos * 2 * d + d; });
-    }
-    wait();
-    project<4>(s_d, d, R, ah, w_row(L.wo, d), x_row(att, d), [&](int n, int r, float y) { stage[r * ldd + n - s_d.n0] = xbuf[cur][r * d + n] + y; });
-    turn(s_d, stage, ldd, xbuf[cur ^ 1], d, s_d, d, w_row(L.cwq, d));
-    cur ^= 1;
-    normalise(p, xbuf[cur], xn, v + 2 * d, v + 3 * d);
-    project<4>(s_d, d, R, ah, w_row(L.cwq, d), x_row(xn, d), [&](int n, int r, float y) { stage[r * ldd + n - s_d.n0] = y; });
-    turn(s_d, stage, ldd, qkv, 3 * d, s_d, d, w_row(L.cwo, d));
-    for (int item = item0; item < R * p.H; item += kCtas * (kThreads / 32)) {
-      const int r = item / p.H, h = item % p.H, b = r / p.rpb;
-      const float* kv = L.crosskv + (size_t)b * p.max_src * 2 * d + h * DH;
-      share_head(r, h, attend<DH>(p, qkv + r * 3 * d + h * DH, 0, s_src[b], item == item0 ? s_src[b] : 0, aa,
-                                  [&](int pos) { return kv + (size_t)pos * 2 * d; }, [&](int pos) { return kv + (size_t)pos * 2 * d + d; }));
-    }
-    arrive();
-    wait();
-    project<4>(s_d, d, R, ah, w_row(L.cwo, d), x_row(att, d), [&](int n, int r, float y) { stage[r * ldd + n - s_d.n0] = xbuf[cur][r * d + n] + y; });
-    turn(s_d, stage, ldd, xbuf[cur ^ 1], d, s_f1, d, w_row(L.w1, d));
-    cur ^= 1;
-    normalise(p, xbuf[cur], xn, v + 4 * d, v + 5 * d);
-    project<4>(s_f1, d, R, ah, w_row(L.w1, d), x_row(xn, d), [&](int n, int r, float y) { stage[r * ldf + n - s_f1.n0] = fmaxf(y + v[7 * d + n], 0.f); });
-    turn(s_f1, stage, ldf, hidden, ff, s_f2, ff, w_row(L.w2, ff));
-    project<4>(s_f2, ff, R, ah, w_row(L.w2, ff), x_row(hidden, ff), [&](int n, int r, float y) {
-      stage[r * ldd + n - s_f2.n0] = xbuf[cur][r * d + n] + y + v[6 * d + n];
-    });
-    if (l + 1 < p.L) turn(s_f2, stage, ldd, xbuf[cur ^ 1], d, s_qkv, d, w_row(p.layers[l + 1].wqkv, d));
-    else turn(s_f2, stage, ldd, xbuf[cur ^ 1], d, s_h1, d, w_row(p.hw1, d));
-    cur ^= 1;
-  }
-  // heads
-  normalise(p, xbuf[cur], xn, lnf, lnf + d);
-  if (rank == 0)
-    for (int i = tid; i < R * d; i += kThreads) p.h_f32[i] = xn[i];
-  const int ldh = ((s_h1.n1 - s_h1.n0) + 3) & ~3, ldo = ((s_h2.n1 - s_h2.n0) + 3) & ~3;
-  project<4>(s_h1, d, R, ah, w_row(p.hw1, d), x_row(xn, d), [&](int n, int r, float y) { stage[r * ldh + n - s_h1.n0] = fmaxf(y + hb1[n], 0.f); });
-  turn(s_h1, stage, ldh, u, hid, s_h2, K2, w_row(p.hw2, K2));
-  project<4>(s_h2, K2, R, ah, w_row(p.hw2, K2), [&](int n, int r) { return u + r * hid + (p.blockdiag ? (n / d) * p.fh : 0); }, [&](int n, int r, float y) {
-    const float h = xn[r * d + n % d];
-    stage[r * ldo + n - s_h2.n0] = (p.p1_identity && n < d) ? h : y + hb2[n] + h;
-  });
-  turn(s_h2, stage, ldo, o, kh * d, s_v, d, w_row(p.out_proj, d));
-  // vocabulary top-1: 16 rows at a time; lane s of a feature's lanes keeps the best of rows s, s + ks, ..
-  for (int rb = 0; rb < R2; rb += 16) {
-    const int nr = min(16, R2 - rb);
-    unsigned long long mine[16];
-#pragma unroll
-    for (int i = 0; i < 16; ++i) mine[i] = 0ull;
-    project<16>(s_v, d, nr, ah, w_row(p.out_proj, d), [&](int, int r) { return o + (rb + r) * d; }, [&](int n, int r, float y) {
-      const unsigned long long key = ((unsigned long long)order_bits(y) << 32) | (0xffffffffu - (unsigned)n);
-#pragma unroll
-      for (int i = 0; i < 16; ++i) if (i == r && key > mine[i]) mine[i] = key;
-    });
-#pragma unroll
-    for (int i = 0; i < 16; ++i) {
-      // the maximum of a row over the warp: the ordered value first, then the lowest index that has it
-      const unsigned top = __reduce_max_sync(0xffffffffu, (unsigned)(mine[i] >> 32));
-      const unsigned low = __reduce_max_sync(0xffffffffu, (unsigned)(mine[i] >> 32) == top ? (unsigned)mine[i] : 0u);
-      if (lane == 0) wbest[warp * 16 + i] = ((unsigned long long)top << 32) | low;
-    }
-    __syncthreads();
-    if (tid < nr) {
-      unsigned long long k = wbest[tid];
-#pragma unroll
-      for (int w = 1; w < 8; ++w) if (wbest[w * 16 + tid] > k) k = wbest[w * 16 + tid];
-      asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(remote(best + rank * R2 + rb + tid, 0)), "l"(k) : "memory");
-    }
-    __syncthreads();
-  }
-  arrive();
-  wait();
-  if (rank != 0) return;
-  for (int r = tid; r < R2; r += kThreads) {
-    unsigned long long k = best[r];
-#pragma unroll
-    for (int c = 1; c < kCtas; ++c) if (best[c * R2 + r] > k) k = best[c * R2 + r];
-    st.table[r] = (int)(0xffffffffu - (unsigned)(k & 0xffffffffull));
-  }
-  __syncthreads();
-  verify_commit(p.verify);
-}
-
-}  // namespace tiny
-}  // namespace bpd

@@ -85,37 +85,3 @@ def test_many_row_attention_decodes_like_the_oracle(bpd, batch, k, max_src, tgt,
             break
     s.close()
     model.close()
-
-
-# the one-launch pass of small fp32 models against the launch-per-step path: widths that leave CTAs without features, feature
-# counts and vocabularies with remainders, one and 16 rows, more than one chunk of 32 keys, both head layouts
-@pytest.mark.parametrize("d,heads,ff,vocab,k,hidden,batch,layout,local", [
-    (16, 1, 8, 5, 1, 8, 1, 0, 0), (48, 3, 72, 37, 3, 40, 5, 0, 0), (64, 2, 264, 513, 4, 256, 4, 1, 0), (128, 4, 136, 300, 8, 24, 2, 0, 0),
-    (64, 4, 256, 512, 4, 256, 3, 0, 16)])
-def test_small_fp32_pass_in_one_launch(bpd, d, heads, ff, vocab, k, hidden, batch, layout, local):
-    from bpd_inputs import ModelConfig, make_weights
-    cfg = ModelConfig(1, 2, d, heads, ff, vocab, k, hidden, dtype=0, head_layout=layout, local_q=local, local_m=local // 2)
-    model = bpd.Model(make_weights(cfg, 9, 0.15))
-    rng = np.random.default_rng(d + k)
-    S, N = 41, 50
-    lens = rng.integers(1, S + 1, batch).astype(np.int32)
-    src = rng.integers(0, vocab, (batch, S)).astype(np.int32)
-    got = {}
-    for one in (1, 0):
-        s = bpd.Session(model, batch, S, N, options={} if one else {"persistent_layers": 0})
-        s.bpd_encode(src, lens)
-        steps = [s.bpd_iteration(k, N, want_hidden=True, accept_mode=k << 16) for _ in range(-(-N // k))]
-        s.bpd_encode(src, lens)
-        launches = bpd.bpd_kernel_launches()
-        ids = s.bpd_decode_greedy(N)[0]
-        launches = bpd.bpd_kernel_launches() - launches
-        s.bpd_encode(src, lens)
-        blockwise = s.bpd_decode_blockwise(k, N)[0]
-        s.close()
-        assert np.array_equal(ids, blockwise)
-        assert (launches <= N + 3) == bool(one)
-        got[one] = ids, steps
-    for a, b in zip(got[1][1], got[0][1]):
-        np.testing.assert_allclose(a["hidden"].cpu().numpy(), b["hidden"].cpu().numpy(), atol=2e-5)
-    assert np.array_equal(got[1][0], got[0][0])
-    model.close()
