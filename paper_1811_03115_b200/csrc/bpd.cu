@@ -254,7 +254,10 @@ static size_t plan_session(const Config& c, int B, int max_src, int max_tgt, cha
   return align_up(a.off);
 }
 
-static size_t fold_floats(const Config& c) { return c.dtype == 1 ? (size_t)c.n_dec * 2 * (3 * c.d + c.d + c.d_ff) : 0; }
+static size_t fold_floats(const Config& c) {
+  if (c.dtype != 1) return 0;
+  return (size_t)c.n_dec * 2 * (3 * c.d + c.d + c.d_ff + 2 * c.d) + (size_t)c.n_enc * 2 * (3 * c.d + c.d_ff);
+}
 static size_t weight_bytes_for(const ParsedBlob& pb) { return align_up(pb.total) + align_up(fold_floats(pb.cfg) * sizeof(float)); }
 
 // ------------------------------------------------------------------ launches
@@ -518,6 +521,24 @@ static int run_encoder_tc(bpd_session* s) {
   memset(&ep, 0, sizeof(ep));
   ep.table = m->src_embed; ep.pe = s->pe; ep.npos = s->npos; ep.x = s->x; ep.rows = E; ep.rows_per_b = s->max_src;
   ep.d = d; ep.vocab = c.V; ep.st = s->st; ep.src = s->src_dev;
+  // Layer norms folded into the projections behind them, statistics as per-tile partial results (see TcParams::stat_out).
+  // The encoder is a chain of launches that wait on one another, about 5 us each at these sizes whatever they move, so what
+  // counts is their number: 50 -> 32 for six layers, with all keys and values for the decoder in one launch.  One 25-word
+  // sentence (base model) 231 -> 198 us, five ragged ones 316 -> 261, 32 sentences (big) 1180 -> 1152.
+  const bool fold = s->fold_enc != 0;
+  auto planes_of = [&](tc::TcParams& q, const void* gain) {
+    if (!fold) return;
+    q.g_next = static_cast<const bf16*>(gain); q.xg_hi = static_cast<bf16*>(s->xn); q.xg_plane = s->pl_xn;
+    q.stat_out = s->ln_stats; q.stat_T = E;
+  };
+  auto norm_of = [&](tc::TcParams& q, const float* fs, const float* fc) {
+    if (!fold) return;
+    q.stat_in = s->ln_stats; q.stat_parts = d / 128; q.stat_T = E; q.ln_s = fs; q.ln_c = fc; q.ln_eps = c.eps;
+  };
+  if (fold) {
+    ep.gain = static_cast<const bf16*>(m->enc[0].ln1g); ep.xg_hi = static_cast<bf16*>(s->xn); ep.xg_plane = s->pl_xn;
+    ep.stat_out = s->ln_stats; ep.stat_T = E;
+  }
   embed_kernel<bf16><<<E, 128, 0, st>>>(ep);
   ++g_launches;
   const tc::Operands xn{nullptr, 0, s->xn, s->pl_xn, d, s->rows_all, d};
@@ -526,9 +547,10 @@ static int run_encoder_tc(bpd_session* s) {
   auto with_w = [](tc::Operands o, const void* w, int rows) { o.w = w; o.w_rows = rows; return o; };
   for (int l = 0; l < c.n_enc; ++l) {
     const EncLayer& L = m->enc[l];
-    launch_ln<bf16, float>(s->x, L.ln1g, L.ln1b, s->xn, nullptr, E, d, c.eps, nullptr, st, s->pl_xn, pdl);
+    if (!fold) launch_ln<bf16, float>(s->x, L.ln1g, L.ln1b, s->xn, nullptr, E, d, c.eps, nullptr, st, s->pl_xn, pdl);
     tc::TcParams pq = tc_params(nullptr, 0, nullptr);
     pq.out_f32 = static_cast<float*>(s->qbuf); pq.ldo = 3 * d;
+    norm_of(pq, L.s_qkv, L.c_qkv);
     BPD_TRY(tc::launch<tc::kTcF32>(with_w(xn, L.wqkv, 3 * d), 3 * d, d, E, pq, sc, st, 1, 0, 0, pdl)); ++g_launches;
     AttnParams ap;
     memset(&ap, 0, sizeof(ap));
@@ -540,20 +562,33 @@ static int run_encoder_tc(bpd_session* s) {
     BPD_TRY(attend<float>(ap, s->max_src, s->max_src, false, st, pdl));
     tc::TcParams po = tc_params(nullptr, 0, nullptr);
     po.out_f32 = s->x; po.ldo = d;
+    planes_of(po, L.ln2g);
     BPD_TRY(tc::launch<tc::kTcResidual>(with_w(at, L.wo, d), d, d, E, po, sc, st, 1, 0, 0, pdl)); ++g_launches;
-    launch_ln<bf16, float>(s->x, L.ln2g, L.ln2b, s->xn, nullptr, E, d, c.eps, nullptr, st, s->pl_xn, pdl);
+    if (!fold) launch_ln<bf16, float>(s->x, L.ln2g, L.ln2b, s->xn, nullptr, E, d, c.eps, nullptr, st, s->pl_xn, pdl);
     tc::TcParams p1 = tc_params(L.b1, 1, nullptr);
     p1.out_hi = static_cast<bf16*>(s->ffh); p1.plane = s->pl_ffh; p1.ldo = f;
+    norm_of(p1, L.s_f1, L.c_f1);
     BPD_TRY(tc::launch<tc::kTcPlanes>(with_w(xn, L.w1, f), f, d, E, p1, sc, st, 1, 0, 0, pdl)); ++g_launches;
     tc::TcParams p2 = tc_params(L.b2, 0, nullptr);
     p2.out_f32 = s->x; p2.ldo = d;
+    planes_of(p2, l + 1 < c.n_enc ? m->enc[l + 1].ln1g : m->enc_lnf_g);
     BPD_TRY(tc::launch<tc::kTcResidual>(with_w(fh, L.w2, d), d, f, E, p2, sc, st, 1, 0, 0, pdl)); ++g_launches;
   }
-  launch_ln<bf16, float>(s->x, m->enc_lnf_g, m->enc_lnf_b, s->xn, nullptr, E, d, c.eps, nullptr, st, s->pl_xn, pdl);
-  for (int l = 0; l < c.n_dec; ++l) {
+  if (!fold) launch_ln<bf16, float>(s->x, m->enc_lnf_g, m->enc_lnf_b, s->xn, nullptr, E, d, c.eps, nullptr, st, s->pl_xn, pdl);
+  // keys and values of all decoder layers: one launch where the layers' weights lie a whole number of rows apart (they do
+  // in a blob written layer after layer), else one per layer
+  const long long row = 2LL * d, step = c.n_dec > 1 ? (const char*)m->dec[1].cwkv - (const char*)m->dec[0].cwkv : 0;
+  bool regular = step % row == 0 && step >= 0 && step / row < (1 << 24);
+  for (int l = 1; l + 1 < c.n_dec; ++l) regular = regular && (const char*)m->dec[l + 1].cwkv - (const char*)m->dec[l].cwkv == step;
+  const int slices = regular ? c.n_dec : 1;
+  for (int l = 0; l < c.n_dec; l += slices) {
     tc::TcParams pk = tc_params(nullptr, 0, nullptr);
     pk.out_f32 = static_cast<float*>(s->crosskv[l]); pk.ldo = 2 * d;
-    BPD_TRY(tc::launch<tc::kTcF32>(with_w(xn, m->dec[l].cwkv, 2 * d), 2 * d, d, E, pk, sc, st, 1, 0, 0, pdl)); ++g_launches;
+    norm_of(pk, m->dec[l].s_ckv, m->dec[l].c_ckv);
+    if (slices > 1) { pk.zofs_out = static_cast<float*>(s->crosskv[1]) - static_cast<float*>(s->crosskv[0]); pk.zofs_ln = 4 * d; }
+    const int rows_apart = (int)(step / row);
+    BPD_TRY(tc::launch<tc::kTcF32>(with_w(xn, m->dec[l].cwkv, (slices - 1) * rows_apart + 2 * d), 2 * d, d, E, pk, sc, st, slices, slices > 1 ? rows_apart : 0, 0, pdl));
+    ++g_launches;
   }
   BPD_CUDA(cudaGetLastError());
   return BPD_OK;
@@ -1279,6 +1314,13 @@ int bpd_load_weights(const void* blob, size_t blob_bytes, void* dev_weight_buf, 
       fold(L.cwq, L.ln2g, L.ln2b, nullptr, d, &L.s_cq, &L.c_cq);
       fold(L.w1, L.ln3g, L.ln3b, L.b1, f, &L.s_f1, &L.c_f1);
     }
+    for (int l = 0; l < c.n_enc; ++l) {
+      EncLayer& L = m->enc[l];
+      fold(L.wqkv, L.ln1g, L.ln1b, nullptr, 3 * d, &L.s_qkv, &L.c_qkv);
+      fold(L.w1, L.ln2g, L.ln2b, L.b1, f, &L.s_f1, &L.c_f1);
+    }
+    // in layer order, so that one launch over all layers steps through them (TcParams::zofs_ln)
+    for (int l = 0; l < c.n_dec; ++l) fold(m->dec[l].cwkv, m->enc_lnf_g, m->enc_lnf_b, nullptr, 2 * d, &m->dec[l].s_ckv, &m->dec[l].c_ckv);
     e = cudaGetLastError();
   }
   if (e == cudaSuccess) e = cudaStreamSynchronize(m->stream);
@@ -1340,6 +1382,7 @@ int bpd_session_create_opt(const bpd_model* model, int batch, int max_src, int m
   // passes of at most 16 rows take the statistics from the stream itself; wider ones need whole 128-feature tiles (and
   // the embedding kernel whole warps: d_model a multiple of 256)
   s->fold_ln = (s->tc && o.fold_layer_norms != 0 && (batch * model->cfg.k_model <= 16 || model->cfg.d % 256 == 0)) ? 1 : 0;
+  s->fold_enc = (s->tc && o.fold_layer_norms != 0 && model->cfg.d % 256 == 0) ? 1 : 0;
   s->fused = (s->tc && fused::supported(model->cfg.d, model->cfg.H, model->cfg.d_ff, batch * model->cfg.k_model) &&
               o.cluster_layers != 0) ? 1 : 0;
   s->opt.persistent_layers = o.persistent_layers;   // -1: where its lean variant applies (measured faster there), 0: never, 1: wherever it runs

@@ -71,6 +71,7 @@ struct TcParams {
   const float* h; int d;       // kTcHeadOut residual; kTcQkv model width
   int head_identity;
   int zofs_n;                  // column offset of this z-slice inside the output row (block-diagonal heads)
+  int zofs_ln; long long zofs_out;   // wide kernel: offset of a z-slice in ln_s / ln_c, and in out_f32 (kTcF32)
   bf16* kcache; bf16* vcache;  // kTcQkv
   RowState st; int rows_per_b;
   // split-K workspace

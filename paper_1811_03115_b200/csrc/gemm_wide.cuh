@@ -79,7 +79,7 @@ __device__ __forceinline__ void finish_setup(const TcParams& p, int z, int tile,
   c.folded = (p.stat_in != nullptr);
   if (c.n >= p.N) return;
   if (c.folded) {
-    const float4 s4 = *reinterpret_cast<const float4*>(p.ln_s + c.n), c4 = *reinterpret_cast<const float4*>(p.ln_c + c.n);
+    const float4 s4 = *reinterpret_cast<const float4*>(p.ln_s + c.n + p.zofs_ln * z), c4 = *reinterpret_cast<const float4*>(p.ln_c + c.n + p.zofs_ln * z);
     c.lns[0] = s4.x; c.lns[1] = s4.y; c.lns[2] = s4.z; c.lns[3] = s4.w;
     c.bias[0] = c4.x; c.bias[1] = c4.y; c.bias[2] = c4.z; c.bias[3] = c4.w;
   } else if (p.bias && p.vec) {
@@ -128,7 +128,7 @@ __device__ __forceinline__ void finish_item(const TcParams& p, const FinishCtx& 
     *reinterpret_cast<uint2*>(p.out_hi + o) = pack4_bf16(hi);
     *reinterpret_cast<uint2*>(p.out_hi + o + p.plane) = pack4_bf16(lo);
   } else if (EPI == kTcF32) {
-    float* y = p.out_f32 + (long long)t * p.ldo + n;
+    float* y = p.out_f32 + p.zofs_out * z + (long long)t * p.ldo + n;
     if (p.vec) {
       *reinterpret_cast<float4*>(y) = make_float4(v[0], v[1], v[2], v[3]);
     } else {

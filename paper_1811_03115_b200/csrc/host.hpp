@@ -111,11 +111,13 @@ int parse_blob(const void* blob, size_t n, ParsedBlob* out);
 
 struct EncLayer {
   const void *ln1g, *ln1b, *wqkv, *wo, *ln2g, *ln2b, *w1, *b1, *w2, *b2;
+  float *s_qkv, *c_qkv, *s_f1, *c_f1;   // layer norms folded into the projections that follow them (bf16 models)
 };
 struct DecLayer {
   const void *ln1g, *ln1b, *wqkv, *wo, *ln2g, *ln2b, *cwq, *cwkv, *cwo, *ln3g, *ln3b, *w1, *b1, *w2, *b2;
   // layer norms folded into the projections that follow them (bf16 models): per-feature s and c vectors
   float *s_qkv, *c_qkv, *s_cq, *c_cq, *s_f1, *c_f1;
+  float *s_ckv, *c_ckv;    // the encoder's final layer norm, folded into the keys and values of this layer's cross-attention
 };
 
 }  // namespace bpd
@@ -185,6 +187,7 @@ struct bpd_session {
   int lazy_heads;          // two-stage head evaluation (p_1 everywhere, all heads only at the accepted position)
   int last_pass_lazy;
   void* u2; long long pl_u2; float* h2; int *table2, *table_full;
+  int fold_enc;            // the same in the encoder
   int fold_ln;             // decoder layer norms are folded into the projections that follow them
   float* ln_stats;         // [d / 128][rows][2]: per-tile mean and squared deviations of the residual stream (passes of more than 16 rows)
   int fused;               // decoder layers as three launches each (clusters; at most 16 rows per pass)

@@ -314,7 +314,7 @@ int launch(const Operands& op, int N, int K, int T, TcParams p, const Scratch& s
   {
     // vector stores in the epilogue: every row offset and pointer involved must allow them
     auto al = [](const void* q, size_t a) { return q == nullptr || (uintptr_t)q % a == 0; };
-    p.vec = (N % 4 == 0 && p.ldo % 4 == 0 && p.plane % 4 == 0 && p.xg_plane % 4 == 0 && p.zofs_n % 4 == 0 &&
+    p.vec = (N % 4 == 0 && p.ldo % 4 == 0 && p.plane % 4 == 0 && p.xg_plane % 4 == 0 && p.zofs_n % 4 == 0 && p.zofs_ln % 4 == 0 && p.zofs_out % 4 == 0 &&
              (p.d % 4 == 0) && al(p.out_f32, 16) && al(p.out_hi, 8) && al(p.xg_hi, 8) && al(p.h, 16) && al(p.bias, 8) &&
              al(p.g_next, 8) && al(p.kcache, 8) && al(p.vcache, 8)) ? 1 : 0;
   }

@@ -85,3 +85,29 @@ def test_many_row_attention_decodes_like_the_oracle(bpd, batch, k, max_src, tgt,
             break
     s.close()
     model.close()
+
+
+# the encoder with its layer norms folded into the projections (widths of whole pairs of tiles) and with layer-norm kernels,
+# one decoder layer (its own launch of keys and values) and several (one launch), from one encoder row to several token tiles
+@pytest.mark.parametrize("batch,max_src,d,n_dec", [(1, 1, 256, 2), (2, 9, 256, 1), (5, 60, 512, 3), (3, 40, 192, 2)])
+def test_encoder_feeds_the_decoder_like_the_oracle(bpd, batch, max_src, d, n_dec):
+    from bpd_inputs import ModelConfig, make_weights
+    from oracle.decode import TransformerScorer
+    from oracle.model import parse_blob
+    blob = make_weights(ModelConfig(2, n_dec, d, d // 64, 2 * d, 300, 4, 64), 5, 0.06)
+    rng = np.random.default_rng(d + batch)
+    lens = rng.integers(1, max_src + 1, batch).astype(np.int32)
+    lens[-1] = max_src
+    src = rng.integers(2, 300, (batch, max_src)).astype(np.int32)
+    model = bpd.Model(blob)
+    s = bpd.Session(model, batch, max_src, 8)
+    s.bpd_encode(src, lens)
+    r = s.bpd_iteration(4, 8, want_hidden=True)
+    model_o = parse_blob(blob)
+    for b in range(batch):
+        scorer = TransformerScorer(model_o, src[b], int(lens[b]), cached=True, capacity=14)
+        scorer([0], 1)
+        scorer([0] + [int(t) for t in r["block"][b]], 4)
+        np.testing.assert_allclose(r["hidden"][b].cpu().numpy(), scorer.last_hidden, atol=8e-3)     # the cache is bf16
+    s.close()
+    model.close()
