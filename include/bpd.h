@@ -104,12 +104,13 @@ typedef struct {
   int32_t dependent_launch;   /* programmatic dependent launch between the kernels of a pass               */
   int32_t lazy_heads;         /* two-stage heads: p_1 at all k positions, all heads only at the accepted
                                  one (default: on when batch * k_model >= 64)                              */
-  int32_t fold_layer_norms;   /* decoder layer norms folded into the projections after them (<= 16 rows)   */
+  int32_t fold_layer_norms;   /* layer norms folded into the projections after them (encoder, and decoder) */
   int32_t cluster_layers;     /* decoder layers as three cluster launches each (<= 16 rows per pass)        */
   int32_t persistent_layers;  /* all decoder layers of a pass in one persistent TMA-fed kernel (<= 16 rows
                                  per pass, d_model 256 / 512 / 1024; takes precedence over cluster_layers).
                                  Default: on for sessions of at most 256 positions whose encoder rows fit
-                                 the staging tile (measured faster there) while no other live session of
+                                 the staging tile, and for one sequence of any length where a CTA has an
+                                 SM to itself (measured faster there), while no other live session of
                                  the device has it, off elsewhere; 1 asks for it wherever it runs.  See
                                  bpd_session_create_opt for what it needs                                  */
   int32_t stage_encoder_rows; /* encoder keys / values staged in shared memory for cross-attention          */
