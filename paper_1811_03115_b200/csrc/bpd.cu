@@ -165,6 +165,25 @@ static int session_wide_rows(const Config& c, int B) {
   return rmax > tc::kNarrowBN ? rmax : 0;
 }
 
+// Shapes the persistent kernel is built for.
+static bool stack_shapes_ok(const Config& c, int rows) {
+  const int d = c.d, H = c.H;
+  if (c.dtype != 1 || H < 1 || d != H * fused::kDH || (d != 256 && d != 512 && d != 1024)) return false;
+  if (c.d_ff % H || (c.d_ff / H != 128 && c.d_ff / H != 256)) return false;   // hidden units per cluster
+  if (rows < 1 || rows > fused::kMaxRows || c.n_dec > 64) return false;
+  return true;
+}
+
+// Sessions of several sequences whose passes have more rows than one set of clusters of the persistent layer kernel takes
+// in its fastest shape (8): groups of sequences, each with H clusters of its own.  At two CTAs per SM 33 clusters of 8 are
+// resident.  0: no groups.
+static int stack_groups(const Config& c, int B, int* seqs) {
+  *seqs = std::max(1, 8 / c.k_model);
+  const int groups = ceil_div(B, *seqs);
+  return B > 1 && B * c.k_model > (c.H <= 15 ? 8 : fused::kMaxRows) && c.k_model <= fused::kMaxRows && groups * c.H <= 33 &&
+         groups <= stack::kMaxGroups ? groups : 0;
+}
+
 // Lays the session out; with base == nullptr only measures.
 static size_t plan_session(const Config& c, int B, int max_src, int max_tgt, char* base, bpd_session* s) {
   Arena a;
@@ -232,8 +251,11 @@ static size_t plan_session(const Config& c, int B, int max_src, int max_tgt, cha
   float* fused_ws = a.take<float>(fused_ok ? fused_parts * Rmax * d : 0);
   unsigned* fused_counters = a.take<unsigned>(fused::kC);
   // persistent layer stack: tensor maps, per-layer pointers, the clusters' partial outputs, the join's words
-  void* stack_layers = a.take_bytes(fused_ok ? (size_t)c.n_dec * sizeof(stack::LayerPtrs) : 0);
-  unsigned long long* stack_ws = a.take<unsigned long long>(fused_ok ? (size_t)2 * (c.H + 1) * fused::kMaxRows * d : 0);
+  void* stack_layers = a.take_bytes((size_t)c.n_dec * sizeof(stack::LayerPtrs));
+  int group_seqs;
+  const int groups = c.dtype == 1 && stack_shapes_ok(c, c.k_model) ? stack_groups(c, B, &group_seqs) : 0;
+  const size_t stack_sets = std::max<size_t>(groups, fused_ok ? 1 : 0);
+  unsigned long long* stack_ws = a.take<unsigned long long>(stack_sets * 2 * (c.H + 1) * fused::kMaxRows * d);
   unsigned* stack_bar = a.take<unsigned>(stack::kBarWords);
   float* ln_stats = a.take<float>((size_t)ceil_div(d, 128) * Rall * 2);
   if (s) {
@@ -677,7 +699,7 @@ static int run_layers_fused(bpd_session* s, const PassArgs& a) {
 static bool stack_plan(const Config& c, int rows, int nb, int ppr, int cross_rows, bool long_seq, int lean, size_t budget,
                        stack::Layout* out) {
   const int NT = rows > 8 ? 2 : 1, RP = NT * 8;
-  const stack::Geo g = stack::make_geo(c.d, c.H, c.d_ff, c.n_dec, cross_rows, lean >= 2);
+  const stack::Geo g = stack::make_geo(c.d, c.H, c.d_ff, c.n_dec, cross_rows, lean == 2 || lean == 3);
   auto up = [](size_t v, size_t a) { return (v + a - 1) / a * a; };
   size_t off = 0;
   stack::Layout L;
@@ -692,7 +714,7 @@ static bool stack_plan(const Config& c, int rows, int nb, int ppr, int cross_row
   const size_t chunk = std::max((size_t)NT * 3 * fused::kDH * 4, (size_t)g.UPR * RP * 4);
   const size_t states = (size_t)fused::kC * rows * stack::kState * 4;
   const size_t window = lean == 2 ? stack::kLongKeys : stack::kShortKeys;
-  if (lean >= 2) {
+  if (lean == 2 || lean == 3) {
     // scores share the outbox, the ranks' states the inbox: their uses never overlap (see share_states)
     L.outbox = L.sc = take(std::max(fused::kC * chunk, (size_t)16 * (window + 4) * 4));
     L.inbox = L.lvl2 = take(std::max(fused::kC * chunk, states));
@@ -749,15 +771,6 @@ static int stack_clusters(const void* kernel, size_t smem, int H, int* out) {
   return BPD_OK;
 }
 
-// Shapes the persistent kernel is built for.
-static bool stack_shapes_ok(const Config& c, int rows) {
-  const int d = c.d, H = c.H;
-  if (c.dtype != 1 || H < 1 || d != H * fused::kDH || (d != 256 && d != 512 && d != 1024)) return false;
-  if (c.d_ff % H || (c.d_ff / H != 128 && c.d_ff / H != 256)) return false;   // hidden units per cluster
-  if (rows < 1 || rows > fused::kMaxRows || c.n_dec > 64) return false;
-  return true;
-}
-
 // Live sessions per device whose decoder layers run in the persistent kernel.  Two such kernels on one GPU at the
 // same time can starve each other of SMs (each waits for clusters the other keeps from being scheduled) until their
 // bounded waits expire, so the library's own choice gives the persistent kernel to one session per device at a time;
@@ -773,20 +786,24 @@ static int stack_live(int dev, int delta) {
 
 // Decides whether the session runs its decoder layers in the persistent kernel and prepares what it needs:
 // a shared-memory plan under which all H clusters are resident at once, tensor maps and per-layer pointers.
-static int stack_setup(bpd_session* s) {
+static int stack_setup(bpd_session* s, bool try_groups) {
   const bpd_model* m = s->m;
   const Config& c = m->cfg;
   s->stack = 0;
-  const int rows = s->B * c.k_model;
-  if (!s->tc || !s->opt.persistent_layers || !stack_shapes_ok(c, rows)) return BPD_OK;
   const bool long_seq = s->max_tgt + 1 + c.k_model > 32 * fused::kC;
+  int seqs = s->B, per_group = 0;
+  int groups = try_groups ? stack_groups(c, s->B, &per_group) : 0;
+  if (groups && (long_seq || s->max_src > 256 || !s->opt.stage_encoder_rows)) groups = 0;
+  if (groups) seqs = per_group;
+  const int rows = seqs * c.k_model;
+  if (!s->tc || !s->opt.persistent_layers || !stack_shapes_ok(c, rows)) return BPD_OK;
   const bool only_lean = s->opt.persistent_layers < 0;   // the library's own choice: sessions a lean kernel takes
   const bool stageable = s->opt.stage_encoder_rows && s->B * s->max_src <= 256;
   // one sequence: the variants that split the keys over the ranks (they need an SM per CTA; measured against the short
   // one on one box: 138 -> 134 us for the base model's layers, and 272 -> 201 against the cluster launches for a long
   // sequence); otherwise the short one
   const int split = (s->B == 1 && s->max_src <= fused::kC * stack::kLongCross) ? (long_seq ? 2 : 3) : 0;
-  const int want = split ? split : (stageable && !long_seq ? 1 : 0);
+  const int want = groups ? 4 : (split ? split : (stageable && !long_seq ? 1 : 0));
   if (only_lean && want == 0) return BPD_OK;
   cudaDeviceProp prop;
   int dev = 0;
@@ -804,18 +821,20 @@ static int stack_setup(bpd_session* s) {
     for (int attempt = 0; attempt < 3 && !ok; ++attempt) {
       // the lean variant, else the general one with and without staged encoder rows
       lean = attempt == 0 ? want : 0;
-      if (lean >= 2 && minb == 2) lean = (stageable && !long_seq) ? 1 : 0;
+      if (groups && (attempt > 0 || minb == 1)) continue;      // groups need two CTAs per SM
+      if ((lean == 2 || lean == 3) && minb == 2) lean = (stageable && !long_seq) ? 1 : 0;
       if ((attempt == 0 && !lean) || (attempt > 0 && only_lean) || (attempt == 1 && !stageable)) continue;
-      staged = lean >= 2 ? s->opt.stage_encoder_rows : (attempt < 2 ? 1 : 0);
-      cross_rows = lean >= 2 ? (ceil_div(s->max_src, fused::kC) + 7) / 8 * 8 : (staged ? s->B * s->max_src : 0);
-      if (budget <= 1024 || !stack_plan(c, rows, s->B, s->ppr, staged ? cross_rows : 0, long_seq, lean, budget - 1024, &lay)) continue;
+      staged = lean == 2 || lean == 3 ? s->opt.stage_encoder_rows : (attempt < 2 ? 1 : 0);
+      cross_rows = lean == 2 || lean == 3 ? (ceil_div(s->max_src, fused::kC) + 7) / 8 * 8 : (staged ? (groups ? 1 : s->B) * s->max_src : 0);
+      if (budget <= 1024 || !stack_plan(c, rows, seqs, s->ppr, staged ? cross_rows : 0, long_seq, lean, budget - 1024, &lay)) continue;
       lay.total += 1024;                       // slack for aligning the ring to 1024 bytes
       int n1 = 0, n2 = 0;
       const size_t sm = (size_t)lay.total;
       const int ksteps = c.d == 256 ? 2 : 4, H = c.H;
       BPD_TRY(stack_clusters(stack::kernel_for(1, ksteps, minb, lean), sm, H, &n1));
       BPD_TRY(stack_clusters(stack::kernel_for(2, ksteps, minb, lean), sm, H, &n2));
-      ok = n1 >= c.H && n2 >= c.H;
+      const int need = std::max(1, groups) * c.H;
+      ok = n1 >= need && n2 >= need;
     }
     if (ok) break;
   }
@@ -823,7 +842,7 @@ static int stack_setup(bpd_session* s) {
   // tensor maps over all layers at once: weight slices as boxes of 64 (32 for d_model 256) reduction columns,
   // encoder keys / values.  The layers' tensors must lie at a constant stride (they do in a blob written tensor
   // by tensor, layer after layer; the session's encoder keys / values are laid out the same way).
-  const stack::Geo g = stack::make_geo(c.d, c.H, c.d_ff, c.n_dec, staged ? cross_rows : 0, lean >= 2);
+  const stack::Geo g = stack::make_geo(c.d, c.H, c.d_ff, c.n_dec, staged ? cross_rows : 0, lean == 2 || lean == 3);
   std::vector<stack::LayerPtrs> lp(c.n_dec);
   const int d = c.d, f = c.d_ff, nl = c.n_dec;
   auto stride_of = [&](auto get, long long* out) {
@@ -868,6 +887,7 @@ static int stack_setup(bpd_session* s) {
   static_assert(sizeof(stack::Layout) <= sizeof(s->stack_layout), "layout does not fit its opaque copy");
   memcpy(s->stack_layout, &lay, sizeof(lay));
   s->stack_cross_rows = cross_rows; s->stack_staged = staged; s->stack_long = long_seq ? 1 : 0; s->stack_minb = minb; s->stack_lean = lean;
+  s->stack_groups = std::max(1, groups); s->stack_group_seqs = seqs;
   s->stack = 1;
   s->stack_dev = dev;
   stack_live(dev, +1);
@@ -882,24 +902,24 @@ static int run_layers_stack(bpd_session* s, const PassArgs& a) {
   stack::StackParams p;
   memset(&p, 0, sizeof(p));
   p.layers = static_cast<const stack::LayerPtrs*>(s->stack_layers);
-  p.L = c.n_dec; p.d = c.d; p.H = c.H; p.ff = c.d_ff; p.R = s->B * a.kcur; p.rows_per_b = a.kcur; p.nb = s->B; p.eps = c.eps;
+  p.L = c.n_dec; p.d = c.d; p.H = c.H; p.ff = c.d_ff; p.R = s->B * a.kcur; p.rows_per_b = a.kcur; p.nb = s->B; p.group_seqs = s->stack_group_seqs; p.eps = c.eps;
   p.tgt_embed = static_cast<const bf16*>(m->tgt_embed); p.pe = s->pe; p.npos = s->npos; p.vocab = c.V;
   p.st = s->st; p.forced = a.forced; p.forced_rows = a.forced_rows; p.kforced = a.kforced;
   p.local_q = c.local_q; p.local_m = c.local_m; p.max_src = s->max_src; p.scale = 1.0f / sqrtf((float)fused::kDH);
-  p.cross_rows = s->stack_cross_rows; p.cross_staged = s->stack_staged; p.cross_split = s->stack_lean >= 2; p.long_seq = s->stack_long;
+  p.cross_rows = s->stack_cross_rows; p.cross_staged = s->stack_staged; p.cross_split = s->stack_lean == 2 || s->stack_lean == 3; p.long_seq = s->stack_long;
   p.lnf_g = static_cast<const bf16*>(m->dec_lnf_g); p.lnf_b = static_cast<const bf16*>(m->dec_lnf_b);
   p.xn_hi = static_cast<bf16*>(s->xn); p.xn_plane = s->pl_xn; p.h_f32 = s->h_f32;
   p.layer_dump = a.layer_dump;
-  p.ws = s->stack_ws; p.gather = s->stack_ws + (size_t)2 * c.H * fused::kMaxRows * c.d; p.bar = s->stack_bar; p.error = s->st.error; p.all_done = s->st.all_done;
+  p.ws = s->stack_ws; p.gather = s->stack_ws + (size_t)s->stack_groups * 2 * c.H * fused::kMaxRows * c.d; p.bar = s->stack_bar; p.error = s->st.error; p.all_done = s->st.all_done;
   p.spin = stack::kSpin;
   memcpy(&p.lay, s->stack_layout, sizeof(p.lay));
-  const dim3 grid(fused::kC, c.H), block(stack::kThreads);
+  const dim3 grid(fused::kC, c.H, s->stack_groups), block(stack::kThreads);
   const bool pdl = s->use_pdl != 0;
   stack::StackMaps maps;
   memcpy(&maps, s->stack_maps, sizeof(maps));
   const size_t smem = (size_t)p.lay.total;
   // reduction panels of 32 columns (two steps of 16) for d_model 256, else 64 (four steps); one or two CTAs per SM
-  const int nt = p.R > 8 ? 2 : 1, ksteps = c.d == 256 ? 2 : 4;
+  const int nt = s->stack_group_seqs * a.kcur > 8 ? 2 : 1, ksteps = c.d == 256 ? 2 : 4;
   const void* kernel = stack::kernel_for(nt, ksteps, s->stack_minb, s->stack_lean);
   if (!kernel) return fail(BPD_E_UNSUPPORTED, "no such instantiation of the persistent layer kernel");
   BPD_CUDA(launch_kc(kernel, grid, block, smem, s->stream, pdl, maps, p));
@@ -1426,7 +1446,8 @@ int bpd_session_create_opt(const bpd_model* model, int batch, int max_src, int m
     delete s;
     return fail(BPD_E_CUDA, "session set-up failed: %s", cudaGetErrorString(e));
   }
-  const int rc_stack = stack_setup(s);
+  int rc_stack = stack_setup(s, true);
+  if (!rc_stack && !s->stack) rc_stack = stack_setup(s, false);
   if (rc_stack) { bpd_session_destroy(s); return rc_stack; }
   *out = s;
   return BPD_OK;

@@ -199,10 +199,10 @@ struct bpd_session {
   int stack;
   unsigned char stack_maps[8 * 128] __attribute__((aligned(64)));   // stack::StackMaps (eight tensor maps over all layers)
   void* stack_layers;      // device: stack::LayerPtrs [n_dec]
-  unsigned long long* stack_ws;   // device: [2][H][16][d] words (value, tag): the clusters' shares of the projection outputs
+  unsigned long long* stack_ws;   // device: per group [2][H][16][d] words (value, tag): the clusters' shares of the projection outputs
   unsigned* stack_bar;     // device: words of the device-wide join
   float* stack_dump;       // device: [n_dec][rows][d] residual stream after every layer (debug dump), or null
-  int stack_cross_rows, stack_staged, stack_long, stack_minb, stack_lean, stack_dev;
+  int stack_cross_rows, stack_staged, stack_long, stack_minb, stack_lean, stack_dev, stack_groups, stack_group_seqs;
   int stack_layout[24];    // stack::Layout, kept opaque here
   std::map<GraphKey, GraphEntry> graphs;
   GraphEntry enc_graph;    // the encoder's launch sequence (fixed for a session), captured on its second use

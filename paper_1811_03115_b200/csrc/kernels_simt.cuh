@@ -1267,11 +1267,10 @@ static __global__ void reset_rows_kernel(ResetParams p) {
     p.st.signal[1] = 0;
     for (int i = 0; i < 4 + kMaxK + 1; ++i) p.st.stats[i] = 0;
   }
-  // the abort word is cleared; word 32 numbers the kernel's reductions over the whole life of the session (its
-  // workspace keeps the tags of earlier decodes) and stays
+  // the abort word is cleared; words 32 and up number the kernel's reductions over the whole life of the session (its
+  // workspace keeps the tags of earlier decodes) and stay
   if (p.join_words)
-    for (int i = threadIdx.x; i < 64; i += blockDim.x)
-      if (i != 32) p.join_words[i] = 0u;
+    for (int i = threadIdx.x; i < 32; i += blockDim.x) p.join_words[i] = 0u;
 }
 
 }  // namespace bpd

@@ -14,6 +14,7 @@ const void* kernel_for(int nt, int ksteps, int minb, int lean) {
   BPD_V(1, 2, 2, 1); BPD_V(2, 2, 2, 1); BPD_V(1, 4, 2, 1); BPD_V(2, 4, 2, 1);
   BPD_V(1, 2, 1, 2); BPD_V(2, 2, 1, 2); BPD_V(1, 4, 1, 2); BPD_V(2, 4, 1, 2);
   BPD_V(1, 2, 1, 3); BPD_V(2, 2, 1, 3); BPD_V(1, 4, 1, 3); BPD_V(2, 4, 1, 3);
+  BPD_V(1, 2, 2, 4); BPD_V(2, 2, 2, 4); BPD_V(1, 4, 2, 4); BPD_V(2, 4, 2, 4);
 #undef BPD_V
   return nullptr;
 }

@@ -68,6 +68,7 @@ constexpr unsigned long long kSpin = 2000000000ull;   // about a second
 constexpr int kBarAbort = 1;               // non-zero: some wait expired, nobody waits any more
 constexpr int kBarBase = 32;               // reductions done so far in this session: the next launch's tags go on from here (never reset)
 constexpr int kBarWords = 64;
+constexpr int kMaxGroups = 16;              // one word each from kBarBase on
 
 // Tensor maps over all decoder layers at once (the layers' tensors lie at a constant stride): dimensions
 // (columns, rows, layer).  Passed as a kernel parameter, so that issuing a load never waits for a descriptor.
@@ -92,6 +93,7 @@ struct Layout {
 struct StackParams {
   const LayerPtrs* layers;                 // [L], device memory
   int L, d, H, ff, R, rows_per_b, nb;
+  int group_seqs;                          // LEAN = 4: sequences of a group (a group = a z slice of the grid, H clusters)
   float eps;
   // embedding of the block (Section 6's decoder input)
   const bf16* tgt_embed; const float* pe; int npos, vocab;
@@ -211,7 +213,7 @@ __host__ __device__ inline Geo make_geo(int d, int H, int ff, int L, int cross_r
 }
 __host__ __device__ inline int round1k(int v) { return (v + 1023) & ~1023; }
 // Tile i of a layer (i in [0, ntl)) for rank c of cluster j.  Sizes are multiples of the ring's 1024-byte grain.
-__host__ __device__ inline TileDesc make_tile(const Geo& g, int i, int cross_rows, int d, int c, int j) {
+__host__ __device__ inline TileDesc make_tile(const Geo& g, int i, int cross_rows, int d, int c, int j, int cross_y = 0) {
   TileDesc t;
   t.map2 = -1; t.x2 = 0; t.off2 = 0; t.bytes2 = 0; t.dx = 0; t.dstep = 0; t.nbox = 1;
   if (i < g.P) {                                               // Q, K, V rows of the head, one panel: three boxes
@@ -231,7 +233,7 @@ __host__ __device__ inline TileDesc make_tile(const Geo& g, int i, int cross_row
   if (g.staged) {
     if (i == 0) {                                              // encoder keys (two halves of 32 floats), then values
       const int kb = round1k(cross_rows * 128);
-      t.map = kMapCk; t.nbox = 2; t.box_bytes = cross_rows * 128; t.x = j * kDH; t.y = g.split ? c * cross_rows : 0; t.dx = 32; t.dstep = kb;
+      t.map = kMapCk; t.nbox = 2; t.box_bytes = cross_rows * 128; t.x = j * kDH; t.y = g.split ? c * cross_rows : cross_y; t.dx = 32; t.dstep = kb;
       t.map2 = kMapCv; t.x2 = d + j * kDH; t.off2 = 2 * kb; t.bytes2 = cross_rows * 256;
       t.bytes = 2 * kb + round1k(cross_rows * 256);
       return t;
@@ -254,6 +256,7 @@ struct Cta {                               // what the device functions below sh
   Ctl* ctl;
   uint32_t ring;                           // shared-memory address of the ring
   int c, j, tid, warp, lane;
+  int R;                                   // rows of this launch, or of this group
   unsigned long long policy;
 };
 
@@ -364,7 +367,7 @@ __device__ __forceinline__ Words load_words(const Cta& k, const bf16* v) {
 #pragma unroll
   for (int u = 0; u < 2; ++u) {
     const int idx = k.tid + u * kThreads;
-    o.w[u] = (v != nullptr && idx < k.p->R * n4) ? *reinterpret_cast<const uint2*>(v + k.c * k.g.ks + (idx & (n4 - 1)) * 4) : make_uint2(0u, 0u);
+    o.w[u] = (v != nullptr && idx < k.R * n4) ? *reinterpret_cast<const uint2*>(v + k.c * k.g.ks + (idx & (n4 - 1)) * 4) : make_uint2(0u, 0u);
   }
   return o;
 }
@@ -374,7 +377,7 @@ __device__ __forceinline__ Words load_words(const Cta& k, const bf16* v) {
 __device__ __forceinline__ void reduce_slice(const Cta& k, float* x_s, const unsigned long long* ws, const Words& bias,
                                              unsigned tag, int nfree) {
   const StackParams& p = *k.p;
-  const int ks = k.g.ks, n4 = ks >> 2, R = p.R, d = p.d, H = p.H;
+  const int ks = k.g.ks, n4 = ks >> 2, R = k.R, d = p.d, H = p.H;
   __syncthreads();                                             // every warp is done with the tiles released here
   if (k.tid == kPumpThread && nfree) release_tiles(k, nfree);
 #pragma unroll
@@ -449,7 +452,7 @@ __device__ __forceinline__ bool ll_wait4(const Cta& k, const unsigned long long*
 __device__ __forceinline__ void reduce_slice_2hop(const Cta& k, float* x_s, const unsigned long long* ws, unsigned long long* gather,
                                                   const Words& bias, unsigned tag, int nfree) {
   const StackParams& p = *k.p;
-  const int ks = k.g.ks, n4 = ks >> 2, R = p.R, d = p.d, H = p.H, j = blockIdx.y;
+  const int ks = k.g.ks, n4 = ks >> 2, R = k.R, d = p.d, H = p.H, j = blockIdx.y;
   __syncthreads();                                             // every warp is done with the tiles released here
   if (k.tid == kPumpThread && nfree) release_tiles(k, nfree);
   const int ipp = (R * n4) / H;                                // items of a part: n4 = 2H, so 2R
@@ -557,7 +560,7 @@ __device__ __forceinline__ void planes_and_stats(const Cta& k, const float* x_s,
 // Row statistics from the eight slices, merged in rank order (threads t < R); needs a barrier afterwards.
 __device__ __forceinline__ void merge_stats(const Cta& k, const float* stats_in, float* s_mean, float* s_rstd) {
   const int t = k.tid;
-  if (t < k.p->R) {
+  if (t < k.R) {
     const float n1 = (float)k.g.ks;
     float mean = stats_in[t * 2], m2 = stats_in[t * 2 + 1], n = n1;
 #pragma unroll
@@ -694,8 +697,8 @@ __device__ __forceinline__ void send_rows(const Cta& k, int n, uint8_t* buf0, ui
   if (k.tid == kPumpThread && nfree) release_tiles(k, nfree);   // behind the barrier: every warp is done with those tiles
   int mine = 0;
 #pragma unroll
-  for (int slot = 0; slot < NT; ++slot) mine += (slot * kC + k.c < k.p->R) ? 1 : 0;
-  if (k.tid == 0) xchg_expect(k, n, (uint32_t)(k.p->R - mine) * row_bytes * (buf1 ? 2u : 1u));
+  for (int slot = 0; slot < NT; ++slot) mine += (slot * kC + k.c < k.R) ? 1 : 0;
+  if (k.tid == 0) xchg_expect(k, n, (uint32_t)(k.R - mine) * row_bytes * (buf1 ? 2u : 1u));
   if (!is_zombie(k)) {                     // after an expired wait nothing new goes into flight
     const int ppr = (int)(row_bytes >> 4), per_dst = mine * ppr * (buf1 ? 2 : 1);
     const uint32_t bar = tc::smem_u32(&k.ctl->ex[n & 1]);
@@ -769,7 +772,7 @@ __device__ __forceinline__ void long_prefetch(const Cta& k, const LongCtx& lc, c
 __device__ __forceinline__ void long_queries(const Cta& k, const LongCtx& lc, const uint8_t* kvq) {
   const int row = k.tid >> 4, col = (k.tid & 15) * 4;
   float4 q = make_float4(0.f, 0.f, 0.f, 0.f);
-  if (row < k.p->R) q = *reinterpret_cast<const float4*>(kvq + row * 512 + 256 + col * 4);
+  if (row < k.R) q = *reinterpret_cast<const float4*>(kvq + row * 512 + 256 + col * 4);
   uint32_t a[3], b[3];
   attn::split3_pair(q.x, q.y, a);
   attn::split3_pair(q.z, q.w, b);
@@ -818,7 +821,7 @@ __device__ __forceinline__ void long_rescale(const Cta& k, const LongCtx& lc, fl
 }
 // This rank's state into its block of the table: warp w holds dims 8w .. 8w + 7 of all rows.
 __device__ __forceinline__ void long_state(const Cta& k, const LongCtx& lc, const float (&acc)[4][4], float* lvl2) {
-  const int g = k.lane >> 2, R = k.p->R;
+  const int g = k.lane >> 2, R = k.R;
 #pragma unroll
   for (int half = 0; half < 2; ++half) {
     const int row = g + 8 * half;
@@ -901,7 +904,7 @@ template <int KW>
 __device__ __forceinline__ void long_cross_attention(const Cta& k, const LongCtx& lc, const LayerPtrs& LP, const uint8_t* kvq, const uint8_t* k0t,
                                                      const uint8_t* k1t, const uint8_t* vt, int limit, float* lvl2) {
   constexpr int sp = KW + 4, pp = kLongCross + 8;
-  const int lane = k.lane, warp = k.warp, g = lane >> 2, t4 = lane & 3, R = k.p->R;
+  const int lane = k.lane, warp = k.warp, g = lane >> 2, t4 = lane & 3, R = k.R;
   const int rows = k.p->cross_rows, first = k.c * rows, nk16 = (rows + 15) & ~15;   // at most kLongCross
   float acc[4][4] = {};
   long_queries(k, lc, kvq);
@@ -959,7 +962,7 @@ __device__ __forceinline__ void long_cross_attention(const Cta& k, const LongCtx
 
 // The ranks' states to every rank (exchange n), merged in rank order into the planes of the attention output.
 __device__ __forceinline__ void share_states(const Cta& k, int n, float* lvl2, uint8_t* oh, uint8_t* ol, int nfree = 0) {
-  const int R = k.p->R;
+  const int R = k.R;
   float* mine = lvl2 + (size_t)k.c * R * kState;
   const uint32_t bytes = (uint32_t)(R * kState * 4);
   fence_async_smem();
@@ -995,6 +998,9 @@ constexpr int kTracePts = 256;
 // path (the short self-attention schedule, the staged cross-attention); the general kernel (0) needs far more than the
 // 128 registers a thread has when two CTAs share an SM.  LEAN = 2, 3: sessions of one sequence of any length (2)
 // or of at most 256 positions (3); both attentions split the keys over the ranks and run on mma.sync.
+// LEAN = 4: the short variant for more sequences than one set of H clusters takes.  The grid's z slices are groups of H
+// clusters that work on a few sequences each (at most 8 rows, or one sequence) and know nothing of one another: shares,
+// tags and rows of their own.  A rank then attends for rows of one sequence only and stages just that one's encoder rows.
 template <int NT, int KS, int MINB, int LEAN>
 __global__ void __cluster_dims__(kC, 1, 1) __launch_bounds__(kThreads, MINB)
 layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant__ StackParams p) {
@@ -1018,7 +1024,12 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
   k.policy = tc::l2_evict_first();
   const Geo& g = k.g;
   const int c = k.c, j = k.j, tid = k.tid, warp = k.warp, lane = k.lane;
-  const int d = p.d, ks = g.ks, R = p.R, nb = p.nb, rpb = p.rows_per_b;
+  constexpr bool GROUPS = LEAN == 4;
+  const int grp = GROUPS ? (int)blockIdx.z : 0, b0 = GROUPS ? grp * p.group_seqs : 0;
+  const int d = p.d, ks = g.ks, rpb = p.rows_per_b, nb = GROUPS ? min(p.group_seqs, p.nb - b0) : p.nb, R = GROUPS ? nb * rpb : p.R;
+  k.R = R;
+  unsigned long long* const ws_g = p.ws + (GROUPS ? (size_t)grp * 2 * p.H * kMaxRows * d : 0);
+  unsigned long long* const gather_g = p.gather + (GROUPS ? (size_t)grp * 2 * kMaxRows * d : 0);
   const int lg = lane >> 2, t4 = lane & 3;
   float* x_s = reinterpret_cast<float*>(ssm + p.lay.x);
   uint8_t* xh = ssm + p.lay.xh;
@@ -1054,13 +1065,13 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
     k.ctl->cyc_wait = 0; k.ctl->cyc_pump = 0; k.ctl->cyc_poll = 0;
 #endif
   }
-  if (tid < g.ntl) k.ctl->tiles[tid] = make_tile(g, tid, p.cross_rows, d, c, j);
+  if (tid < g.ntl) k.ctl->tiles[tid] = make_tile(g, tid, p.cross_rows, d, c, j, GROUPS ? (b0 + min(c / rpb, nb - 1)) * p.max_src : 0);
   __syncthreads();
   // Weights and page tables do not depend on anything earlier in the stream.  The encoder's keys and values do:
   // the launches before this one (the encoder's, right after bpd_encode) may still be running, so the first
   // tile that carries them is not requested before the dependency wait.
   if (tid == kPumpThread) pump(k, g.staged ? g.P + 2 : 0x7fffffff);
-  for (int i = tid; i < nb * p.st.pages_per_row; i += kThreads) s_pt[i] = p.st.page_table[i];
+  for (int i = tid; i < nb * p.st.pages_per_row; i += kThreads) s_pt[i] = p.st.page_table[b0 * p.st.pages_per_row + i];
   for (int i = tid; i < p.L * (int)(sizeof(LayerPtrs) / 8); i += kThreads)
     reinterpret_cast<unsigned long long*>(layers_s)[i] = reinterpret_cast<const unsigned long long*>(p.layers)[i];
   // rows beyond R of the planes are never written: zero them once so that no NaN pattern reaches an MMA
@@ -1075,8 +1086,8 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
     return;
   }
   if (tid == kPumpThread) pump(k);
-  const unsigned base = __ldcg(p.bar + kBarBase);
-  if (tid < nb) { s_len[tid] = p.st.len[tid]; s_src[tid] = p.st.src_len[tid]; }
+  const unsigned base = __ldcg(p.bar + kBarBase + grp);
+  if (tid < nb) { s_len[tid] = p.st.len[b0 + tid]; s_src[tid] = p.st.src_len[b0 + tid]; }
   __syncthreads();
 
   // ---- embedding of the block: x[t] = E[token] sqrt(d) + PE(position), this rank's columns
@@ -1085,14 +1096,14 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
     const float scale = sqrtf((float)d);
     for (int idx = tid; idx < R * n4; idx += kThreads) {
       const int t = idx >> g.lg_n4, c4 = idx & (n4 - 1);
-      const int b = t / rpb, i = t % rpb;
+      const int bl = t / rpb, i = t % rpb, b = b0 + bl;
       int tok = p.st.block[b * kMaxK + i];
       if (p.forced && i >= 1 && i < p.kforced) {
         const int jb = p.st.j[b];
         if (p.forced_rows == 1) tok = p.forced[(size_t)b * (p.kforced - 1) + (i - 1)];
         else if (jb < p.forced_rows) tok = p.forced[((size_t)b * p.forced_rows + jb) * (p.kforced - 1) + (i - 1)];
       }
-      int pos = s_len[b] + i;
+      int pos = s_len[bl] + i;
       if (j == 0 && c == 0 && c4 == 0) p.st.cur_block[b * kMaxK + i] = tok;
       if (tok < 0 || tok >= p.vocab || pos >= p.npos) {     // never index outside the tables; report instead
         atomicCAS(p.error, 0, 1);
@@ -1122,7 +1133,7 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
       one_chunk_per_rank = one_chunk_per_rank && ((s_len[b] + rpb + 31) >> 5) - (attn_first_key(ap, s_len[b]) >> 5) <= kC;
   }
 
-  constexpr bool SPLIT = LEAN >= 2;         // keys split over the ranks
+  constexpr bool SPLIT = LEAN == 2 || LEAN == 3;         // keys split over the ranks
   constexpr int KW = LEAN == 2 ? kLongKeys : kShortKeys;
   const LongCtx lc = SPLIT ? long_ctx<KW>(k, ap, ssm, s_pt, s_len[0]) : LongCtx{};
   if (SPLIT) long_prefetch<KW>(k, lc, layers_s[0], 0);
@@ -1166,13 +1177,13 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
       const Words bw = load_words(k, layers_s[l - 1].b2);
       ++nbar;
       BPD_TR();
-      if (p.H == 16) reduce_slice_2hop(k, x_s, p.ws + (size_t)((nbar - 1) & 1) * p.H * kMaxRows * d, p.gather + (size_t)((nbar - 1) & 1) * kMaxRows * d, bw, base + nbar, g.PH);
-      else reduce_slice(k, x_s, p.ws + (size_t)((nbar - 1) & 1) * p.H * kMaxRows * d, bw, base + nbar, g.PH);
+      if (p.H == 16) reduce_slice_2hop(k, x_s, ws_g + (size_t)((nbar - 1) & 1) * p.H * kMaxRows * d, gather_g + (size_t)((nbar - 1) & 1) * kMaxRows * d, bw, base + nbar, g.PH);
+      else reduce_slice(k, x_s, ws_g + (size_t)((nbar - 1) & 1) * p.H * kMaxRows * d, bw, base + nbar, g.PH);
       BPD_TR();
       if (p.layer_dump && j == 0) {
         __syncthreads();
         for (int idx = tid; idx < R * ks; idx += kThreads)
-          p.layer_dump[((size_t)(l - 1) * R + idx / ks) * d + c * ks + idx % ks] = x_s[idx];
+          p.layer_dump[((size_t)(l - 1) * p.R + b0 * rpb + idx / ks) * d + c * ks + idx % ks] = x_s[idx];
       }
     }
     planes_and_stats<NT>(k, x_s, gw, xh, xl, stats_mine);
@@ -1239,7 +1250,7 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
         if (l + 1 < p.L) long_prefetch<KW>(k, lc, layers_s[l + 1], 0);
         share_states(k, xn, lvl2, oh, ol);
         ++xn;
-      } else if (LEAN == 1 || one_chunk_per_rank) {
+      } else if (LEAN == 1 || GROUPS || one_chunk_per_rank) {
         // this rank attends for its own rows; warp w folds the chunk that belongs to rank w
         for (int slot = 0; slot < NT; ++slot) {
           const int token = slot * kC + c;
@@ -1331,7 +1342,7 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
     BPD_TR();
     // this head's share of the output projection for feature slice c
     {
-      unsigned long long* wsj = p.ws + ((size_t)(nbar & 1) * p.H + j) * kMaxRows * d;
+      unsigned long long* wsj = ws_g + ((size_t)(nbar & 1) * p.H + j) * kMaxRows * d;
       const unsigned tag_out = base + nbar + 1;            // the reduction that consumes these shares
       for (int mt = warp; mt < ks / 16; mt += kWarps) {
         float acc[NT][4];
@@ -1358,8 +1369,8 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
     if (tid < kDH) { fs = LP.s_cq[j * kDH + tid]; fc = LP.c_cq[j * kDH + tid]; }
     ++nbar;
     BPD_TR();
-    if (p.H == 16) reduce_slice_2hop(k, x_s, p.ws + (size_t)((nbar - 1) & 1) * p.H * kMaxRows * d, p.gather + (size_t)((nbar - 1) & 1) * kMaxRows * d, nobias, base + nbar, 1);
-      else reduce_slice(k, x_s, p.ws + (size_t)((nbar - 1) & 1) * p.H * kMaxRows * d, nobias, base + nbar, 1);
+    if (p.H == 16) reduce_slice_2hop(k, x_s, ws_g + (size_t)((nbar - 1) & 1) * p.H * kMaxRows * d, gather_g + (size_t)((nbar - 1) & 1) * kMaxRows * d, nobias, base + nbar, 1);
+      else reduce_slice(k, x_s, ws_g + (size_t)((nbar - 1) & 1) * p.H * kMaxRows * d, nobias, base + nbar, 1);
     BPD_TR();
     planes_and_stats<NT>(k, x_s, gw, xh, xl, stats_mine);
     __syncthreads();
@@ -1423,7 +1434,7 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
           __syncthreads();
           const int b = token / rpb;
           float ov;
-          if (LEAN == 1 || g.staged) ov = cross_attention_tile(ckv_g, ckv_g + kb, ckv_g + 2 * kb, b * p.max_src, s_src[b], sm);
+          if (LEAN == 1 || GROUPS || g.staged) ov = cross_attention_tile(ckv_g, ckv_g + kb, ckv_g + 2 * kb, GROUPS ? 0 : b * p.max_src, s_src[b], sm);
           else ov = attention_head<float, kDH, kWarps, false>(ap, b, j, 0, s_src[b], sm);
           if (tid < kDH) store_attn_out(oh, ol, token, tid, ov);
           __syncthreads();
@@ -1441,7 +1452,7 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
     ++xn;
     BPD_TR();
     {
-      unsigned long long* wsj = p.ws + ((size_t)(nbar & 1) * p.H + j) * kMaxRows * d;
+      unsigned long long* wsj = ws_g + ((size_t)(nbar & 1) * p.H + j) * kMaxRows * d;
       const unsigned tag_out = base + nbar + 1;            // the reduction that consumes these shares
       for (int mt = warp; mt < ks / 16; mt += kWarps) {
         float acc[NT][4];
@@ -1474,8 +1485,8 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
     }
     ++nbar;
     BPD_TR();
-    if (p.H == 16) reduce_slice_2hop(k, x_s, p.ws + (size_t)((nbar - 1) & 1) * p.H * kMaxRows * d, p.gather + (size_t)((nbar - 1) & 1) * kMaxRows * d, nobias, base + nbar, 1);
-      else reduce_slice(k, x_s, p.ws + (size_t)((nbar - 1) & 1) * p.H * kMaxRows * d, nobias, base + nbar, 1);
+    if (p.H == 16) reduce_slice_2hop(k, x_s, ws_g + (size_t)((nbar - 1) & 1) * p.H * kMaxRows * d, gather_g + (size_t)((nbar - 1) & 1) * kMaxRows * d, nobias, base + nbar, 1);
+      else reduce_slice(k, x_s, ws_g + (size_t)((nbar - 1) & 1) * p.H * kMaxRows * d, nobias, base + nbar, 1);
     BPD_TR();
     planes_and_stats<NT>(k, x_s, gw, xh, xl, stats_mine);
     __syncthreads();
@@ -1533,7 +1544,7 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
     BPD_TR();
     // the hidden units times slice c of the second projection: this cluster's share of the block's output
     {
-      unsigned long long* wsj = p.ws + ((size_t)(nbar & 1) * p.H + j) * kMaxRows * d;
+      unsigned long long* wsj = ws_g + ((size_t)(nbar & 1) * p.H + j) * kMaxRows * d;
       const unsigned tag_out = base + nbar + 1;            // the reduction that consumes these shares
       for (int mt = warp; mt < ks / 16; mt += kWarps) {
         float acc[NT][4];
@@ -1571,13 +1582,13 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
     ++nbar;
     BPD_TR();
     pdl_launch_dependents();
-    if (p.H == 16) reduce_slice_2hop(k, x_s, p.ws + (size_t)((nbar - 1) & 1) * p.H * kMaxRows * d, p.gather + (size_t)((nbar - 1) & 1) * kMaxRows * d, bw, base + nbar, g.PH);
-      else reduce_slice(k, x_s, p.ws + (size_t)((nbar - 1) & 1) * p.H * kMaxRows * d, bw, base + nbar, g.PH);
+    if (p.H == 16) reduce_slice_2hop(k, x_s, ws_g + (size_t)((nbar - 1) & 1) * p.H * kMaxRows * d, gather_g + (size_t)((nbar - 1) & 1) * kMaxRows * d, bw, base + nbar, g.PH);
+      else reduce_slice(k, x_s, ws_g + (size_t)((nbar - 1) & 1) * p.H * kMaxRows * d, bw, base + nbar, g.PH);
     BPD_TR();
     if (p.layer_dump && j == 0) {
       __syncthreads();
       for (int idx = tid; idx < R * ks; idx += kThreads)
-        p.layer_dump[((size_t)(p.L - 1) * R + idx / ks) * d + c * ks + idx % ks] = x_s[idx];
+        p.layer_dump[((size_t)(p.L - 1) * p.R + b0 * rpb + idx / ks) * d + c * ks + idx % ks] = x_s[idx];
     }
     planes_and_stats<NT>(k, x_s, gw, xh, xl, stats_mine);   // the planes are not used; the statistics are
     BPD_TR();
@@ -1606,12 +1617,12 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
       uint32_t hi[4], lo[4];
 #pragma unroll
       for (int e = 0; e < 4; ++e) fused::split_bits(o[e], hi[e], lo[e]);
-      bf16* yp = p.xn_hi + (size_t)t * d + col;
+      bf16* yp = p.xn_hi + (size_t)(b0 * rpb + t) * d + col;
       *reinterpret_cast<uint2*>(yp) = make_uint2(hi[0] | (hi[1] << 16), hi[2] | (hi[3] << 16));
       *reinterpret_cast<uint2*>(yp + p.xn_plane) = make_uint2(lo[0] | (lo[1] << 16), lo[2] | (lo[3] << 16));
-      *reinterpret_cast<float4*>(p.h_f32 + (size_t)t * d + col) = make_float4(o[0], o[1], o[2], o[3]);
+      *reinterpret_cast<float4*>(p.h_f32 + (size_t)(b0 * rpb + t) * d + col) = make_float4(o[0], o[1], o[2], o[3]);
     }
-    if (c == 0 && tid == 0) p.bar[kBarBase] = base + nbar;         // tags of the next launch go on from here
+    if (c == 0 && tid == 0) p.bar[kBarBase + grp] = base + nbar;         // tags of the next launch go on from here
   }
 #ifdef BPD_STACK_TRACE
   if (g_stack_trace && tid == 0) {
