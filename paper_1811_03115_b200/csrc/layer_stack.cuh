@@ -524,7 +524,7 @@ template <int NT>
 __device__ __forceinline__ void planes_and_stats(const Cta& k, const float* x_s, const Words& gain, uint8_t* xh, uint8_t* xl,
                                                  float* stats_mine) {
   const StackParams& p = *k.p;
-  const int ks = k.g.ks, n4 = ks >> 2, R = p.R, PW = k.g.PW;
+  const int ks = k.g.ks, n4 = ks >> 2, R = k.R, PW = k.g.PW;
   constexpr int RP = NT * 8;
 #pragma unroll
   for (int it = 0; it < 2; ++it) {
