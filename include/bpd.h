@@ -111,7 +111,9 @@ typedef struct {
                                  Default: on for sessions of at most 256 positions whose encoder rows fit
                                  the staging tile, and for one sequence of any length where a CTA has an
                                  SM to itself (measured faster there), while no other live session of
-                                 the device has it, off elsewhere; 1 asks for it wherever it runs.  See
+                                 the device has it, off elsewhere; 1 asks for it wherever it runs.
+                                 Several sequences (also more than 16 rows) run as groups side by side
+                                 where the device holds n_heads * 8 CTAs for each group.  See
                                  bpd_session_create_opt for what it needs                                  */
   int32_t stage_encoder_rows; /* encoder keys / values staged in shared memory for cross-attention          */
   int32_t l2_stream_hints;    /* weights read once per pass are loaded "evict first"                        */

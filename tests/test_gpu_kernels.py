@@ -111,3 +111,36 @@ def test_encoder_feeds_the_decoder_like_the_oracle(bpd, batch, max_src, d, n_dec
         np.testing.assert_allclose(r["hidden"][b].cpu().numpy(), scorer.last_hidden, atol=8e-3)     # the cache is bf16
     s.close()
     model.close()
+
+
+# the persistent layer kernel with groups of sequences: a last group that is full and one that is not, two sequences per
+# group and one, one token tile and two, lengths up to the limit of 256 positions, one encoder row and 256
+@pytest.mark.parametrize("batch,k,heads,max_src,tgt", [(3, 4, 4, 61, 30), (8, 4, 4, 9, 251), (5, 3, 8, 1, 20), (2, 10, 8, 33, 40), (4, 16, 8, 24, 48),
+                                                       (9, 4, 4, 7, 12)])
+def test_groups_of_sequences_decode_like_the_oracle(bpd, batch, k, heads, max_src, tgt):
+    from bpd_inputs import ModelConfig, make_weights
+    from oracle.decode import TransformerScorer
+    from oracle.model import parse_blob
+    blob = make_weights(ModelConfig(1, 2, 64 * heads, heads, 128 * heads, 300, k, 64), 5, 0.06)
+    rng = np.random.default_rng(batch * k)
+    lens = rng.integers(1, max_src + 1, batch).astype(np.int32)
+    lens[-1] = max_src
+    src = rng.integers(2, 300, (batch, max_src)).astype(np.int32)
+    model = bpd.Model(blob)
+    s = bpd.Session(model, batch, max_src, tgt)
+    assert s.layer_path == 2
+    s.bpd_encode(src, lens)
+    model_o, rows = parse_blob(blob), sorted({0, 1, batch - 1})
+    scorers = {b: TransformerScorer(model_o, src[b], int(lens[b]), cached=True, capacity=tgt + k + 2) for b in rows}
+    inputs = {b: [0] for b in rows}
+    for b in rows:
+        scorers[b](inputs[b], 1)
+    while len(inputs[0]) <= tgt:
+        r = s.bpd_iteration(k, tgt, want_hidden=True, accept_mode=k << 16)      # minimum block k: every proposal is kept
+        for b in rows:
+            block = [int(t) for t in r["block"][b]]
+            scorers[b](inputs[b] + block, k)
+            np.testing.assert_allclose(r["hidden"][b].cpu().numpy(), scorers[b].last_hidden, atol=8e-3)     # the cache is bf16
+            inputs[b] += block[:int(r["khat"][b])]
+    s.close()
+    model.close()
