@@ -319,13 +319,17 @@ _top1_scratch = {}      # (device, stream) -> scratch tensor, address, bytes: ke
 
 
 def _scratch_for(device, stream: int, nbytes: int):
-    """A scratch of at least ``nbytes`` for calls on this device and stream.  Calls on one stream run one after the
-    other and each leaves the scratch cleared, so they may share it -- also when several threads enqueue on the same
-    stream.  At most 64 are kept."""
+    """A scratch of at least ``nbytes`` for calls on this device and stream (the current one).  Calls on one stream run
+    one after the other and each leaves the scratch cleared, so they may share it -- also when several threads enqueue
+    on the same stream.  At most 64 are kept.  A call that is being captured gets a scratch of its own out of the
+    graph's memory: a replay comes on any stream and long after the kept one has been replaced."""
+    import torch
+    if torch.cuda.is_current_stream_capturing():
+        t = torch.empty(nbytes, dtype=torch.uint8, device=device)
+        return t, t.data_ptr(), nbytes
     key = (device, stream)
     have = _top1_scratch.get(key)
     if have is None or have[2] < nbytes:
-        import torch
         if len(_top1_scratch) >= 64:
             _top1_scratch.clear()
         t = torch.empty(nbytes, dtype=torch.uint8, device=device)

@@ -51,6 +51,36 @@ def test_fp32_projection_at_tile_edges(bpd, rows, in_f, out_f):
         np.testing.assert_allclose(v.cpu().numpy(), want.max(-1), atol=1e-5)
 
 
+# the fp32 top-1 only enqueues, so a program may capture it: replays after the kept scratch of the stream was replaced
+# by a larger call's, with eager calls in between, on the stream of the capture and on another
+def test_captured_fp32_top1_replays_after_its_stream_saw_larger_calls(bpd):
+    import torch
+    g = torch.Generator().manual_seed(3)
+    w = (torch.randn(1000, 64, generator=g) * 0.05).cuda()
+    x = torch.empty(37, 64, device="cuda")
+    big = torch.randn(300, 64, generator=g).cuda()
+    s = torch.cuda.Stream()
+    with torch.cuda.stream(s):
+        bpd.bpd_op_vocab_argmax(big[:37], w)                   # loads the kernel, leaves a small scratch kept for this stream
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=s):
+            idx, val = bpd.bpd_op_vocab_argmax(x, w, want_val=True)
+        bpd.bpd_op_vocab_argmax(big, w)
+        torch.cuda.synchronize()
+        canary = [torch.full((64, n), 7, dtype=torch.uint8, device="cuda") for n in (256, 1024, 4096)]
+        torch.cuda.synchronize()
+        for on in (s, torch.cuda.Stream()):
+            x.copy_(torch.randn(37, 64, generator=g))
+            torch.cuda.synchronize()
+            with torch.cuda.stream(on):
+                graph.replay()
+            torch.cuda.synchronize()
+            want = x.double().cpu().numpy() @ w.double().cpu().numpy().T
+            np.testing.assert_allclose(want[np.arange(37), idx.cpu().numpy()], want.max(-1), atol=1e-5)
+            np.testing.assert_allclose(val.cpu().numpy(), want.max(-1), atol=1e-5)
+    assert all(bool((c == 7).all()) for c in canary)
+
+
 # attention of many-row sessions against the oracle's decoder: one chunk and several (96 encoder rows per chunk), query tiles
 # of up to 16 rows, sources from one id on, sequences long enough for a second chunk of 256 cached keys, local attention
 @pytest.mark.parametrize("batch,k,max_src,tgt,local", [(3, 8, 33, 20, 0), (9, 2, 100, 12, 0), (10, 16, 17, 40, 0), (19, 3, 5, 300, 0), (19, 3, 97, 290, 64)])
