@@ -280,9 +280,11 @@ static size_t plan_session(const Config& c, int B, int max_src, int max_tgt, cha
   return align_up(a.off);
 }
 
+// Shares of the folded vectors' sums, one per 128 columns, where the encoder's planes are centred.
+static int fold_parts(const Config& c) { return c.d % 256 == 0 ? c.d / 128 : 0; }
 static size_t fold_floats(const Config& c) {
   if (c.dtype != 1) return 0;
-  return (size_t)c.n_dec * 2 * (3 * c.d + c.d + c.d_ff + 2 * c.d) + (size_t)c.n_enc * 2 * (3 * c.d + c.d_ff);
+  return (size_t)c.n_dec * 2 * (3 * c.d + c.d + c.d_ff) + (size_t)(2 + fold_parts(c)) * (c.n_dec * 2 * c.d + c.n_enc * (3 * c.d + c.d_ff));
 }
 static size_t weight_bytes_for(const ParsedBlob& pb) { return align_up(pb.total) + align_up(fold_floats(pb.cfg) * sizeof(float)); }
 
@@ -548,22 +550,24 @@ static int run_encoder_tc(bpd_session* s) {
   ep.table = m->src_embed; ep.pe = s->pe; ep.npos = s->npos; ep.x = s->x; ep.rows = E; ep.rows_per_b = s->max_src;
   ep.d = d; ep.vocab = c.V; ep.st = s->st; ep.src = s->src_dev;
   // Layer norms folded into the projections behind them, statistics as per-tile partial results (see TcParams::stat_out).
-  // The encoder is a chain of launches that wait on one another, about 5 us each at these sizes whatever they move, so what
-  // counts is their number: 50 -> 32 for six layers, with all keys and values for the decoder in one launch.  One 25-word
-  // sentence (base model) 231 -> 198 us, five ragged ones 316 -> 261, 32 sentences (big) 1180 -> 1152.
+  // With few rows the encoder is a chain of launches that wait on one another, about 5 us each whatever they move, so what
+  // counts is their number: 50 -> 32 for six layers, with all keys and values for the decoder in one launch (where the line
+  // lies: bpd_session_create_opt).  The planes are centred tile by tile (TcParams::ln_parts): without that rows of mean m
+  // and deviation s lost m / s times the precision of the layer-norm kernel (keys and values off by 1.9e-4 of their norm at
+  // m / s = 64; centred 6.5e-6, layer-norm kernels 6.5e-6; 2.5e-6 each at a mean near zero).
   const bool fold = s->fold_enc != 0;
   auto planes_of = [&](tc::TcParams& q, const void* gain) {
     if (!fold) return;
     q.g_next = static_cast<const bf16*>(gain); q.xg_hi = static_cast<bf16*>(s->xn); q.xg_plane = s->pl_xn;
-    q.stat_out = s->ln_stats; q.stat_T = E;
+    q.stat_out = s->ln_stats; q.stat_T = E; q.centred = 1;
   };
-  auto norm_of = [&](tc::TcParams& q, const float* fs, const float* fc) {
+  auto norm_of = [&](tc::TcParams& q, const float* shares, const float* fc) {
     if (!fold) return;
-    q.stat_in = s->ln_stats; q.stat_parts = d / 128; q.stat_T = E; q.ln_s = fs; q.ln_c = fc; q.ln_eps = c.eps;
+    q.stat_in = s->ln_stats; q.stat_parts = d / 128; q.stat_T = E; q.ln_parts = shares; q.ln_c = fc; q.ln_eps = c.eps;
   };
   if (fold) {
     ep.gain = static_cast<const bf16*>(m->enc[0].ln1g); ep.xg_hi = static_cast<bf16*>(s->xn); ep.xg_plane = s->pl_xn;
-    ep.stat_out = s->ln_stats; ep.stat_T = E;
+    ep.stat_out = s->ln_stats; ep.stat_T = E; ep.centred = 1;
   }
   embed_kernel<bf16><<<E, 128, 0, st>>>(ep);
   ++g_launches;
@@ -576,7 +580,7 @@ static int run_encoder_tc(bpd_session* s) {
     if (!fold) launch_ln<bf16, float>(s->x, L.ln1g, L.ln1b, s->xn, nullptr, E, d, c.eps, nullptr, st, s->pl_xn, pdl);
     tc::TcParams pq = tc_params(nullptr, 0, nullptr);
     pq.out_f32 = static_cast<float*>(s->qbuf); pq.ldo = 3 * d;
-    norm_of(pq, L.s_qkv, L.c_qkv);
+    norm_of(pq, L.p_qkv, L.c_qkv);
     BPD_TRY(tc::launch<tc::kTcF32>(with_w(xn, L.wqkv, 3 * d), 3 * d, d, E, pq, sc, st, 1, 0, 0, pdl)); ++g_launches;
     AttnParams ap;
     memset(&ap, 0, sizeof(ap));
@@ -593,7 +597,7 @@ static int run_encoder_tc(bpd_session* s) {
     if (!fold) launch_ln<bf16, float>(s->x, L.ln2g, L.ln2b, s->xn, nullptr, E, d, c.eps, nullptr, st, s->pl_xn, pdl);
     tc::TcParams p1 = tc_params(L.b1, 1, nullptr);
     p1.out_hi = static_cast<bf16*>(s->ffh); p1.plane = s->pl_ffh; p1.ldo = f;
-    norm_of(p1, L.s_f1, L.c_f1);
+    norm_of(p1, L.p_f1, L.c_f1);
     BPD_TRY(tc::launch<tc::kTcPlanes>(with_w(xn, L.w1, f), f, d, E, p1, sc, st, 1, 0, 0, pdl)); ++g_launches;
     tc::TcParams p2 = tc_params(L.b2, 0, nullptr);
     p2.out_f32 = s->x; p2.ldo = d;
@@ -610,8 +614,11 @@ static int run_encoder_tc(bpd_session* s) {
   for (int l = 0; l < c.n_dec; l += slices) {
     tc::TcParams pk = tc_params(nullptr, 0, nullptr);
     pk.out_f32 = static_cast<float*>(s->crosskv[l]); pk.ldo = 2 * d;
-    norm_of(pk, m->dec[l].s_ckv, m->dec[l].c_ckv);
-    if (slices > 1) { pk.zofs_out = static_cast<float*>(s->crosskv[1]) - static_cast<float*>(s->crosskv[0]); pk.zofs_ln = 4 * d; }
+    norm_of(pk, m->dec[l].p_ckv, m->dec[l].c_ckv);
+    if (slices > 1) {
+      pk.zofs_out = static_cast<float*>(s->crosskv[1]) - static_cast<float*>(s->crosskv[0]);
+      pk.zofs_ln = (2 + fold_parts(c)) * 2 * d;
+    }
     const int rows_apart = (int)(step / row);
     BPD_TRY(tc::launch<tc::kTcF32>(with_w(xn, m->dec[l].cwkv, (slices - 1) * rows_apart + 2 * d), 2 * d, d, E, pk, sc, st, slices, slices > 1 ? rows_apart : 0, 0, pdl));
     ++g_launches;
@@ -1325,11 +1332,12 @@ int bpd_load_weights(const void* blob, size_t blob_bytes, void* dev_weight_buf, 
   cudaError_t e = cudaMemcpyAsync(m->base, blob, pb.total, cudaMemcpyHostToDevice, m->stream);
   if (c.dtype == 1 && e == cudaSuccess) {
     float* fp = reinterpret_cast<float*>(m->base + align_up(pb.total));
-    auto fold = [&](const void* w, const void* g, const void* b, const void* bias, int N, float** s_out, float** c_out) {
+    auto fold = [&](const void* w, const void* g, const void* b, const void* bias, int N, float** s_out, float** c_out, float** shares = nullptr) {
       *s_out = fp; fp += N;
       *c_out = fp; fp += N;
+      if (shares) { *shares = fold_parts(c) ? fp : nullptr; fp += (size_t)fold_parts(c) * N; }
       FoldParams p{static_cast<const bf16*>(w), static_cast<const bf16*>(g), static_cast<const bf16*>(b),
-                   static_cast<const bf16*>(bias), *s_out, *c_out, N, d};
+                   static_cast<const bf16*>(bias), *s_out, *c_out, shares ? *shares : nullptr, N, d};
       fold_ln_kernel<<<ceil_div(N, 4), 128, 0, m->stream>>>(p);
     };
     for (int l = 0; l < c.n_dec; ++l) {
@@ -1340,11 +1348,11 @@ int bpd_load_weights(const void* blob, size_t blob_bytes, void* dev_weight_buf, 
     }
     for (int l = 0; l < c.n_enc; ++l) {
       EncLayer& L = m->enc[l];
-      fold(L.wqkv, L.ln1g, L.ln1b, nullptr, 3 * d, &L.s_qkv, &L.c_qkv);
-      fold(L.w1, L.ln2g, L.ln2b, L.b1, f, &L.s_f1, &L.c_f1);
+      fold(L.wqkv, L.ln1g, L.ln1b, nullptr, 3 * d, &L.s_qkv, &L.c_qkv, &L.p_qkv);
+      fold(L.w1, L.ln2g, L.ln2b, L.b1, f, &L.s_f1, &L.c_f1, &L.p_f1);
     }
     // in layer order, so that one launch over all layers steps through them (TcParams::zofs_ln)
-    for (int l = 0; l < c.n_dec; ++l) fold(m->dec[l].cwkv, m->enc_lnf_g, m->enc_lnf_b, nullptr, 2 * d, &m->dec[l].s_ckv, &m->dec[l].c_ckv);
+    for (int l = 0; l < c.n_dec; ++l) fold(m->dec[l].cwkv, m->enc_lnf_g, m->enc_lnf_b, nullptr, 2 * d, &m->dec[l].s_ckv, &m->dec[l].c_ckv, &m->dec[l].p_ckv);
     e = cudaGetLastError();
   }
   if (e == cudaSuccess) e = cudaStreamSynchronize(m->stream);
@@ -1406,7 +1414,12 @@ int bpd_session_create_opt(const bpd_model* model, int batch, int max_src, int m
   // passes of at most 16 rows take the statistics from the stream itself; wider ones need whole 128-feature tiles (and
   // the embedding kernel whole warps: d_model a multiple of 256)
   s->fold_ln = (s->tc && o.fold_layer_norms != 0 && (batch * model->cfg.k_model <= 16 || model->cfg.d % 256 == 0)) ? 1 : 0;
-  s->fold_enc = (s->tc && o.fold_layer_norms != 0 && model->cfg.d % 256 == 0) ? 1 : 0;
+  // In the encoder a folded layer norm saves a dependent launch and costs its consumer eight products per output (see
+  // TcParams::ln_parts); a call, folded against layer-norm kernels: 40 rows 214 / 227 us (base) and 246 / 267 (big), 305
+  // rows 270 / 285 and 358 / 374, 768 rows 327 / 333 and 549 / 547, 1280 rows 411 / 407 and 790 / 755, 2560 rows
+  // 650 / 627 and 1275 / 1240.
+  s->fold_enc = (s->tc && o.fold_layer_norms != 0 && model->cfg.d % 256 == 0 &&
+                 (o.fold_layer_norms > 0 || (long long)batch * max_src <= 768)) ? 1 : 0;
   s->fused = (s->tc && fused::supported(model->cfg.d, model->cfg.H, model->cfg.d_ff, batch * model->cfg.k_model) &&
               o.cluster_layers != 0) ? 1 : 0;
   s->opt.persistent_layers = o.persistent_layers;   // -1: where its lean variant applies (measured faster there), 0: never, 1: wherever it runs

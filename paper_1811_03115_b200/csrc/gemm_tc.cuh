@@ -87,6 +87,10 @@ struct TcParams {
   // epilogue finishes y = rstd * (acc - mean * ln_s[n]) + ln_c[n] with per-token statistics of ln_x
   const float* ln_x; int ln_d; float ln_eps;   // residual stream [rows, ln_d] fp32, or null
   const float* ln_s; const float* ln_c;        // [N]: sum_c gain_c w[n][c]  and  sum_c shift_c w[n][c] + bias[n]
+  // wide kernel, `centred`: the planes hold (x - m) * gain, m the mean of the token's 128 features of the tile (stat_in),
+  // and y = rstd * (acc + sum_i (m_i - mean) ln_parts[i][n]) + ln_c[n]: a row's mean, however large against its
+  // deviations, costs the planes no bits
+  const float* ln_parts; int centred;          // [stat_parts][N] shares of ln_s (consumer); 1: write such planes (producer)
   // kTcResidual: also write planes of the updated stream times the next layer norm's gain
   const bf16* g_next; bf16* xg_hi; long long xg_plane;
   // Wide token tiles (more than 16 tokens) cannot afford to read whole rows of the residual stream for the folded

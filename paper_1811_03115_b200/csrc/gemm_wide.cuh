@@ -27,8 +27,10 @@ constexpr int kWidePitch = kBM + 4; // floats between the rows (tokens) of a til
 constexpr int kWideStages = 8;
 
 __host__ __device__ inline size_t wide_stage_bytes(int bn, int planes) { return (size_t)kBM * 128 + (size_t)planes * bn * 128; }
-__host__ __device__ inline size_t wide_smem_bytes(int bn, int planes, int stages) {
-  const size_t ring = stages * wide_stage_bytes(bn, planes), tile = (size_t)bn * kWidePitch * sizeof(float);
+// (centred: 32 bytes per token behind the tile, see centre_shares; they change neither the stages nor the CTAs per SM:
+// a tile with them is 80 KB at the 144 tokens that two CTAs take, 140 KB at 256)
+__host__ __device__ inline size_t wide_smem_bytes(int bn, int planes, int stages, bool centred = false) {
+  const size_t ring = stages * wide_stage_bytes(bn, planes), tile = (size_t)bn * (kWidePitch * sizeof(float) + (centred ? 32 : 0));
   return (ring > tile ? ring : tile) + 1024 /*alignment*/ + 256 /*barriers, control words*/;
 }
 
@@ -67,7 +69,7 @@ __device__ __forceinline__ void report(const TcParams& p, int code) {
 // A warp finishes the 128 features of a token, four consecutive ones per lane.  Per-thread constants of the four:
 struct FinishCtx {
   float bias[4], gn[4], lns[4];
-  bool folded;     // y = rstd * (acc - mean * ln_s) + ln_c; ln_c holds the bias
+  bool folded;     // y = rstd * (acc - mean * ln_s) + ln_c; ln_c holds the bias (ln_s: 0 with centred planes, see centre_terms)
   int n, g;
 };
 template <int EPI>
@@ -79,8 +81,11 @@ __device__ __forceinline__ void finish_setup(const TcParams& p, int z, int tile,
   c.folded = (p.stat_in != nullptr);
   if (c.n >= p.N) return;
   if (c.folded) {
-    const float4 s4 = *reinterpret_cast<const float4*>(p.ln_s + c.n + p.zofs_ln * z), c4 = *reinterpret_cast<const float4*>(p.ln_c + c.n + p.zofs_ln * z);
-    c.lns[0] = s4.x; c.lns[1] = s4.y; c.lns[2] = s4.z; c.lns[3] = s4.w;
+    const float4 c4 = *reinterpret_cast<const float4*>(p.ln_c + c.n + p.zofs_ln * z);
+    if (!p.ln_parts) {
+      const float4 s4 = *reinterpret_cast<const float4*>(p.ln_s + c.n + p.zofs_ln * z);
+      c.lns[0] = s4.x; c.lns[1] = s4.y; c.lns[2] = s4.z; c.lns[3] = s4.w;
+    }
     c.bias[0] = c4.x; c.bias[1] = c4.y; c.bias[2] = c4.z; c.bias[3] = c4.w;
   } else if (p.bias && p.vec) {
     const uint2 bw = *reinterpret_cast<const uint2*>(p.bias + c.n + p.zofs_n * z);
@@ -96,9 +101,19 @@ __device__ __forceinline__ void finish_setup(const TcParams& p, int z, int tile,
     c.gn[2] = __uint_as_float(gw.y << 16); c.gn[3] = __uint_as_float(gw.y & 0xffff0000u);
   }
 }
+// Planes of the updated stream, less `centre`, times the next layer norm's gain.
+__device__ __forceinline__ void store_planes_next(const TcParams& p, const FinishCtx& c, int t, const float4& x, float centre) {
+  const float v[4] = {x.x - centre, x.y - centre, x.z - centre, x.w - centre};
+  bf16 hi[4], lo[4];
+#pragma unroll
+  for (int e = 0; e < 4; ++e) split_bf16(v[e] * c.gn[e], hi[e], lo[e]);
+  bf16* at = p.xg_hi + (long long)t * p.ldo + c.n;
+  *reinterpret_cast<uint2*>(at) = pack4_bf16(hi);
+  *reinterpret_cast<uint2*>(at + p.xg_plane) = pack4_bf16(lo);
+}
 // One item: token t (row tr of the tile), features c.n .. c.n + 3, accumulated values a; `old` is the residual stream's
 // content, fetched by the caller (kTcResidual only), and returns the new content.
-template <int EPI>
+template <int EPI, bool CENTRED>
 __device__ __forceinline__ void finish_item(const TcParams& p, const FinishCtx& c, int z, int t, int tr, const float4& a,
                                             float4& old, const unsigned long long* s_slot, const float* s_mean,
                                             const float* s_rstd) {
@@ -139,13 +154,7 @@ __device__ __forceinline__ void finish_item(const TcParams& p, const FinishCtx& 
     const float xn[4] = {old.x + v[0], old.y + v[1], old.z + v[2], old.w + v[3]};
     old = make_float4(xn[0], xn[1], xn[2], xn[3]);
     *reinterpret_cast<float4*>(p.out_f32 + (long long)t * p.ldo + n) = old;
-    if (p.g_next) {
-      bf16 hi[4], lo[4];
-#pragma unroll
-      for (int e = 0; e < 4; ++e) split_bf16(xn[e] * c.gn[e], hi[e], lo[e]);
-      *reinterpret_cast<uint2*>(p.xg_hi + (long long)t * p.ldo + n) = pack4_bf16(hi);
-      *reinterpret_cast<uint2*>(p.xg_hi + (long long)t * p.ldo + n + p.xg_plane) = pack4_bf16(lo);
-    }
+    if (!CENTRED && p.g_next) store_planes_next(p, c, t, old, 0.f);      // centred: by tile_stats
   } else if (EPI == kTcQkv) {
     const int d = p.d;
     if (n < d) {
@@ -161,7 +170,7 @@ __device__ __forceinline__ void finish_item(const TcParams& p, const FinishCtx& 
 // each token, four per lane (N is a multiple of 128 here: every lane is live).  Sums of deviations from the token's
 // first value in the tile, and of their squares, are reduced for all TB tokens together so that the shuffles of one
 // token hide behind those of the others; mean and squared deviations about the mean follow exactly from the two.
-template <int TB>
+template <int TB, bool CENTRED>
 __device__ __forceinline__ void tile_stats(const TcParams& p, const FinishCtx& c, int t0, int tb, int hi, const float4 (&xn)[TB]) {
   float s1[TB], s2[TB], pivot[TB];
 #pragma unroll
@@ -179,16 +188,31 @@ __device__ __forceinline__ void tile_stats(const TcParams& p, const FinishCtx& c
       s2[i] += __shfl_xor_sync(0xffffffffu, s2[i], o);
     }
   }
-  if (c.g == 0) {
 #pragma unroll
-    for (int i = 0; i < TB; ++i) {
-      const int tr = tb + kEpiWarps * i;
-      if (tr < hi) {
-        const float dm = s1[i] * (1.0f / kBM);              // mean - pivot
-        reinterpret_cast<float2*>(p.stat_out)[(size_t)(c.n / kBM) * p.stat_T + t0 + tr] =
-            make_float2(pivot[i] + dm, fmaxf(s2[i] - s1[i] * dm, 0.f));
-      }
+  for (int i = 0; i < TB; ++i) {
+    const int tr = tb + kEpiWarps * i;
+    if (tr < hi) {
+      const float dm = s1[i] * (1.0f / kBM), mean = pivot[i] + dm;   // dm: mean - pivot
+      if (c.g == 0) reinterpret_cast<float2*>(p.stat_out)[(size_t)(c.n / kBM) * p.stat_T + t0 + tr] = make_float2(mean, fmaxf(s2[i] - s1[i] * dm, 0.f));
+      if (CENTRED) store_planes_next(p, c, t0 + tr, xn[i], mean);
     }
+  }
+}
+// Centred planes (TcParams::ln_parts) leave out of a token's sum: over the up to eight tiles (d_model 1024), (tile mean -
+// row mean) times the tile's share of ln_s.  A lane keeps the shares of its four features; the differences of a token are
+// eight words of shared memory behind the tile.
+__device__ __forceinline__ void centre_shares(const TcParams& p, const FinishCtx& c, int z, float4 (&share)[8]) {
+#pragma unroll
+  for (int q = 0; q < 8; ++q)
+    share[q] = q < p.stat_parts ? __ldg(reinterpret_cast<const float4*>(p.ln_parts + (size_t)q * p.N + c.n + p.zofs_ln * z)) : make_float4(0.f, 0.f, 0.f, 0.f);
+}
+__device__ __forceinline__ void add_centre(const float4 (&share)[8], const float4* diff, float4& v) {
+  const float4 a = diff[0], b = diff[1];
+  const float w[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    v.x = fmaf(w[q], share[q].x, v.x); v.y = fmaf(w[q], share[q].y, v.y);
+    v.z = fmaf(w[q], share[q].z, v.z); v.w = fmaf(w[q], share[q].w, v.w);
   }
 }
 
@@ -196,13 +220,16 @@ __device__ __forceinline__ void tile_stats(const TcParams& p, const FinishCtx& c
 // Tokens lo .. hi - 1 of the tile, whose S partial tiles lie in the shared memories of the cluster's CTAs (`tile_addr`:
 // this CTA's, the same offset in every CTA).  Warp w takes tokens lo + w, lo + w + 8, ..., TB of them at a time:
 // S x TB 16-byte reads (and the old residual values) are in flight per lane; the partial tiles are added in rank order.
-template <int EPI, int S, int TB>
+template <int EPI, bool CENTRED, int S, int TB>
 __device__ __forceinline__ void finish_tokens(const TcParams& p, int z, int t0, int lo, int hi, int tile, uint32_t tile_addr,
                                               const unsigned long long* s_slot, int warp, int lane, const float* s_mean,
-                                              const float* s_rstd) {
+                                              const float* s_rstd, const float4* s_diff) {
   FinishCtx c;
   finish_setup<EPI>(p, z, tile, lane, c);
   const bool live = c.n < p.N;                         // lanes beyond the last feature only keep the warp together
+  constexpr bool TERMS = CENTRED && EPI != kTcResidual;
+  float4 share[TERMS ? 8 : 1];
+  if constexpr (TERMS) centre_shares(p, c, z, share);
   uint32_t part[S];
 #pragma unroll
   for (int s = 0; s < S; ++s) part[s] = (S > 1 ? map_to_rank(tile_addr, s) : tile_addr) + lane * 16;
@@ -236,6 +263,10 @@ __device__ __forceinline__ void finish_tokens(const TcParams& p, int z, int t0, 
       for (int s = 1; s < S; ++s) {
         v[0][i].x += v[s][i].x; v[0][i].y += v[s][i].y; v[0][i].z += v[s][i].z; v[0][i].w += v[s][i].w;
       }
+    }
+    if constexpr (TERMS) {
+#pragma unroll
+      for (int i = 0; i < TB; ++i) add_centre(share, s_diff + 2 * min(tb + kEpiWarps * i, hi - 1), v[0][i]);
     }
     if constexpr (EPI == kTcArgmax) {
 #pragma unroll
@@ -275,9 +306,9 @@ __device__ __forceinline__ void finish_tokens(const TcParams& p, int z, int t0, 
 #pragma unroll
       for (int i = 0; i < TB; ++i) {
         const int tr = tb + kEpiWarps * i;
-        if (tr < hi && live) finish_item<EPI>(p, c, z, t0 + tr, tr, v[0][i], old[i], s_slot, s_mean, s_rstd);
+        if (tr < hi && live) finish_item<EPI, CENTRED>(p, c, z, t0 + tr, tr, v[0][i], old[i], s_slot, s_mean, s_rstd);
       }
-      if (EPI == kTcResidual && p.stat_out) tile_stats<TB>(p, c, t0, tb, hi, old);
+      if (EPI == kTcResidual && p.stat_out) tile_stats<TB, CENTRED>(p, c, t0, tb, hi, old);
     }
   }
 }
@@ -285,7 +316,10 @@ __device__ __forceinline__ void finish_tokens(const TcParams& p, int z, int t0, 
 // ---------------------------------------------------------------- the kernel
 // grid = (token tiles x slices, K splits, feature tiles), clusters of (1, K splits, 1): the CTAs that share a weight tile
 // are neighbours in x.  tmA: weights [N, K]; tmBh / tmBl: activation planes [rows, K]; boxes (64, 128) and (64, bn).
-template <int EPI, int PL>
+// CENTRED: the planes read (kTcResidual: written) are, see
+// TcParams::ln_parts.  Kernels of their own, because the code costs the decoder's launches more than it does the encoder's:
+// in one kernel a pass of 320 rows took 1 % longer.
+template <int EPI, int PL, bool CENTRED>
 __global__ void __launch_bounds__(kWideThreads, 2)
 gemm_wide_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmBh,
                  const __grid_constant__ CUtensorMap tmBl, const __grid_constant__ TcParams p, int ttiles, int stages,
@@ -298,6 +332,7 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
   __shared__ uint32_t s_ctl[2];                                     // tensor-memory base, "this CTA merges the top-1"
   __shared__ float s_mean[kWideBN], s_rstd[kWideBN];
   __shared__ unsigned long long s_slot[EPI == kTcQkv ? kWideBN : 1];
+  constexpr bool TERMS = CENTRED && EPI != kTcResidual;
   const int bn = p.bn;
   const uint32_t stage_sz = (uint32_t)wide_stage_bytes(bn, PL);
   const uint32_t bars = smem_u32(s_bar);                             // full[stages], empty[stages], accumulator
@@ -393,6 +428,7 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     const int et = threadIdx.x - 64, ew = warp - 2;   // 0..255, 0..7
     // this CTA's share of the tile's tokens
     const int per = (nt + S - 1) / S, lo = min(nt, split * per), hi = min(nt, lo + per);
+    float diff[TERMS ? 8 : 1] = {};                  // tile means less the row's mean, of this thread's token
     if (EPI == kTcQkv && !skip) {
       const int tr = lo + et;
       if (tr < hi) {
@@ -426,6 +462,10 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
       }
       s_mean[tr] = mean;
       s_rstd[tr] = rsqrtf(m2 / cnt + p.ln_eps);
+      if constexpr (TERMS) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) diff[i] = i < p.stat_parts ? part[i].x - mean : 0.f;
+      }
     }
     bool done = !skip;
     if (done && nchunks > 0) done = mbar_wait(acc_bar, 0);
@@ -446,6 +486,13 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
 #pragma unroll
         for (int c = 0; c < 16; ++c) s_t[(cb + c) * kWidePitch + row] = v[c];
       }
+      if constexpr (TERMS) {
+        float4* at = reinterpret_cast<float4*>(s_t + bn * kWidePitch) + 2 * (lo + et);
+        if (lo + et < hi) {
+          at[0] = make_float4(diff[0], diff[1], diff[2], diff[3]);
+          at[1] = make_float4(diff[4], diff[5], diff[6], diff[7]);
+        }
+      }
     }
     s_ctl[1] = 0;
   }
@@ -456,10 +503,11 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
   if (warp >= 2 && !skip_all) {
     const int et = threadIdx.x - 64, ew = warp - 2;
     const int per = (nt + S - 1) / S, lo = min(nt, split * per), hi = min(nt, lo + per);
-    if (S == 1) finish_tokens<EPI, 1, 4>(p, slice, t0, lo, hi, tile, base, s_slot, ew, lane, s_mean, s_rstd);
-    else if (S == 2) finish_tokens<EPI, 2, 4>(p, slice, t0, lo, hi, tile, base, s_slot, ew, lane, s_mean, s_rstd);
-    else if (S == 4) finish_tokens<EPI, 4, 2>(p, slice, t0, lo, hi, tile, base, s_slot, ew, lane, s_mean, s_rstd);
-    else finish_tokens<EPI, 8, 1>(p, slice, t0, lo, hi, tile, base, s_slot, ew, lane, s_mean, s_rstd);
+    const float4* s_diff = reinterpret_cast<const float4*>(gen_base + (size_t)bn * kWidePitch * sizeof(float));
+    if (S == 1) finish_tokens<EPI, CENTRED, 1, 4>(p, slice, t0, lo, hi, tile, base, s_slot, ew, lane, s_mean, s_rstd, s_diff);
+    else if (S == 2) finish_tokens<EPI, CENTRED, 2, 4>(p, slice, t0, lo, hi, tile, base, s_slot, ew, lane, s_mean, s_rstd, s_diff);
+    else if (S == 4) finish_tokens<EPI, CENTRED, 4, 2>(p, slice, t0, lo, hi, tile, base, s_slot, ew, lane, s_mean, s_rstd, s_diff);
+    else finish_tokens<EPI, CENTRED, 8, 1>(p, slice, t0, lo, hi, tile, base, s_slot, ew, lane, s_mean, s_rstd, s_diff);
     if (EPI == kTcArgmax) {
       // the CTA that completes the last tile hands the winners out
       asm volatile("bar.sync 1, 256;" ::: "memory");

@@ -111,13 +111,14 @@ int parse_blob(const void* blob, size_t n, ParsedBlob* out);
 
 struct EncLayer {
   const void *ln1g, *ln1b, *wqkv, *wo, *ln2g, *ln2b, *w1, *b1, *w2, *b2;
-  float *s_qkv, *c_qkv, *s_f1, *c_f1;   // layer norms folded into the projections that follow them (bf16 models)
+  // layer norms folded into the projections that follow them (bf16 models); p_: the shares of s_ (see FoldParams)
+  float *s_qkv, *c_qkv, *p_qkv, *s_f1, *c_f1, *p_f1;
 };
 struct DecLayer {
   const void *ln1g, *ln1b, *wqkv, *wo, *ln2g, *ln2b, *cwq, *cwkv, *cwo, *ln3g, *ln3b, *w1, *b1, *w2, *b2;
   // layer norms folded into the projections that follow them (bf16 models): per-feature s and c vectors
   float *s_qkv, *c_qkv, *s_cq, *c_cq, *s_f1, *c_f1;
-  float *s_ckv, *c_ckv;    // the encoder's final layer norm, folded into the keys and values of this layer's cross-attention
+  float *s_ckv, *c_ckv, *p_ckv;    // the encoder's final layer norm, folded into the keys and values of this layer's cross-attention
 };
 
 }  // namespace bpd

@@ -27,6 +27,7 @@ struct EmbedParams {
   const bf16* gain;        // optional: also write planes (hi, lo) of x * gain for a projection with a folded layer norm
   bf16* xg_hi; long long xg_plane;
   float* stat_out; int stat_T;   // optional: mean and squared deviations of every 128 consecutive features of a row, [d / 128][stat_T][2]
+  int centred;             // 1 (with stat_out): the planes hold (x - mean of the 128 features) * gain
   const int* all_done;
 };
 
@@ -68,6 +69,7 @@ __device__ __forceinline__ void embed_row(const EmbedParams& p, int r) {
     for (int i = 0; i < 8; ++i) v[i] = w[i] * scale + e[i];
     out[0] = make_float4(v[0], v[1], v[2], v[3]);
     out[1] = make_float4(v[4], v[5], v[6], v[7]);
+    float centre = 0.f;
     if (p.stat_out) {
       // 16 consecutive lanes hold 128 consecutive features (d is a multiple of 128 here, so half-warps are whole)
       float sum = ((v[0] + v[1]) + (v[2] + v[3])) + ((v[4] + v[5]) + (v[6] + v[7]));
@@ -80,6 +82,7 @@ __device__ __forceinline__ void embed_row(const EmbedParams& p, int r) {
 #pragma unroll
       for (int o = 8; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
       if ((threadIdx.x & 15) == 0) reinterpret_cast<float2*>(p.stat_out)[(size_t)(c >> 7) * p.stat_T + r] = make_float2(mean, sq);
+      if (p.centred) centre = mean;
     }
     if (p.gain) {
       float g[8];
@@ -87,7 +90,7 @@ __device__ __forceinline__ void embed_row(const EmbedParams& p, int r) {
       bf16 hi[8], lo[8];
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
-        const float xg = v[i] * g[i];
+        const float xg = (v[i] - centre) * g[i];
         hi[i] = __float2bfloat16_rn(xg);
         lo[i] = __float2bfloat16_rn(xg - __bfloat162float(hi[i]));
       }
@@ -109,9 +112,11 @@ __global__ void embed_kernel(EmbedParams p) {
 // ------------------------------------------------------------------ folding a layer norm into the projection after it
 // LN(x) w^T = rstd * (x*gain) w^T - rstd * mean * s + c   with   s[n] = sum_c gain[c] w[n][c],
 // c[n] = sum_c shift[c] w[n][c] + bias[n].  One warp per output feature, accumulated in double (load time only).
+// parts[i][n]: s[n]'s share of features 128 i .. 128 i + 127, for planes that hold x - mean of the 128 (K is a multiple
+// of 256 then, so a half-warp's loads are one share), or null.
 struct FoldParams {
   const bf16* w; const bf16* gain; const bf16* shift; const bf16* bias;
-  float* s; float* c;
+  float* s; float* c; float* parts;
   int N, K;
 };
 static __global__ void __launch_bounds__(128) fold_ln_kernel(FoldParams p) {
@@ -124,8 +129,15 @@ static __global__ void __launch_bounds__(128) fold_ln_kernel(FoldParams p) {
     load8(p.w + (size_t)n * p.K + k, w);
     load8(p.gain + k, g);
     load8(p.shift + k, b);
+    double sk = 0.0;
 #pragma unroll
-    for (int e = 0; e < 8; ++e) { ss += (double)g[e] * (double)w[e]; cc += (double)b[e] * (double)w[e]; }
+    for (int e = 0; e < 8; ++e) { sk += (double)g[e] * (double)w[e]; cc += (double)b[e] * (double)w[e]; }
+    ss += sk;
+    if (p.parts) {
+#pragma unroll
+      for (int o = 8; o > 0; o >>= 1) sk += __shfl_xor_sync(0xffffffffu, sk, o);
+      if ((lane & 15) == 0) p.parts[(size_t)(k >> 7) * p.N + n] = (float)sk;
+    }
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {

@@ -321,12 +321,16 @@ int launch(const Operands& op, int N, int K, int T, TcParams p, const Scratch& s
   if (p.ln_x || (!p.vec && EPI != kTcF32 && EPI != kTcArgmax)) return fail(BPD_E_UNSUPPORTED, "operands of the wide projection kernel are misaligned");
   if ((p.stat_in || p.stat_out) && !(p.vec && N % kBM == 0 && EPI != kTcArgmax))
     return fail(BPD_E_UNSUPPORTED, "per-tile layer-norm statistics need whole, aligned feature tiles (N = %d)", N);
-  const void* kernel = planes == 2 ? reinterpret_cast<const void*>(gemm_wide_kernel<EPI, 2>) : nullptr;
+  const void* kernel = planes == 2 && !p.ln_parts && !p.centred ? reinterpret_cast<const void*>(gemm_wide_kernel<EPI, 2, false>) : nullptr;
   if constexpr (EPI == kTcF32 || EPI == kTcArgmax) {
-    if (planes == 1) kernel = reinterpret_cast<const void*>(gemm_wide_kernel<EPI, 1>);
+    if (planes == 1 && !p.ln_parts) kernel = reinterpret_cast<const void*>(gemm_wide_kernel<EPI, 1, false>);
   }
-  if (!kernel) return fail(BPD_E_UNSUPPORTED, "single-plane activations with this epilogue");
-  const size_t smem = wide_smem_bytes(bn, planes, wp.stages);
+  if constexpr (EPI == kTcF32 || EPI == kTcPlanes || EPI == kTcResidual) {
+    if (planes == 2 && (EPI == kTcResidual ? p.centred && p.stat_out : p.ln_parts && p.stat_in)) kernel = reinterpret_cast<const void*>(gemm_wide_kernel<EPI, 2, true>);
+  }
+  if (p.ln_parts && p.stat_parts > 8) return fail(BPD_E_UNSUPPORTED, "centred activations of %d tiles", p.stat_parts);
+  if (!kernel) return fail(BPD_E_UNSUPPORTED, "single-plane or centred activations with this epilogue");
+  const size_t smem = wide_smem_bytes(bn, planes, wp.stages, p.ln_parts != nullptr);
   if ((rc = ensure_smem_limit(kernel, smem))) return rc;
   BPD_CUDA(launch_cluster(kernel, dim3(wp.ttiles * zslices, wp.splits, wp.tiles), dim3(kWideThreads), smem, st, pdl, wp.splits,
                           ma, mh, ml, p, wp.ttiles, wp.stages, a_rows_per_slice, b_cols_per_slice));

@@ -143,6 +143,57 @@ def test_encoder_feeds_the_decoder_like_the_oracle(bpd, batch, max_src, d, n_dec
     model.close()
 
 
+# With the decoder's self-attention output projections at zero nothing that reaches the hidden states is rounded to the
+# cache's bf16: encoder, cross-attention and feed-forward layers carry fp32 throughout (two bf16 planes per activation, three
+# in the attention kernels), in every form the layers take.  Rows far from zero mean (64 standard deviations) must cost the
+# encoder nothing.  An activation's planes round at 2^-18 of its value, the hidden states are normalised (elements up to
+# about 4) and some 15 such roundings lie on the way, so 15 * 4 * 2^-18 = 2.3e-4 at worst; 1e-4 is five times what is
+# seen.  Losing a plane costs 2^-9 of a value, uncentred planes of the shifted rows 64 * 2^-18.
+@pytest.mark.parametrize("shift", [0, 64])
+@pytest.mark.parametrize("batch,k,heads,max_src,tgt,options", [
+    (1, 4, 4, 40, 20, {}),                                           # persistent kernel: one short sequence
+    (1, 4, 8, 100, 600, {}),                                         # one long
+    (2, 4, 4, 40, 20, {}),                                           # several in one set of clusters
+    (5, 4, 8, 40, 20, {}),                                           # groups
+    (2, 4, 8, 40, 20, {"persistent_layers": 0}),                     # cluster launches
+    (2, 4, 4, 40, 20, {"persistent_layers": 0, "cluster_layers": 0}),    # one kernel per projection, few rows
+    (24, 4, 8, 97, 20, {}),                                          # many rows, layer-norm kernels in the encoder
+    (24, 4, 8, 97, 20, {"fold_layer_norms": 1}),                     # and folded, several token tiles
+    (9, 4, 16, 85, 20, {}),                                          # the most rows that are folded, eight tiles of statistics
+    (3, 8, 3, 33, 20, {}),                                           # widths without folded layer norms
+])
+def test_fp32_paths_keep_their_precision(bpd, batch, k, heads, max_src, tgt, options, shift):
+    import torch
+    from bpd_inputs import ModelConfig, make_weights
+    from bpd_inputs.blob import blob_layout
+    from oracle.decode import TransformerScorer
+    from oracle.model import parse_blob
+    cfg = ModelConfig(2, 2, 64 * heads, heads, 128 * heads, 300, k, 64)
+    blob = make_weights(cfg, 5, 0.06)
+    for name, shape, _, off, nbytes in blob_layout(cfg)[0]:
+        if name.endswith("self.wo"):
+            blob[off:off + nbytes] = 0
+        if name == "src_embed":
+            t = torch.from_numpy(blob[off:off + nbytes].view(np.int16)).view(torch.bfloat16)
+            t.copy_((t.float() + shift * 0.06).bfloat16())
+    rng = np.random.default_rng(batch)
+    lens = rng.integers(1, max_src + 1, batch).astype(np.int32)
+    lens[-1] = max_src
+    src = rng.integers(2, 300, (batch, max_src)).astype(np.int32)
+    model = bpd.Model(blob)
+    s = bpd.Session(model, batch, max_src, tgt, options=options)
+    s.bpd_encode(src, lens)
+    r = s.bpd_iteration(k, tgt, want_hidden=True)
+    model_o = parse_blob(blob)
+    for b in sorted({0, 1, batch - 1} & set(range(batch))):
+        scorer = TransformerScorer(model_o, src[b], int(lens[b]), cached=True, capacity=tgt + k + 2)
+        scorer([0], 1)
+        scorer([0] + [int(t) for t in r["block"][b]], k)
+        np.testing.assert_allclose(r["hidden"][b].cpu().numpy(), scorer.last_hidden, atol=1e-4)
+    s.close()
+    model.close()
+
+
 # the persistent layer kernel with groups of sequences: a last group that is full and one that is not, two sequences per
 # group and one, one token tile and two, lengths up to the limit of 256 positions, one encoder row and 256
 @pytest.mark.parametrize("batch,k,heads,max_src,tgt", [(3, 4, 4, 61, 30), (8, 4, 4, 9, 251), (5, 3, 8, 1, 20), (2, 10, 8, 33, 40), (4, 16, 8, 24, 48),
