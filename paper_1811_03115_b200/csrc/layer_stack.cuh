@@ -1009,10 +1009,16 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
   uint8_t* ssm = ssm_raw + ((1024u - (tc::smem_u32(ssm_raw) & 1023u)) & 1023u);
   cg::cluster_group cluster = cg::this_cluster();
   constexpr int RP = NT * 8;
+  constexpr bool GROUPS = LEAN == 4;
+  constexpr bool SPLIT = LEAN == 2 || LEAN == 3;         // keys split over the ranks
   Cta k;
   k.p = &p;
   k.maps = &maps;
-  k.g = make_geo(p.d, p.H, p.ff, p.L, p.cross_staged ? p.cross_rows : 0, p.cross_split);
+  // Two parameters that only the variants which split the keys need are constants in the others: there they cost variant 1
+  // 24 bytes of spills, 192.6 instead of 191.6 us for the six layers of a 16-head model and 1.8 % of its greedy decode
+  // (28930 / 28412 us), variant 4 1 % of a decode of
+  // five sentences (4631 / 4581 us).  (As constants in variants 2 and 3 too: 4008 against 3971 us for a base sentence.)
+  k.g = make_geo(p.d, p.H, p.ff, p.L, (LEAN == 1 || GROUPS || p.cross_staged) ? p.cross_rows : 0, SPLIT ? p.cross_split : 0);
   k.sm = ssm;
   k.ctl = reinterpret_cast<Ctl*>(ssm + p.lay.misc);
   k.ring = tc::smem_u32(ssm);
@@ -1024,7 +1030,6 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
   k.policy = tc::l2_evict_first();
   const Geo& g = k.g;
   const int c = k.c, j = k.j, tid = k.tid, warp = k.warp, lane = k.lane;
-  constexpr bool GROUPS = LEAN == 4;
   const int grp = GROUPS ? (int)blockIdx.z : 0, b0 = GROUPS ? grp * p.group_seqs : 0;
   const int d = p.d, ks = g.ks, rpb = p.rows_per_b, nb = GROUPS ? min(p.group_seqs, p.nb - b0) : p.nb, R = GROUPS ? nb * rpb : p.R;
   k.R = R;
@@ -1133,7 +1138,6 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
       one_chunk_per_rank = one_chunk_per_rank && ((s_len[b] + rpb + 31) >> 5) - (attn_first_key(ap, s_len[b]) >> 5) <= kC;
   }
 
-  constexpr bool SPLIT = LEAN == 2 || LEAN == 3;         // keys split over the ranks
   constexpr int KW = LEAN == 2 ? kLongKeys : kShortKeys;
   const LongCtx lc = SPLIT ? long_ctx<KW>(k, ap, ssm, s_pt, s_len[0]) : LongCtx{};
   if (SPLIT) long_prefetch<KW>(k, lc, layers_s[0], 0);
