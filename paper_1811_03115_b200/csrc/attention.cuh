@@ -281,10 +281,15 @@ __global__ void __launch_bounds__(kThreads, 3) attention_mma_kernel(const __grid
 }
 
 // Whether a launch takes this kernel; `block`: the most query rows per sequence of any launch of the session (the choice
-// must not depend on the pass).  With a CTA on half the SMs it is the faster one at any length.  Launches of fewer CTAs
-// stay with the kernel that gives every row a CTA of its own where a CTA would have less than half of its 16 rows to work
-// on (5 sentences of 4 rows, 8 heads: 315 against 324 us per pass; 3 sentences of 8 rows, 16 heads: 447 against 413), or
-// where it would walk more than 512 keys alone (about 5 us per 1000).
+// must not depend on the pass).  With a CTA on half the SMs (74 items) it is the faster one at any length.  Launches of fewer
+// CTAs stay with the kernels that give rows CTAs of their own where a CTA would have less than half of its 16 rows to work
+// on, or would walk more than 512 keys alone.  us per pass with the row kernels / with this one in every launch:
+//   items (sequences x heads)   48        48        48        64        64        72        80        80        96
+//   rows of a sequence           4         6         8         5         7         4         4         8         2
+//   up to 140 keys             487/500   357/352   405/375   372/353   417/378   374/332   367/351   490/401   350/312
+//   48 items of 8 rows over 450 / 600 / 1200 / 2400 keys: 431/393, 444/402, 492/459, 568/560 (this one for the encoder's
+//   rows and the row kernels for the cache: 542); 72 of 8 over 600: 575/407; 80 of 4 over 1200: 685/423
+// So the line is on the careful side: of these only 48 items of 4 rows lose with this kernel, and 64 to 73 items win.
 inline bool applies(const AttnParams& a, int max_keys, int block) {
   const int items = (a.rows / a.rows_per_b) * a.H * ((block + kRows - 1) / kRows);
   return a.dh == 64 && (items >= 74 || (block >= kRows / 2 && max_keys <= 512));

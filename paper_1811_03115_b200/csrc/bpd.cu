@@ -177,10 +177,13 @@ static bool stack_shapes_ok(const Config& c, int rows) {
 // Sessions of several sequences whose passes have more rows than one set of clusters of the persistent layer kernel takes
 // in its fastest shape (8): groups of sequences, each with H clusters of its own.  A pass of kernel-per-projection layers is
 // 55 launches of about 5 us each whatever they move; the groups' chains run side by side, and what they fetch twice comes
-// out of L2.  Five sentences of the base model (20 rows): 315 -> 200 us per pass, four (16 rows, one set of clusters with
-// two token tiles before) 249 -> 222 per single iteration.  The line: 33 clusters of 8 are resident at two CTAs per SM, so
-// four groups of 8 heads or two of 16; models of 16 heads with at most 16 rows stay with the cluster launches, which take
-// them whole.  0: no groups.
+// out of L2.  Five sentences of the base model (20 rows): 315 -> 200 us per pass.  The line: 33 clusters of 8 are resident
+// at two CTAs per SM, so four groups of 8 heads or two of 16.  (33 is a B200's count.  It sizes the session's buffer, for
+// which no device is asked; whether the clusters fit, stack_setup asks the device.)  At 9 to 16 rows one set of clusters with
+// two token tiles takes the pass whole, and models of 16 heads the cluster launches; us per pass, whole / in groups:
+//   8 heads   3 x 3 rows 211/190   2 x 5 210/195   2 x 8 231/207   4 x 4 225/199   8 x 2 223/197
+//   16 heads  2 x 5 383/232   3 x 4 421/233   2 x 8 465/262   4 x 4 446/248   8 x 2 450/245
+// So 16 heads could take groups from 9 rows on as well; the rule does not do it yet.  0: no groups.
 static int stack_groups(const Config& c, int B, int* seqs) {
   *seqs = std::max(1, 8 / c.k_model);
   const int groups = ceil_div(B, *seqs);
@@ -284,7 +287,8 @@ static size_t plan_session(const Config& c, int B, int max_src, int max_tgt, cha
 static int fold_parts(const Config& c) { return c.d % 256 == 0 ? c.d / 128 : 0; }
 static size_t fold_floats(const Config& c) {
   if (c.dtype != 1) return 0;
-  return (size_t)c.n_dec * 2 * (3 * c.d + c.d + c.d_ff) + (size_t)(2 + fold_parts(c)) * (c.n_dec * 2 * c.d + c.n_enc * (3 * c.d + c.d_ff));
+  const size_t decoder = (size_t)c.n_dec * 2 * (3 * c.d + c.d + c.d_ff), encoder = (size_t)c.n_dec * 2 * c.d + (size_t)c.n_enc * (3 * c.d + c.d_ff);
+  return decoder + (fold_parts(c) ? (1 + fold_parts(c)) * encoder : 0);
 }
 static size_t weight_bytes_for(const ParsedBlob& pb) { return align_up(pb.total) + align_up(fold_floats(pb.cfg) * sizeof(float)); }
 
@@ -617,7 +621,7 @@ static int run_encoder_tc(bpd_session* s) {
     norm_of(pk, m->dec[l].p_ckv, m->dec[l].c_ckv);
     if (slices > 1) {
       pk.zofs_out = static_cast<float*>(s->crosskv[1]) - static_cast<float*>(s->crosskv[0]);
-      pk.zofs_ln = (2 + fold_parts(c)) * 2 * d;
+      pk.zofs_ln = (1 + fold_parts(c)) * 2 * d;
     }
     const int rows_apart = (int)(step / row);
     BPD_TRY(tc::launch<tc::kTcF32>(with_w(xn, m->dec[l].cwkv, (slices - 1) * rows_apart + 2 * d), 2 * d, d, E, pk, sc, st, slices, slices > 1 ? rows_apart : 0, 0, pdl));
@@ -1332,27 +1336,28 @@ int bpd_load_weights(const void* blob, size_t blob_bytes, void* dev_weight_buf, 
   cudaError_t e = cudaMemcpyAsync(m->base, blob, pb.total, cudaMemcpyHostToDevice, m->stream);
   if (c.dtype == 1 && e == cudaSuccess) {
     float* fp = reinterpret_cast<float*>(m->base + align_up(pb.total));
-    auto fold = [&](const void* w, const void* g, const void* b, const void* bias, int N, float** s_out, float** c_out, float** shares = nullptr) {
-      *s_out = fp; fp += N;
+    auto fold = [&](const void* w, const void* g, const void* b, const void* bias, int N, float** s_out, float** c_out, float** shares) {
       *c_out = fp; fp += N;
-      if (shares) { *shares = fold_parts(c) ? fp : nullptr; fp += (size_t)fold_parts(c) * N; }
+      if (s_out) { *s_out = fp; fp += N; }
+      if (shares) { *shares = fp; fp += (size_t)fold_parts(c) * N; }
       FoldParams p{static_cast<const bf16*>(w), static_cast<const bf16*>(g), static_cast<const bf16*>(b),
-                   static_cast<const bf16*>(bias), *s_out, *c_out, shares ? *shares : nullptr, N, d};
+                   static_cast<const bf16*>(bias), s_out ? *s_out : nullptr, *c_out, shares ? *shares : nullptr, N, d};
       fold_ln_kernel<<<ceil_div(N, 4), 128, 0, m->stream>>>(p);
     };
     for (int l = 0; l < c.n_dec; ++l) {
       DecLayer& L = m->dec[l];
-      fold(L.wqkv, L.ln1g, L.ln1b, nullptr, 3 * d, &L.s_qkv, &L.c_qkv);
-      fold(L.cwq, L.ln2g, L.ln2b, nullptr, d, &L.s_cq, &L.c_cq);
-      fold(L.w1, L.ln3g, L.ln3b, L.b1, f, &L.s_f1, &L.c_f1);
+      fold(L.wqkv, L.ln1g, L.ln1b, nullptr, 3 * d, &L.s_qkv, &L.c_qkv, nullptr);
+      fold(L.cwq, L.ln2g, L.ln2b, nullptr, d, &L.s_cq, &L.c_cq, nullptr);
+      fold(L.w1, L.ln3g, L.ln3b, L.b1, f, &L.s_f1, &L.c_f1, nullptr);
     }
-    for (int l = 0; l < c.n_enc; ++l) {
+    for (int l = 0; l < c.n_enc && fold_parts(c); ++l) {
       EncLayer& L = m->enc[l];
-      fold(L.wqkv, L.ln1g, L.ln1b, nullptr, 3 * d, &L.s_qkv, &L.c_qkv, &L.p_qkv);
-      fold(L.w1, L.ln2g, L.ln2b, L.b1, f, &L.s_f1, &L.c_f1, &L.p_f1);
+      fold(L.wqkv, L.ln1g, L.ln1b, nullptr, 3 * d, nullptr, &L.c_qkv, &L.p_qkv);
+      fold(L.w1, L.ln2g, L.ln2b, L.b1, f, nullptr, &L.c_f1, &L.p_f1);
     }
     // in layer order, so that one launch over all layers steps through them (TcParams::zofs_ln)
-    for (int l = 0; l < c.n_dec; ++l) fold(m->dec[l].cwkv, m->enc_lnf_g, m->enc_lnf_b, nullptr, 2 * d, &m->dec[l].s_ckv, &m->dec[l].c_ckv, &m->dec[l].p_ckv);
+    for (int l = 0; l < c.n_dec && fold_parts(c); ++l)
+      fold(m->dec[l].cwkv, m->enc_lnf_g, m->enc_lnf_b, nullptr, 2 * d, nullptr, &m->dec[l].c_ckv, &m->dec[l].p_ckv);
     e = cudaGetLastError();
   }
   if (e == cudaSuccess) e = cudaStreamSynchronize(m->stream);
@@ -1425,7 +1430,7 @@ int bpd_session_create_opt(const bpd_model* model, int batch, int max_src, int m
   s->opt.persistent_layers = o.persistent_layers;   // -1: where its lean variant applies (measured faster there), 0: never, 1: wherever it runs
   s->opt.stage_encoder_rows = o.stage_encoder_rows != 0 ? 1 : 0;
   s->opt.l2_stream_hints = o.l2_stream_hints != 0 ? 1 : 0;
-  s->stack = 0; s->stack_dump = nullptr;
+  s->stack = 0;
   s->timed = 0;
   s->phase = kPhaseCreated; s->plan_len = 0; s->plan_k = 0; s->invocations = 0; s->pinned = nullptr;
   plan_session(model->cfg, batch, max_src, max_tgt, s->base, s);

@@ -80,14 +80,6 @@ __device__ __forceinline__ float warp_max(float v) {
 __device__ __forceinline__ bool better(float v, int i, float bv, int bi) {
   return (v > bv) || (v == bv && i < bi);
 }
-__device__ __forceinline__ void warp_argmax(float& v, int& i) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    float ov = __shfl_xor_sync(0xffffffffu, v, o);
-    int oi = __shfl_xor_sync(0xffffffffu, i, o);
-    if (better(ov, oi, v, i)) { v = ov; i = oi; }
-  }
-}
 
 // (value, index) packed so that an unsigned 64-bit max picks the larger value and, among equal values, the lower index.
 // Zero is below every real entry.  Every row's key has a 128-byte line of its own: hundreds of tiles send one atomic

@@ -40,7 +40,6 @@ __device__ __forceinline__ void tc_stamp(int region, int slot) {
 
 constexpr int kBM = 128;          // features per tile (MMA M)
 constexpr int kBK = 64;           // K elements per pipeline stage (128 bytes of bf16: one swizzle row)
-constexpr int kMaxStages = 4;     // pipeline depth is chosen per launch (2..4) so that two CTAs fit on an SM when possible
 constexpr int kThreads = 192;     // warp 0: TMA, warp 1: MMA + tensor-memory allocation, warps 2-5: epilogue
 constexpr int kMaxBN = 16;        // tokens per CTA (MMA N); wider launches take gemm_wide.cuh
 constexpr unsigned long long kSpinCycles = 2000000000ull;   // about a second
@@ -210,8 +209,8 @@ __device__ __forceinline__ void split_bf16(float v, bf16& hi, bf16& lo) {
 
 // Shared-memory footprint of one CTA.
 __host__ __device__ inline size_t stage_bytes(int bn) { return (size_t)kBM * 128 + 2 * (size_t)bn * 128; }
-__host__ __device__ inline int stages_for(int) { return 5; }
-__host__ __device__ inline size_t smem_bytes(int bn) { return stages_for(bn) * stage_bytes(bn) + 1024 /*alignment*/ + 256; }
+constexpr int kStages = 5;        // K chunks in flight; 101 KB at 16 tokens, so two CTAs fit on an SM
+__host__ __device__ inline size_t smem_bytes(int bn) { return kStages * stage_bytes(bn) + 1024 /*alignment*/ + 256; }
 
 // ---------------------------------------------------------------- final epilogue for one (feature, token)
 // Finishes up to 8 tokens of one feature.  Everything that has to be read (old residual values, the head
@@ -491,7 +490,6 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;      // swizzled tiles need 1024-byte alignment
   uint8_t* gen_base = smem_raw + (base - smem_u32(smem_raw));
   const int bn = p.bn;
-  const int kStages = stages_for(bn);
   const uint32_t stage_sz = (uint32_t)stage_bytes(bn);
   const uint32_t bars = base + kStages * stage_sz;                   // full[kStages], empty[kStages], accum
   volatile uint32_t* ctl = reinterpret_cast<volatile uint32_t*>(gen_base + kStages * stage_sz + 128);

@@ -111,14 +111,14 @@ int parse_blob(const void* blob, size_t n, ParsedBlob* out);
 
 struct EncLayer {
   const void *ln1g, *ln1b, *wqkv, *wo, *ln2g, *ln2b, *w1, *b1, *w2, *b2;
-  // layer norms folded into the projections that follow them (bf16 models); p_: the shares of s_ (see FoldParams)
-  float *s_qkv, *c_qkv, *p_qkv, *s_f1, *c_f1, *p_f1;
+  // layer norms folded into the projections that follow them (bf16 models): c, and s as its shares (see FoldParams)
+  float *c_qkv, *p_qkv, *c_f1, *p_f1;
 };
 struct DecLayer {
   const void *ln1g, *ln1b, *wqkv, *wo, *ln2g, *ln2b, *cwq, *cwkv, *cwo, *ln3g, *ln3b, *w1, *b1, *w2, *b2;
   // layer norms folded into the projections that follow them (bf16 models): per-feature s and c vectors
   float *s_qkv, *c_qkv, *s_cq, *c_cq, *s_f1, *c_f1;
-  float *s_ckv, *c_ckv, *p_ckv;    // the encoder's final layer norm, folded into the keys and values of this layer's cross-attention
+  float *c_ckv, *p_ckv;    // the encoder's final layer norm, folded into the keys and values of this layer's cross-attention
 };
 
 }  // namespace bpd
@@ -202,7 +202,6 @@ struct bpd_session {
   void* stack_layers;      // device: stack::LayerPtrs [n_dec]
   unsigned long long* stack_ws;   // device: per group [2][H][16][d] words (value, tag): the clusters' shares of the projection outputs
   unsigned* stack_bar;     // device: words of the device-wide join
-  float* stack_dump;       // device: [n_dec][rows][d] residual stream after every layer (debug dump), or null
   int stack_cross_rows, stack_staged, stack_long, stack_minb, stack_lean, stack_dev, stack_groups, stack_group_seqs;
   int stack_layout[24];    // stack::Layout, kept opaque here
   std::map<GraphKey, GraphEntry> graphs;

@@ -101,6 +101,9 @@ __device__ __forceinline__ void embed_row(const EmbedParams& p, int r) {
   }
 }
 
+// The first kernel of a pass and of the encoder, launched without the programmatic attribute: kernels behind it read the
+// rows' lengths, committed cache entries and the encoder's rows before their own dependency wait, and only this full
+// dependency says that the pass before (its verify kernel) has ended by then.
 template <typename WT>
 __global__ void embed_kernel(EmbedParams p) {
   pdl_launch_dependents();
@@ -113,10 +116,10 @@ __global__ void embed_kernel(EmbedParams p) {
 // LN(x) w^T = rstd * (x*gain) w^T - rstd * mean * s + c   with   s[n] = sum_c gain[c] w[n][c],
 // c[n] = sum_c shift[c] w[n][c] + bias[n].  One warp per output feature, accumulated in double (load time only).
 // parts[i][n]: s[n]'s share of features 128 i .. 128 i + 127, for planes that hold x - mean of the 128 (K is a multiple
-// of 256 then, so a half-warp's loads are one share), or null.
+// of 256 then, so a half-warp's loads are one share).
 struct FoldParams {
   const bf16* w; const bf16* gain; const bf16* shift; const bf16* bias;
-  float* s; float* c; float* parts;
+  float* s; float* c; float* parts;    // s and parts: or null
   int N, K;
 };
 static __global__ void __launch_bounds__(128) fold_ln_kernel(FoldParams p) {
@@ -145,7 +148,7 @@ static __global__ void __launch_bounds__(128) fold_ln_kernel(FoldParams p) {
     cc += __shfl_xor_sync(0xffffffffu, cc, o);
   }
   if (lane == 0) {
-    p.s[n] = (float)ss;
+    if (p.s) p.s[n] = (float)ss;
     p.c[n] = (float)(cc + (p.bias ? (double)__bfloat162float(p.bias[n]) : 0.0));
   }
 }

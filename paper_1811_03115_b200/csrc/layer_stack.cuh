@@ -523,7 +523,6 @@ static __global__ void tagged_wait_probe_kernel(int* error, unsigned long long l
 template <int NT>
 __device__ __forceinline__ void planes_and_stats(const Cta& k, const float* x_s, const Words& gain, uint8_t* xh, uint8_t* xl,
                                                  float* stats_mine) {
-  const StackParams& p = *k.p;
   const int ks = k.g.ks, n4 = ks >> 2, R = k.R, PW = k.g.PW;
   constexpr int RP = NT * 8;
 #pragma unroll
@@ -1016,8 +1015,8 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
   k.maps = &maps;
   // Two parameters that only the variants which split the keys need are constants in the others: there they cost variant 1
   // 24 bytes of spills, 192.6 instead of 191.6 us for the six layers of a 16-head model and 1.8 % of its greedy decode
-  // (28930 / 28412 us), variant 4 1 % of a decode of
-  // five sentences (4631 / 4581 us).  (As constants in variants 2 and 3 too: 4008 against 3971 us for a base sentence.)
+  // (28930 / 28412 us), variant 4 1 % of a decode of five sentences (4631 / 4581 us).  As constants in variants 2 and 3 too:
+  // 4008 against 3971 us for a base sentence.
   k.g = make_geo(p.d, p.H, p.ff, p.L, (LEAN == 1 || GROUPS || p.cross_staged) ? p.cross_rows : 0, SPLIT ? p.cross_split : 0);
   k.sm = ssm;
   k.ctl = reinterpret_cast<Ctl*>(ssm + p.lay.misc);
@@ -1645,7 +1644,8 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
 }
 
 // The kernel's instantiations (layer_stack.cu): token tiles (1 or 2 of 8 rows), reduction steps per panel (2: d_model
-// 256, else 4), CTAs per SM (1 or 2), lean (short sequences and staged encoder rows only); null if there is none.
+// 256, else 4), CTAs per SM (1 or 2), variant (LEAN, see the kernel: 0 general, 1 short sequences with staged encoder
+// rows, 2 one long sequence, 3 one short sequence, 4 groups of sequences); null if there is none.
 const void* kernel_for(int nt, int ksteps, int minb, int lean);
 
 }  // namespace stack

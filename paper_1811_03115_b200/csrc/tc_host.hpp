@@ -15,7 +15,8 @@
 namespace bpd {
 namespace tc {
 
-// Resident CTA slots the planner aims to fill: 2 CTAs on each of the 148 SMs of a B200.
+// Resident CTA slots the planner aims to fill: 2 CTAs on each of the 148 SMs of a B200.  Constants of that chip, as are the
+// cluster counts in wide_tiling: a plan fixes the order of sums, which a model's results should not owe to the device asked.
 constexpr int kSms = 148;
 constexpr int kSlots = 2 * kSms;
 constexpr int kMinChunksPerSplit = 2;
@@ -197,34 +198,9 @@ inline int make_map(const void* ptr, uint64_t rows, uint64_t cols, uint64_t ld, 
   return BPD_OK;
 }
 
-// A general 2-D map (not cached): `rows` x `cols` elements of `elem_bytes` (2: bf16, 4: fp32) with `ld` elements
-// between rows, boxes of box_cols x box_rows, swizzle chosen by the box's inner extent in bytes (128 -> 128-byte
-// mode, 64 -> 64-byte mode, anything else -> none).
-inline int make_map_2d(const void* ptr, int elem_bytes, uint64_t rows, uint64_t cols, uint64_t ld, uint32_t box_cols,
-                       uint32_t box_rows, bool swizzle, CUtensorMap* out) {
-  if ((uintptr_t)ptr % 16 || (ld * elem_bytes) % 16) return fail(BPD_E_INVALID, "tensor-map operand is not 16-byte aligned");
-  if (box_rows < 1 || box_rows > 256 || box_cols < 1 || box_cols > 256) return fail(BPD_E_INVALID, "tensor-map box %u x %u", box_cols, box_rows);
-  EncodeTiledFn enc;
-  int rc = get_encode_fn(&enc);
-  if (rc) return rc;
-  const uint32_t inner = box_cols * (uint32_t)elem_bytes;
-  CUtensorMapSwizzle sw = CU_TENSOR_MAP_SWIZZLE_NONE;
-  if (swizzle && inner == 128) sw = CU_TENSOR_MAP_SWIZZLE_128B;
-  else if (swizzle && inner == 64) sw = CU_TENSOR_MAP_SWIZZLE_64B;
-  else if (swizzle) return fail(BPD_E_INVALID, "no swizzle mode for boxes of %u bytes per row", inner);
-  const cuuint64_t dims[2] = {cols, rows};
-  const cuuint64_t strides[1] = {ld * (uint64_t)elem_bytes};
-  const cuuint32_t box[2] = {box_cols, box_rows};
-  const cuuint32_t estr[2] = {1, 1};
-  CUresult r = enc(out, elem_bytes == 2 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2,
-                   const_cast<void*>(ptr), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, sw,
-                   CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  if (r != CUDA_SUCCESS) return fail(BPD_E_CUDA, "cuTensorMapEncodeTiled failed with code %d", (int)r);
-  return BPD_OK;
-}
-
-// The same over `layers` tensors that lie `layer_stride_bytes` apart: dimensions (columns, rows, layer), boxes of
-// box_cols x box_rows x 1.
+// A 3-D map (not cached): `layers` matrices of `rows` x `cols` elements of `elem_bytes` (2: bf16, 4: fp32), `ld` elements
+// between rows and `layer_stride_bytes` between matrices; boxes of box_cols x box_rows x 1, swizzle chosen by the box's
+// inner extent in bytes (128 -> 128-byte mode, 64 -> 64-byte mode).
 inline int make_map_3d(const void* ptr, int elem_bytes, uint64_t layers, uint64_t layer_stride_bytes, uint64_t rows, uint64_t cols,
                        uint64_t ld, uint32_t box_cols, uint32_t box_rows, bool swizzle, CUtensorMap* out) {
   if ((uintptr_t)ptr % 16 || (ld * elem_bytes) % 16 || layer_stride_bytes % 16)

@@ -195,9 +195,10 @@ def test_fp32_paths_keep_their_precision(bpd, batch, k, heads, max_src, tgt, opt
 
 
 # the persistent layer kernel with groups of sequences: a last group that is full and one that is not, two sequences per
-# group and one, one token tile and two, lengths up to the limit of 256 positions, one encoder row and 256
+# group and one, one token tile and two, lengths up to the limit of 256 positions, one encoder row and the most (a
+# multiple of 8) whose staging tile fits beside the working buffers of each shape: 136, 104 and 48
 @pytest.mark.parametrize("batch,k,heads,max_src,tgt", [(3, 4, 4, 61, 30), (8, 4, 4, 9, 251), (5, 3, 8, 1, 20), (2, 10, 8, 33, 40), (4, 16, 8, 24, 48),
-                                                       (9, 4, 4, 7, 12)])
+                                                       (9, 4, 4, 7, 12), (3, 4, 4, 136, 20), (5, 3, 8, 104, 20), (2, 10, 8, 48, 20)])
 def test_groups_of_sequences_decode_like_the_oracle(bpd, batch, k, heads, max_src, tgt):
     from bpd_inputs import ModelConfig, make_weights
     from oracle.decode import TransformerScorer
