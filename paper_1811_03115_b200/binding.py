@@ -318,18 +318,19 @@ def bpd_kernel_launches() -> int:
 _top1_scratch = {}      # (device, stream) -> scratch tensor, address, bytes: kept from call to call (see _scratch_for)
 
 
-def _scratch_for(device, stream: int, nbytes: int):
-    """A scratch of at least ``nbytes`` for calls on this device and stream (the current one).  Calls on one stream run
-    one after the other and each leaves the scratch cleared, so they may share it -- also when several threads enqueue
-    on the same stream.  At most 64 are kept.  A call that is being captured gets a scratch of its own out of the
-    graph's memory: a replay comes on any stream and long after the kept one has been replaced."""
-    import torch
-    if torch.cuda.is_current_stream_capturing():
+def _scratch_for(device, stream: int, nbytes: int, captured: bool):
+    """A scratch of at least ``nbytes`` for calls on this device and stream.  Calls on one stream run one after the other
+    and each leaves the scratch cleared, so they may share it -- also when several threads enqueue on the same stream.
+    At most 64 are kept.  A call that is being captured gets a scratch of its own out of the graph's memory: a replay
+    comes on any stream and long after the kept one has been replaced."""
+    if captured:
+        import torch
         t = torch.empty(nbytes, dtype=torch.uint8, device=device)
         return t, t.data_ptr(), nbytes
     key = (device, stream)
     have = _top1_scratch.get(key)
     if have is None or have[2] < nbytes:
+        import torch
         if len(_top1_scratch) >= 64:
             _top1_scratch.clear()
         t = torch.empty(nbytes, dtype=torch.uint8, device=device)
@@ -344,7 +345,9 @@ def bpd_op_vocab_argmax(x, w, want_val: bool = False):
     vocab = w.shape[0]
     dtype = 0 if x.dtype == torch.float32 else 1
     device, stream = x.device, _stream()
-    scratch = _scratch_for(device, stream, max(lib.bpd_op_vocab_argmax_scratch_bytes(rows, d, vocab, dtype), 256))
+    # (the bf16 call waits for its result: it cannot be captured)
+    scratch = _scratch_for(device, stream, max(lib.bpd_op_vocab_argmax_scratch_bytes(rows, d, vocab, dtype), 256),
+                           dtype == 0 and torch.cuda.is_current_stream_capturing())
     idx = torch.empty(rows, dtype=torch.int32, device=device)
     val = torch.empty(rows, dtype=torch.float32, device=device) if want_val else None
     _check(lib.bpd_op_vocab_argmax(x.data_ptr(), w.data_ptr(), rows, d, vocab, dtype, scratch[1], scratch[2],

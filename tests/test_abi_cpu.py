@@ -103,12 +103,10 @@ def test_top1_scratch_of_a_captured_call_is_its_own(lib, monkeypatch):
     """The kept scratch is replaced by a larger call's: a captured graph, which outlives that, must not point at it."""
     import torch
     monkeypatch.setattr(lib, "_top1_scratch", {})
-    monkeypatch.setattr(torch.cuda, "is_current_stream_capturing", lambda: False)
     cpu = torch.device("cpu")
-    kept = lib._scratch_for(cpu, 5, 512)
-    assert lib._scratch_for(cpu, 5, 256)[1] == kept[1]
-    monkeypatch.setattr(torch.cuda, "is_current_stream_capturing", lambda: True)
-    captured = lib._scratch_for(cpu, 5, 512)
+    kept = lib._scratch_for(cpu, 5, 512, False)
+    assert lib._scratch_for(cpu, 5, 256, False)[1] == kept[1]
+    captured = lib._scratch_for(cpu, 5, 512, True)
     assert captured[1] != kept[1] and captured[2] >= 512
-    larger = lib._scratch_for(cpu, 6, 1024)
+    larger = lib._scratch_for(cpu, 6, 1024, True)
     assert larger[2] >= 1024 and list(lib._top1_scratch) == [(cpu, 5)] and lib._top1_scratch[(cpu, 5)][1] == kept[1]
