@@ -104,7 +104,8 @@ typedef struct {
   int32_t dependent_launch;   /* programmatic dependent launch between the kernels of a pass               */
   int32_t lazy_heads;         /* two-stage heads: p_1 at all k positions, all heads only at the accepted
                                  one (default: on when batch * k_model >= 64)                              */
-  int32_t fold_layer_norms;   /* layer norms folded into the projections after them (encoder, and decoder) */
+  int32_t fold_layer_norms;   /* layer norms folded into the projections after them (decoder, and encoder;
+                                 default in the encoder: up to batch * max_src = 768)                      */
   int32_t cluster_layers;     /* decoder layers as three cluster launches each (<= 16 rows per pass)        */
   int32_t persistent_layers;  /* all decoder layers of a pass in one persistent TMA-fed kernel (<= 16 rows
                                  per pass, d_model 256 / 512 / 1024; takes precedence over cluster_layers).

@@ -1014,9 +1014,8 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
   k.p = &p;
   k.maps = &maps;
   // Two parameters that only the variants which split the keys need are constants in the others: there they cost variant 1
-  // 24 bytes of spills, 192.6 instead of 191.6 us for the six layers of a 16-head model and 1.8 % of its greedy decode
-  // (28930 / 28412 us), variant 4 1 % of a decode of five sentences (4631 / 4581 us).  As constants in variants 2 and 3 too:
-  // 4008 against 3971 us for a base sentence.
+  // 24 bytes of spills and variant 4 28.  Medians over 15 placements of the buffers (where they lie in memory moves a pass
+  // by up to 3 us): headline pass 330.1 -> 329.2 us, five base sentences 203.6 -> 203.1, one greedy row 218.2 -> 218.4.
   k.g = make_geo(p.d, p.H, p.ff, p.L, (LEAN == 1 || GROUPS || p.cross_staged) ? p.cross_rows : 0, SPLIT ? p.cross_split : 0);
   k.sm = ssm;
   k.ctl = reinterpret_cast<Ctl*>(ssm + p.lay.misc);
