@@ -9,7 +9,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB_PATH = os.path.join(HERE, "libbpd.so")
 OBJ_DIR = os.path.join(HERE, "build")
-SOURCES = ["layer_stack.cu", "fused_layer.cu", "gemm_tc.cu", "attention.cu", "bpd.cu", "noalloc.cu"]
+SOURCES = ["layer_stack.cu", "layer_stack_512.cu", "layer_stack_256.cu", "fused_layer.cu", "gemm_tc.cu", "attention.cu", "bpd.cu", "noalloc.cu"]
 
 
 def _nvcc() -> str:

@@ -845,9 +845,9 @@ static int stack_setup(bpd_session* s, bool try_groups) {
       lay.total += 1024;                       // slack for aligning the ring to 1024 bytes
       int n1 = 0, n2 = 0;
       const size_t sm = (size_t)lay.total;
-      const int ksteps = c.d == 256 ? 2 : 4, H = c.H;
-      BPD_TRY(stack_clusters(stack::kernel_for(1, ksteps, minb, lean), sm, H, &n1));
-      BPD_TRY(stack_clusters(stack::kernel_for(2, ksteps, minb, lean), sm, H, &n2));
+      const int H = c.H;
+      BPD_TRY(stack_clusters(stack::kernel_for(1, c.d, c.d_ff / c.H, minb, lean), sm, H, &n1));
+      BPD_TRY(stack_clusters(stack::kernel_for(2, c.d, c.d_ff / c.H, minb, lean), sm, H, &n2));
       const int need = std::max(1, groups) * c.H;
       ok = n1 >= need && n2 >= need;
     }
@@ -933,9 +933,8 @@ static int run_layers_stack(bpd_session* s, const PassArgs& a) {
   stack::StackMaps maps;
   memcpy(&maps, s->stack_maps, sizeof(maps));
   const size_t smem = (size_t)p.lay.total;
-  // reduction panels of 32 columns (two steps of 16) for d_model 256, else 64 (four steps); one or two CTAs per SM
-  const int nt = s->stack_group_seqs * a.kcur > 8 ? 2 : 1, ksteps = c.d == 256 ? 2 : 4;
-  const void* kernel = stack::kernel_for(nt, ksteps, s->stack_minb, s->stack_lean);
+  const int nt = s->stack_group_seqs * a.kcur > 8 ? 2 : 1;
+  const void* kernel = stack::kernel_for(nt, c.d, c.d_ff / c.H, s->stack_minb, s->stack_lean);
   if (!kernel) return fail(BPD_E_UNSUPPORTED, "no such instantiation of the persistent layer kernel");
   BPD_CUDA(launch_kc(kernel, grid, block, smem, s->stream, pdl, maps, p));
   ++g_launches;

@@ -257,6 +257,7 @@ struct Cta {                               // what the device functions below sh
   uint32_t ring;                           // shared-memory address of the ring
   int c, j, tid, warp, lane;
   int R;                                   // rows of this launch, or of this group
+  int d, H;
   unsigned long long policy;
 };
 
@@ -266,7 +267,7 @@ struct Cta {                               // what the device functions below sh
 __device__ __forceinline__ void pump(const Cta& k, int stop_before = 0x7fffffff) {
   Ctl* ctl = k.ctl;
   if (ctl->zombie) return;                 // nothing new goes into flight once a wait has expired
-  const int ring_bytes = k.p->lay.ring_bytes, total = min(k.g.total_tiles, stop_before), ntl = k.g.ntl, dmodel = k.p->d;
+  const int ring_bytes = k.p->lay.ring_bytes, total = min(k.g.total_tiles, stop_before), ntl = k.g.ntl, dmodel = k.d;
   int issued = ctl->issued, head = ctl->head, idx = ctl->issue_idx, layer = ctl->issue_layer;
   const int freed = ctl->freed;
   int tail = ctl->off[freed & (kNB - 1)];
@@ -377,7 +378,7 @@ __device__ __forceinline__ Words load_words(const Cta& k, const bf16* v) {
 __device__ __forceinline__ void reduce_slice(const Cta& k, float* x_s, const unsigned long long* ws, const Words& bias,
                                              unsigned tag, int nfree) {
   const StackParams& p = *k.p;
-  const int ks = k.g.ks, n4 = ks >> 2, R = k.R, d = p.d, H = p.H;
+  const int ks = k.g.ks, n4 = ks >> 2, R = k.R, d = k.d, H = k.H;
   __syncthreads();                                             // every warp is done with the tiles released here
   if (k.tid == kPumpThread && nfree) release_tiles(k, nfree);
 #pragma unroll
@@ -451,8 +452,7 @@ __device__ __forceinline__ bool ll_wait4(const Cta& k, const unsigned long long*
 }
 __device__ __forceinline__ void reduce_slice_2hop(const Cta& k, float* x_s, const unsigned long long* ws, unsigned long long* gather,
                                                   const Words& bias, unsigned tag, int nfree) {
-  const StackParams& p = *k.p;
-  const int ks = k.g.ks, n4 = ks >> 2, R = k.R, d = p.d, H = p.H, j = blockIdx.y;
+  const int ks = k.g.ks, n4 = ks >> 2, R = k.R, d = k.d, H = k.H, j = blockIdx.y;
   __syncthreads();                                             // every warp is done with the tiles released here
   if (k.tid == kPumpThread && nfree) release_tiles(k, nfree);
   const int ipp = (R * n4) / H;                                // items of a part: n4 = 2H, so 2R
@@ -756,7 +756,7 @@ __device__ __forceinline__ int long_pos(const LongCtx& lc, int i) { return ((lc.
 // Committed keys and values of this rank's keys i0 .. i0 + KW - 1 on their way into shared memory.
 template <int KW>
 __device__ __forceinline__ void long_prefetch(const Cta& k, const LongCtx& lc, const LayerPtrs& LP, int i0) {
-  const int n = min(KW, lc.n_my * 32 - i0), d = k.p->d;
+  const int n = min(KW, lc.n_my * 32 - i0), d = k.d;
   const uint32_t ks = tc::smem_u32(lc.kb), vs = tc::smem_u32(lc.vb);
   for (int w = k.tid; w < n * 8; w += kThreads) {
     const int i = w >> 3, piece = w & 7, pos = long_pos(lc, i0 + i);
@@ -914,7 +914,7 @@ __device__ __forceinline__ void long_cross_attention(const Cta& k, const LongCtx
   for (int n0 = warp * 8; n0 < nk16; n0 += 64) {
     float c[4][4] = {};
     const int row = min(n0 + g, rows - 1);                 // rows beyond the last repeat it with weight 0
-    const float* unstaged = LP.crosskv + (size_t)min(first + row, k.p->max_src - 1) * (2 * k.p->d) + k.j * kDH;
+    const float* unstaged = LP.crosskv + (size_t)min(first + row, k.p->max_src - 1) * (2 * k.d) + k.j * kDH;
 #pragma unroll
     for (int kk = 0; kk < 4; ++kk) {
       const uint8_t* base = kk < 2 ? k0t : k1t;
@@ -944,7 +944,7 @@ __device__ __forceinline__ void long_cross_attention(const Cta& k, const LongCtx
     auto at = [&](int r) {
       const int row = min(k0 + r, rows - 1), dim = warp * 8 + g;
       if (k.g.staged) return *reinterpret_cast<const float*>(vt + (size_t)row * 256 + dim * 4);
-      return LP.crosskv[(size_t)min(first + row, k.p->max_src - 1) * (2 * k.p->d) + k.p->d + k.j * kDH + dim];
+      return LP.crosskv[(size_t)min(first + row, k.p->max_src - 1) * (2 * k.d) + k.d + k.j * kDH + dim];
     };
     attn::split3_pair(at(t4 * 2), at(t4 * 2 + 1), b0);
     attn::split3_pair(at(t4 * 2 + 8), at(t4 * 2 + 9), b1);
@@ -981,7 +981,7 @@ __device__ __forceinline__ void share_states(const Cta& k, int n, float* lvl2, u
 
 // ------------------------------------------------------------------ development trace
 #ifdef BPD_STACK_TRACE
-__device__ unsigned long long* g_stack_trace = nullptr;
+static __device__ unsigned long long* g_stack_trace = nullptr;
 constexpr int kTracePts = 256;
 #define BPD_TR() do { if (g_stack_trace && tid == 0 && tp < kTracePts - 4) { unsigned long long t_; asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t_)); \
                         g_stack_trace[(size_t)(blockIdx.y * kC + c) * kTracePts + tp] = t_; } ++tp; } while (0)
@@ -1000,23 +1000,29 @@ constexpr int kTracePts = 256;
 // LEAN = 4: the short variant for more sequences than one set of H clusters takes.  The grid's z slices are groups of H
 // clusters that work on a few sequences each (at most 8 rows, or one sequence) and know nothing of one another: shares,
 // tags and rows of their own.  A rank then attends for rows of one sequence only and stages just that one's encoder rows.
-template <int NT, int KS, int MINB, int LEAN>
+// NT: token tiles of eight rows; D: d_model; HCT: hidden units per cluster.  With the model's shape as constants the offsets and
+// masks of every step fold into its instructions, and what decides between shapes is gone: with few dependent
+// instructions between any two waits that is what a step's time is made of.  us per pass, shape in registers / d_model
+// constant / hidden units too: big model, block of 8 rows 318.4 / 307.9 / 302.0, one row 220 / 215 / 201; base model 165.0 / 150.6 /
+// 146.7 and 155.8 / 140.3 / 136.7; five base sentences 205 / 174 / 175.5; 1000 intensities 235 / 217 / 214.
+template <int NT, int D, int HCT, int MINB, int LEAN>
 __global__ void __cluster_dims__(kC, 1, 1) __launch_bounds__(kThreads, MINB)
 layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant__ StackParams p) {
   extern __shared__ __align__(1024) uint8_t ssm_raw[];
   // swizzled tiles need 1024-byte alignment (the launch carries 1024 bytes of slack for this)
   uint8_t* ssm = ssm_raw + ((1024u - (tc::smem_u32(ssm_raw) & 1023u)) & 1023u);
   cg::cluster_group cluster = cg::this_cluster();
-  constexpr int RP = NT * 8;
+  constexpr int RP = NT * 8, H = D / kDH, KS = D == 256 ? 2 : 4;      // steps of 16 columns per panel
   constexpr bool GROUPS = LEAN == 4;
   constexpr bool SPLIT = LEAN == 2 || LEAN == 3;         // keys split over the ranks
   Cta k;
   k.p = &p;
+  k.d = D; k.H = H;
   k.maps = &maps;
   // Two parameters that only the variants which split the keys need are constants in the others: there they cost variant 1
   // 24 bytes of spills and variant 4 28.  Medians over 15 placements of the buffers (where they lie in memory moves a pass
   // by up to 3 us): headline pass 330.1 -> 329.2 us, five base sentences 203.6 -> 203.1, one greedy row 218.2 -> 218.4.
-  k.g = make_geo(p.d, p.H, p.ff, p.L, (LEAN == 1 || GROUPS || p.cross_staged) ? p.cross_rows : 0, SPLIT ? p.cross_split : 0);
+  k.g = make_geo(D, H, HCT * H, p.L, (LEAN == 1 || GROUPS || p.cross_staged) ? p.cross_rows : 0, SPLIT ? p.cross_split : 0);
   k.sm = ssm;
   k.ctl = reinterpret_cast<Ctl*>(ssm + p.lay.misc);
   k.ring = tc::smem_u32(ssm);
@@ -1029,9 +1035,10 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
   const Geo& g = k.g;
   const int c = k.c, j = k.j, tid = k.tid, warp = k.warp, lane = k.lane;
   const int grp = GROUPS ? (int)blockIdx.z : 0, b0 = GROUPS ? grp * p.group_seqs : 0;
-  const int d = p.d, ks = g.ks, rpb = p.rows_per_b, nb = GROUPS ? min(p.group_seqs, p.nb - b0) : p.nb, R = GROUPS ? nb * rpb : p.R;
+  constexpr int d = D;
+  const int ks = g.ks, rpb = p.rows_per_b, nb = GROUPS ? min(p.group_seqs, p.nb - b0) : p.nb, R = GROUPS ? nb * rpb : p.R;
   k.R = R;
-  unsigned long long* const ws_g = p.ws + (GROUPS ? (size_t)grp * 2 * p.H * kMaxRows * d : 0);
+  unsigned long long* const ws_g = p.ws + (GROUPS ? (size_t)grp * 2 * H * kMaxRows * d : 0);
   unsigned long long* const gather_g = p.gather + (GROUPS ? (size_t)grp * 2 * kMaxRows * d : 0);
   const int lg = lane >> 2, t4 = lane & 3;
   float* x_s = reinterpret_cast<float*>(ssm + p.lay.x);
@@ -1128,7 +1135,7 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
 
   AttnParams ap;
   memset(&ap, 0, sizeof(ap));
-  ap.rows = R; ap.rows_per_b = rpb; ap.H = p.H; ap.dh = kDH; ap.causal = 1; ap.local_q = p.local_q; ap.local_m = p.local_m;
+  ap.rows = R; ap.rows_per_b = rpb; ap.H = H; ap.dh = kDH; ap.causal = 1; ap.local_q = p.local_q; ap.local_m = p.local_m;
   ap.ldkv = d; ap.paged = 1; ap.st = p.st; ap.st.page_table = s_pt; ap.scale = p.scale;
   bool one_chunk_per_rank = true;
   if (LEAN == 0) {
@@ -1179,8 +1186,8 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
       const Words bw = load_words(k, layers_s[l - 1].b2);
       ++nbar;
       BPD_TR();
-      if (p.H == 16) reduce_slice_2hop(k, x_s, ws_g + (size_t)((nbar - 1) & 1) * p.H * kMaxRows * d, gather_g + (size_t)((nbar - 1) & 1) * kMaxRows * d, bw, base + nbar, g.PH);
-      else reduce_slice(k, x_s, ws_g + (size_t)((nbar - 1) & 1) * p.H * kMaxRows * d, bw, base + nbar, g.PH);
+      if constexpr (H == 16) reduce_slice_2hop(k, x_s, ws_g + (size_t)((nbar - 1) & 1) * H * kMaxRows * d, gather_g + (size_t)((nbar - 1) & 1) * kMaxRows * d, bw, base + nbar, g.PH);
+      else reduce_slice(k, x_s, ws_g + (size_t)((nbar - 1) & 1) * H * kMaxRows * d, bw, base + nbar, g.PH);
       BPD_TR();
       if (p.layer_dump && j == 0) {
         __syncthreads();
@@ -1344,7 +1351,7 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
     BPD_TR();
     // this head's share of the output projection for feature slice c
     {
-      unsigned long long* wsj = ws_g + ((size_t)(nbar & 1) * p.H + j) * kMaxRows * d;
+      unsigned long long* wsj = ws_g + ((size_t)(nbar & 1) * H + j) * kMaxRows * d;
       const unsigned tag_out = base + nbar + 1;            // the reduction that consumes these shares
       for (int mt = warp; mt < ks / 16; mt += kWarps) {
         float acc[NT][4];
@@ -1371,8 +1378,8 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
     if (tid < kDH) { fs = LP.s_cq[j * kDH + tid]; fc = LP.c_cq[j * kDH + tid]; }
     ++nbar;
     BPD_TR();
-    if (p.H == 16) reduce_slice_2hop(k, x_s, ws_g + (size_t)((nbar - 1) & 1) * p.H * kMaxRows * d, gather_g + (size_t)((nbar - 1) & 1) * kMaxRows * d, nobias, base + nbar, 1);
-      else reduce_slice(k, x_s, ws_g + (size_t)((nbar - 1) & 1) * p.H * kMaxRows * d, nobias, base + nbar, 1);
+    if constexpr (H == 16) reduce_slice_2hop(k, x_s, ws_g + (size_t)((nbar - 1) & 1) * H * kMaxRows * d, gather_g + (size_t)((nbar - 1) & 1) * kMaxRows * d, nobias, base + nbar, 1);
+      else reduce_slice(k, x_s, ws_g + (size_t)((nbar - 1) & 1) * H * kMaxRows * d, nobias, base + nbar, 1);
     BPD_TR();
     planes_and_stats<NT>(k, x_s, gw, xh, xl, stats_mine);
     __syncthreads();
@@ -1454,7 +1461,7 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
     ++xn;
     BPD_TR();
     {
-      unsigned long long* wsj = ws_g + ((size_t)(nbar & 1) * p.H + j) * kMaxRows * d;
+      unsigned long long* wsj = ws_g + ((size_t)(nbar & 1) * H + j) * kMaxRows * d;
       const unsigned tag_out = base + nbar + 1;            // the reduction that consumes these shares
       for (int mt = warp; mt < ks / 16; mt += kWarps) {
         float acc[NT][4];
@@ -1487,8 +1494,8 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
     }
     ++nbar;
     BPD_TR();
-    if (p.H == 16) reduce_slice_2hop(k, x_s, ws_g + (size_t)((nbar - 1) & 1) * p.H * kMaxRows * d, gather_g + (size_t)((nbar - 1) & 1) * kMaxRows * d, nobias, base + nbar, 1);
-      else reduce_slice(k, x_s, ws_g + (size_t)((nbar - 1) & 1) * p.H * kMaxRows * d, nobias, base + nbar, 1);
+    if constexpr (H == 16) reduce_slice_2hop(k, x_s, ws_g + (size_t)((nbar - 1) & 1) * H * kMaxRows * d, gather_g + (size_t)((nbar - 1) & 1) * kMaxRows * d, nobias, base + nbar, 1);
+      else reduce_slice(k, x_s, ws_g + (size_t)((nbar - 1) & 1) * H * kMaxRows * d, nobias, base + nbar, 1);
     BPD_TR();
     planes_and_stats<NT>(k, x_s, gw, xh, xl, stats_mine);
     __syncthreads();
@@ -1546,7 +1553,7 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
     BPD_TR();
     // the hidden units times slice c of the second projection: this cluster's share of the block's output
     {
-      unsigned long long* wsj = ws_g + ((size_t)(nbar & 1) * p.H + j) * kMaxRows * d;
+      unsigned long long* wsj = ws_g + ((size_t)(nbar & 1) * H + j) * kMaxRows * d;
       const unsigned tag_out = base + nbar + 1;            // the reduction that consumes these shares
       for (int mt = warp; mt < ks / 16; mt += kWarps) {
         float acc[NT][4];
@@ -1584,8 +1591,8 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
     ++nbar;
     BPD_TR();
     pdl_launch_dependents();
-    if (p.H == 16) reduce_slice_2hop(k, x_s, ws_g + (size_t)((nbar - 1) & 1) * p.H * kMaxRows * d, gather_g + (size_t)((nbar - 1) & 1) * kMaxRows * d, bw, base + nbar, g.PH);
-      else reduce_slice(k, x_s, ws_g + (size_t)((nbar - 1) & 1) * p.H * kMaxRows * d, bw, base + nbar, g.PH);
+    if constexpr (H == 16) reduce_slice_2hop(k, x_s, ws_g + (size_t)((nbar - 1) & 1) * H * kMaxRows * d, gather_g + (size_t)((nbar - 1) & 1) * kMaxRows * d, bw, base + nbar, g.PH);
+      else reduce_slice(k, x_s, ws_g + (size_t)((nbar - 1) & 1) * H * kMaxRows * d, bw, base + nbar, g.PH);
     BPD_TR();
     if (p.layer_dump && j == 0) {
       __syncthreads();
@@ -1642,10 +1649,23 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
   cluster.sync();
 }
 
-// The kernel's instantiations (layer_stack.cu): token tiles (1 or 2 of 8 rows), reduction steps per panel (2: d_model
-// 256, else 4), CTAs per SM (1 or 2), variant (LEAN, see the kernel: 0 general, 1 short sequences with staged encoder
-// rows, 2 one long sequence, 3 one short sequence, 4 groups of sequences); null if there is none.
-const void* kernel_for(int nt, int ksteps, int minb, int lean);
+// The kernel's instantiations: token tiles (1 or 2 of 8 rows), d_model, hidden units per cluster (128 or 256), CTAs per SM
+// (1 or 2), variant (LEAN, see the kernel: 0 general, 1 short sequences with staged encoder rows, 2 one long sequence,
+// 3 one short sequence, 4 groups of sequences); null if there is none.  One translation unit per d_model
+// (layer_stack.cu, layer_stack_512.cu, layer_stack_256.cu), compiled side by side.
+const void* kernel_for(int nt, int d, int hct, int minb, int lean);
+template <int D> const void* kernel_of(int nt, int hct, int minb, int lean);
+#define BPD_STACK_V(D, NT, MB, LN) \
+  if (nt == NT && hct == 128 && minb == MB && lean == LN) return reinterpret_cast<const void*>(layer_stack_kernel<NT, D, 128, MB, LN>); \
+  if (nt == NT && hct == 256 && minb == MB && lean == LN) return reinterpret_cast<const void*>(layer_stack_kernel<NT, D, 256, MB, LN>)
+#define BPD_STACK_KERNELS(D) \
+  template <> const void* kernel_of<D>(int nt, int hct, int minb, int lean) { \
+    BPD_STACK_V(D, 1, 1, 0); BPD_STACK_V(D, 2, 1, 0); BPD_STACK_V(D, 1, 2, 0); BPD_STACK_V(D, 2, 2, 0); \
+    BPD_STACK_V(D, 1, 1, 1); BPD_STACK_V(D, 2, 1, 1); BPD_STACK_V(D, 1, 2, 1); BPD_STACK_V(D, 2, 2, 1); \
+    BPD_STACK_V(D, 1, 1, 2); BPD_STACK_V(D, 2, 1, 2); BPD_STACK_V(D, 1, 1, 3); BPD_STACK_V(D, 2, 1, 3); \
+    BPD_STACK_V(D, 1, 2, 4); BPD_STACK_V(D, 2, 2, 4); \
+    return nullptr; \
+  }
 
 }  // namespace stack
 }  // namespace bpd

@@ -1,0 +1,11 @@
+// The persistent layer kernel for d_model 256.
+#include "host.hpp"
+#include "layer_stack.cuh"
+
+namespace bpd {
+namespace stack {
+
+BPD_STACK_KERNELS(256)
+
+}  // namespace stack
+}  // namespace bpd
