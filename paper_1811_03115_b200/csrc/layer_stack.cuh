@@ -182,6 +182,7 @@ struct Ctl {
   int off[kNB];                            // ring offset of the tile in that slot
   int head, issued, freed, zombie;
   int issue_layer, issue_idx;              // layer and index within the layer of the next tile to request
+  int tok_b[2], tok_i[2], tok_at[2];       // this rank's tokens: sequence, place in the block, physical cache row of its key and value
   TileDesc tiles[kMaxTiles];
 #ifdef BPD_STACK_TRACE
   long long cyc_wait, cyc_pump, cyc_poll;   // thread 0: cycles spent waiting for tiles, requesting tiles, polling the join
@@ -323,8 +324,9 @@ __device__ __forceinline__ uint32_t tile_wait(const Cta& k, int seq) {
 #ifdef BPD_STACK_TRACE
   const long long t0 = clock64();
 #endif
-  if (!is_zombie(k)) {
-    if (!tc::mbar_wait(tc::smem_u32(&k.ctl->full[slot]), (uint32_t)(seq / kNB) & 1u, k.p->spin)) raise_abort(k, 105);
+  const uint32_t bar = tc::smem_u32(&k.ctl->full[slot]), phase = (uint32_t)(seq / kNB) & 1u;
+  if (!tc::mbar_try_wait(bar, phase) && !is_zombie(k)) {       // mostly there: the common case looks at nothing else
+    if (!tc::mbar_wait(bar, phase, k.p->spin)) raise_abort(k, 105);
   }
 #ifdef BPD_STACK_TRACE
   if (k.tid == 0) k.ctl->cyc_wait += clock64() - t0;
@@ -344,8 +346,9 @@ __device__ __forceinline__ void xchg_send(const Cta& k, int n, int rank, const v
 }
 // All threads: wait for everything exchange n brings.
 __device__ __forceinline__ void xchg_wait(const Cta& k, int n) {
-  if (!is_zombie(k)) {
-    if (!tc::mbar_wait(tc::smem_u32(&k.ctl->ex[n & 1]), (uint32_t)(n >> 1) & 1u, k.p->spin)) raise_abort(k, 106);
+  const uint32_t bar = tc::smem_u32(&k.ctl->ex[n & 1]), phase = (uint32_t)(n >> 1) & 1u;
+  if (!tc::mbar_try_wait(bar, phase) && !is_zombie(k)) {
+    if (!tc::mbar_wait(bar, phase, k.p->spin)) raise_abort(k, 106);
   }
 }
 
@@ -575,42 +578,58 @@ __device__ __forceinline__ void merge_stats(const Cta& k, const float* stats_in,
   }
 }
 
-// ------------------------------------------------------------------ cross-attention over a staged tile
-// Keys: two boxes [rows][32 floats] in the 128-byte swizzle (lane = key reads 16 bytes per step without bank
-// conflicts); values: [rows][64 floats] as they are.  Warp w folds chunks w, w + 8, ... of 32 positions in order,
-// the warps' states are merged in warp order.  Threads c < kDH return output element c.
-__device__ __forceinline__ float cross_attention_tile(const uint8_t* k0, const uint8_t* k1, const uint8_t* vv, int row0,
-                                                      int limit, AttnSmem<kDH, kWarps>& sm) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+// ------------------------------------------------------------------ cross-attention
+// Keys: two boxes [rows][32 floats] in the 128-byte swizzle; values: [rows][64 floats] as they are.  Warp w folds chunks w,
+// w + 8, ... of 8 positions in order, four lanes to a key: chunks of 32 with a lane to a key kept one or two of the eight
+// warps busy at the usual source lengths, each with a chain of 64 products.  The warps' states are merged in warp
+// order.  Threads c < kDH return output element c.  (Base model's layers: with this, one wait per panel and the constant sizes of
+// send_rows 146.9 -> 144.1 us per pass, five sentences 173.4 -> 166.2, 1000 intensities 213.2 -> 209.4; big model 306.4 / 306.7.)
+// TILE = false: sources that are not staged; the rows come out of L2 (`rows`: the sequence's first key of this head, its value
+// d elements behind, 2 d elements between rows), the same arithmetic in the same order.
+template <bool TILE>
+__device__ __forceinline__ float cross_attention(const uint8_t* k0, const uint8_t* k1, const uint8_t* vv, int row0, const float* rows, int d_model,
+                                                 int limit, AttnSmem<kDH, kWarps>& sm) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, quarter = lane & 3, own = lane >> 2;
   float m_run = -INFINITY, l_run = 0.f, a0 = 0.f, a1 = 0.f;
-  for (int c0 = warp * 32; c0 < limit; c0 += kWarps * 32) {
-    const int nk = min(32, limit - c0);
-    float sc = -INFINITY;
-    if (lane < nk) {
-      const uint32_t row = (uint32_t)(row0 + c0 + lane) * 128;
-      const float4* qv = reinterpret_cast<const float4*>(sm.q);
-      float dot = 0.f;
+  // this lane's sixteen dimensions of the query: pieces quarter, quarter + 4, ... of four
+  float4 q4[4];
 #pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const float4 k4 = *reinterpret_cast<const float4*>(k0 + swz(row + u * 16, 7u)), q4 = qv[u];
-        dot = fmaf(q4.x, k4.x, dot); dot = fmaf(q4.y, k4.y, dot); dot = fmaf(q4.z, k4.z, dot); dot = fmaf(q4.w, k4.w, dot);
-      }
+  for (int u = 0; u < 4; ++u) q4[u] = reinterpret_cast<const float4*>(sm.q)[quarter + 4 * u];
+#pragma unroll 1
+  for (int c0 = warp * 8; c0 < limit; c0 += kWarps * 8) {
+    const int nk = min(8, limit - c0);
+    const int key = c0 + min(own, nk - 1);
+    const uint32_t row = (uint32_t)(row0 + key) * 128;
+    float d[4];
 #pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const float4 k4 = *reinterpret_cast<const float4*>(k1 + swz(row + u * 16, 7u)), q4 = qv[8 + u];
-        dot = fmaf(q4.x, k4.x, dot); dot = fmaf(q4.y, k4.y, dot); dot = fmaf(q4.z, k4.z, dot); dot = fmaf(q4.w, k4.w, dot);
-      }
-      sc = dot;
+    for (int u = 0; u < 4; ++u) {
+      const float4 k4 = TILE ? *reinterpret_cast<const float4*>((u < 2 ? k0 : k1) + swz(row + (quarter + 4 * (u & 1)) * 16, 7u))
+                             : __ldcg(reinterpret_cast<const float4*>(rows + (size_t)key * (2 * d_model)) + quarter + 4 * u);
+      d[u] = fmaf(q4[u].w, k4.w, fmaf(q4[u].z, k4.z, fmaf(q4[u].y, k4.y, q4[u].x * k4.x)));
     }
-    const float m_new = fmaxf(m_run, warp_max(sc));
+    float dot = (d[0] + d[1]) + (d[2] + d[3]);
+    dot += __shfl_xor_sync(0xffffffffu, dot, 1);
+    dot += __shfl_xor_sync(0xffffffffu, dot, 2);
+    const float sc = own < nk ? dot : -INFINITY;
+    float top = fmaxf(sc, __shfl_xor_sync(0xffffffffu, sc, 4));
+    top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, 8));
+    top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, 16));
+    const float m_new = fmaxf(m_run, top);
     const float corr = expf(m_run - m_new);
-    const float pj = (lane < nk) ? expf(sc - m_new) : 0.f;
-    l_run = l_run * corr + warp_sum(pj);
+    const float pj = own < nk ? expf(sc - m_new) : 0.f;
+    float sum = pj + __shfl_xor_sync(0xffffffffu, pj, 4);
+    sum += __shfl_xor_sync(0xffffffffu, sum, 8);
+    sum += __shfl_xor_sync(0xffffffffu, sum, 16);
+    l_run = fmaf(l_run, corr, sum);
     a0 *= corr;
     a1 *= corr;
-    for (int jj = 0; jj < nk; ++jj) {
-      const float pw = __shfl_sync(0xffffffffu, pj, jj);
-      const float2 v2 = *reinterpret_cast<const float2*>(vv + (size_t)(row0 + c0 + jj) * 256 + lane * 8);
+    const uint8_t* vr = vv + (size_t)(row0 + c0) * 256 + lane * 8;
+#pragma unroll
+    for (int jj = 0; jj < 8; ++jj) {
+      const float pw = __shfl_sync(0xffffffffu, pj, 4 * jj);
+      const int r = min(jj, nk - 1);                         // rows beyond the last repeat it with weight 0
+      const float2 v2 = TILE ? *reinterpret_cast<const float2*>(vr + r * 256)
+                             : __ldcg(reinterpret_cast<const float2*>(rows + (size_t)(c0 + r) * (2 * d_model) + d_model) + lane);
       a0 = fmaf(pw, v2.x, a0);
       a1 = fmaf(pw, v2.y, a1);
     }
@@ -690,24 +709,25 @@ __device__ __forceinline__ void chunk_fetch_mixed(const bf16* Kc, const bf16* Vc
 // thread, straight out of this CTA's rows, no staging fence) arrive sooner than bulk copies set up for so little --
 // measured on the headline shape: 0.3-0.5 us per exchange.  The larger exchanges (partial sums, hidden units: up to
 // a kilobyte per destination) stay bulk copies: as per-thread stores they measured slower.
-template <int NT>
-__device__ __forceinline__ void send_rows(const Cta& k, int n, uint8_t* buf0, uint8_t* buf1, uint32_t row_bytes, int nfree) {
+template <int NT, int ROW_BYTES, bool TWO>
+__device__ __forceinline__ void send_rows(const Cta& k, int n, uint8_t* buf0, uint8_t* buf1, int nfree) {
+  constexpr int PPR = ROW_BYTES >> 4, PPD = PPR * (TWO ? 2 : 1);           // 16-byte pieces per row, per destination
+  static_assert((kC - 1) * PPD <= kThreads, "one piece per thread");
   __syncthreads();
   if (k.tid == kPumpThread && nfree) release_tiles(k, nfree);   // behind the barrier: every warp is done with those tiles
   int mine = 0;
 #pragma unroll
   for (int slot = 0; slot < NT; ++slot) mine += (slot * kC + k.c < k.R) ? 1 : 0;
-  if (k.tid == 0) xchg_expect(k, n, (uint32_t)(k.R - mine) * row_bytes * (buf1 ? 2u : 1u));
-  if (!is_zombie(k)) {                     // after an expired wait nothing new goes into flight
-    const int ppr = (int)(row_bytes >> 4), per_dst = mine * ppr * (buf1 ? 2 : 1);
-    const uint32_t bar = tc::smem_u32(&k.ctl->ex[n & 1]);
-    for (int idx = k.tid; idx < (kC - 1) * per_dst; idx += kThreads) {
-      const int di = idx / per_dst, piece = idx - di * per_dst, rank = di < k.c ? di : di + 1;
-      const int pb = piece / ppr, off = (piece - pb * ppr) << 4;           // (row, buffer) pair and byte offset in the row
-      const int slot = buf1 ? pb >> 1 : pb;
-      uint8_t* at = ((buf1 && (pb & 1)) ? buf1 : buf0) + (slot * kC + k.c) * row_bytes + off;
-      dsmem_store16(map_rank(tc::smem_u32(at), rank), *reinterpret_cast<const uint4*>(at), map_rank(bar, rank));
-    }
+  if (k.tid == 0) xchg_expect(k, n, (uint32_t)(k.R - mine) * (ROW_BYTES * (TWO ? 2u : 1u)));
+  if (k.tid < (kC - 1) * PPD && !is_zombie(k)) {                // after an expired wait nothing new goes into flight
+    const int di = k.tid / PPD, piece = k.tid % PPD, rank = di < k.c ? di : di + 1;
+    const uint32_t bar = map_rank(tc::smem_u32(&k.ctl->ex[n & 1]), rank);
+#pragma unroll
+    for (int slot = 0; slot < NT; ++slot)
+      if (slot * kC + k.c < k.R) {
+        uint8_t* at = ((TWO && piece >= PPR) ? buf1 : buf0) + (slot * kC + k.c) * ROW_BYTES + (piece % PPR) * 16;
+        dsmem_store16(map_rank(tc::smem_u32(at), rank), *reinterpret_cast<const uint4*>(at), bar);
+      }
   }
   xchg_wait(k, n);
 }
@@ -1013,6 +1033,8 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
   uint8_t* ssm = ssm_raw + ((1024u - (tc::smem_u32(ssm_raw) & 1023u)) & 1023u);
   cg::cluster_group cluster = cg::this_cluster();
   constexpr int RP = NT * 8, H = D / kDH, KS = D == 256 ? 2 : 4;      // steps of 16 columns per panel
+  constexpr int kPanels = D / kC <= 64 ? 1 : D / kC / 64;             // panels of a rank's columns
+  constexpr bool kHoist = kPanels == 1;      // wait for a panel once, not once per row tile (two panels cost more registers than the waits)
   constexpr bool GROUPS = LEAN == 4;
   constexpr bool SPLIT = LEAN == 2 || LEAN == 3;         // keys split over the ranks
   Cta k;
@@ -1130,6 +1152,11 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
       *reinterpret_cast<float4*>(x_s + t * ks + c4 * 4) = v;
     }
   }
+  if (tid < NT) {
+    const int token = min(tid * kC + c, R - 1), b = token / rpb, i = token - b * rpb, pos = s_len[b] + i;
+    k.ctl->tok_b[tid] = b; k.ctl->tok_i[tid] = i;
+    k.ctl->tok_at[tid] = s_pt[b * p.st.pages_per_row + pos / kPage] * kPage + pos % kPage;
+  }
   fused::cluster_arrive();
   fused::cluster_wait();                    // every CTA of the cluster runs: its shared memory and mbarriers may be written
 
@@ -1199,12 +1226,15 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
     __syncthreads();
     BPD_TR();
     // Q, K, V of the head over this rank's columns; token t's partial goes to rank t % 8
+    uint32_t wt[kPanels];
+#pragma unroll
+    for (int q = 0; q < kPanels; ++q) wt[q] = kHoist ? tile_wait(k, seq + q) : 0u;
     for (int mt = warp; mt < 3 * kDH / 16; mt += kWarps) {
       float acc[NT][4];
 #pragma unroll
       for (int nt = 0; nt < NT; ++nt) acc[nt][0] = acc[nt][1] = acc[nt][2] = acc[nt][3] = 0.f;
-      for (int q = 0; q < g.P; ++q) {
-        const uint32_t a = tile_wait(k, seq + q) + ((mt / 4) * 64 + (mt % 4) * 16) * xrow, b = x_plane + q * RP * xrow;
+      for (int q = 0; q < kPanels; ++q) {
+        const uint32_t a = (kHoist ? wt[q] : tile_wait(k, seq + q)) + mt * 16 * xrow, b = x_plane + q * RP * xrow;
 #pragma unroll
         for (int kk = 0; kk < KS; ++kk) mma_step<NT>(acc, a + (ax_pre ^ (kk << 5)), b + (bx_pre ^ (kk << 5)), 8 * xrow);
       }
@@ -1225,6 +1255,7 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
     __syncthreads();
     // this rank's tokens: partials in rank order, layer norm; the row's key and value (rounded as the cache holds
     // them) go into the cache for later passes and, with the scaled query, into this rank's copy of the block's rows
+#pragma unroll
     for (int slot = 0; slot < NT; ++slot) {
       const int token = slot * kC + c;
       if (token < R && tid < 3 * kDH) {
@@ -1237,17 +1268,13 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
         if (sect == 0) {
           reinterpret_cast<float*>(row + 256)[f] = y * p.scale;
         } else {
-          const int b = token / rpb, i = token % rpb;
-          const int pos = s_len[b] + i;
-          const int page = s_pt[b * p.st.pages_per_row + pos / kPage];
-          const size_t at = ((size_t)page * kPage + (pos % kPage)) * d + j * kDH + f;
           const bf16 yb = __float2bfloat16_rn(y);
-          (sect == 1 ? LP.kcache : LP.vcache)[at] = yb;
+          (sect == 1 ? LP.kcache : LP.vcache)[(size_t)k.ctl->tok_at[slot] * d + j * kDH + f] = yb;
           reinterpret_cast<bf16*>(row + (sect - 1) * 128)[f] = yb;
         }
       }
     }
-    send_rows<NT>(k, xn, kvq, nullptr, 512, 0);  // every rank now holds the keys, values and queries of all block rows
+    send_rows<NT, 512, false>(k, xn, kvq, nullptr, 0);  // every rank now holds the keys, values and queries of all block rows
     ++xn;
     BPD_TR();
     {
@@ -1261,10 +1288,11 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
         ++xn;
       } else if (LEAN == 1 || GROUPS || one_chunk_per_rank) {
         // this rank attends for its own rows; warp w folds the chunk that belongs to rank w
+#pragma unroll
         for (int slot = 0; slot < NT; ++slot) {
           const int token = slot * kC + c;
           if (token < R) {                                           // uniform over the CTA
-            const int b = token / rpb, i = token % rpb;
+            const int b = k.ctl->tok_b[slot], i = k.ctl->tok_i[slot];
             const int len = s_len[b], lim_max = len + rpb;
             const int fk = attn_first_key(ap, len + i), ch0 = attn_first_key(ap, len) >> 5;
             const int ch = ch0 + ((warp - ch0) & (kC - 1));
@@ -1288,7 +1316,7 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
             }
           }
         }
-        send_rows<NT>(k, xn, oh, ol, 128, 0);
+        send_rows<NT, 128, true>(k, xn, oh, ol, 0);
         ++xn;
       } else {
         // long sequences: rank c folds its own chunks for every row (keys fetched once per sequence), the ranks'
@@ -1389,7 +1417,7 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
 #pragma unroll
       for (int nt = 0; nt < NT; ++nt) acc[nt][0] = acc[nt][1] = acc[nt][2] = acc[nt][3] = 0.f;
       const uint32_t a0 = tile_wait(k, seq);
-      for (int q = 0; q < g.P; ++q) {
+      for (int q = 0; q < kPanels; ++q) {
         const uint32_t a = a0 + (q * 64 + mt * 16) * xrow, b = x_plane + q * RP * xrow;
 #pragma unroll
         for (int kk = 0; kk < KS; ++kk) mma_step<NT>(acc, a + (ax_pre ^ (kk << 5)), b + (bx_pre ^ (kk << 5)), 8 * xrow);
@@ -1427,10 +1455,11 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
             reinterpret_cast<float*>(kvq + token * 512 + 256)[tid] = (s_rstd[token] * (a - s_mean[token] * fs) + fc) * p.scale;
           }
         }
-        send_rows<NT>(k, xn, kvq, nullptr, 512, 0);
+        send_rows<NT, 512, false>(k, xn, kvq, nullptr, 0);
         ++xn;
         long_cross_attention<KW>(k, lc, LP, kvq, ckv_g, ckv_g + kb, ckv_g + 2 * kb, s_src[0], lvl2);
       } else {
+#pragma unroll
       for (int slot = 0; slot < NT; ++slot) {
         const int token = slot * kC + c;
         if (token < R) {                     // uniform over the CTA
@@ -1441,10 +1470,10 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
             sm.q[tid] = (s_rstd[token] * (a - s_mean[token] * fs) + fc) * p.scale;
           }
           __syncthreads();
-          const int b = token / rpb;
+          const int b = k.ctl->tok_b[slot];
           float ov;
-          if (LEAN == 1 || GROUPS || g.staged) ov = cross_attention_tile(ckv_g, ckv_g + kb, ckv_g + 2 * kb, GROUPS ? 0 : b * p.max_src, s_src[b], sm);
-          else ov = attention_head<float, kDH, kWarps, false>(ap, b, j, 0, s_src[b], sm);
+          if (LEAN == 1 || GROUPS || g.staged) ov = cross_attention<true>(ckv_g, ckv_g + kb, ckv_g + 2 * kb, GROUPS ? 0 : b * p.max_src, nullptr, d, s_src[b], sm);
+          else ov = cross_attention<false>(nullptr, nullptr, nullptr, 0, LP.crosskv + (size_t)b * p.max_src * (2 * d) + j * kDH, d, s_src[b], sm);
           if (tid < kDH) store_attn_out(oh, ol, token, tid, ov);
           __syncthreads();
         }
@@ -1456,7 +1485,7 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
     if constexpr (SPLIT) {
       share_states(k, xn, lvl2, oh, ol, g.staged);
     } else {
-      send_rows<NT>(k, xn, oh, ol, 128, g.staged);
+      send_rows<NT, 128, true>(k, xn, oh, ol, g.staged);
     }
     ++xn;
     BPD_TR();
@@ -1501,12 +1530,14 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
     __syncthreads();
     BPD_TR();
     // the cluster's hidden units over this rank's columns; unit f belongs to rank f / UPR
+#pragma unroll
+    for (int q = 0; q < kPanels; ++q) wt[q] = kHoist ? tile_wait(k, seq + q) : 0u;
     for (int mt = warp; mt < g.HCt / 16; mt += kWarps) {
       float acc[NT][4];
 #pragma unroll
       for (int nt = 0; nt < NT; ++nt) acc[nt][0] = acc[nt][1] = acc[nt][2] = acc[nt][3] = 0.f;
-      for (int q = 0; q < g.P; ++q) {
-        const uint32_t a = tile_wait(k, seq + q) + mt * 16 * xrow, b = x_plane + q * RP * xrow;
+      for (int q = 0; q < kPanels; ++q) {
+        const uint32_t a = (kHoist ? wt[q] : tile_wait(k, seq + q)) + mt * 16 * xrow, b = x_plane + q * RP * xrow;
 #pragma unroll
         for (int kk = 0; kk < KS; ++kk) mma_step<NT>(acc, a + (ax_pre ^ (kk << 5)), b + (bx_pre ^ (kk << 5)), 8 * xrow);
       }

@@ -194,6 +194,36 @@ def test_fp32_paths_keep_their_precision(bpd, batch, k, heads, max_src, tgt, opt
     model.close()
 
 
+# Cross-attention of the persistent kernel takes the encoder's rows in chunks of 8, one per warp: one row, a chunk's edges and
+# the edges of a second round of the eight warps.  Tolerance as above (fp32 throughout, the same roundings on the way).
+@pytest.mark.parametrize("heads", [4, 8])
+def test_source_lengths_around_a_chunk_of_encoder_rows(bpd, heads):
+    from bpd_inputs import ModelConfig, make_weights
+    from bpd_inputs.blob import blob_layout
+    from oracle.decode import TransformerScorer
+    from oracle.model import parse_blob
+    lens = np.array([1, 7, 8, 9, 63, 64, 65, 72], np.int32)
+    cfg = ModelConfig(2, 2, 64 * heads, heads, 128 * heads, 300, 2, 64)
+    blob = make_weights(cfg, 5, 0.06)
+    for name, shape, _, off, nbytes in blob_layout(cfg)[0]:
+        if name.endswith("self.wo"):
+            blob[off:off + nbytes] = 0
+    src = np.random.default_rng(heads).integers(2, 300, (8, 72)).astype(np.int32)
+    model = bpd.Model(blob)
+    s = bpd.Session(model, 8, 72, 20)
+    assert s.layer_path == 2
+    s.bpd_encode(src, lens)
+    r = s.bpd_iteration(2, 20, want_hidden=True)
+    model_o = parse_blob(blob)
+    for b in range(8):
+        scorer = TransformerScorer(model_o, src[b], int(lens[b]), cached=True, capacity=24)
+        scorer([0], 1)
+        scorer([0] + [int(t) for t in r["block"][b]], 2)
+        np.testing.assert_allclose(r["hidden"][b].cpu().numpy(), scorer.last_hidden, atol=1e-4)
+    s.close()
+    model.close()
+
+
 # the persistent layer kernel with groups of sequences: a last group that is full and one that is not, two sequences per
 # group and one, one token tile and two, lengths up to the limit of 256 positions, one encoder row and the most (a
 # multiple of 8) whose staging tile fits beside the working buffers of each shape: 136, 104 and 48
