@@ -363,56 +363,69 @@ __device__ __forceinline__ void ll_load2(const unsigned long long* at, unsigned 
 }
 
 // ------------------------------------------------------------------ x slice: reduce, planes, statistics
-// Static words of a thread's (at most two) items, fetched before the join: four gains or four bias values each.
-struct Words { uint2 w[2]; };
-__device__ __forceinline__ Words load_words(const Cta& k, const bf16* v) {
-  Words o;
-  const int n4 = k.g.ks >> 2;
+// An item is V neighbouring columns of a row (four, or two where a rank has at most 64 columns: with four rows and eight heads
+// a quarter of the threads would have all the loads to do, sixteen each; us per pass with items of four / two, base model: block
+// of four rows 144.6 / 139.0, one row 135.7 / 128.5, five sentences 167.2 / 162.5, 1000 intensities 210.4 / 210.1).
+template <int V> struct Words { uint32_t w[2][V / 2]; };       // of a thread's (at most two) items: gains or bias values, fetched before the join
+template <int V>
+__device__ __forceinline__ Words<V> load_words(const Cta& k, const bf16* v) {
+  Words<V> o;
+  const int nv = k.g.ks / V;
 #pragma unroll
   for (int u = 0; u < 2; ++u) {
     const int idx = k.tid + u * kThreads;
-    o.w[u] = (v != nullptr && idx < k.R * n4) ? *reinterpret_cast<const uint2*>(v + k.c * k.g.ks + (idx & (n4 - 1)) * 4) : make_uint2(0u, 0u);
+    const bool live = v != nullptr && idx < k.R * nv;
+    const uint32_t* at = reinterpret_cast<const uint32_t*>(v + k.c * k.g.ks + (idx & (nv - 1)) * V);
+    if constexpr (V == 4) {
+      const uint2 x = live ? *reinterpret_cast<const uint2*>(at) : make_uint2(0u, 0u);
+      o.w[u][0] = x.x; o.w[u][1] = x.y;
+    } else {
+      o.w[u][0] = live ? *at : 0u;
+    }
   }
   return o;
 }
 // After a join: x[t][col] += bias[col] + sum over the H clusters' partial outputs, in cluster order, for this
-// rank's columns.  Item = (row, four columns); rows are aligned to groups of lanes.  The loads of up to 16
+// rank's columns.  Item = (row, V columns); rows are aligned to groups of lanes.  The loads of up to 16
 // partials are all in flight before the first is added.
-__device__ __forceinline__ void reduce_slice(const Cta& k, float* x_s, const unsigned long long* ws, const Words& bias,
+template <int V>
+__device__ __forceinline__ void reduce_slice(const Cta& k, float* x_s, const unsigned long long* ws, const Words<V>& bias,
                                              unsigned tag, int nfree) {
   const StackParams& p = *k.p;
-  const int ks = k.g.ks, n4 = ks >> 2, R = k.R, d = k.d, H = k.H;
+  const int ks = k.g.ks, nv = ks / V, R = k.R, d = k.d, H = k.H;
   __syncthreads();                                             // every warp is done with the tiles released here
   if (k.tid == kPumpThread && nfree) release_tiles(k, nfree);
 #pragma unroll
   for (int it = 0; it < 2; ++it) {
     const int idx = k.tid + it * kThreads;
-    if (idx >= R * n4) break;
-    const int t = idx >> k.g.lg_n4, c4 = idx & (n4 - 1);
-    const unsigned long long* src = ws + (size_t)t * d + k.c * ks + c4 * 4;
+    if (idx >= R * nv) break;
+    const int t = idx / nv, cv = idx & (nv - 1);
+    const unsigned long long* src = ws + (size_t)t * d + k.c * ks + cv * V;
     const size_t step = (size_t)kMaxRows * d;
-    float4 acc = *reinterpret_cast<const float4*>(x_s + t * ks + c4 * 4);
-    {
-      const uint2 bw = bias.w[it];
-      acc.x += __uint_as_float(bw.x << 16); acc.y += __uint_as_float(bw.x & 0xffff0000u);
-      acc.z += __uint_as_float(bw.y << 16); acc.w += __uint_as_float(bw.y & 0xffff0000u);
+    float* x = x_s + t * ks + cv * V;
+    float acc[V];
+#pragma unroll
+    for (int e = 0; e < V; e += 2) {
+      const float2 old = *reinterpret_cast<const float2*>(x + e);
+      const uint32_t bw = bias.w[it][e / 2];
+      acc[e] = old.x + __uint_as_float(bw << 16); acc[e + 1] = old.y + __uint_as_float(bw & 0xffff0000u);
     }
     for (int p0 = 0; p0 < H; p0 += 8) {
       // eight producers per round; a round is repeated as a whole until every word carries this reduction's tag
-      unsigned long long v[8][4];
+      unsigned long long v[8][V];
       const unsigned long long t0 = clock64();
       for (unsigned spins = 0;; ++spins) {
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
           const unsigned long long* at = src + (size_t)min(p0 + u, H - 1) * step;
-          ll_load2(at, v[u][0], v[u][1]);
-          ll_load2(at + 2, v[u][2], v[u][3]);
+#pragma unroll
+          for (int e = 0; e < V; e += 2) ll_load2(at + e, v[u][e], v[u][e + 1]);
         }
         bool ready = true;
 #pragma unroll
         for (int u = 0; u < 8; ++u)
-          ready = ready && (unsigned)(v[u][0] >> 32) == tag && (unsigned)(v[u][1] >> 32) == tag &&
-                  (unsigned)(v[u][2] >> 32) == tag && (unsigned)(v[u][3] >> 32) == tag;
+#pragma unroll
+          for (int e = 0; e < V; ++e) ready = ready && (unsigned)(v[u][e] >> 32) == tag;
         if (ready || is_zombie(k)) break;
         if ((spins & 15u) == 15u) {
           if (__ldcg(p.bar + kBarAbort) != 0u) { *reinterpret_cast<volatile int*>(&k.ctl->zombie) = 1; break; }
@@ -421,12 +434,12 @@ __device__ __forceinline__ void reduce_slice(const Cta& k, float* x_s, const uns
       }
 #pragma unroll
       for (int u = 0; u < 8; ++u)
-        if (p0 + u < H) {
-          acc.x += __uint_as_float((unsigned)v[u][0]); acc.y += __uint_as_float((unsigned)v[u][1]);
-          acc.z += __uint_as_float((unsigned)v[u][2]); acc.w += __uint_as_float((unsigned)v[u][3]);
-        }
+        if (p0 + u < H)
+#pragma unroll
+          for (int e = 0; e < V; ++e) acc[e] += __uint_as_float((unsigned)v[u][e]);
     }
-    *reinterpret_cast<float4*>(x_s + t * ks + c4 * 4) = acc;
+#pragma unroll
+    for (int e = 0; e < V; e += 2) *reinterpret_cast<float2*>(x + e) = make_float2(acc[e], acc[e + 1]);
   }
 }
 
@@ -454,7 +467,7 @@ __device__ __forceinline__ bool ll_wait4(const Cta& k, const unsigned long long*
   return true;
 }
 __device__ __forceinline__ void reduce_slice_2hop(const Cta& k, float* x_s, const unsigned long long* ws, unsigned long long* gather,
-                                                  const Words& bias, unsigned tag, int nfree) {
+                                                  const Words<4>& bias, unsigned tag, int nfree) {
   const int ks = k.g.ks, n4 = ks >> 2, R = k.R, d = k.d, H = k.H, j = blockIdx.y;
   __syncthreads();                                             // every warp is done with the tiles released here
   if (k.tid == kPumpThread && nfree) release_tiles(k, nfree);
@@ -484,11 +497,8 @@ __device__ __forceinline__ void reduce_slice_2hop(const Cta& k, float* x_s, cons
     if (idx >= R * n4) break;
     const int t = idx >> k.g.lg_n4, c4 = idx & (n4 - 1);
     float4 acc = *reinterpret_cast<const float4*>(x_s + t * ks + c4 * 4);
-    {
-      const uint2 bw = bias.w[it];
-      acc.x += __uint_as_float(bw.x << 16); acc.y += __uint_as_float(bw.x & 0xffff0000u);
-      acc.z += __uint_as_float(bw.y << 16); acc.w += __uint_as_float(bw.y & 0xffff0000u);
-    }
+    acc.x += __uint_as_float(bias.w[it][0] << 16); acc.y += __uint_as_float(bias.w[it][0] & 0xffff0000u);
+    acc.z += __uint_as_float(bias.w[it][1] << 16); acc.w += __uint_as_float(bias.w[it][1] & 0xffff0000u);
     float4 v;
     ll_wait4(k, gather + (size_t)t * d + k.c * ks + c4 * 4, tag, v);
     acc.x += v.x; acc.y += v.y; acc.z += v.z; acc.w += v.w;
@@ -523,39 +533,57 @@ static __global__ void tagged_wait_probe_kernel(int* error, unsigned long long l
 // into this rank's block of the statistics table (sent to the other ranks with the next exchange).  A thread
 // reads back the items it wrote itself in reduce_slice / the embedding (same idx -> thread mapping): no barrier
 // is needed in between.
-template <int NT>
-__device__ __forceinline__ void planes_and_stats(const Cta& k, const float* x_s, const Words& gain, uint8_t* xh, uint8_t* xl,
+template <int NT, int V>
+__device__ __forceinline__ void planes_and_stats(const Cta& k, const float* x_s, const Words<V>& gain, uint8_t* xh, uint8_t* xl,
                                                  float* stats_mine) {
-  const int ks = k.g.ks, n4 = ks >> 2, R = k.R, PW = k.g.PW;
+  const int ks = k.g.ks, nv = ks / V, R = k.R, PW = k.g.PW;
   constexpr int RP = NT * 8;
 #pragma unroll
   for (int it = 0; it < 2; ++it) {
     const int idx = k.tid + it * kThreads;
-    if (idx >= ((R * n4 + 31) & ~31)) break;                 // whole warps leave together
-    const bool live = idx < R * n4;
-    const int t = live ? idx >> k.g.lg_n4 : 0, c4 = live ? idx & (n4 - 1) : 0;
-    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (idx >= ((R * nv + 31) & ~31)) break;                 // whole warps leave together
+    const bool live = idx < R * nv;
+    const int t = live ? idx / nv : 0, cv = live ? idx & (nv - 1) : 0;
+    float v[V] = {};
     if (live) {
-      v = *reinterpret_cast<const float4*>(x_s + t * ks + c4 * 4);
-      const uint2 gw = gain.w[it];
-      const float w[4] = {v.x * __uint_as_float(gw.x << 16), v.y * __uint_as_float(gw.x & 0xffff0000u),
-                          v.z * __uint_as_float(gw.y << 16), v.w * __uint_as_float(gw.y & 0xffff0000u)};
-      uint32_t hi[4], lo[4];
+      if constexpr (V == 4) {
+        const float4 x = *reinterpret_cast<const float4*>(x_s + t * ks + cv * 4);
+        v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
+      } else {
+        const float2 x = *reinterpret_cast<const float2*>(x_s + t * ks + cv * 2);
+        v[0] = x.x; v[1] = x.y;
+      }
+      uint32_t hi[V / 2], lo[V / 2];
 #pragma unroll
-      for (int e = 0; e < 4; ++e) fused::split_bits(w[e], hi[e], lo[e]);
-      const int col = c4 * 4, panel = col >> k.g.lg_pw, within = col & (PW - 1);
+      for (int e = 0; e < V; e += 2) {
+        const uint32_t gw = gain.w[it][e / 2];
+        uint32_t h0, l0, h1, l1;
+        fused::split_bits(v[e] * __uint_as_float(gw << 16), h0, l0);
+        fused::split_bits(v[e + 1] * __uint_as_float(gw & 0xffff0000u), h1, l1);
+        hi[e / 2] = h0 | (h1 << 16); lo[e / 2] = l0 | (l1 << 16);
+      }
+      const int col = cv * V, panel = col >> k.g.lg_pw, within = col & (PW - 1);
       const uint32_t at = panel * (RP * PW * 2) + swz((uint32_t)(t * PW * 2 + within * 2), k.g.xmask);
-      *reinterpret_cast<uint2*>(xh + at) = make_uint2(hi[0] | (hi[1] << 16), hi[2] | (hi[3] << 16));
-      *reinterpret_cast<uint2*>(xl + at) = make_uint2(lo[0] | (lo[1] << 16), lo[2] | (lo[3] << 16));
+      if constexpr (V == 4) {
+        *reinterpret_cast<uint2*>(xh + at) = make_uint2(hi[0], hi[1]);
+        *reinterpret_cast<uint2*>(xl + at) = make_uint2(lo[0], lo[1]);
+      } else {
+        *reinterpret_cast<uint32_t*>(xh + at) = hi[0];
+        *reinterpret_cast<uint32_t*>(xl + at) = lo[0];
+      }
     }
-    // the n4 lanes of a row (a power of two, at most 32, aligned) add up in a fixed butterfly
-    float s = (v.x + v.y) + (v.z + v.w);
-    for (int o = 1; o < n4; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    // the nv lanes of a row (a power of two, at most 32, aligned) add up in a fixed butterfly
+    float s = v[0] + v[1];
+    if constexpr (V == 4) s += v[2] + v[3];
+    for (int o = 1; o < nv; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     const float mean = s / (float)ks;
-    const float d0 = v.x - mean, d1 = v.y - mean, d2 = v.z - mean, d3 = v.w - mean;
-    float m2 = (d0 * d0 + d1 * d1) + (d2 * d2 + d3 * d3);
-    for (int o = 1; o < n4; o <<= 1) m2 += __shfl_xor_sync(0xffffffffu, m2, o);
-    if (live && c4 == 0) { stats_mine[t * 2] = mean; stats_mine[t * 2 + 1] = m2; }
+    float dv[V];
+#pragma unroll
+    for (int e = 0; e < V; ++e) dv[e] = v[e] - mean;
+    float m2 = dv[0] * dv[0] + dv[1] * dv[1];
+    if constexpr (V == 4) m2 += dv[2] * dv[2] + dv[3] * dv[3];
+    for (int o = 1; o < nv; o <<= 1) m2 += __shfl_xor_sync(0xffffffffu, m2, o);
+    if (live && cv == 0) { stats_mine[t * 2] = mean; stats_mine[t * 2 + 1] = m2; }
   }
 }
 
@@ -1034,6 +1062,7 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
   cg::cluster_group cluster = cg::this_cluster();
   constexpr int RP = NT * 8, H = D / kDH, KS = D == 256 ? 2 : 4;      // steps of 16 columns per panel
   constexpr int kPanels = D / kC <= 64 ? 1 : D / kC / 64;             // panels of a rank's columns
+  constexpr int V = D == 1024 ? 4 : 2;                                // columns of an item, see Words
   constexpr bool kHoist = kPanels == 1;      // wait for a panel once, not once per row tile (two panels cost more registers than the waits)
   constexpr bool GROUPS = LEAN == 4;
   constexpr bool SPLIT = LEAN == 2 || LEAN == 3;         // keys split over the ranks
@@ -1202,7 +1231,7 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
     const LayerPtrs& LP = layers_s[l];
     // =================================================================== self-attention block
     // static words first (gains, folded layer-norm vectors, bias): their latency hides behind the join
-    Words gw = load_words(k, LP.g1);
+    Words<V> gw = load_words<V>(k, LP.g1);
     float fs = 0.f, fc = 0.f;
     if (tid < 3 * kDH) {
       const int n = (tid / kDH) * d + j * kDH + (tid % kDH);
@@ -1210,11 +1239,11 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
       fc = LP.c_qkv[n];
     }
     if (l > 0) {
-      const Words bw = load_words(k, layers_s[l - 1].b2);
+      const Words<V> bw = load_words<V>(k, layers_s[l - 1].b2);
       ++nbar;
       BPD_TR();
       if constexpr (H == 16) reduce_slice_2hop(k, x_s, ws_g + (size_t)((nbar - 1) & 1) * H * kMaxRows * d, gather_g + (size_t)((nbar - 1) & 1) * kMaxRows * d, bw, base + nbar, g.PH);
-      else reduce_slice(k, x_s, ws_g + (size_t)((nbar - 1) & 1) * H * kMaxRows * d, bw, base + nbar, g.PH);
+      else reduce_slice<V>(k, x_s, ws_g + (size_t)((nbar - 1) & 1) * H * kMaxRows * d, bw, base + nbar, g.PH);
       BPD_TR();
       if (p.layer_dump && j == 0) {
         __syncthreads();
@@ -1222,7 +1251,7 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
           p.layer_dump[((size_t)(l - 1) * p.R + b0 * rpb + idx / ks) * d + c * ks + idx % ks] = x_s[idx];
       }
     }
-    planes_and_stats<NT>(k, x_s, gw, xh, xl, stats_mine);
+    planes_and_stats<NT, V>(k, x_s, gw, xh, xl, stats_mine);
     __syncthreads();
     BPD_TR();
     // Q, K, V of the head over this rank's columns; token t's partial goes to rank t % 8
@@ -1401,15 +1430,15 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
     BPD_TR();
 
     // =================================================================== cross-attention block
-    gw = load_words(k, LP.g2);
-    const Words nobias = load_words(k, nullptr);
+    gw = load_words<V>(k, LP.g2);
+    const Words<V> nobias = load_words<V>(k, nullptr);
     if (tid < kDH) { fs = LP.s_cq[j * kDH + tid]; fc = LP.c_cq[j * kDH + tid]; }
     ++nbar;
     BPD_TR();
     if constexpr (H == 16) reduce_slice_2hop(k, x_s, ws_g + (size_t)((nbar - 1) & 1) * H * kMaxRows * d, gather_g + (size_t)((nbar - 1) & 1) * kMaxRows * d, nobias, base + nbar, 1);
-      else reduce_slice(k, x_s, ws_g + (size_t)((nbar - 1) & 1) * H * kMaxRows * d, nobias, base + nbar, 1);
+      else reduce_slice<V>(k, x_s, ws_g + (size_t)((nbar - 1) & 1) * H * kMaxRows * d, nobias, base + nbar, 1);
     BPD_TR();
-    planes_and_stats<NT>(k, x_s, gw, xh, xl, stats_mine);
+    planes_and_stats<NT, V>(k, x_s, gw, xh, xl, stats_mine);
     __syncthreads();
     BPD_TR();
     for (int mt = warp; mt < kDH / 16; mt += kWarps) {
@@ -1512,7 +1541,7 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
     BPD_TR();
 
     // =================================================================== feed-forward block
-    gw = load_words(k, LP.g3);
+    gw = load_words<V>(k, LP.g3);
     float fs1[2], fc1[2];                    // folded vectors of the (at most two) hidden units this thread finishes
 #pragma unroll
     for (int u = 0; u < 2; ++u) {
@@ -1524,9 +1553,9 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
     ++nbar;
     BPD_TR();
     if constexpr (H == 16) reduce_slice_2hop(k, x_s, ws_g + (size_t)((nbar - 1) & 1) * H * kMaxRows * d, gather_g + (size_t)((nbar - 1) & 1) * kMaxRows * d, nobias, base + nbar, 1);
-      else reduce_slice(k, x_s, ws_g + (size_t)((nbar - 1) & 1) * H * kMaxRows * d, nobias, base + nbar, 1);
+      else reduce_slice<V>(k, x_s, ws_g + (size_t)((nbar - 1) & 1) * H * kMaxRows * d, nobias, base + nbar, 1);
     BPD_TR();
-    planes_and_stats<NT>(k, x_s, gw, xh, xl, stats_mine);
+    planes_and_stats<NT, V>(k, x_s, gw, xh, xl, stats_mine);
     __syncthreads();
     BPD_TR();
     // the cluster's hidden units over this rank's columns; unit f belongs to rank f / UPR
@@ -1618,19 +1647,19 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
   }
   // =================================================================== final layer norm
   {
-    const Words bw = load_words(k, layers_s[p.L - 1].b2), gw = load_words(k, p.lnf_g);
+    const Words<V> bw = load_words<V>(k, layers_s[p.L - 1].b2), gw = load_words<V>(k, p.lnf_g);
     ++nbar;
     BPD_TR();
     pdl_launch_dependents();
     if constexpr (H == 16) reduce_slice_2hop(k, x_s, ws_g + (size_t)((nbar - 1) & 1) * H * kMaxRows * d, gather_g + (size_t)((nbar - 1) & 1) * kMaxRows * d, bw, base + nbar, g.PH);
-      else reduce_slice(k, x_s, ws_g + (size_t)((nbar - 1) & 1) * H * kMaxRows * d, bw, base + nbar, g.PH);
+      else reduce_slice<V>(k, x_s, ws_g + (size_t)((nbar - 1) & 1) * H * kMaxRows * d, bw, base + nbar, g.PH);
     BPD_TR();
     if (p.layer_dump && j == 0) {
       __syncthreads();
       for (int idx = tid; idx < R * ks; idx += kThreads)
         p.layer_dump[((size_t)(p.L - 1) * p.R + b0 * rpb + idx / ks) * d + c * ks + idx % ks] = x_s[idx];
     }
-    planes_and_stats<NT>(k, x_s, gw, xh, xl, stats_mine);   // the planes are not used; the statistics are
+    planes_and_stats<NT, V>(k, x_s, gw, xh, xl, stats_mine);   // the planes are not used; the statistics are
     BPD_TR();
   }
   fence_async_smem();
