@@ -1189,10 +1189,9 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
   fused::cluster_arrive();
   fused::cluster_wait();                    // every CTA of the cluster runs: its shared memory and mbarriers may be written
 
-  AttnParams ap;
+  AttnParams ap;                            // what attn_first_key looks at
   memset(&ap, 0, sizeof(ap));
-  ap.rows = R; ap.rows_per_b = rpb; ap.H = H; ap.dh = kDH; ap.causal = 1; ap.local_q = p.local_q; ap.local_m = p.local_m;
-  ap.ldkv = d; ap.paged = 1; ap.st = p.st; ap.st.page_table = s_pt; ap.scale = p.scale;
+  ap.causal = 1; ap.local_q = p.local_q; ap.local_m = p.local_m;
   bool one_chunk_per_rank = true;
   if (LEAN == 0) {
     for (int b = 0; b < nb; ++b)
@@ -1307,7 +1306,6 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
     ++xn;
     BPD_TR();
     {
-      ap.k = LP.kcache; ap.v = LP.vcache;
       const bf16* Kc = LP.kcache;
       const bf16* Vc = LP.vcache;
       if constexpr (SPLIT) {
@@ -1471,8 +1469,6 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
       if (g.staged) ckv = tile_wait(k, seq);
       const uint8_t* ckv_g = ssm + (ckv - k.ring);
       const int kb = round1k(p.cross_rows * 128);
-      ap.causal = 0; ap.limit_b = s_src; ap.k = LP.crosskv; ap.v = LP.crosskv + d; ap.ldkv = 2 * d;
-      ap.bstride = (long long)p.max_src * 2 * d; ap.paged = 0;
       if constexpr (SPLIT) {
         // every rank needs all queries: finished rows travel like the keys and values of the self-attention block
         for (int slot = 0; slot < NT; ++slot) {
@@ -1508,7 +1504,6 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
         }
       }
       }
-      ap.causal = 1; ap.ldkv = d; ap.paged = 1;
       seq += g.staged;
     }
     if constexpr (SPLIT) {
