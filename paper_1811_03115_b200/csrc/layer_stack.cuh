@@ -1008,6 +1008,10 @@ __device__ __forceinline__ void long_cross_attention(const Cta& k, const LongCtx
 }
 
 // The ranks' states to every rank (exchange n), merged in rank order into the planes of the attention output.
+// Where the table may lie: no rank hears from another that it has merged until that one sends again, and the next thing
+// every rank sends to every other are partial sums into the inboxes, so the table is not the inbox.  It is the hidden planes:
+// a rank sends states or hidden units only after the partial sums of all ranks have reached it, and a rank sends those only
+// after it has read whatever the table or the planes held before.
 __device__ __forceinline__ void share_states(const Cta& k, int n, float* lvl2, uint8_t* oh, uint8_t* ol, int nfree = 0) {
   const int R = k.R;
   float* mine = lvl2 + (size_t)k.c * R * kState;
