@@ -33,6 +33,9 @@ int main() {
           printf("%d %d %d %d  %d %d  %d %d  %d %d  %d %d\n", d, units, rows, lean, L.inbox, fused::kC * chunk, L.lvl2,
                  (int)(fused::kC * rows * stack::kState * 4), L.hid, fused::kC * 2 * RP * UPR * 2, L.stats, fused::kC * fused::kMaxRows * 8);
         }
+  printf("rows\n");
+  for (int rows = 1; rows <= fused::kMaxRows; ++rows)
+    for (int c = 0; c < fused::kC; ++c) printf("%d %d\n", stack::row_bytes_sent(c, rows, 512), stack::row_bytes_awaited(c, rows, 512));
 }
 """
 
@@ -44,9 +47,9 @@ def plans(tmp_path_factory):
     (tmp / "plans.cu").write_text(PLANS)
     subprocess.run([nvcc, "-std=c++17", "-gencode", "arch=compute_100a,code=sm_100a", "-I", CSRC, "-o", str(tmp / "plans"), str(tmp / "plans.cu")], check=True)
     out = subprocess.run([str(tmp / "plans")], check=True, capture_output=True, text=True).stdout
-    rows = [[int(v) for v in line.split()] for line in out.splitlines()]
-    assert rows
-    return rows
+    shapes, sent = ([[int(v) for v in line.split()] for line in part.splitlines() if line] for part in out.split("rows"))
+    assert shapes and len(sent) == 16 * RANKS
+    return shapes, [sent[i:i + RANKS] for i in range(0, len(sent), RANKS)]
 
 
 def _faults(exchanges):
@@ -54,13 +57,15 @@ def _faults(exchanges):
     send m, wait for m, read, send m + 1.  known[c][r]: the latest exchange of which c knows that r has sent its part, hence
     has finished its reads after the one before.  Returns what a rank may overwrite too early."""
     found = set()
-    known = [[-1] * RANKS for _ in range(RANKS)]
+    known = [[-1] * RANKS for _ in range(RANKS)]        # two barriers alternate: r must have passed exchange m - 2
     overlap = lambda a, b: a[0] < b[0] + b[1] and b[0] < a[0] + a[1]
     for m, (writes, _, senders) in enumerate(exchanges):
         for c in senders:
             for r in range(RANKS):
                 if r == c:
                     continue
+                if m >= 2 and known[c][r] < m - 1:
+                    found.add((m, m - 2))
                 for q in range(m):
                     for w in writes:
                         for t in exchanges[q][1]:
@@ -76,12 +81,20 @@ def _faults(exchanges):
 
 
 def test_no_rank_overwrites_what_another_still_reads(plans):
-    for d, units, rows, lean, *at in plans:
-        if lean not in (2, 3) or rows < RANKS:
-            continue
+    for d, units, rows, lean, *at in plans[0]:
         inbox, states, hidden, stats = zip(at[0::2], at[1::2])
         every = range(RANKS)
-        partials = ((inbox, stats), (inbox, stats), every)
-        layer = [partials, ((), (), every), ((states,), (states,), every),          # keys, values and queries; states
-                 partials, ((), (), every), ((states,), (states,), every), partials, ((hidden,), (hidden,), every)]
+        with_rows = [c for c in every if plans[1][rows - 1][c][0] > 0]
+        partials, finish = ((inbox, stats), (inbox, stats), every), ((hidden,), (hidden,), every)
+        share, some = ((states,), (states,), every), ((), (), with_rows)
+        if lean in (2, 3):        # keys, values and queries, then states, in both attentions
+            layer = [partials, some, share, partials, some, share, partials, finish]
+        else:                     # keys, values and queries, finished rows (or states), finished rows
+            layer = [partials, some, share if lean == 0 else some, partials, some, partials, finish]
         assert not _faults(layer * 3), (d, units, rows, lean)
+
+
+def test_an_exchange_of_rows_awaits_what_is_sent(plans):
+    for sent in plans[1]:
+        for c in range(RANKS):
+            assert sent[c][0] > 0 and sent[c][1] == sum(n for n, _ in sent) - sent[c][0]
