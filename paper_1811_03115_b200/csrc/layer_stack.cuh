@@ -326,7 +326,7 @@ __device__ __forceinline__ uint32_t tile_wait(const Cta& k, int seq) {
   const long long t0 = clock64();
 #endif
   const uint32_t bar = tc::smem_u32(&k.ctl->full[slot]), phase = (uint32_t)(seq / kNB) & 1u;
-  if (!tc::mbar_try_wait(bar, phase) && !is_zombie(k)) {       // mostly there: the common case looks at nothing else
+  if (!tc::mbar_test(bar, phase) && !is_zombie(k)) {           // mostly there: the common case looks at nothing else
     if (!tc::mbar_wait(bar, phase, k.p->spin)) raise_abort(k, 105);
   }
 #ifdef BPD_STACK_TRACE
@@ -348,7 +348,7 @@ __device__ __forceinline__ void xchg_send(const Cta& k, int n, int rank, const v
 // All threads: wait for everything exchange n brings.
 __device__ __forceinline__ void xchg_wait(const Cta& k, int n) {
   const uint32_t bar = tc::smem_u32(&k.ctl->ex[n & 1]), phase = (uint32_t)(n >> 1) & 1u;
-  if (!tc::mbar_try_wait(bar, phase) && !is_zombie(k)) {
+  if (!tc::mbar_test(bar, phase) && !is_zombie(k)) {
     if (!tc::mbar_wait(bar, phase, k.p->spin)) raise_abort(k, 106);
   }
 }
@@ -509,7 +509,8 @@ __device__ __forceinline__ void reduce_slice_2hop(const Cta& k, float* x_s, cons
 
 // Self test of the bounded wait on tagged words: one warp waits for a tag that nobody writes, gives up after
 // `limit_cycles`, records the error code a real pass would (104) and raises the abort word; the kernel returns
-// normally and the context stays usable.
+// normally and the context stays usable.  From then on waits for tiles and exchanges must not wait: 64 of each, for barriers that
+// nothing arrives on, take about 70 cycles apiece (a try_wait, which may put the thread to sleep, took 7800).
 static __device__ unsigned long long g_probe_words[4];
 static __device__ unsigned g_probe_bar[kBarWords];
 static __global__ void tagged_wait_probe_kernel(int* error, unsigned long long limit_cycles) {
@@ -520,12 +521,20 @@ static __global__ void tagged_wait_probe_kernel(int* error, unsigned long long l
     sp.error = error; sp.bar = g_probe_bar; sp.spin = limit_cycles;
     g_probe_bar[kBarAbort] = 0u;
     for (int i = 0; i < 4; ++i) g_probe_words[i] = 0ull;          // tag 0: never the tag of a reduction
+    tc::mbar_init(tc::smem_u32(&ctl.full[0]), 1);
+    tc::mbar_init(tc::smem_u32(&ctl.ex[0]), 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    ctl.off[0] = 0;
   }
   __syncthreads();
   Cta k;
-  k.p = &sp; k.ctl = &ctl; k.tid = threadIdx.x;
+  k.p = &sp; k.ctl = &ctl; k.tid = threadIdx.x; k.ring = 0;
   float4 v;
   ll_wait4(k, g_probe_words, 1u, v);
+  __syncthreads();
+  const long long t0 = clock64();
+  for (int i = 0; i < 64; ++i) { tile_wait(k, 0); xchg_wait(k, 0); }
+  if (threadIdx.x == 0 && clock64() - t0 > 64 * 2 * 1000) atomicExch(error, -2);
   __syncthreads();
   if (threadIdx.x == 0 && (ctl.zombie == 0 || g_probe_bar[kBarAbort] == 0u)) atomicExch(error, -1);   // the wait ended some other way
 }
