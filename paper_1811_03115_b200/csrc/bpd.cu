@@ -709,9 +709,10 @@ static int run_layers_fused(bpd_session* s, const PassArgs& a) {
 }
 
 // ------------------------------------------------------------------ persistent layer stack (few rows per pass)
-// How many clusters of the given instantiation can be resident at once.
+// How many clusters of the given instantiation can be resident at once; none of one that does not exist.
 static int stack_clusters(const void* kernel, size_t smem, int H, int* out) {
-  if (!kernel) return fail(BPD_E_UNSUPPORTED, "no such instantiation of the persistent layer kernel");
+  *out = 0;
+  if (!kernel) return BPD_OK;
   BPD_TRY(ensure_smem_limit(kernel, smem));
   cudaLaunchConfig_t cfg;
   memset(&cfg, 0, sizeof(cfg));
@@ -781,13 +782,12 @@ static int stack_setup(bpd_session* s, bool try_groups) {
       cross_rows = lean == 2 || lean == 3 ? (ceil_div(s->max_src, fused::kC) + 7) / 8 * 8 : (staged ? (groups ? 1 : s->B) * s->max_src : 0);
       if (budget <= 1024 || !stack_plan(c, rows, seqs, s->ppr, staged ? cross_rows : 0, long_seq, lean, budget - 1024, &lay)) continue;
       lay.total += 1024;                       // slack for aligning the ring to 1024 bytes
-      int n1 = 0, n2 = 0;
-      const size_t sm = (size_t)lay.total;
-      const int H = c.H;
-      BPD_TRY(stack_clusters(stack::kernel_for(1, c.d, c.d_ff / c.H, minb, lean), sm, H, &n1));
-      BPD_TRY(stack_clusters(stack::kernel_for(2, c.d, c.d_ff / c.H, minb, lean), sm, H, &n2));
-      const int need = std::max(1, groups) * c.H;
-      ok = n1 >= need && n2 >= need;
+      ok = true;                               // the widest pass and narrower ones
+      for (int nt = 1; nt <= (rows > 8 ? 2 : 1) && ok; ++nt) {
+        int n = 0;
+        BPD_TRY(stack_clusters(stack::kernel_for(nt, c.d, c.d_ff / c.H, minb, lean), (size_t)lay.total, c.H, &n));
+        ok = n >= std::max(1, groups) * c.H;
+      }
     }
     if (ok) break;
   }

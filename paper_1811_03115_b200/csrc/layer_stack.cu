@@ -6,7 +6,7 @@
 namespace bpd {
 namespace stack {
 
-BPD_STACK_KERNELS(1024)
+BPD_STACK_KERNELS_HALF_SM(1024)
 template <> const void* kernel_of<512>(int nt, int hct, int minb, int lean);
 template <> const void* kernel_of<256>(int nt, int hct, int minb, int lean);
 

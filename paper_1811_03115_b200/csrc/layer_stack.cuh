@@ -1739,6 +1739,9 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
 // (1 or 2), variant (LEAN, see the kernel: 0 general, 1 short sequences with staged encoder rows, 2 one long sequence,
 // 3 one short sequence, 4 groups of sequences); null if there is none.  One translation unit per d_model
 // (layer_stack.cu, layer_stack_512.cu, layer_stack_256.cu), compiled side by side.
+// There are those that a session can get on a B200.  4 or 8 clusters (d_model 256, 512) always have an SM to themselves per CTA,
+// and what does not fit a whole SM does not fit half a one; groups need two CTAs per SM.  16 clusters (d_model 1024) need
+// two (15 are resident at one), and half an SM has no room for two token tiles, which groups of 16 heads always have.
 const void* kernel_for(int nt, int d, int hct, int minb, int lean);
 template <int D> const void* kernel_of(int nt, int hct, int minb, int lean);
 #define BPD_STACK_V(D, NT, MB, LN) \
@@ -1746,10 +1749,14 @@ template <int D> const void* kernel_of(int nt, int hct, int minb, int lean);
   if (nt == NT && hct == 256 && minb == MB && lean == LN) return reinterpret_cast<const void*>(layer_stack_kernel<NT, D, 256, MB, LN>)
 #define BPD_STACK_KERNELS(D) \
   template <> const void* kernel_of<D>(int nt, int hct, int minb, int lean) { \
-    BPD_STACK_V(D, 1, 1, 0); BPD_STACK_V(D, 2, 1, 0); BPD_STACK_V(D, 1, 2, 0); BPD_STACK_V(D, 2, 2, 0); \
-    BPD_STACK_V(D, 1, 1, 1); BPD_STACK_V(D, 2, 1, 1); BPD_STACK_V(D, 1, 2, 1); BPD_STACK_V(D, 2, 2, 1); \
+    BPD_STACK_V(D, 1, 1, 0); BPD_STACK_V(D, 2, 1, 0); BPD_STACK_V(D, 1, 1, 1); BPD_STACK_V(D, 2, 1, 1); \
     BPD_STACK_V(D, 1, 1, 2); BPD_STACK_V(D, 2, 1, 2); BPD_STACK_V(D, 1, 1, 3); BPD_STACK_V(D, 2, 1, 3); \
     BPD_STACK_V(D, 1, 2, 4); BPD_STACK_V(D, 2, 2, 4); \
+    return nullptr; \
+  }
+#define BPD_STACK_KERNELS_HALF_SM(D) \
+  template <> const void* kernel_of<D>(int nt, int hct, int minb, int lean) { \
+    BPD_STACK_V(D, 1, 2, 0); BPD_STACK_V(D, 1, 2, 1); \
     return nullptr; \
   }
 
