@@ -839,7 +839,7 @@ static int stack_setup(bpd_session* s, bool try_groups) {
   BPD_CUDA(cudaStreamSynchronize(s->stream));
   static_assert(sizeof(stack::Layout) <= sizeof(s->stack_layout), "layout does not fit its opaque copy");
   memcpy(s->stack_layout, &lay, sizeof(lay));
-  s->stack_cross_rows = cross_rows; s->stack_staged = staged; s->stack_long = long_seq ? 1 : 0; s->stack_minb = minb; s->stack_lean = lean;
+  s->stack_cross_rows = cross_rows; s->stack_staged = staged; s->stack_minb = minb; s->stack_lean = lean;
   s->stack_groups = std::max(1, groups); s->stack_group_seqs = seqs;
   s->stack = 1;
   s->stack_dev = dev;
@@ -855,11 +855,11 @@ static int run_layers_stack(bpd_session* s, const PassArgs& a) {
   stack::StackParams p;
   memset(&p, 0, sizeof(p));
   p.layers = static_cast<const stack::LayerPtrs*>(s->stack_layers);
-  p.L = c.n_dec; p.d = c.d; p.H = c.H; p.ff = c.d_ff; p.R = s->B * a.kcur; p.rows_per_b = a.kcur; p.nb = s->B; p.group_seqs = s->stack_group_seqs; p.eps = c.eps;
+  p.L = c.n_dec; p.R = s->B * a.kcur; p.rows_per_b = a.kcur; p.nb = s->B; p.group_seqs = s->stack_group_seqs; p.eps = c.eps;
   p.tgt_embed = static_cast<const bf16*>(m->tgt_embed); p.pe = s->pe; p.npos = s->npos; p.vocab = c.V;
   p.st = s->st; p.forced = a.forced; p.forced_rows = a.forced_rows; p.kforced = a.kforced;
   p.local_q = c.local_q; p.local_m = c.local_m; p.max_src = s->max_src; p.scale = 1.0f / sqrtf((float)fused::kDH);
-  p.cross_rows = s->stack_cross_rows; p.cross_staged = s->stack_staged; p.cross_split = s->stack_lean == 2 || s->stack_lean == 3; p.long_seq = s->stack_long;
+  p.cross_rows = s->stack_cross_rows; p.cross_staged = s->stack_staged; p.cross_split = s->stack_lean == 2 || s->stack_lean == 3;
   p.lnf_g = static_cast<const bf16*>(m->dec_lnf_g); p.lnf_b = static_cast<const bf16*>(m->dec_lnf_b);
   p.xn_hi = static_cast<bf16*>(s->xn); p.xn_plane = s->pl_xn; p.h_f32 = s->h_f32;
   p.layer_dump = a.layer_dump;

@@ -16,13 +16,3 @@ BPD_TC_LAUNCH(kTcArgmax);
 
 }  // namespace tc
 }  // namespace bpd
-
-#ifdef BPD_TC_TRACE
-// Development builds only: where the projection kernel writes its per-CTA step timestamps (4096 * 16 unsigned 64-bit
-// words of device memory), or null to stop.
-extern "C" int bpd_debug_set_tc_trace(void* dev_buffer) {
-  unsigned long long* ptr = static_cast<unsigned long long*>(dev_buffer);
-  BPD_CUDA(cudaMemcpyToSymbol(bpd::tc::g_tc_trace, &ptr, sizeof(ptr)));
-  return BPD_OK;
-}
-#endif

@@ -21,23 +21,6 @@
 namespace bpd {
 namespace tc {
 
-#ifdef BPD_TC_TRACE
-// Development builds only: per-CTA step timestamps of the projection kernel (16 words per CTA, up to 4096 CTAs of
-// the launches that run while the pointer is set; 128 regions chosen by the host's launch counter).
-__device__ unsigned long long* g_tc_trace = nullptr;
-__device__ __forceinline__ void tc_stamp(int region, int slot) {
-  if (!g_tc_trace) return;
-  const unsigned cta = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
-  if (cta >= 2047) return;
-  unsigned long long t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  g_tc_trace[((size_t)region * 2048 + cta) * 16 + slot] = t;
-}
-#define BPD_TC_STAMP(slot) tc_stamp(p.trace_id, slot)
-#else
-#define BPD_TC_STAMP(slot) do { } while (0)
-#endif
-
 constexpr int kBM = 128;          // features per tile (MMA M)
 constexpr int kBK = 64;           // K elements per pipeline stage (128 bytes of bf16: one swizzle row)
 constexpr int kThreads = 192;     // warp 0: TMA, warp 1: MMA + tensor-memory allocation, warps 2-5: epilogue
@@ -97,9 +80,6 @@ struct TcParams {
   // the sum of squared deviations of its 128 new values (stat_out, [tiles][stat_T][2]); the projection that
   // consumes the normalised stream merges the stat_parts tiles of a token in tile order (stat_in).
   float* stat_out; const float* stat_in; int stat_parts; int stat_T;
-#ifdef BPD_TC_TRACE
-  int trace_id;
-#endif
   int* error;                  // error word
   int error_on_host;           // 1 (wide kernel only): the word lies in pinned host memory
   const int* all_done;
@@ -397,7 +377,6 @@ __device__ __forceinline__ void tc_epilogue(const TcParams& p, const EpiShared& 
     if (nchunks > 0 && !skip) done = mbar_wait(u.acc_bar, u.acc_parity);
     if (!done && !skip) atomicCAS(p.error, 0, 103);
     ctl[3] = done ? 1u : 0u;
-    BPD_TC_STAMP(5);
   }
   asm volatile("bar.sync 1, 128;" ::: "memory");
   const bool ok = (ctl[3] != 0);
@@ -422,10 +401,8 @@ __device__ __forceinline__ void tc_epilogue(const TcParams& p, const EpiShared& 
         if (c < nt) wsz[((size_t)split * bn + c) * kBM + row] = v[c];
       asm volatile("bar.sync 1, 128;" ::: "memory");
       if (et == 0) {
-        BPD_TC_STAMP(6);
         const unsigned prev = atom_add_acq_rel(&p.tile_counters[(size_t)u.zidx * ntiles + tile], 1u);
         ctl[1] = (prev == (unsigned)p.splits - 1) ? 1u : 0u;
-        BPD_TC_STAMP(7);
       }
       asm volatile("bar.sync 1, 128;" ::: "memory");
       if (ctl[1]) {
@@ -486,16 +463,6 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                const __grid_constant__ CUtensorMap tmBl, TcParams p, int zslices, int a_rows_per_slice,
                int b_cols_per_slice) {
   pdl_launch_dependents();
-  if (threadIdx.x == 0) {
-    BPD_TC_STAMP(0);
-#ifdef BPD_TC_TRACE
-    if (g_tc_trace && blockIdx.x + blockIdx.y + blockIdx.z == 0) {
-      unsigned long long* h = g_tc_trace + ((size_t)p.trace_id * 2048 + 2047) * 16;
-      h[10] = EPI; h[11] = p.N; h[12] = p.K; h[13] = p.T; h[14] = p.splits;
-      h[15] = gridDim.x | (gridDim.y << 12) | ((unsigned long long)gridDim.z << 24) | ((unsigned long long)p.bn << 40);
-    }
-#endif
-  }
   extern __shared__ uint8_t smem_raw[];
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;      // swizzled tiles need 1024-byte alignment
   uint8_t* gen_base = smem_raw + (base - smem_u32(smem_raw));
@@ -535,7 +502,6 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   tc_fence_after();
   const uint32_t tmem = ctl[0];
   bool ok = true;
-  if (threadIdx.x == 0) BPD_TC_STAMP(1);
 
   if (warp == 0 && lane == 0) {
     // ---------------- TMA producer.  Weights do not depend on the preceding kernel: the first stages'
@@ -548,7 +514,6 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       else tma_load_2d(base + it * stage_sz, &tmA, bars + 8 * it, (c0 + it) * kBK, a_row);
     }
     pdl_wait();
-    BPD_TC_STAMP(2);
     const bool skip = p.all_done && *p.all_done;
     for (int it = 0; it < npre; ++it) {
       const uint32_t sa = base + it * stage_sz;
@@ -588,7 +553,6 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       if (in_group == p.group_chunks) { in_group = 0; acc += 16; }
       if (!mbar_wait(bars + 8 * s, ph)) { ok = false; break; }
       tc_fence_after();
-      if (it == 0) BPD_TC_STAMP(3);
       const uint32_t sa = base + s * stage_sz;
 #pragma unroll
       for (int kk = 0; kk < kBK / 16; ++kk) {
@@ -601,7 +565,6 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       umma_commit(bars + 8 * (kStages + s));       // frees the stage once these MMAs have read it
     }
     if (!skip) umma_commit(bars + 8 * 2 * kStages);            // accumulator complete
-    BPD_TC_STAMP(4);
     if (!ok) atomicCAS(p.error, 0, 102);
   } else if (warp >= 2) {
     // ---------------- epilogue: thread = one feature row, registers = tokens
@@ -613,7 +576,6 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   }
   tc_fence_before();
   __syncthreads();
-  if (threadIdx.x == 0) BPD_TC_STAMP(9);
   if (warp == 1) {
     tc_fence_after();
     tmem_dealloc(tmem, ncols);

@@ -202,7 +202,7 @@ struct bpd_session {
   void* stack_layers;      // device: stack::LayerPtrs [n_dec]
   unsigned long long* stack_ws;   // device: per group [2][H][16][d] words (value, tag): the clusters' shares of the projection outputs
   unsigned* stack_bar;     // device: words of the device-wide join
-  int stack_cross_rows, stack_staged, stack_long, stack_minb, stack_lean, stack_dev, stack_groups, stack_group_seqs;
+  int stack_cross_rows, stack_staged, stack_minb, stack_lean, stack_dev, stack_groups, stack_group_seqs;
   int stack_layout[24];    // stack::Layout, kept opaque here
   std::map<GraphKey, GraphEntry> graphs;
   GraphEntry enc_graph;    // the encoder's launch sequence (fixed for a session), captured on its second use

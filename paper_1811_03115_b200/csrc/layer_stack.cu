@@ -16,13 +16,3 @@ const void* kernel_for(int nt, int d, int hct, int minb, int lean) {
 
 }  // namespace stack
 }  // namespace bpd
-
-#ifdef BPD_STACK_TRACE
-// Development builds only: where the persistent layer kernel (of this translation unit's d_model) writes its per-CTA step
-// timestamps (device memory, clusters * 8 * 256 unsigned 64-bit words), or null to stop.
-extern "C" int bpd_debug_set_stack_trace(void* dev_buffer) {
-  unsigned long long* ptr = static_cast<unsigned long long*>(dev_buffer);
-  BPD_CUDA(cudaMemcpyToSymbol(bpd::stack::g_stack_trace, &ptr, sizeof(ptr)));
-  return BPD_OK;
-}
-#endif

@@ -1,9 +1,9 @@
 // The whole decoder layer stack of a pass as ONE persistent kernel (sessions with at most 16 rows per pass).
 //
 // A pass over few rows is a chain of small dependent steps; what costs time is what separates them.  Here the
-// launch boundaries of the layer-by-layer path become device-wide counter joins, the residual stream never
-// leaves the chip between layers, and the weights of the next steps are already on their way into shared
-// memory (TMA, cp.async.bulk.tensor) while the current step computes.
+// launch boundaries of the layer-by-layer path become sums over words that say themselves when they are there, the
+// residual stream never leaves the chip between layers, and the weights of the next steps are already on their way
+// into shared memory (TMA, cp.async.bulk.tensor) while the current step computes.
 //
 // Work split.  One thread-block cluster of 8 CTAs per attention head (the same clusters take ff / H hidden units
 // of the feed-forward block).  Rank c of a cluster owns columns [c d/8, (c+1) d/8) of the residual stream x and
@@ -16,8 +16,8 @@
 //   feed-forward     the cluster's hidden units over this rank's columns -> exchange -> ReLU -> all ranks ->
 //                    the hidden units times slice c of the second projection -> workspace
 //
-// After each of the three blocks every CTA arrives on a device-wide counter, waits for all, and then adds the
-// H partial outputs of its own column slice in cluster order to its copy of x: every cluster holds the same x,
+// After each of the three blocks every CTA polls the H partial outputs of its own column slice (words that carry the
+// reduction's number, see ll_store) and adds them in cluster order to its copy of x: every cluster holds the same x,
 // computed by the same sums in the same order, so nothing has to be broadcast.  The layer norm that follows is
 // folded into the next projection (y = rstd (acc - mean s) + c); its row statistics are merged from the eight
 // slices in rank order.  All sums have an order that depends on neither the number of rows nor on timing.
@@ -33,7 +33,8 @@
 // waits on -- one transfer per destination instead of thousands of scalar remote stores, and no cluster-wide
 // barrier.  The smallest exchanges (single rows) go as 16-byte asynchronous stores (st.async) counted on the same
 // mbarriers.  Two mbarriers alternate between successive exchanges, so a fast sender's next exchange can never be
-// counted into the one a receiver is still waiting for.
+// counted into the one a receiver is still waiting for: in each exchange every rank sends something to every other, so
+// a rank that has passed one knows that all ranks have passed the one before and read what that brought.
 //
 // Every wait is bounded.  When one expires the CTA records an error, raises a device-wide flag and stops
 // waiting: it (and, through the flag, every other CTA) runs the remaining steps without waits, so that all
@@ -56,15 +57,15 @@ using fused::kMaxRows;
 constexpr int kThreads = 256;
 constexpr int kWarps = 8;
 constexpr int kNB = 16;                    // tiles resident or in flight at most (one mbarrier each)
-constexpr int kPumpThread = 32;            // the thread that requests tiles: not thread 0, which arrives on and polls the
-                                           // device-wide join and sends to rank 0, so the two work side by side
+constexpr int kPumpThread = 32;            // the thread that requests tiles: not in the first warp, whose threads announce an
+                                           // exchange and send it, so the two work side by side
 constexpr int kMaps = 8;
 enum MapKind { kMapQkv = 0, kMapWo = 1, kMapCq = 2, kMapCwo = 3, kMapW1 = 4, kMapW2 = 5, kMapCk = 6, kMapCv = 7 };
 constexpr int kMaxTiles = 16;              // tiles per layer at most
 constexpr int kState = 68;                 // floats per partial attention state: 64 outputs, maximum, weight sum, and
                                            // padding to a multiple of 16 bytes
 constexpr unsigned long long kSpin = 2000000000ull;   // about a second
-// words of the device-wide join
+// words that all CTAs share
 constexpr int kBarAbort = 1;               // non-zero: some wait expired, nobody waits any more
 constexpr int kBarBase = 32;               // reductions done so far in this session: the next launch's tags go on from here (never reset)
 constexpr int kBarWords = 64;
@@ -92,7 +93,7 @@ struct Layout {
 
 struct StackParams {
   const LayerPtrs* layers;                 // [L], device memory
-  int L, d, H, ff, R, rows_per_b, nb;
+  int L, R, rows_per_b, nb;
   int group_seqs;                          // LEAN = 4: sequences of a group (a group = a z slice of the grid, H clusters)
   float eps;
   // embedding of the block (Section 6's decoder input)
@@ -104,7 +105,6 @@ struct StackParams {
   float scale;
   int cross_rows, cross_split;             // encoder rows per CTA: all nb * max_src, or (split) rows rank * cross_rows ..
   int cross_staged;                        // 1: in a tile of the ring, 0: read from L2
-  int long_seq;                            // 1: sequences may exceed 256 keys (buffers of the shared-key schedule exist)
   // final layer norm -> planes for the head's first projection and the fp32 residual of the heads
   const bf16 *lnf_g, *lnf_b;
   bf16* xn_hi; long long xn_plane; float* h_f32;
@@ -185,9 +185,6 @@ struct Ctl {
   int no_row;                              // bytes that an exchange of rows brings from the ranks without a row
   int tok_b[2], tok_i[2], tok_at[2];       // this rank's tokens: sequence, place in the block, physical cache row of its key and value
   TileDesc tiles[kMaxTiles];
-#ifdef BPD_STACK_TRACE
-  long long cyc_wait, cyc_pump, cyc_poll;   // thread 0: cycles spent waiting for tiles, requesting tiles, polling the join
-#endif
 };
 
 struct Geo {                               // derived sizes, the same in every CTA
@@ -302,14 +299,8 @@ __device__ __forceinline__ void pump(const Cta& k, int stop_before = 0x7fffffff)
 }
 // One thread, after a barrier behind the last read of the tiles: release the n oldest tiles and refill the ring.
 __device__ __forceinline__ void release_tiles(const Cta& k, int n) {
-#ifdef BPD_STACK_TRACE
-  const long long t0 = clock64();
-#endif
   k.ctl->freed += n;
   pump(k);
-#ifdef BPD_STACK_TRACE
-  k.ctl->cyc_pump += clock64() - t0;
-#endif
 }
 
 __device__ __forceinline__ void raise_abort(const Cta& k, int code) {
@@ -322,16 +313,10 @@ __device__ __forceinline__ bool is_zombie(const Cta& k) { return *reinterpret_ca
 // All threads: wait until tile `seq` has landed; returns its shared-memory address.
 __device__ __forceinline__ uint32_t tile_wait(const Cta& k, int seq) {
   const int slot = seq & (kNB - 1);
-#ifdef BPD_STACK_TRACE
-  const long long t0 = clock64();
-#endif
   const uint32_t bar = tc::smem_u32(&k.ctl->full[slot]), phase = (uint32_t)(seq / kNB) & 1u;
   if (!tc::mbar_test(bar, phase) && !is_zombie(k)) {           // mostly there: the common case looks at nothing else
     if (!tc::mbar_wait(bar, phase, k.p->spin)) raise_abort(k, 105);
   }
-#ifdef BPD_STACK_TRACE
-  if (k.tid == 0) k.ctl->cyc_wait += clock64() - t0;
-#endif
   return k.ring + *reinterpret_cast<volatile int*>(&k.ctl->off[slot]);
 }
 
@@ -367,7 +352,7 @@ __device__ __forceinline__ void ll_load2(const unsigned long long* at, unsigned 
 // An item is V neighbouring columns of a row (four, or two where a rank has at most 64 columns: with four rows and eight heads
 // a quarter of the threads would have all the loads to do, sixteen each; us per pass with items of four / two, base model: block
 // of four rows 144.6 / 139.0, one row 135.7 / 128.5, five sentences 167.2 / 162.5, 1000 intensities 210.4 / 210.1).
-template <int V> struct Words { uint32_t w[2][V / 2]; };       // of a thread's (at most two) items: gains or bias values, fetched before the join
+template <int V> struct Words { uint32_t w[2][V / 2]; };       // of a thread's (at most two) items: gains or bias values, fetched before the reduction
 template <int V>
 __device__ __forceinline__ Words<V> load_words(const Cta& k, const bf16* v) {
   Words<V> o;
@@ -386,9 +371,9 @@ __device__ __forceinline__ Words<V> load_words(const Cta& k, const bf16* v) {
   }
   return o;
 }
-// After a join: x[t][col] += bias[col] + sum over the H clusters' partial outputs, in cluster order, for this
-// rank's columns.  Item = (row, V columns); rows are aligned to groups of lanes.  The loads of up to 16
-// partials are all in flight before the first is added.
+// x[t][col] += bias[col] + sum over the H clusters' partial outputs, in cluster order, for this rank's columns.
+// Item = (row, V columns); rows are aligned to groups of lanes.  The loads of eight producers are all in flight
+// before the first is added.
 template <int V>
 __device__ __forceinline__ void reduce_slice(const Cta& k, float* x_s, const unsigned long long* ws, const Words<V>& bias,
                                              unsigned tag, int nfree) {
@@ -540,9 +525,9 @@ static __global__ void tagged_wait_probe_kernel(int* error, unsigned long long l
 }
 
 // Planes (hi, lo) of x * gain for this rank's columns, and the slice's per-row (mean, sum of squared deviations)
-// into this rank's block of the statistics table (sent to the other ranks with the next exchange).  A thread
-// reads back the items it wrote itself in reduce_slice / the embedding (same idx -> thread mapping): no barrier
-// is needed in between.
+// into this rank's block of the statistics table (sent to the other ranks with the next exchange).  After a reduction a
+// thread reads back the items it wrote itself (the same idx -> thread mapping): no barrier is needed in between.  The
+// embedding writes items of four columns whatever V is; the cluster barrier behind it makes them visible.
 template <int NT, int V>
 __device__ __forceinline__ void planes_and_stats(const Cta& k, const float* x_s, const Words<V>& gain, uint8_t* xh, uint8_t* xl,
                                                  float* stats_mine) {
@@ -621,7 +606,8 @@ __device__ __forceinline__ void merge_stats(const Cta& k, const float* stats_in,
 // w + 8, ... of 8 positions in order, four lanes to a key: chunks of 32 with a lane to a key kept one or two of the eight
 // warps busy at the usual source lengths, each with a chain of 64 products.  The warps' states are merged in warp
 // order.  Threads c < kDH return output element c.  (Base model's layers: with this, one wait per panel and the constant sizes of
-// send_rows 146.9 -> 144.1 us per pass, five sentences 173.4 -> 166.2, 1000 intensities 213.2 -> 209.4; big model 306.4 / 306.7.)
+// send_rows 146.9 -> 144.1 us per pass, five sentences 173.4 -> 166.2, 1000 intensities 213.2 -> 209.4.  The big model's
+// 40 encoder rows gain nothing, 306.4 / 306.7; it has the form of the others.)
 // TILE = false: sources that are not staged; the rows come out of L2 (`rows`: the sequence's first key of this head, its value
 // d elements behind, 2 d elements between rows), the same arithmetic in the same order.
 template <bool TILE>
@@ -1057,16 +1043,6 @@ __device__ __forceinline__ void share_states(const Cta& k, int n, float* lvl2, u
   __syncthreads();
 }
 
-// ------------------------------------------------------------------ development trace
-#ifdef BPD_STACK_TRACE
-static __device__ unsigned long long* g_stack_trace = nullptr;
-constexpr int kTracePts = 256;
-#define BPD_TR() do { if (g_stack_trace && tid == 0 && tp < kTracePts - 4) { unsigned long long t_; asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t_)); \
-                        g_stack_trace[(size_t)(blockIdx.y * kC + c) * kTracePts + tp] = t_; } ++tp; } while (0)
-#else
-#define BPD_TR() do { } while (0)
-#endif
-
 // ------------------------------------------------------------------ the kernel
 // grid = (8, H), clusters of 8 along x.  All clusters must be resident at once (the host checks the occupancy).
 // MINB: CTAs per SM the kernel is compiled for.  Models with at most 15 heads have an SM to themselves per CTA (no
@@ -1091,7 +1067,7 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
   uint8_t* ssm = ssm_raw + ((1024u - (tc::smem_u32(ssm_raw) & 1023u)) & 1023u);
   cg::cluster_group cluster = cg::this_cluster();
   constexpr int RP = NT * 8, H = D / kDH, KS = D == 256 ? 2 : 4;      // steps of 16 columns per panel
-  constexpr int kPanels = D / kC <= 64 ? 1 : D / kC / 64;             // panels of a rank's columns
+  constexpr int kPanels = D / kC <= 64 ? 1 : D / kC / 64;             // panels of a rank's columns (Geo::P as a constant)
   constexpr int V = D == 1024 ? 4 : 2;                                // columns of an item, see Words
   constexpr bool kHoist = kPanels == 1;      // wait for a panel once, not once per row tile (two panels cost more registers than the waits)
   constexpr bool GROUPS = LEAN == 4;
@@ -1100,9 +1076,7 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
   k.p = &p;
   k.d = D; k.H = H;
   k.maps = &maps;
-  // Two parameters that only the variants which split the keys need are constants in the others: there they cost variant 1
-  // 24 bytes of spills and variant 4 28.  Medians over 15 placements of the buffers (where they lie in memory moves a pass
-  // by up to 3 us): headline pass 330.1 -> 329.2 us, five base sentences 203.6 -> 203.1, one greedy row 218.2 -> 218.4.
+  // two parameters that only the variants which split the keys need are constants in the others, which spill
   k.g = make_geo(D, H, HCT * H, p.L, (LEAN == 1 || GROUPS || p.cross_staged) ? p.cross_rows : 0, SPLIT ? p.cross_split : 0);
   k.sm = ssm;
   k.ctl = reinterpret_cast<Ctl*>(ssm + p.lay.misc);
@@ -1152,9 +1126,6 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
     tc::mbar_init(tc::smem_u32(&k.ctl->ex[1]), 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     k.ctl->head = 0; k.ctl->issued = 0; k.ctl->freed = 0; k.ctl->zombie = 0; k.ctl->issue_layer = 0; k.ctl->issue_idx = 0;
-#ifdef BPD_STACK_TRACE
-    k.ctl->cyc_wait = 0; k.ctl->cyc_pump = 0; k.ctl->cyc_poll = 0;
-#endif
   }
   if (tid < g.ntl) k.ctl->tiles[tid] = make_tile(g, tid, p.cross_rows, d, c, j, GROUPS ? (b0 + min(c / rpb, nb - 1)) * p.max_src : 0);
   __syncthreads();
@@ -1233,18 +1204,9 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
   const LongCtx lc = SPLIT ? long_ctx<KW>(k, ap, ssm, s_pt, s_len[0]) : LongCtx{};
   if (SPLIT) long_prefetch<KW>(k, lc, layers_s[0], 0);
 
-  unsigned nbar = 0;                        // joins passed so far in this launch
+  unsigned nbar = 0;                        // reductions done so far in this launch
   int seq = 0;                              // next tile to consume
   int xn = 0;                               // exchanges inside the cluster so far
-#ifdef BPD_STACK_TRACE
-  int tp = 0;
-  if (g_stack_trace && tid == 0) {
-    unsigned smid;
-    asm volatile("mov.u32 %0, %%smid;" : "=r"(smid));
-    g_stack_trace[(size_t)(blockIdx.y * kC + c) * kTracePts + kTracePts - 1] = smid;
-  }
-#endif
-  BPD_TR();
   // this lane's ldmatrix offsets: weight boxes (row lane % 16, second half of the step for lanes >= 16) and planes
   // (token lane % 8, second half for lanes 8-15 and 24-31; lanes >= 16 address the lo plane)
   const uint32_t a_lane_row = (uint32_t)(lane & 15), a_lane_half = (uint32_t)(lane >> 4) * 16;
@@ -1260,7 +1222,7 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
   for (int l = 0; l < p.L; ++l) {
     const LayerPtrs& LP = layers_s[l];
     // =================================================================== self-attention block
-    // static words first (gains, folded layer-norm vectors, bias): their latency hides behind the join
+    // static words first (gains, folded layer-norm vectors, bias): their latency hides behind the reduction
     Words<V> gw = load_words<V>(k, LP.g1);
     float fs = 0.f, fc = 0.f;
     if (tid < 3 * kDH) {
@@ -1271,10 +1233,8 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
     if (l > 0) {
       const Words<V> bw = load_words<V>(k, layers_s[l - 1].b2);
       ++nbar;
-      BPD_TR();
       if constexpr (H == 16) reduce_slice_2hop(k, x_s, ws_g + (size_t)((nbar - 1) & 1) * H * kMaxRows * d, gather_g + (size_t)((nbar - 1) & 1) * kMaxRows * d, bw, base + nbar, g.PH);
       else reduce_slice<V>(k, x_s, ws_g + (size_t)((nbar - 1) & 1) * H * kMaxRows * d, bw, base + nbar, g.PH);
-      BPD_TR();
       if (p.layer_dump && j == 0) {
         __syncthreads();
         for (int idx = tid; idx < R * ks; idx += kThreads)
@@ -1283,7 +1243,6 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
     }
     planes_and_stats<NT, V>(k, x_s, gw, xh, xl, stats_mine);
     __syncthreads();
-    BPD_TR();
     // Q, K, V of the head over this rank's columns; token t's partial goes to rank t % 8
     uint32_t wt[kPanels];
 #pragma unroll
@@ -1306,10 +1265,8 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
         }
     }
     seq += g.P;
-    BPD_TR();
     send_partials(k, xn, outbox, inbox, NT * 3 * kDH * 4, stats_in, g.P);
     ++xn;
-    BPD_TR();
     merge_stats(k, stats_in, s_mean, s_rstd);
     __syncthreads();
     // this rank's tokens: partials in rank order, layer norm; the row's key and value (rounded as the cache holds
@@ -1335,7 +1292,6 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
     }
     send_rows<NT, 512, false>(k, xn, kvq, nullptr, 0);  // every rank now holds the keys, values and queries of all block rows
     ++xn;
-    BPD_TR();
     {
       const bf16* Kc = LP.kcache;
       const bf16* Vc = LP.vcache;
@@ -1434,7 +1390,6 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
         __syncthreads();
       }
     }
-    BPD_TR();
     // this head's share of the output projection for feature slice c
     {
       unsigned long long* wsj = ws_g + ((size_t)(nbar & 1) * H + j) * kMaxRows * d;
@@ -1456,20 +1411,16 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
       }
       seq += 1;
     }
-    BPD_TR();
 
     // =================================================================== cross-attention block
     gw = load_words<V>(k, LP.g2);
     const Words<V> nobias = load_words<V>(k, nullptr);
     if (tid < kDH) { fs = LP.s_cq[j * kDH + tid]; fc = LP.c_cq[j * kDH + tid]; }
     ++nbar;
-    BPD_TR();
     if constexpr (H == 16) reduce_slice_2hop(k, x_s, ws_g + (size_t)((nbar - 1) & 1) * H * kMaxRows * d, gather_g + (size_t)((nbar - 1) & 1) * kMaxRows * d, nobias, base + nbar, 1);
       else reduce_slice<V>(k, x_s, ws_g + (size_t)((nbar - 1) & 1) * H * kMaxRows * d, nobias, base + nbar, 1);
-    BPD_TR();
     planes_and_stats<NT, V>(k, x_s, gw, xh, xl, stats_mine);
     __syncthreads();
-    BPD_TR();
     for (int mt = warp; mt < kDH / 16; mt += kWarps) {
       float acc[NT][4];
 #pragma unroll
@@ -1489,10 +1440,8 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
         }
     }
     seq += 1;
-    BPD_TR();
     send_partials(k, xn, outbox, inbox, NT * kDH * 4, stats_in, 1);
     ++xn;
-    BPD_TR();
     merge_stats(k, stats_in, s_mean, s_rstd);
     __syncthreads();
     {
@@ -1543,7 +1492,6 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
       send_rows<NT, 128, true>(k, xn, oh, ol, g.staged);
     }
     ++xn;
-    BPD_TR();
     {
       unsigned long long* wsj = ws_g + ((size_t)(nbar & 1) * H + j) * kMaxRows * d;
       const unsigned tag_out = base + nbar + 1;            // the reduction that consumes these shares
@@ -1564,7 +1512,6 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
       }
       seq += 1;
     }
-    BPD_TR();
 
     // =================================================================== feed-forward block
     gw = load_words<V>(k, LP.g3);
@@ -1577,13 +1524,10 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
       fc1[u] = idx < g.UPR * R ? LP.c_f1[unit] : 0.f;
     }
     ++nbar;
-    BPD_TR();
     if constexpr (H == 16) reduce_slice_2hop(k, x_s, ws_g + (size_t)((nbar - 1) & 1) * H * kMaxRows * d, gather_g + (size_t)((nbar - 1) & 1) * kMaxRows * d, nobias, base + nbar, 1);
       else reduce_slice<V>(k, x_s, ws_g + (size_t)((nbar - 1) & 1) * H * kMaxRows * d, nobias, base + nbar, 1);
-    BPD_TR();
     planes_and_stats<NT, V>(k, x_s, gw, xh, xl, stats_mine);
     __syncthreads();
-    BPD_TR();
     // the cluster's hidden units over this rank's columns; unit f belongs to rank f / UPR
 #pragma unroll
     for (int q = 0; q < kPanels; ++q) wt[q] = kHoist ? tile_wait(k, seq + q) : 0u;
@@ -1605,10 +1549,8 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
         }
     }
     seq += g.P;
-    BPD_TR();
     send_partials(k, xn, outbox, inbox, g.UPR * RP * 4, stats_in, g.P);
     ++xn;
-    BPD_TR();
     merge_stats(k, stats_in, s_mean, s_rstd);
     __syncthreads();
     // ranks in order, layer norm, bias, ReLU -> this rank's block of the hidden planes, which goes to every rank
@@ -1636,7 +1578,6 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
       xchg_wait(k, xn);
       ++xn;
     }
-    BPD_TR();
     // the hidden units times slice c of the second projection: this cluster's share of the block's output
     {
       unsigned long long* wsj = ws_g + ((size_t)(nbar & 1) * H + j) * kMaxRows * d;
@@ -1669,24 +1610,20 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
       }
       seq += g.PH;
     }
-    BPD_TR();
   }
   // =================================================================== final layer norm
   {
     const Words<V> bw = load_words<V>(k, layers_s[p.L - 1].b2), gw = load_words<V>(k, p.lnf_g);
     ++nbar;
-    BPD_TR();
     pdl_launch_dependents();
     if constexpr (H == 16) reduce_slice_2hop(k, x_s, ws_g + (size_t)((nbar - 1) & 1) * H * kMaxRows * d, gather_g + (size_t)((nbar - 1) & 1) * kMaxRows * d, bw, base + nbar, g.PH);
       else reduce_slice<V>(k, x_s, ws_g + (size_t)((nbar - 1) & 1) * H * kMaxRows * d, bw, base + nbar, g.PH);
-    BPD_TR();
     if (p.layer_dump && j == 0) {
       __syncthreads();
       for (int idx = tid; idx < R * ks; idx += kThreads)
         p.layer_dump[((size_t)(p.L - 1) * p.R + b0 * rpb + idx / ks) * d + c * ks + idx % ks] = x_s[idx];
     }
     planes_and_stats<NT, V>(k, x_s, gw, xh, xl, stats_mine);   // the planes are not used; the statistics are
-    BPD_TR();
   }
   fence_async_smem();
   __syncthreads();
@@ -1694,7 +1631,6 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
   if (tid < kC && tid != c) xchg_send(k, xn, tid, stats_mine, stats_mine, kMaxRows * 8u);
   xchg_wait(k, xn);
   ++xn;
-  BPD_TR();
   merge_stats(k, stats_in, s_mean, s_rstd);
   __syncthreads();
   if (j == 0) {
@@ -1719,12 +1655,6 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
     }
     if (c == 0 && tid == 0) p.bar[kBarBase + grp] = base + nbar;         // tags of the next launch go on from here
   }
-#ifdef BPD_STACK_TRACE
-  if (g_stack_trace && tid == 0) {
-    unsigned long long* tr = g_stack_trace + (size_t)(blockIdx.y * kC + c) * kTracePts;
-    tr[kTracePts - 2] = k.ctl->cyc_wait; tr[kTracePts - 3] = k.ctl->cyc_pump; tr[kTracePts - 4] = k.ctl->cyc_poll;
-  }
-#endif
   if (tid == kPumpThread && k.ctl->zombie) {
     // a wait expired somewhere: tiles may still be in flight; give each slot's last request a bounded chance to land
     for (int s2 = max(0, k.ctl->issued - kNB); s2 < k.ctl->issued; ++s2)
@@ -1741,22 +1671,24 @@ layer_stack_kernel(const __grid_constant__ StackMaps maps, const __grid_constant
 // (layer_stack.cu, layer_stack_512.cu, layer_stack_256.cu), compiled side by side.
 // There are those that a session can get on a B200.  4 or 8 clusters (d_model 256, 512) always have an SM to themselves per CTA,
 // and what does not fit a whole SM does not fit half a one; groups need two CTAs per SM.  16 clusters (d_model 1024) need
-// two (15 are resident at one), and half an SM has no room for two token tiles, which groups of 16 heads always have.
+// two (15 are resident at one), and half an SM has no room for two token tiles, which groups of 16 heads always have.  Nor
+// has it for those of 8 heads with 256 hidden units.
 const void* kernel_for(int nt, int d, int hct, int minb, int lean);
 template <int D> const void* kernel_of(int nt, int hct, int minb, int lean);
-#define BPD_STACK_V(D, NT, MB, LN) \
-  if (nt == NT && hct == 128 && minb == MB && lean == LN) return reinterpret_cast<const void*>(layer_stack_kernel<NT, D, 128, MB, LN>); \
-  if (nt == NT && hct == 256 && minb == MB && lean == LN) return reinterpret_cast<const void*>(layer_stack_kernel<NT, D, 256, MB, LN>)
-#define BPD_STACK_KERNELS(D) \
+#define BPD_STACK_V(D, HCT, NT, MB, LN) \
+  if (nt == NT && hct == HCT && minb == MB && lean == LN) return reinterpret_cast<const void*>(layer_stack_kernel<NT, D, HCT, MB, LN>);
+#define BPD_STACK_VV(D, NT, MB, LN) BPD_STACK_V(D, 128, NT, MB, LN) BPD_STACK_V(D, 256, NT, MB, LN)
+// MORE: further variants
+#define BPD_STACK_KERNELS(D, MORE) \
   template <> const void* kernel_of<D>(int nt, int hct, int minb, int lean) { \
-    BPD_STACK_V(D, 1, 1, 0); BPD_STACK_V(D, 2, 1, 0); BPD_STACK_V(D, 1, 1, 1); BPD_STACK_V(D, 2, 1, 1); \
-    BPD_STACK_V(D, 1, 1, 2); BPD_STACK_V(D, 2, 1, 2); BPD_STACK_V(D, 1, 1, 3); BPD_STACK_V(D, 2, 1, 3); \
-    BPD_STACK_V(D, 1, 2, 4); BPD_STACK_V(D, 2, 2, 4); \
+    BPD_STACK_VV(D, 1, 1, 0) BPD_STACK_VV(D, 2, 1, 0) BPD_STACK_VV(D, 1, 1, 1) BPD_STACK_VV(D, 2, 1, 1) \
+    BPD_STACK_VV(D, 1, 1, 2) BPD_STACK_VV(D, 2, 1, 2) BPD_STACK_VV(D, 1, 1, 3) BPD_STACK_VV(D, 2, 1, 3) \
+    BPD_STACK_VV(D, 1, 2, 4) BPD_STACK_V(D, 128, 2, 2, 4) MORE \
     return nullptr; \
   }
 #define BPD_STACK_KERNELS_HALF_SM(D) \
   template <> const void* kernel_of<D>(int nt, int hct, int minb, int lean) { \
-    BPD_STACK_V(D, 1, 2, 0); BPD_STACK_V(D, 1, 2, 1); \
+    BPD_STACK_VV(D, 1, 2, 0) BPD_STACK_VV(D, 1, 2, 1) \
     return nullptr; \
   }
 

@@ -5,7 +5,7 @@
 namespace bpd {
 namespace stack {
 
-BPD_STACK_KERNELS(512)
+BPD_STACK_KERNELS(512, )
 
 }  // namespace stack
 }  // namespace bpd

@@ -270,9 +270,6 @@ int launch(const Operands& op, int N, int K, int T, TcParams p, const Scratch& s
   if (rc) return rc;
   p.T = T; p.N = N; p.K = K; p.bn = bn;
   p.splits = wide ? wp.splits : pl.splits; p.chunks_per_split = wide ? wp.chunks_per_split : pl.chunks_per_split;
-#ifdef BPD_TC_TRACE
-  { static int next_trace_id = 0; p.trace_id = next_trace_id++ & 127; }
-#endif
   p.ws = sc.ws; p.tile_counters = sc.tile_counters; p.done_counter = sc.done_counter;
   p.best = sc.best; p.error = sc.error; p.error_on_host = sc.error_on_host;
   p.stream_weights = ((!wide || wp.ttiles == 1) && sc.l2_hints) ? 1 : 0;
