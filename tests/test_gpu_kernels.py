@@ -195,33 +195,93 @@ def test_fp32_paths_keep_their_precision(bpd, batch, k, heads, max_src, tgt, opt
 
 
 # Cross-attention of the persistent kernel takes the encoder's rows in chunks of 8, one per warp: one row, a chunk's edges and
-# the edges of a second round of the eight warps.  Tolerance as above (fp32 throughout, the same roundings on the way).
-@pytest.mark.parametrize("heads", [4, 8])
-def test_source_lengths_around_a_chunk_of_encoder_rows(bpd, heads):
+# the edges of a second round of the eight warps; rows staged for groups of sequences, for all sequences (as many as fit), and
+# read out of L2; one CTA per SM and two (16 heads).  Tolerance as above (fp32 throughout, the same roundings on the way).
+UNSTAGED = {"persistent_layers": 1, "stage_encoder_rows": 0}
+
+
+@pytest.mark.parametrize("heads,lens,options", [
+    (4, (1, 7, 8, 9, 63, 64, 65, 72), {}), (8, (1, 7, 8, 9, 63, 64, 65, 72), {}),
+    (4, (63, 64, 72), {}), (8, (1, 7, 8, 9), {}), (8, (63, 64, 65), {}), (16, (1, 7, 8, 9), {}), (16, (63,), {}), (16, (64,), {}),
+    (4, (1, 7, 8, 9, 63, 64, 65, 72), UNSTAGED), (8, (1, 7, 8, 9, 63, 64, 65, 72), UNSTAGED),
+    (16, (1, 7, 8, 9), UNSTAGED), (16, (63, 64, 65, 72), UNSTAGED)])
+def test_source_lengths_around_a_chunk_of_encoder_rows(bpd, heads, lens, options):
     from bpd_inputs import ModelConfig, make_weights
     from bpd_inputs.blob import blob_layout
     from oracle.decode import TransformerScorer
     from oracle.model import parse_blob
-    lens = np.array([1, 7, 8, 9, 63, 64, 65, 72], np.int32)
     cfg = ModelConfig(2, 2, 64 * heads, heads, 128 * heads, 300, 2, 64)
     blob = make_weights(cfg, 5, 0.06)
     for name, shape, _, off, nbytes in blob_layout(cfg)[0]:
         if name.endswith("self.wo"):
             blob[off:off + nbytes] = 0
-    src = np.random.default_rng(heads).integers(2, 300, (8, 72)).astype(np.int32)
+    src = np.random.default_rng(heads).integers(2, 300, (len(lens), max(lens))).astype(np.int32)
     model = bpd.Model(blob)
-    s = bpd.Session(model, 8, 72, 20)
+    s = bpd.Session(model, len(lens), max(lens), 20, options=options)
     assert s.layer_path == 2
-    s.bpd_encode(src, lens)
+    s.bpd_encode(src, np.array(lens, np.int32))
     r = s.bpd_iteration(2, 20, want_hidden=True)
     model_o = parse_blob(blob)
-    for b in range(8):
-        scorer = TransformerScorer(model_o, src[b], int(lens[b]), cached=True, capacity=24)
+    for b in range(len(lens)):
+        scorer = TransformerScorer(model_o, src[b], lens[b], cached=True, capacity=24)
         scorer([0], 1)
         scorer([0] + [int(t) for t in r["block"][b]], 2)
         np.testing.assert_allclose(r["hidden"][b].cpu().numpy(), scorer.last_hidden, atol=1e-4)
     s.close()
     model.close()
+
+
+# Every instantiation of the persistent kernel: width, hidden units per cluster, variant, token tiles.  First with the
+# self-attention's output projections at zero, tolerance as above; then whole, over several blocks: a cached key or value is
+# off by 2^-9 of itself.  Weights of 0.06 sqrt(256 / d) keep products at 0.96 of their input at every width, hence scores and
+# attention outputs at a standard deviation of 0.9; a score is then off by 0.9 * 2^-9 and so is a weight, a value by 2^-9, an
+# output by 0.9 * 1.9 * 2^-9 = 3.4e-3, and two layers add up to 6.7e-3.  (At 0.06 the 1024-wide model's scores have a
+# deviation of 3.7: four times as much in the scores, four times in the outputs.)
+@pytest.mark.parametrize("units", [128, 256])
+@pytest.mark.parametrize("heads,batch,k,max_src,tgt,options", [
+    (heads, *case) for heads in (4, 8) for case in [
+        (2, 3, 20, 20, UNSTAGED), (3, 4, 20, 20, UNSTAGED), (2, 3, 20, 300, UNSTAGED), (2, 7, 20, 300, UNSTAGED),     # general, short and long
+        (2, 4, 20, 20, {}), (2, 8, 112, 20, {}),                            # short; too many encoder rows for groups
+        (1, 4, 20, 600, {}), (1, 10, 20, 600, {}), (1, 4, 20, 20, {}), (1, 10, 20, 20, {}),      # one long, one short sequence
+        (5, 3, 20, 20, {}), (3, 10, 20, 20, {})]                            # groups
+] + [(16, 2, 4, 20, 20, UNSTAGED), (16, 1, 2, 20, 300, {"persistent_layers": 1}), (16, 4, 2, 9, 20, {})])
+def test_every_shape_of_the_persistent_kernel_scores_like_the_oracle(bpd, heads, batch, k, max_src, tgt, options, units):
+    from bpd_inputs import ModelConfig, make_weights
+    from bpd_inputs.blob import blob_layout
+    from oracle.decode import TransformerScorer
+    from oracle.model import parse_blob
+    cfg = ModelConfig(1, 2, 64 * heads, heads, units * heads, 300, k, 64)
+    rng = np.random.default_rng(batch * k)
+    lens = rng.integers(1, max_src + 1, batch).astype(np.int32)
+    lens[-1] = max_src
+    src = rng.integers(2, 300, (batch, max_src)).astype(np.int32)
+    blob = make_weights(cfg, 5, 0.06 * (4 / heads) ** 0.5)
+    kept = blob.copy()
+    for name, shape, _, off, nbytes in blob_layout(cfg)[0]:
+        if name.endswith("self.wo"):
+            blob[off:off + nbytes] = 0
+    for weights, blocks, atol in ((blob, 1, 1e-4), (kept, 3, 8e-3)):
+        model = bpd.Model(weights)
+        s = bpd.Session(model, batch, max_src, tgt, options=options)
+        no_room = units == 256 and (heads, batch, k, tgt) in ((8, 3, 10, 20), (16, 1, 2, 300))
+        assert (s.layer_path == 2) != no_room
+        s.bpd_encode(src, lens)
+        model_o, rows = parse_blob(weights), sorted({0, batch - 1})
+        scorers = {b: TransformerScorer(model_o, src[b], int(lens[b]), cached=True, capacity=tgt + k + 2) for b in rows}
+        inputs = {b: [0] for b in rows}
+        for b in rows:
+            scorers[b](inputs[b], 1)
+        for _ in range(blocks):
+            r = s.bpd_iteration(k, tgt, want_hidden=True, accept_mode=k << 16)      # minimum block k: every proposal is kept
+            for b in rows:
+                block = [int(t) for t in r["block"][b]]
+                scorers[b](inputs[b] + block, k)
+                np.testing.assert_allclose(r["hidden"][b].cpu().numpy(), scorers[b].last_hidden, atol=atol)
+                inputs[b] += block[:int(r["khat"][b])]
+            if len(inputs[0]) > tgt:
+                break
+        s.close()
+        model.close()
 
 
 # the persistent layer kernel with groups of sequences: a last group that is full and one that is not, two sequences per
