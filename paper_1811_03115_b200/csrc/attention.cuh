@@ -289,7 +289,8 @@ __global__ void __launch_bounds__(kThreads, 3) attention_mma_kernel(const __grid
 //   up to 140 keys             487/500   357/352   405/375   372/353   417/378   374/332   367/351   490/401   350/312
 //   48 items of 8 rows over 450 / 600 / 1200 / 2400 keys: 431/393, 444/402, 492/459, 568/560 (this one for the encoder's
 //   rows and the row kernels for the cache: 542); 72 of 8 over 600: 575/407; 80 of 4 over 1200: 685/423
-// So the line is on the careful side: of these only 48 items of 4 rows lose with this kernel, and 64 to 73 items win.
+// By this table the line belongs at 64 items and, for 6 rows and more, at 48: of these only 48 items of 4 rows lose with this
+// kernel.  It has not been moved there yet.
 inline bool applies(const AttnParams& a, int max_keys, int block) {
   const int items = (a.rows / a.rows_per_b) * a.H * ((block + kRows - 1) / kRows);
   return a.dh == 64 && (items >= 74 || (block >= kRows / 2 && max_keys <= 512));

@@ -184,7 +184,8 @@ static bool stack_shapes_ok(const Config& c, int rows) {
 // two token tiles takes the pass whole, and models of 16 heads the cluster launches; us per pass, whole / in groups:
 //   8 heads   3 x 3 rows 211/190   2 x 5 210/195   2 x 8 231/207   4 x 4 225/199   8 x 2 223/197
 //   16 heads  2 x 5 383/232   3 x 4 421/233   2 x 8 465/262   4 x 4 446/248   8 x 2 450/245
-// So 16 heads could take groups from 9 rows on as well; the rule does not do it yet.  0: no groups.
+// So 16 heads could take groups from 9 rows on as well; the rule does not do it yet, nor is the groups' variant with one token
+// tile instantiated for them.  0: no groups.
 static int stack_groups(const Config& c, int B, int* seqs) {
   *seqs = std::max(1, 8 / c.k_model);
   const int groups = ceil_div(B, *seqs);
